@@ -136,10 +136,9 @@ struct MemberArgs {
     int32_t M;             // tokens of this member
 };
 
-// Forward / backward-input for `count` weights of one shape in one launch (count == 1: the plain calls).  The members
-// may have different token counts (several adapters on one weight: one member per token group).
-lowra_status run_members(bool backward, const MemberArgs* mem, int count, int32_t r, float s, void* workspace,
-                         size_t workspace_bytes, void* stream_v, bool stream_k = true) {
+// Checks the arguments of a fused call for `count` weights of one shape.
+lowra_status check_members(const MemberArgs* mem, int count, int32_t r, const void* workspace, size_t workspace_bytes,
+                           bool stream_k) {
     if (count < 1 || count > kMaxBatch) return LOWRA_ERR_SHAPE;
     for (int i = 0; i < count; ++i) {
         lowra_status st = check_layout(mem[i].layout);
@@ -150,12 +149,11 @@ lowra_status run_members(bool backward, const MemberArgs* mem, int count, int32_
     const int N = mem[0].layout->N, K = mem[0].layout->K;
     if (!rank_ok(r) || N % 8 != 0 || N > 64 * kMaxGroups64 || (uint64_t)N * (uint64_t)(K / 64) >= (1ull << 32))
         return LOWRA_ERR_SHAPE;
-    int Ms[kMaxBatch], M = 0;
+    int Ms[kMaxBatch];
     for (int i = 0; i < count; ++i) {
         const MemberArgs& m = mem[i];
         if (m.M < 1) return LOWRA_ERR_SHAPE;
         Ms[i] = m.M;
-        M = m.M > M ? m.M : M;
         if (m.layout->N != N || m.layout->K != K) return LOWRA_ERR_SHAPE;                 // one shape per launch
         if (count > 1 && m.layout->deal_dev == nullptr) return LOWRA_ERR_NULL;            // a batch has no prologue launch
         if (!aligned16(m.packed) || !aligned16(m.absmax) || !aligned16(m.maps) || !aligned16(m.act) || !aligned16(m.A) ||
@@ -164,13 +162,37 @@ lowra_status run_members(bool backward, const MemberArgs* mem, int count, int32_
     }
     const Workspace w = plan_workspace(N, K, Ms, count, r, stream_k);
     if (workspace_bytes < w.total || (reinterpret_cast<uintptr_t>(workspace) & 255u) != 0) return LOWRA_ERR_WORKSPACE;
-    lowra_status st = check_device();
+    return check_device();
+}
+
+lowra_status run_small(const MemberArgs* mem, uint16_t* const* T_of, int count, int32_t r, float s, void* workspace, cudaStream_t stream);
+// The diagnostic lowra_diag_drop_t_flags is about flags, which the path for few tokens has none of: it leaves that path out.
+bool takes_small_path(bool backward, int M) { return !backward && M <= kSmallTokens && g_drop_t_flags.load(std::memory_order_relaxed) == 0; }
+
+// Forward / backward-input for `count` weights of one shape in one launch (count == 1: the plain calls).  The members
+// may have different token counts (several adapters on one weight: one member per token group).
+lowra_status run_members(bool backward, const MemberArgs* mem, int count, int32_t r, float s, void* workspace,
+                         size_t workspace_bytes, void* stream_v, bool stream_k = true) {
+    lowra_status st = check_members(mem, count, r, workspace, workspace_bytes, stream_k);
     if (st != LOWRA_OK) return st;
+    const int N = mem[0].layout->N, K = mem[0].layout->K;
+    int Ms[kMaxBatch], M = 0;
+    for (int i = 0; i < count; ++i) {
+        Ms[i] = mem[i].M;
+        M = Ms[i] > M ? Ms[i] : M;
+    }
+    const Workspace w = plan_workspace(N, K, Ms, count, r, stream_k);
     cudaStream_t stream = (cudaStream_t)stream_v;
 
     unsigned char* ws = static_cast<unsigned char*>(workspace);
     uint32_t* status = reinterpret_cast<uint32_t*>(ws);
     uint32_t* flags = reinterpret_cast<uint32_t*>(ws + w.off_flags);
+
+    if (takes_small_path(backward, M)) {   // (M: the largest member's tokens)
+        uint16_t* T_of[kMaxBatch];
+        for (int i = 0; i < count; ++i) T_of[i] = reinterpret_cast<uint16_t*>(ws + w.off_T[i]);
+        return run_small(mem, T_of, count, r, s, workspace, stream);
+    }
 
     GemmParams G;
     memset(&G, 0, sizeof(G));
@@ -267,6 +289,30 @@ lowra_status run_members(bool backward, const MemberArgs* mem, int count, int32_
         }
     }
     return launch_fused(backward ? kModeBackward : kModeForward, G, TM, stream);
+}
+
+// Forward pass of members of few tokens each (any number of them, one shape): two launches for every kSmallMembers.
+// Their arguments have been checked as run_members does.  T_of: where member i's down-projected tokens go.
+lowra_status run_small(const MemberArgs* mem, uint16_t* const* T_of, int count, int32_t r, float s, void* workspace, cudaStream_t stream) {
+    SmallParams P;
+    memset(&P, 0, sizeof(P));
+    P.N = mem[0].layout->N;
+    P.K = mem[0].layout->K;
+    P.r = r;
+    P.rp = (r + 63) / 64 * 64;
+    P.s = s;
+    P.status = static_cast<uint32_t*>(workspace);
+    for (int first = 0; first < count; first += kSmallMembers) {
+        P.count = count - first < kSmallMembers ? count - first : kSmallMembers;
+        P.clear_status = first == 0 && mem[0].layout->deal_dev == nullptr;
+        for (int i = 0; i < P.count; ++i) {
+            const MemberArgs& m = mem[first + i];
+            P.m[i] = SmallMember{make_row_layout(m.layout), m.packed, m.absmax, m.maps, m.act, m.A, m.B, m.out, T_of[first + i], m.M};
+        }
+        const lowra_status st = launch_small(P, stream);
+        if (st != LOWRA_OK) return st;
+    }
+    return LOWRA_OK;
 }
 
 lowra_status run_lora(bool backward, const lowra_layout* layout, const uint8_t* packed, const float* absmax,
@@ -421,14 +467,34 @@ extern "C" lowra_status lowra_lora_forward_adapters(const lowra_layout* layout, 
     // every group is a launch of its own.
     const bool together = layout->deal_dev != nullptr &&
                           workspace_bytes >= plan_workspace(layout->N, layout->K, M, r, true, kMaxBatch).total;
-    MemberArgs mem[kMaxBatch];
-    int n = 0;
+    // Groups of few tokens take the path for those, all of them together and first; their T lies where the tokens' own
+    // rows lie in the T of a call for all M tokens.
+    auto member = [&](int a) {
+        const int m0 = group_start_host[a];
+        return MemberArgs{layout, packed_dev, absmax_dev, maps_dev + (size_t)a * N * kTableStride, X_dev + (size_t)m0 * K,
+                          A_dev + (size_t)a * K * (size_t)r, B_dev + (size_t)a * (size_t)r * N, Y_dev + (size_t)m0 * N,
+                          group_start_host[a + 1] - m0};
+    };
+    auto is_small = [&](int a) { return takes_small_path(false, group_start_host[a + 1] - group_start_host[a]); };
+    MemberArgs mem[kMaxBatch], few[kSmallMembers];
+    uint16_t* few_T[kSmallMembers];
+    int n = 0, n_few = 0;
+    for (int a = 0; a <= n_adapters; ++a) {
+        if (a < n_adapters && group_start_host[a + 1] > group_start_host[a] && is_small(a)) {
+            if (n_few == 0 && (st = check_members(&(few[0] = member(a)), 1, r, workspace_dev, workspace_bytes, true)) != LOWRA_OK) return st;
+            few_T[n_few] = reinterpret_cast<uint16_t*>(static_cast<unsigned char*>(workspace_dev) + kStatusBytes) +
+                           (size_t)group_start_host[a] * (size_t)((r + 63) / 64 * 64);
+            few[n_few++] = member(a);
+        }
+        if (n_few > 0 && (a == n_adapters || n_few == kSmallMembers)) {
+            if ((st = run_small(few, few_T, n_few, r, s, workspace_dev, (cudaStream_t)stream)) != LOWRA_OK) return st;
+            n_few = 0;
+        }
+    }
     for (int a = 0; a <= n_adapters; ++a) {
         if (a < n_adapters) {
-            const int m0 = group_start_host[a], m = group_start_host[a + 1] - m0;
-            if (m == 0) continue;
-            mem[n++] = MemberArgs{layout, packed_dev, absmax_dev, maps_dev + (size_t)a * N * kTableStride, X_dev + (size_t)m0 * K,
-                                  A_dev + (size_t)a * K * (size_t)r, B_dev + (size_t)a * (size_t)r * N, Y_dev + (size_t)m0 * N, m};
+            if (group_start_host[a + 1] == group_start_host[a] || is_small(a)) continue;
+            mem[n++] = member(a);
         }
         if (n > 0 && (a == n_adapters || n == (together ? kMaxBatch : 1))) {
             st = run_members(false, mem, n, r, s, workspace_dev, workspace_bytes, stream);

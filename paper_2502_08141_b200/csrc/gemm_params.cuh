@@ -153,6 +153,27 @@ static_assert(kGemmSmemBytes <= 232448, "227 KB of shared memory per CTA");
 
 lowra_status launch_fused(int mode, const GemmParams& G, const BatchMaps& TM, cudaStream_t stream);
 
+// ---- forward pass for few tokens (gemm_small.cu) --------------------------------------------
+constexpr int kSmallTokens = 64;    // members of up to so many tokens take it
+constexpr int kSmallMembers = 8;    // per launch
+struct SmallMember {
+    RowLayout L;
+    const uint8_t* packed;
+    const float* absmax;
+    const float* maps;
+    const uint16_t *X, *A, *B;
+    uint16_t *Y, *T;          // T [M, rp]: s X A, as the fused calls leave it
+    int M;
+};
+struct SmallParams {
+    SmallMember m[kSmallMembers];
+    int count, N, K, r, rp;
+    float s;
+    uint32_t* status;
+    int clear_status;         // the call brings no deal: its status word starts from zero
+};
+lowra_status launch_small(const SmallParams& P, cudaStream_t stream);
+
 // One skinny product D [R, rp] = P . Q (see gemm_grad.cu), written in bf16 as out [R, ld_out] or, transposed,
 // as out [n_cols, ld_out].
 struct SkinnyArgs {

@@ -1,0 +1,486 @@
+// Forward pass for few tokens (generation, short prompts, small token groups of several adapters):
+//     Y = X . deq(Wq)^T + s * (X . A) . B
+// With a handful of tokens the work is reading the weight's codes once (1 - 2 bits per weight), a few microseconds of memory
+// time: what counts is how many SMs share it and how long the longest chain of dependent steps is.  The persistent
+// tensor-core kernel (gemm_fused.cu) gives a 256-token tile 128 channels and the whole contraction: 32 clusters busy on
+// a 4096 x 4096 weight, 64 stages in series, 50 us.  Here two launches share the work finely instead:
+//   project_kernel   T = bf16(s X A): a CTA per 16 tokens and slice of the contraction, the slices of a cluster added up
+//                    through distributed shared memory.
+//   small_kernel     a CTA takes 64 stored rows of one precision and a slice of the contraction, its warps 16 rows and half
+//                    of that slice each.  The weights never leave the registers: in a block of 256 input features lane
+//                    (g, t) of a warp holds the 64-element absmax block t of the rows g and g + 8 - one wide load of codes,
+//                    one absmax - and dequantises it straight into the A fragments of mma.m16n8k16.  The order in which the
+//                    contraction indices are fed is free as long as both operands agree, so lane t's fragments are
+//                    simply its own next four elements, for the weights and for the tokens alike.  The tokens of the slice
+//                    lie in shared memory.  Slices are added up as above; the low-rank term enters as further steps of
+//                    the same accumulation.
+// It starts while project_kernel runs and waits for it only before the low-rank term (programmatic dependent launch).
+// No flags, no waits that need a limit, any number of such calls may share the GPU.
+#include "gemm_params.cuh"
+#include "ptx.cuh"
+
+namespace lowra {
+
+namespace {
+
+constexpr int kSmallThreads = 256;
+constexpr int kSmallRows = 64;          // stored rows per CTA
+constexpr int kSmallSpan = 256;         // contraction indices per step of a warp: one absmax block for each of four lanes
+constexpr int kPartPitch = kSmallRows + 4;   // fp32 words: neighbouring tokens of a partial tile 4 banks apart
+
+struct Unit { int member, m0; };        // up to 8 NT8 tokens of one member
+__device__ __forceinline__ Unit unit_at(const SmallParams& P, int u, int tokens) {
+    Unit r = {0, 0};
+    for (int i = 0; i + 1 < P.count; ++i) {
+        const int n = (P.m[i].M + tokens - 1) / tokens;
+        if (u < n) break;
+        u -= n;
+        r.member = i + 1;
+    }
+    r.m0 = u * tokens;
+    return r;
+}
+
+__device__ __forceinline__ void mma_bf16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+                 : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void cp_async_16_zfill(uint32_t saddr, const void* gptr, bool valid) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(saddr), "l"(gptr), "r"(valid ? 16u : 0u) : "memory");
+}
+__device__ __forceinline__ uint4 ld_shared_v4(uint32_t saddr) {
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(saddr) : "memory");
+    return v;
+}
+__device__ __forceinline__ float ld_cluster_f32(uint32_t caddr) {
+    float v;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(caddr) : "memory");
+    return v;
+}
+
+// ------------------------------------------------------------------------------------------------ T = bf16(s X A)
+constexpr int kProjectBatch = 4;        // steps of 16 contraction indices a warp fetches at a time
+
+// Grid: (slices of the contraction = cluster, tiles of 16 tokens of all members).
+__global__ void __launch_bounds__(kSmallThreads) project_kernel(const __grid_constant__ SmallParams P) {
+    extern __shared__ __align__(16) unsigned char project_smem[];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // the next kernel reads its operands right away, so it may start only now that everything before this kernel is complete
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (P.clear_status && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *P.status = 0u;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const int slices = (int)gridDim.x, slice = (int)blockIdx.x;
+    const Unit un = unit_at(P, (int)blockIdx.y, 16);
+    const SmallMember& W = P.m[un.member];
+    const int n_steps = P.K / 16;
+    const int s0 = (int)((long long)slice * n_steps / slices), s1 = (int)((long long)(slice + 1) * n_steps / slices);
+    const int pitch = P.r * 2 + 16;                                   // bytes per contraction index of A in shared memory
+    unsigned char* mine = project_smem + (size_t)warp * (kProjectBatch * 16 * pitch);
+    const int n_j8 = P.r / 8;
+    float acc[16][4];
+#pragma unroll
+    for (int j = 0; j < 16; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.0f;
+    const int row0 = un.m0 + g, row1 = row0 + 8;
+    const uint32_t* x0 = reinterpret_cast<const uint32_t*>(W.X + (size_t)row0 * P.K) + t;
+    const uint32_t* x1 = reinterpret_cast<const uint32_t*>(W.X + (size_t)row1 * P.K) + t;
+    const bool v0 = row0 < W.M, v1 = row1 < W.M;
+    constexpr int kWarps = kSmallThreads / 32;
+    for (int first = s0 + warp; first < s1; first += kWarps * kProjectBatch) {
+        uint32_t xa[kProjectBatch][4];
+        __syncwarp();   // the previous batch has been read
+#pragma unroll
+        for (int u = 0; u < kProjectBatch; ++u) {
+            const int st = first + u * kWarps;
+            xa[u][0] = xa[u][1] = xa[u][2] = xa[u][3] = 0u;
+            if (st < s1) {
+                for (int c = lane; c < 16 * n_j8; c += 32) {
+                    const int k = c / n_j8, j = c - k * n_j8;
+                    cp_async_16_zfill(ptx::smem_u32(mine + (u * 16 + k) * pitch + j * 16), W.A + (size_t)(st * 16 + k) * P.r + j * 8, true);
+                }
+                if (v0) { xa[u][0] = __ldg(x0 + st * 8); xa[u][2] = __ldg(x0 + st * 8 + 4); }
+                if (v1) { xa[u][1] = __ldg(x1 + st * 8); xa[u][3] = __ldg(x1 + st * 8 + 4); }
+            }
+        }
+        ptx::cp_async_commit();
+        ptx::cp_async_wait<0>();
+        __syncwarp();
+#pragma unroll
+        for (int u = 0; u < kProjectBatch; ++u) {
+            if (first + u * kWarps >= s1) break;
+            const uint32_t a_row = ptx::smem_u32(mine + (u * 16 + (lane & 15)) * pitch + (lane >> 4) * 16);
+#pragma unroll
+            for (int j = 0; j < 16; j += 2) {
+                if (j >= n_j8) break;
+                uint32_t b0, b1, b2, b3;
+                asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                             : "=r"(b0), "=r"(b1), "=r"(b2), "=r"(b3) : "r"(a_row + (uint32_t)j * 16u) : "memory");
+                mma_bf16(acc[j], xa[u][0], xa[u][1], xa[u][2], xa[u][3], b0, b1);
+                mma_bf16(acc[j + 1], xa[u][0], xa[u][1], xa[u][2], xa[u][3], b2, b3);
+            }
+        }
+    }
+    // the warps' sums, then the CTA's, then the cluster's, each in a fixed order
+    __syncthreads();
+    float* red = reinterpret_cast<float*>(project_smem);              // [warps][16 tokens][r]
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+        if (j >= n_j8) break;
+        float* d = red + (warp * 16 + g) * P.r + j * 8 + 2 * t;
+        d[0] = acc[j][0]; d[1] = acc[j][1];
+        d[8 * P.r] = acc[j][2]; d[8 * P.r + 1] = acc[j][3];
+    }
+    __syncthreads();
+    float* part = red + kWarps * 16 * P.r;                            // [16][r]
+    for (int i = threadIdx.x; i < 16 * P.r; i += kSmallThreads) {
+        float sum = 0.0f;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) sum += red[w * 16 * P.r + i];
+        part[i] = sum;
+    }
+    ptx::cluster_sync();
+    const uint32_t part_addr = ptx::smem_u32(part);
+    // pairs of neighbouring ranks; columns between the rank and its padded width are zero
+    for (int i = slice * kSmallThreads + (int)threadIdx.x; i < 16 * P.rp / 2; i += slices * kSmallThreads) {
+        const int row = i / (P.rp / 2), col = (i - row * (P.rp / 2)) * 2;
+        if (un.m0 + row >= W.M) continue;
+        float a = 0.0f, b = 0.0f;
+        if (col < P.r) {
+            for (int c = 0; c < slices; ++c) {
+                const uint32_t addr = ptx::map_to_cta(part_addr + (uint32_t)(row * P.r + col) * 4u, (uint32_t)c);
+                a += ld_cluster_f32(addr);
+                b += ld_cluster_f32(addr + 4u);
+            }
+        }
+        *reinterpret_cast<uint32_t*>(W.T + (size_t)(un.m0 + row) * P.rp + col) = pack_bf16x2(P.s * a, P.s * b);
+    }
+    ptx::cluster_sync();   // nobody leaves while a peer still reads its sums
+}
+
+// ------------------------------------------------------------------------------------------------ the product
+// What a lane fetches of one row for one step: the codes of a 64-element block (8, 16 or 32 bytes) and its absmax.
+template <int B>
+struct Codes {
+    uint32_t w[2 * B];
+    float a;
+};
+template <int B>
+__device__ __forceinline__ void fetch_codes(Codes<B>& c, const uint8_t* row, const float* absmax, int blk, bool valid) {
+    if (!valid) {
+#pragma unroll
+        for (int i = 0; i < 2 * B; ++i) c.w[i] = 0u;
+        c.a = 0.0f;
+        return;
+    }
+    const uint8_t* p = row + (size_t)blk * (8 * B);
+    if (B == 1) {
+        const uint2 v = __ldg(reinterpret_cast<const uint2*>(p));
+        c.w[0] = v.x; c.w[1] = v.y;
+    } else {
+#pragma unroll
+        for (int i = 0; i < B / 2; ++i) {
+            const uint4 v = __ldg(reinterpret_cast<const uint4*>(p) + i);
+            c.w[4 * i] = v.x; c.w[4 * i + 1] = v.y; c.w[4 * i + 2] = v.z; c.w[4 * i + 3] = v.w;
+        }
+    }
+    c.a = __ldg(absmax + blk);
+}
+
+// The block's levels, scaled by its absmax and rounded to bf16 as lowra_decode does, in the form that expand16 wants.
+template <int B> struct Scaled;
+template <> struct Scaled<1> {
+    uint32_t base, d, f;     // both halves: the smaller pattern; the difference of the patterns; 0x10001 if level 0 is the larger one
+    __device__ __forceinline__ void set(const float* y, float a) {
+        const uint32_t LH = pack_bf16x2(__fmul_rn(y[0], a), __fmul_rn(y[1], a));
+        const uint32_t L = LH & 0xFFFFu, H = LH >> 16, lo = min(L, H);
+        base = lo * 0x10001u; d = max(L, H) - lo; f = (L > H) ? 0x10001u : 0u;
+    }
+    // elements 16 q .. 16 q + 15 of the block, two per word
+    __device__ __forceinline__ void expand16(const Codes<1>& c, int q, uint32_t (&o)[8]) const {
+        const uint32_t h = (q & 1) ? (c.w[q >> 1] >> 16) : (c.w[q >> 1] & 0xFFFFu);
+        const uint32_t z = h | (h << 15);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) o[i] = (((z >> (2 * i)) & 0x10001u) ^ f) * d + base;
+    }
+};
+template <> struct Scaled<2> {
+    uint32_t e01, e23;
+    __device__ __forceinline__ void set(const float* y, float a) {
+        e01 = pack_bf16x2(__fmul_rn(y[0], a), __fmul_rn(y[1], a));
+        e23 = pack_bf16x2(__fmul_rn(y[2], a), __fmul_rn(y[3], a));
+    }
+    __device__ __forceinline__ void expand16(const Codes<2>& c, int q, uint32_t (&o)[8]) const {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const uint32_t y = c.w[q] >> (4 * i);
+            const uint32_t s = (y & 3u) | ((y << 6) & 0x300u);
+            o[i] = __byte_perm(e01, e23, s * 0x22u + 0x1010u);
+        }
+    }
+};
+template <> struct Scaled<4> {
+    uint32_t lo[4], hi[4];   // low and high bytes of the sixteen patterns
+    __device__ __forceinline__ void set(const float* y, float a) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float4 f = __ldg(reinterpret_cast<const float4*>(y) + i);
+            const uint32_t p = pack_bf16x2(__fmul_rn(f.x, a), __fmul_rn(f.y, a)), r = pack_bf16x2(__fmul_rn(f.z, a), __fmul_rn(f.w, a));
+            lo[i] = __byte_perm(p, r, 0x6420u);
+            hi[i] = __byte_perm(p, r, 0x7531u);
+        }
+    }
+    // four codes at a time: a byte permute looks up the low three bits of each in either half of the table, the fourth bits
+    // choose between the halves
+    __device__ __forceinline__ void expand16(const Codes<4>& c, int q, uint32_t (&o)[8]) const {
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+            const uint32_t x = c.w[2 * q + (h >> 1)] >> (16 * (h & 1));
+            const uint32_t sel = x & 0x7777u;
+            const uint32_t upper = __byte_perm(0x0000FF00u, 0u, (x >> 3) & 0x1111u);   // 0xFF where the code is 8 or more
+            const uint32_t l = (__byte_perm(lo[0], lo[1], sel) & ~upper) | (__byte_perm(lo[2], lo[3], sel) & upper);
+            const uint32_t u = (__byte_perm(hi[0], hi[1], sel) & ~upper) | (__byte_perm(hi[2], hi[3], sel) & upper);
+            o[2 * h] = __byte_perm(l, u, 0x5140u);
+            o[2 * h + 1] = __byte_perm(l, u, 0x7362u);
+        }
+    }
+};
+
+// Where 16-byte piece j (0 .. 7) of block t of token row m lies in a staged [tokens][256] tile: the pieces of a block are
+// exchanged among themselves so that the eight lanes of a shared-memory wavefront read eight different columns.
+__device__ __forceinline__ uint32_t token_piece(int m, int t, int j) {
+    return (uint32_t)(m * (kSmallSpan * 2) + (t * 8 + (j ^ (t | ((m & 1) << 2)))) * 16);
+}
+
+template <int B, int NT8>
+__device__ __forceinline__ void multiply_rows(const SmallParams& P, const SmallMember& W, int m0, int p0, int p_end, int slot, int slots,
+                                              uint32_t x_smem, int half, float (&acc)[NT8][4]) {
+    constexpr int c = B >> 1;
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const int n_span = (P.K + kSmallSpan - 1) / kSmallSpan, nb = P.K / kBlock;
+    const int b0 = (int)((long long)slot * n_span / slots), b1 = (int)((long long)(slot + 1) * n_span / slots);
+    // rows g and g + 8 of the warp's sixteen
+    const bool live0 = p0 + g < p_end, live1 = p0 + g + 8 < p_end;
+    const int q0 = live0 ? p0 + g : p_end - 1, q1 = live1 ? p0 + g + 8 : p_end - 1;
+    const int r0 = __ldg(W.L.perm + q0), r1 = __ldg(W.L.perm + q1);
+    const uint8_t* row0 = W.packed + packed_row_offset(W.L, c, q0, r0);
+    const uint8_t* row1 = W.packed + packed_row_offset(W.L, c, q1, r1);
+    const float* am0 = W.absmax + (size_t)absmax_row_of(W.L, q0, r0) * nb;
+    const float* am1 = W.absmax + (size_t)absmax_row_of(W.L, q1, r1) * nb;
+    const float* y0 = W.maps + (size_t)r0 * kTableStride;
+    const float* y1 = W.maps + (size_t)r1 * kTableStride;
+    // tokens of one step: fetched by the four warps that share it, two steps in flight
+    constexpr uint32_t kStep = 8u * NT8 * kSmallSpan * 2u;
+    const int th = threadIdx.x & 127;
+    auto stage = [&](int b) {
+        if (b < b1) {
+            const uint32_t dst = x_smem + (uint32_t)((b - b0) & 1) * kStep;
+            for (int i = th; i < 8 * NT8 * 32; i += 128) {
+                const int m = i >> 5, t2 = (i >> 3) & 3, j = i & 7, k = b * kSmallSpan + t2 * 64 + j * 8;
+                const bool ok = m0 + m < W.M && k < P.K;
+                cp_async_16_zfill(dst + token_piece(m, t2, j), ok ? W.X + (size_t)(m0 + m) * P.K + k : W.X, ok);
+            }
+        }
+        ptx::cp_async_commit();
+    };
+    Codes<B> n0, n1;
+    auto fetch = [&](int b) {
+        const int blk = 4 * b + t;
+        fetch_codes<B>(n0, row0, am0, blk, live0 && b < b1 && blk < nb);
+        fetch_codes<B>(n1, row1, am1, blk, live1 && b < b1 && blk < nb);
+    };
+    fetch(b0);
+    stage(b0);
+    float ya[4], yb[4];
+    if (B <= 2) {
+#pragma unroll
+        for (int i = 0; i < 2 * B; ++i) { ya[i] = __ldg(y0 + i); yb[i] = __ldg(y1 + i); }
+    }
+    for (int b = b0; b < b1; ++b) {
+        const Codes<B> c0 = n0, c1 = n1;
+        fetch(b + 1);
+        stage(b + 1);
+        Scaled<B> s0, s1;
+        s0.set(B <= 2 ? ya : y0, c0.a);
+        s1.set(B <= 2 ? yb : y1, c1.a);
+        ptx::cp_async_wait<1>();
+        ptx::named_barrier_sync(1 + half, 128);
+        const uint32_t xs = x_smem + (uint32_t)((b - b0) & 1) * kStep;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {   // sixteen elements of the block
+            uint32_t o0[8], o1[8];
+            s0.expand16(c0, q, o0);
+            s1.expand16(c1, q, o1);
+#pragma unroll
+            for (int nt = 0; nt < NT8; ++nt) {
+                const uint4 xl = ld_shared_v4(xs + token_piece(nt * 8 + g, t, 2 * q)), xh = ld_shared_v4(xs + token_piece(nt * 8 + g, t, 2 * q + 1));
+                mma_bf16(acc[nt], o0[0], o1[0], o0[1], o1[1], xl.x, xl.y);
+                mma_bf16(acc[nt], o0[2], o1[2], o0[3], o1[3], xl.z, xl.w);
+                mma_bf16(acc[nt], o0[4], o1[4], o0[5], o1[5], xh.x, xh.y);
+                mma_bf16(acc[nt], o0[6], o1[6], o0[7], o1[7], xh.z, xh.w);
+            }
+        }
+        ptx::named_barrier_sync(1 + half, 128);   // the tokens have been read: the buffer may be filled again
+    }
+}
+
+// Grid: (row groups x slices of the contraction = cluster, token tiles of all members).
+template <int NT8>
+__global__ void __launch_bounds__(kSmallThreads, 2) small_kernel(const __grid_constant__ SmallParams P, const int slices) {
+    extern __shared__ __align__(16) unsigned char small_smem[];
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    constexpr int kTokens = 8 * NT8;
+    constexpr uint32_t kTokenBytes = 2u * kTokens * kSmallSpan * 2u;     // two steps of one half of the warps
+    float* part = reinterpret_cast<float*>(small_smem + 2 * kTokenBytes);   // [2][tokens][kPartPitch]
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const int rank = (int)ptx::cluster_ctarank();
+    int grp = (int)blockIdx.x / slices;
+    const Unit un = unit_at(P, (int)blockIdx.y, kTokens);
+    const SmallMember& W = P.m[un.member];
+    // the group's rows: 64 neighbouring stored rows of one precision class
+    int c = 0;
+    for (; c < 2; ++c) {
+        const int n = (W.L.class_start[c + 1] - W.L.class_start[c] + kSmallRows - 1) / kSmallRows;
+        if (grp < n) break;
+        grp -= n;
+    }
+    const int p_first = W.L.class_start[c] + grp * kSmallRows, p_end = W.L.class_start[c + 1];
+    const bool any = p_first < p_end;                                    // (members with other class counts have fewer groups)
+    const int tile = warp & 3, half = warp >> 2;
+    const int p0 = p_first + tile * 16;
+    const int slot = rank * 2 + half, slots = slices * 2;
+    float acc[NT8][4];
+#pragma unroll
+    for (int i = 0; i < NT8; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.0f;
+    // the up-projection's fragments for this warp's rows: steps of 16 ranks, dealt to the slots
+    const int q0 = min(p0 + g, p_end - 1), q1 = min(p0 + g + 8, p_end - 1);
+    uint32_t up[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int j0 = (slot + i * slots) * 16 + 2 * t;
+        up[i][0] = up[i][1] = up[i][2] = up[i][3] = 0u;
+        if (any && (slot + i * slots) * 16 < P.r) {
+            const uint16_t* b0 = W.B + __ldg(W.L.perm + q0);
+            const uint16_t* b1 = W.B + __ldg(W.L.perm + q1);
+            const size_t N = (size_t)P.N;
+            up[i][0] = (uint32_t)__ldg(b0 + j0 * N) | ((uint32_t)__ldg(b0 + (j0 + 1) * N) << 16);
+            up[i][1] = (uint32_t)__ldg(b1 + j0 * N) | ((uint32_t)__ldg(b1 + (j0 + 1) * N) << 16);
+            up[i][2] = (uint32_t)__ldg(b0 + (j0 + 8) * N) | ((uint32_t)__ldg(b0 + (j0 + 9) * N) << 16);
+            up[i][3] = (uint32_t)__ldg(b1 + (j0 + 8) * N) | ((uint32_t)__ldg(b1 + (j0 + 9) * N) << 16);
+        }
+    }
+    if (any) {
+        const uint32_t xs = ptx::smem_u32(small_smem) + (uint32_t)half * kTokenBytes;
+        if (c == 0) multiply_rows<1, NT8>(P, W, un.m0, p0, p_end, slot, slots, xs, half, acc);
+        else if (c == 1) multiply_rows<2, NT8>(P, W, un.m0, p0, p_end, slot, slots, xs, half, acc);
+        else multiply_rows<4, NT8>(P, W, un.m0, p0, p_end, slot, slots, xs, half, acc);
+    }
+    asm volatile("griddepcontrol.wait;" ::: "memory");                   // T is in place
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        if (!any || (slot + i * slots) * 16 >= P.r) break;
+#pragma unroll
+        for (int nt = 0; nt < NT8; ++nt) {
+            const int m = un.m0 + nt * 8 + g;
+            uint32_t b0 = 0u, b1 = 0u;
+            if (m < W.M) {
+                const uint32_t* tr = reinterpret_cast<const uint32_t*>(W.T + (size_t)m * P.rp + (slot + i * slots) * 16) + t;
+                b0 = __ldcg(tr);
+                b1 = __ldcg(tr + 4);
+            }
+            mma_bf16(acc[nt], up[i][0], up[i][1], up[i][2], up[i][3], b0, b1);
+        }
+    }
+#pragma unroll
+    for (int nt = 0; nt < NT8; ++nt) {
+        float* d = part + (half * kTokens + nt * 8 + 2 * t) * kPartPitch + tile * 16 + g;
+        d[0] = acc[nt][0]; d[kPartPitch] = acc[nt][1];
+        d[8] = acc[nt][2]; d[kPartPitch + 8] = acc[nt][3];
+    }
+    ptx::cluster_sync();
+    // every CTA of the cluster adds up its share of the rows over the slices, in a fixed order
+    const int share = kSmallRows / slices;
+    const uint32_t part_addr = ptx::smem_u32(part);
+    for (int i = threadIdx.x; any && i < share * kTokens; i += kSmallThreads) {
+        const int m = i / share, row = rank * share + (i - m * share);
+        if (un.m0 + m >= W.M || p_first + row >= p_end) continue;
+        float sum = 0.0f;
+        for (int s = 0; s < slices; ++s) {
+            const uint32_t addr = ptx::map_to_cta(part_addr + (uint32_t)(m * kPartPitch + row) * 4u, (uint32_t)s);
+            sum += ld_cluster_f32(addr) + ld_cluster_f32(addr + (uint32_t)(kTokens * kPartPitch) * 4u);
+        }
+        W.Y[(size_t)(un.m0 + m) * P.N + __ldg(W.L.perm + p_first + row)] = (uint16_t)pack_bf16x2(sum, 0.0f);
+    }
+    ptx::cluster_sync();   // nobody leaves while a peer still reads its sums
+}
+
+template <int NT8>
+lowra_status launch_product(const SmallParams& P, int groups, int units, int slices, cudaStream_t stream) {
+    constexpr size_t smem = 4u * (8 * NT8) * kSmallSpan * 2u + 2u * (8 * NT8) * kPartPitch * 4u;
+    static SmemLimit limit = {};
+    if (ensure_smem_limit(reinterpret_cast<const void*>(small_kernel<NT8>), smem, &limit) != LOWRA_OK) return LOWRA_ERR_CUDA;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)slices;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3((unsigned)(groups * slices), (unsigned)units, 1);
+    cfg.blockDim = dim3(kSmallThreads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, small_kernel<NT8>, P, slices) == cudaSuccess ? LOWRA_OK : LOWRA_ERR_CUDA;
+}
+
+}  // namespace
+
+lowra_status launch_small(const SmallParams& P, cudaStream_t stream) {
+    int m16 = 0, groups = 0, most = 0;
+    for (int i = 0; i < P.count; ++i) {
+        const SmallMember& m = P.m[i];
+        m16 += (m.M + 15) / 16;
+        most = m.M > most ? m.M : most;
+        int n = 0;
+        for (int c = 0; c < 3; ++c) n += (m.L.class_start[c + 1] - m.L.class_start[c] + kSmallRows - 1) / kSmallRows;
+        groups = n > groups ? n : groups;
+    }
+    // ---- T: the contraction over up to eight CTAs, 128 indices or more each
+    {
+        int slices = 1;
+        while (slices < 8 && P.K >= 256 * slices) slices *= 2;
+        const size_t fetch = (size_t)8 * kProjectBatch * 16 * (P.r * 2 + 16), sums = (size_t)(8 + 1) * 16 * P.r * 4;
+        const size_t smem = fetch > sums ? fetch : sums;
+        static SmemLimit limit = {};
+        if (ensure_smem_limit(reinterpret_cast<const void*>(project_kernel), smem, &limit) != LOWRA_OK) return LOWRA_ERR_CUDA;
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr[2];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)slices;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[1].val.programmaticStreamSerializationAllowed = 1;
+        cfg.gridDim = dim3((unsigned)slices, (unsigned)m16, 1);
+        cfg.blockDim = dim3(kSmallThreads, 1, 1);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = stream;
+        cfg.attrs = attr;
+        cfg.numAttrs = 2;
+        if (cudaLaunchKernelEx(&cfg, project_kernel, P) != cudaSuccess) return LOWRA_ERR_CUDA;
+    }
+    // ---- the product: slices of the contraction until the grid is about three CTAs per two places, as long as every warp keeps
+    // a step of 256.  The choice depends on the weight's shape alone, so that a member's result does not depend on its company.
+    const int n_span = (P.K + kSmallSpan - 1) / kSmallSpan, by_shape = (P.N + kSmallRows - 1) / kSmallRows;
+    int slices = 1;
+    while (slices < 8 && 4 * slices <= n_span && 2 * slices * by_shape <= 3 * kNumSMs) slices *= 2;
+    const int nt8 = most <= 8 ? 1 : most <= 16 ? 2 : 4;
+    int units = 0;
+    for (int i = 0; i < P.count; ++i) units += (P.m[i].M + 8 * nt8 - 1) / (8 * nt8);
+    if (nt8 == 1) return launch_product<1>(P, groups, units, slices, stream);
+    if (nt8 == 2) return launch_product<2>(P, groups, units, slices, stream);
+    return launch_product<4>(P, groups, units, slices, stream);
+}
+
+}  // namespace lowra
