@@ -192,8 +192,8 @@ lowra_status lowra_channel_errors(int32_t N, int32_t K, const float* W_dev, cons
 
 /* Bytes of device scratch that lowra_lora_forward / lowra_lora_backward_input need for M tokens and
  * LoRA rank r (0 if the arguments are invalid).  The first 256 bytes hold the device status word; the
- * rest: the down-projected activations, flags, the deal of the rows to the dequant warps and 19 MB for
- * the fp32 partial tiles that tiles cut between SMs are handed over in (about 21 MB for a 4096 x 11008
+ * rest: the down-projected activations, flags, the deal of the rows to the dequant warps and 39 MB for
+ * the fp32 partial tiles that tiles cut between SMs are handed over in (about 41 MB for a 4096 x 11008
  * matrix at 4096 tokens). */
 size_t lowra_workspace_bytes(const lowra_layout* layout, int32_t M, int32_t r);
 
@@ -206,8 +206,8 @@ size_t lowra_workspace_bytes(const lowra_layout* layout, int32_t M, int32_t r);
  * of a call (3-6 us less per call on a B200); the workspace then has to be initialised once with
  * lowra_workspace_init before its first use, is written by these calls only, and its status word is no
  * longer cleared per call: lowra_device_status reports the first failure since the initialisation.
- *   lowra_deal_bytes   size of the buffer for this layout (0 if the layout is invalid); about 40 bytes per
- *                      channel (0.44 MB for 11008 channels)
+ *   lowra_deal_bytes   size of the buffer for this layout (0 if the layout is invalid); about 20 bytes per
+ *                      channel (0.22 MB for 11008 channels)
  *   lowra_deal_build   fills deal_dev (256-byte aligned, >= lowra_deal_bytes(layout) bytes) for both the
  *                      forward and the backward-input call; reads layout->precs_dev / inv_perm_dev and
  *                      ignores layout->deal_dev.  The buffer is read-only afterwards and may serve any
@@ -386,7 +386,8 @@ lowra_status lowra_set_wait_limit(uint64_t nanoseconds);
  * library is loaded there until the process exits.  The call allocates nothing, frees nothing and
  * calls no allocating routine; inputs and outputs are still the caller's.
  *
- *   - Same arguments, results and errors as lowra_lora_forward, without the workspace.  If
+ *   - Same arguments, results (up to the order of fp32 sums where lowra_lora_forward cuts tiles between SMs) and errors as
+ *     lowra_lora_forward, without the workspace.  If
  *     the scratch this entry needs (lowra_workspace_bytes(layout, M, r) less the partial tiles, which
  *     it does without: tiles are never cut here) exceeds LOWRA_STATIC_SCRATCH_BYTES the call launches
  *     nothing and returns LOWRA_ERR_LIMIT (for scale: N = K = 8192, M = 8192, r = 64 needs about 1.6 MB).

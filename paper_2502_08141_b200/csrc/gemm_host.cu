@@ -31,37 +31,25 @@ size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 struct Workspace {
     size_t off_T[kMaxBatch];      // per member: its down-projected activations
     int flag0[kMaxBatch];         // per member: index of its first "T ready" flag
-    size_t off_flags, off_items, off_meta, off_part, total;
+    size_t off_flags, off_items, off_part, total;
     int rp, n_flags, sk_flag0;
 };
 
 bool rank_ok(int r) { return r >= 16 && r <= 128 && r % 16 == 0; }
 
-// Sizes of the row deal (see gemm_prep.cu).  Forward: 128 row words per group of 128 channels; backward: 4 work-list
-// entries (a head and 32 row records of 16 bytes each) per group of 64 channels, plus the end markers.
-struct DealSizes {
-    size_t fwd_bytes, rows_bytes, heads_bytes;
-};
-DealSizes deal_sizes(int N) {
-    const size_t groups_per_cta = ((size_t)(N + 63) / 64 + kCluster - 1) / kCluster;
-    const size_t entries = kCluster * (4 * groups_per_cta + kListSlack + kProducerWarps);
-    DealSizes d;
-    d.fwd_bytes = (size_t)((N + 127) / 128) * kItemStride * 4;
-    d.rows_bytes = entries * 32 * 16;
-    d.heads_bytes = entries * 4;
-    return d;
-}
-// A deal kept by the caller (lowra_deal_build): forward row words | backward row records | backward heads
+// Sizes of the row deal (see gemm_prep.cu).  Forward: 128 row words per group of 128 channels; backward: 64 row records of
+// 16 bytes per group of 64 channels.
+size_t deal_forward_bytes(int N) { return (size_t)((N + 127) / 128) * kItemStride * 4; }
+size_t deal_backward_bytes(int N) { return (size_t)((N + 63) / 64) * kGroupRecords * 16; }
+// A deal kept by the caller (lowra_deal_build): forward row words | backward row records
 struct DealBuffer {
-    size_t off_fwd, off_rows, off_heads, total;
+    size_t off_fwd, off_rows, total;
 };
 DealBuffer plan_deal(int N) {
-    const DealSizes z = deal_sizes(N);
     DealBuffer d;
     d.off_fwd = 0;
-    d.off_rows = align256(z.fwd_bytes);
-    d.off_heads = d.off_rows + align256(z.rows_bytes);
-    d.total = d.off_heads + align256(z.heads_bytes);
+    d.off_rows = align256(deal_forward_bytes(N));
+    d.total = d.off_rows + align256(deal_backward_bytes(N));
     return d;
 }
 
@@ -71,22 +59,21 @@ Workspace plan_workspace(int N, int K, const int* Ms, int count, int r, bool str
     Workspace w;
     memset(&w, 0, sizeof(w));
     w.rp = (r + 63) / 64 * 64;
-    const DealSizes z = deal_sizes(N);   // room for the deal of one direction, rebuilt by every call that brings none
     size_t off = kStatusBytes;
     int flags = 0;
     for (int i = 0; i < count; ++i) {
         w.off_T[i] = off;
         off += align256((size_t)Ms[i] * w.rp * 2);
-        // the member's "T ready" flags (a cluster's last token tiles may lie past its tokens)
-        w.flag0[i] = flags;
-        flags += (Ms[i] + kTileT - 1) / kTileT + kCluster;
+        w.flag0[i] = flags;          // the member's "T ready" flags: one per CTA and token tile
+        flags += (Ms[i] + kHalfT - 1) / kHalfT * kCluster;
     }
     w.off_flags = off;
     w.sk_flag0 = flags;                                  // then one "partial tile ready" flag per CTA
     w.n_flags = flags + kMaxClusters * kCluster;
     w.off_items = w.off_flags + align256((size_t)w.n_flags * 4);
-    w.off_meta = w.off_items + align256(z.rows_bytes > z.fwd_bytes ? z.rows_bytes : z.fwd_bytes);
-    w.off_part = w.off_meta + align256(z.heads_bytes);
+    // room for the deal of one direction, rebuilt by every call that brings none
+    const size_t fwd = deal_forward_bytes(N), bwd = deal_backward_bytes(N);
+    w.off_part = w.off_items + align256(fwd > bwd ? fwd : bwd);
     w.total = w.off_part + (stream_k ? align256((size_t)kMaxClusters * kSkSlotFloats * 4) : 0);   // stream-K partial tiles
     return w;
 }
@@ -165,6 +152,13 @@ lowra_status check_members(const MemberArgs* mem, int count, int32_t r, const vo
     return check_device();
 }
 
+// A row of the output is R bf16 values (a multiple of 8), every output pointer a multiple of 16 bytes.
+int out_alignment(const MemberArgs* mem, int count, int R) {
+    bool wide = R % 16 == 0;
+    for (int i = 0; i < count; ++i) wide = wide && (reinterpret_cast<uintptr_t>(mem[i].out) & 31u) == 0;
+    return wide ? 32 : 16;
+}
+
 lowra_status run_small(const MemberArgs* mem, uint16_t* const* T_of, int count, int32_t r, float s, void* workspace, cudaStream_t stream);
 // The diagnostic lowra_diag_drop_t_flags is about flags, which the path for few tokens has none of: it leaves that path out.
 bool takes_small_path(bool backward, int M) { return !backward && M <= kSmallTokens && g_drop_t_flags.load(std::memory_order_relaxed) == 0; }
@@ -210,26 +204,21 @@ lowra_status run_members(bool backward, const MemberArgs* mem, int count, int32_
         g.T = reinterpret_cast<uint16_t*>(ws + w.off_T[i]);
         g.flags = flags + w.flag0[i];
         g.M = m.M;
-        g.st0 = G.super_total;
-        G.super_total += ((m.M + kTileT - 1) / kTileT + kCluster - 1) / kCluster;
         if (m.layout->deal_dev != nullptr) {
             // the rows were dealt once for this weight (lowra_deal_build) and the workspace numbers its calls
             // (lowra_workspace_init): nothing to prepare, the fused kernel is the only launch
             const DealBuffer d = plan_deal(N);
             const unsigned char* deal = static_cast<const unsigned char*>(m.layout->deal_dev);
             g.items = reinterpret_cast<const uint32_t*>(deal + (backward ? d.off_rows : d.off_fwd));
-            g.heads = reinterpret_cast<const uint32_t*>(deal + d.off_heads);
         } else {
             // ---- prologue: clear status and flags, deal the rows (plain calls only)
             uint32_t* items = reinterpret_cast<uint32_t*>(ws + w.off_items);
-            uint32_t* heads = reinterpret_cast<uint32_t*>(ws + w.off_meta);
             PrepParams P;
             memset(&P, 0, sizeof(P));
             P.L = g.L;
             P.precs = m.layout->precs_dev;
             P.inv_perm = m.layout->inv_perm_dev;
             P.items = items;
-            P.heads = heads;
             P.N = N;
             P.group = backward ? 64 : 128;
             P.status = status;
@@ -240,7 +229,6 @@ lowra_status run_members(bool backward, const MemberArgs* mem, int count, int32_
             st = launch_prep(P, stream);
             if (st != LOWRA_OK) return st;
             g.items = items;
-            g.heads = heads;
         }
     }
 
@@ -257,9 +245,10 @@ lowra_status run_members(bool backward, const MemberArgs* mem, int count, int32_
     G.R = backward ? K : N;
     G.C = backward ? N : K;
     G.ld_out = G.R;
+    G.out_align = out_alignment(mem, count, G.R);
     G.main_blocks = (G.C + kTileC - 1) / kTileC;
     G.lora_blocks = w.rp / kTileC;
-    G.tiles_r = (G.R + kTileR - 1) / kTileR;
+    G.tiles_r = (G.R + kPairR - 1) / kPairR;
     for (int i = 0; i < count; ++i) {   // token operands: every distinct one once (q, k, v share X in the forward pass)
         bool seen = false;
         for (int j = 0; j < i; ++j) seen = seen || mem[j].act == mem[i].act;
@@ -276,15 +265,15 @@ lowra_status run_members(bool backward, const MemberArgs* mem, int count, int32_
     for (int i = 0; i < count; ++i) {
         const MemberArgs& m = mem[i];
         MemberMaps& t = TM.m[i];
-        if (!make_map(&t.tmB, m.act, (uint64_t)m.M, (uint64_t)G.C, (uint64_t)G.C, kTileT)) return LOWRA_ERR_CUDA;
-        if (!make_map(&t.tmT, G.mem[i].T, (uint64_t)m.M, (uint64_t)w.rp, (uint64_t)w.rp, kTileT)) return LOWRA_ERR_CUDA;
+        if (!make_map(&t.tmB, m.act, (uint64_t)m.M, (uint64_t)G.C, (uint64_t)G.C, 128)) return LOWRA_ERR_CUDA;
+        if (!make_map(&t.tmT, G.mem[i].T, (uint64_t)m.M, (uint64_t)w.rp, (uint64_t)w.rp, 128)) return LOWRA_ERR_CUDA;
         if (!backward) {
             // T tiles take ranks x features from A [K, r] (64 x 64 boxes); LoRA blocks take channels x ranks from B [r, N]
             if (!make_map(&t.tmFt, m.A, (uint64_t)K, (uint64_t)r, (uint64_t)r, 64)) return LOWRA_ERR_CUDA;
             if (!make_map(&t.tmFl, m.B, (uint64_t)r, (uint64_t)N, (uint64_t)N, 64)) return LOWRA_ERR_CUDA;
         } else {
-            // T tiles take ranks x channels from B [r, N]; LoRA blocks take features x ranks from A [K, r] (64 x 128 boxes)
-            if (!make_map(&t.tmFt, m.B, (uint64_t)r, (uint64_t)N, (uint64_t)N, kTileR)) return LOWRA_ERR_CUDA;
+            // T tiles take ranks x channels from B [r, N] (64 x 64); LoRA blocks take features x ranks from A [K, r] (64 x 128)
+            if (!make_map(&t.tmFt, m.B, (uint64_t)r, (uint64_t)N, (uint64_t)N, 64)) return LOWRA_ERR_CUDA;
             if (!make_map(&t.tmFl, m.A, (uint64_t)K, (uint64_t)r, (uint64_t)r, kTileR)) return LOWRA_ERR_CUDA;
         }
     }
@@ -374,7 +363,6 @@ extern "C" lowra_status lowra_deal_build(const lowra_layout* layout, void* deal_
         P.precs = layout->precs_dev;
         P.inv_perm = layout->inv_perm_dev;
         P.items = reinterpret_cast<uint32_t*>(deal + (backward ? d.off_rows : d.off_fwd));
-        P.heads = reinterpret_cast<uint32_t*>(deal + d.off_heads);
         P.N = N;
         P.group = backward ? 64 : 128;
         P.blocks = ((N + P.group - 1) / P.group + 3) / 4;
@@ -762,13 +750,13 @@ extern "C" lowra_status lowra_dense_nt(const uint16_t* P_dev, const uint16_t* Q_
     G.R = N;
     G.C = K;
     G.ld_out = N;
+    G.out_align = N % 8 == 0 ? 16 : 2;
     G.main_blocks = K / kTileC;
     G.lora_blocks = 0;
-    G.tiles_r = (N + kTileR - 1) / kTileR;
-    G.super_total = (M + kTileT - 1) / kTileT;     // one CTA per "cluster" in the dense mode
+    G.tiles_r = (N + kPairR - 1) / kPairR;
     G.mem[0].M = M;
     G.wait_ns = wait_limit_ns();
-    if (!make_map(&TM.m[0].tmB, P_dev, (uint64_t)M, (uint64_t)K, (uint64_t)K, kTileT)) return LOWRA_ERR_CUDA;
+    if (!make_map(&TM.m[0].tmB, P_dev, (uint64_t)M, (uint64_t)K, (uint64_t)K, 128)) return LOWRA_ERR_CUDA;
     if (!make_map(&TM.m[0].tmFl, Q_dev, (uint64_t)N, (uint64_t)K, (uint64_t)K, kTileR)) return LOWRA_ERR_CUDA;
     TM.m[0].tmT = TM.m[0].tmB;
     TM.m[0].tmFt = TM.m[0].tmB;

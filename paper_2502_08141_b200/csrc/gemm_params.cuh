@@ -9,24 +9,21 @@ namespace lowra {
 
 // ---- prologue ------------------------------------------------------------------------------
 constexpr int kPrepThreads = 128;
-constexpr int kProducerWarps = 8;             // dequant warps of the main kernel
+constexpr int kProducerWarps = 16;            // dequant warps of the main kernel
 constexpr int kItemStride = 128;              // forward: entries per group of 128 rows in the deal table
-constexpr int kStageArrivals = 8;             // arrivals a weight-slot barrier expects from the dequant warps (backward: four chunks x 2)
-constexpr int kCluster = 2;                   // CTAs per cluster; they share every dequantised weight tile
-constexpr int kListWarps = kProducerWarps * kCluster;   // backward: work lists (one per dequant warp of the cluster)
-constexpr int kListSlack = 4 * kProducerWarps;  // backward: all-ones heads written behind the last entry of a CTA's lists
+constexpr int kGroupRecords = 64;             // backward: row records per group of 64 channels
+constexpr int kCluster = 2;                   // CTAs per cluster: the pair that works on one tensor-core tile
 constexpr int kMaxGroups64 = 8192;            // backward: at most this many groups of 64 output channels (N <= 524288)
 
 struct PrepParams {
     // deal of the rows to the dequant threads of the main kernel.  Row word = row offset inside its group
     // (bits 0-6) | class (bits 7-8, 3 = row past N) | stored position (bits 9-31), all ones for "no row".
     //   forward (group 128): items[g * kItemStride + i] = i-th row of group g in precision order
-    //   backward (group 64): per-warp work lists, see deal_backward
+    //   backward (group 64): 64 row records of 16 bytes per group, see deal_backward
     RowLayout L;
     const uint8_t* precs;
     const int32_t* inv_perm;
-    uint32_t* items;      // forward: row words; backward: 16-byte row records of the work-list entries
-    uint32_t* heads;      // backward: [7 * ceil(N / 64) + kListSlack] work-list heads
+    uint32_t* items;      // forward: row words; backward: 16-byte row records
     int N, group;
     uint32_t* status;     // device status word, cleared (null: left alone)
     uint32_t* exits;      // the fused kernel's count of CTAs that have left, cleared (null: left alone)
@@ -38,29 +35,25 @@ struct PrepParams {
 lowra_status launch_prep(const PrepParams& P, cudaStream_t stream);
 
 // ---- fused kernel --------------------------------------------------------------------------
-constexpr int kTileR = 128;       // rows of the MMA A operand per tile (output channels fwd, input features bwd)
-constexpr int kTileT = 256;       // tokens per tile (MMA N)
+constexpr int kTileR = 128;       // operand rows (output channels fwd, input features bwd) per CTA ...
+constexpr int kPairR = 256;       // ... and per tile: the two CTAs of a cluster form one tensor-core tile
+constexpr int kHalfT = 256;       // tokens per MMA (128 in either CTA)
+constexpr int kTileT = 512;       // tokens per tile at most: two MMAs' worth share every dequantised weight
 constexpr int kTileC = 64;        // contraction elements per pipeline stage (= one absmax block, = 128 bytes of bf16)
-constexpr int kStages = 4;        // dense diagnostic: four stages of one weight slot + one token slot
-// Forward / backward: the dequant warps (and the copies between the CTAs of a cluster) need to run further ahead
-// of the tensor core than the TMA loads do, so the ring is split into 16 KB weight slots and 32 KB token slots:
-// five + four in both passes, plus 16 KB for the level tables of 4-bit rows (the token slots hide the L2
-// latency of the TMA loads; a fifth weight slot was worth +9..13 % in the forward pass; a sixth is worth another
-// +3..5 % and takes the place of the table cache in calls on weights without 4-bit rows; reading the tables through
-// L1 instead, or keeping the levels in registers, cost more than the sixth slot gives).  A weight slot
-// is free once the MMAs of that many stages earlier are complete; the weight ring must not be shallower than the
-// token ring (the TMA warp also loads factor tiles into weight slots).
-constexpr int kStagesA_fwd = 5, kStagesA_bwd = 5;
-constexpr int kStagesB_fwd = 4, kStagesB_bwd = 4;
-constexpr int kMaxStagesA = 6;
+// The operand ring: a stage takes one weight slot and an entry for each half of its tokens, 16 KB each.
+constexpr int kSlotsW = 6, kSlotsX = 8;
+// At the start and the end of a tile so many stages are worked on half by half (all of the first half's, then all of the second
+// half's), so that the first half's accumulator is drained while the second half's is still being filled.
+constexpr int kSkew = 4;
+static_assert(kSkew <= kSlotsW && 2 * kSkew <= kSlotsX, "the ring holds the stages that are worked on half by half");
 constexpr int kFirstEpilogueWarp = 2;
-constexpr int kFirstProducerWarp = 6;
-// 16 warps, of which two idle (the two that would share the MMA warp's scheduler): at most four per scheduler,
-// so 128 registers per thread.
-constexpr int kGemmWarps = 16;
+constexpr int kEpilogueWarps = 8;       // two per quarter of the tensor memory's lanes
+constexpr int kFirstProducerWarp = kFirstEpilogueWarp + kEpilogueWarps;
+constexpr int kProducerGroups = kProducerWarps / 4;   // four warps fill the weight slot of a stage, the groups take the stages in turn
+constexpr int kGemmWarps = kFirstProducerWarp + kProducerWarps;
 constexpr int kGemmThreads = 32 * kGemmWarps;
-static_assert(kProducerWarps == 8, "the warp map above places eight dequant warps");
-constexpr int kTmemCols = 512;    // two 128 x 256 fp32 accumulators
+static_assert(kProducerGroups <= kSlotsW, "see stage_free in the kernel");
+constexpr int kTmemCols = 512;    // two 128 x 256 fp32 accumulators per CTA
 
 constexpr int kModeForward = 0, kModeBackward = 1, kModeDense = 2;
 
@@ -72,13 +65,12 @@ struct Member {
     const uint8_t* packed;
     const float* absmax;
     const float* maps;
-    const uint32_t* items;    // from the deal: row words (forward: per tile; backward: per work-list entry)
-    const uint32_t* heads;    // from the deal (backward): work-list heads
+    const uint32_t* items;    // from the deal: row words (forward) or row records (backward)
     uint16_t* out;            // [M, ld_out] bf16
     uint16_t* T;              // [M, rp] bf16: s * X . A (forward) or s * dY . B^T (backward), written by the T tiles
-    uint32_t* flags;          // [tiles_t + kCluster] set to the call's number when T of a token tile is complete
+    uint32_t* flags;          // [token tiles][kCluster] set to the call's number when a CTA's half of T is complete
     int M;                    // this member's tokens (the batch calls: the same for all; several adapters: a group's)
-    int st0;                  // token-tile groups (kCluster tiles each) of the members before this one
+    int st0;                  // token tiles of the members before this one
 };
 
 // Tensor maps of one member: token operand, T, factor of the T tiles, factor of the LoRA blocks.
@@ -107,21 +99,25 @@ struct GemmCommon {
     int rp;                 // LoRA rank rounded up to 64
     int r;                  // LoRA rank
     int M;                  // tokens of the largest member (host: schedule choice)
-    int super_total;        // token-tile groups (kCluster tiles each) of all members
+    int super_total;        // token tiles of all members
     int R;                  // A-operand rows in total: N (forward, dense) or K (backward)
     int C;                  // main contraction length: K (forward, dense) or N (backward)
     int ld_out;             // = R
+    int out_align;          // what every address of a row's 32-column piece is a multiple of: 32, 16 or 2 bytes
     int main_blocks;        // ceil(C / 64)
     int lora_blocks;        // rp / 64 (0 in dense mode)
-    int tiles_r;            // row tiles of a member (all members have one shape)
+    int tiles_r;            // tiles of 256 operand rows of a member (all members have one shape)
     long long operand_bytes;   // token operands of the call, each distinct one counted once (host: schedule choice)
-    // stream-K schedule (set by the launcher; sk == 0: whole tiles, dealt round-robin to the clusters)
-    float* sk_part;         // fp32 partial tiles, one [kCluster][kTileT][kTileR] slot per cluster
-    uint32_t* sk_flags;     // [clusters] raised when a cluster's partial tile is complete
+    // schedule of the tiles that are cut between clusters (set by the launcher; sk == 0: whole tiles, dealt round-robin)
+    float* sk_part;         // fp32 partial tiles, one [kCluster][2 halves][256 rows][128 tokens] slot per cluster
+    uint32_t* sk_flags;     // [clusters][kCluster] raised when a CTA's partial tile is complete
+    int halves;             // token tiles of 256 (1) or 512 tokens (2)
+    int t_split;            // > 1: every T tile is cut between so many clusters, which do nothing else
     int sk;
-    int sk_dp;              // rows of whole pieces (T tiles, then weight tiles, round-robin) before the ranges
-    int sk_late;            // 1: partial tiles are added in the collecting piece's epilogue; 0: preloaded into its accumulator
-    long long sk_total;     // contraction blocks of the weight tiles behind the whole rows
+    int sk_c0;              // the first cluster that gets a range
+    int sk_first;           // first weight tile of the ranges
+    int sk_num;             // contraction blocks of the weight tiles behind the whole rows, plus what follows
+    int sk_extra;           // blocks that a cluster with a T tile is charged (negative: credited) against its range
     unsigned long long wait_ns;   // limit of every device-side wait (lowra_set_wait_limit)
     int diag_drop_t_flags;  // diagnostic (lowra_diag_drop_t_flags): the T tiles do not raise their flags, so the waits
                             // for them run out and the call ends with LOWRA_ERR_TIMEOUT
@@ -133,22 +129,15 @@ struct KParams : GemmCommon {
 using GemmParams = KParams<kMaxBatch>;
 unsigned long long wait_limit_ns();   // the process-wide limit, 1 s unless lowra_set_wait_limit changed it
 constexpr int kMaxClusters = kNumSMs / kCluster;
-constexpr size_t kSkSlotFloats = (size_t)kCluster * kTileT * kTileR;
+constexpr size_t kSkCtaFloats = (size_t)kTileT / kCluster * kPairR;   // a CTA's partial tile: its 256 tokens x 256 rows
+constexpr size_t kSkSlotFloats = (size_t)kCluster * kSkCtaFloats;
 
-constexpr uint32_t kSmemA = kTileR * kTileC * 2;   // 16 KB
-constexpr uint32_t kSmemB = kTileT * kTileC * 2;   // 32 KB
-constexpr uint32_t kSmemStage = kSmemA + kSmemB;
-constexpr uint32_t kSmemRingMax = 224 * 1024;   // operand ring + table cache
-static_assert(kStages * kSmemStage <= kSmemRingMax, "the dense ring fits into the same space");
-constexpr int kEpilogueTokens = 8;                           // tokens per transposition round of the epilogue
-constexpr uint32_t kSmemOut = kEpilogueTokens * kTileR * 2;  // epilogue staging: 8 tokens x 128 channels bf16
+constexpr uint32_t kSmemSlot = 128 * kTileC * 2;   // 16 KB: 128 operand rows or tokens of a stage
+constexpr uint32_t kSmemRing = (kSlotsW + kSlotsX) * kSmemSlot;
 constexpr uint32_t kSmemBarriers = 1024;
-constexpr uint32_t kSmemTab = kProducerWarps * 2048;         // fp32 level tables of the dequant warps' 4-bit rows
-static_assert(kStagesA_bwd * kSmemA + kStagesB_bwd * kSmemB + kSmemTab <= kSmemRingMax, "the backward ring and its table cache fit");
-static_assert(kStagesA_fwd * kSmemA + kStagesB_fwd * kSmemB + kSmemTab <= kSmemRingMax, "the forward ring and its table cache fit");
 // no alignment slack: the dynamic shared memory of a kernel without static shared memory starts 1024-byte
 // aligned (checked by the kernel, which the swizzled operand tiles need)
-constexpr uint32_t kGemmSmemBytes = kSmemRingMax + kSmemOut + kSmemBarriers;
+constexpr uint32_t kGemmSmemBytes = kSmemRing + kSmemBarriers;
 static_assert(kGemmSmemBytes <= 232448, "227 KB of shared memory per CTA");
 
 lowra_status launch_fused(int mode, const GemmParams& G, const BatchMaps& TM, cudaStream_t stream);

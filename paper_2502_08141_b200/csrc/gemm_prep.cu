@@ -63,46 +63,23 @@ __device__ void deal_rows(const PrepParams& P, int blk) {
     }
 }
 
-// Backward-input: every pipeline stage of the main kernel brings a group of 64 consecutive output channels.
-// The CTAs of a cluster take the groups in turn (group g is dequantised by CTA g % kCluster, which then copies
-// the finished operand tile to its peers).  The rows of a group are ordered by precision class (rows past N last)
-// and cut into four chunks of 16 rows; a chunk is the work of one dequant warp on one stage (32 lanes = 16 rows x
-// 2 halves of the tile's 128 features), so most warps see one precision and a few see two.  The chunks of the
-// groups of one CTA are numbered through the whole matrix and chunk n goes to warp n % kProducerWarps of that
-// CTA as entry n / kProducerWarps of the warp's work list, so a warp only ever visits the stages it has work on:
-//   heads[e]         = group index (bits 0-23) | arrivals this entry owes the stage barrier (bits 24-27)
-//   rows[e * 32 + l] = what lane l needs to find its row, ready to use (16 bytes):
+// Backward-input: every pipeline stage of the main kernel brings a group of 64 consecutive output channels.  The rows of a
+// group are ordered by precision class (rows past N last) and cut into four chunks of 16 rows; a chunk is the work of one
+// dequant warp of either CTA on that stage (32 lanes = 16 rows x 2 halves of the CTA's 128 features), so most warps see one
+// precision and a few see two.  Four warps share a group; the chunks differ in cost (the last one
+// holds the group's 4-bit rows, usually next to 2-bit ones: two code paths), so which of the four warps takes which chunk
+// rotates from one round of groups to the next.
+//   rows[(g * 4 + w) * 16 + l] = what lanes l and l + 16 of the warp with number w mod 4 need to find their row (16 bytes):
 //                      x = byte offset of the row in the packed buffer / 16, y = index of the row's first absmax,
 //                      z = index of the row's first level in the maps table,
 //                      w = channel inside the group (bits 0-5) | precision class (bits 8-9; 3 = row past N: zeros)
-// with e = entry * kListWarps + warp * kCluster + CTA.  Every list ends with all-ones heads.
-__device__ __forceinline__ uint32_t list_slot(uint32_t n, int cta) {
-    return (n / kProducerWarps) * kListWarps + (n % kProducerWarps) * kCluster + (uint32_t)cta;
-}
-// The chunks of a group are sorted by precision, so its last chunk is the dearest one (it holds the group's 4-bit
-// rows, usually next to 2-bit ones: two code paths).  Which of a group's four warps takes which chunk therefore
-// rotates from one group pair to the next; a warp still gets one chunk of every second group of its CTA, in order.
-__device__ __forceinline__ uint32_t chunk_slot(uint32_t n0, uint32_t ci, int cta) {
-    const uint32_t pair = n0 / kProducerWarps;                    // n0 = 4 * (group's number within its CTA)
-    return list_slot((n0 & ~3u) + ((ci + pair) & 3u), cta);
-}
-
 __device__ void deal_backward(const PrepParams& P, int blk) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, tid = threadIdx.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     constexpr int kWarps = kPrepThreads / 32;
-    constexpr int kChunks = 4;   // per group of 64 rows
     const int n_groups = (P.N + 63) / 64;
-    if (blk == 0) {   // end markers behind the last entry of every CTA's lists
-        for (int cta = 0; cta < kCluster; ++cta) {
-            const uint32_t total = (uint32_t)kChunks * (uint32_t)((n_groups - cta + kCluster - 1) / kCluster);
-            for (int i = tid; i < kListSlack; i += kPrepThreads) P.heads[list_slot(total + (uint32_t)i, cta)] = 0xFFFFFFFFu;
-        }
-    }
     uint4* rows = reinterpret_cast<uint4*>(P.items);
     // one warp per group
     for (int grp = blk * kWarps + warp; grp < n_groups; grp += P.blocks * kWarps) {
-        const int cta = grp % kCluster;
-        const uint32_t n0 = (uint32_t)kChunks * (uint32_t)(grp / kCluster);   // number of the group's first chunk
         int cls[2];
         uint32_t stored[2];   // stored position of the row (asked for now: the answer is needed last)
         unsigned mask[2][4];
@@ -120,8 +97,6 @@ __device__ void deal_backward(const PrepParams& P, int blk) {
                 mask[i][c] = __ballot_sync(0xffffffffu, cls[i] == c);
             }
         }
-        if (lane < kChunks)
-            P.heads[chunk_slot(n0, (uint32_t)lane, cta)] = (uint32_t)grp | ((uint32_t)(kStageArrivals / kChunks) << 24);
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
 #pragma unroll
@@ -148,9 +123,8 @@ __device__ void deal_backward(const PrepParams& P, int blk) {
                             if (c2 < c || (c2 == c && i2 < i)) rank += __popc(mask[i2][c2] & res_mask);
                     rank += __popc(mask[i][c] & res_mask & ((1u << lane) - 1u));
                     const int pos = rank * 8 + (lane & 7);
-                    uint4* dst = rows + (size_t)chunk_slot(n0, (uint32_t)(pos / 16), cta) * 32 + pos % 16;
-                    dst[0] = rec;
-                    dst[16] = rec;
+                    const int w = (pos / 16 + grp / kProducerGroups) & 3;
+                    rows[((size_t)grp * 4 + w) * 16 + pos % 16] = rec;
                 }
             }
         }

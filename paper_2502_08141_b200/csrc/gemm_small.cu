@@ -16,6 +16,7 @@
 //                    the same accumulation.
 // It starts while project_kernel runs and waits for it only before the low-rank term (programmatic dependent launch).
 // No flags, no waits that need a limit, any number of such calls may share the GPU.
+#include "dequant.cuh"
 #include "gemm_params.cuh"
 #include "ptx.cuh"
 
@@ -187,64 +188,19 @@ __device__ __forceinline__ void fetch_codes(Codes<B>& c, const uint8_t* row, con
     c.a = __ldg(absmax + blk);
 }
 
-// The block's levels, scaled by its absmax and rounded to bf16 as lowra_decode does, in the form that expand16 wants.
-template <int B> struct Scaled;
-template <> struct Scaled<1> {
-    uint32_t base, d, f;     // both halves: the smaller pattern; the difference of the patterns; 0x10001 if level 0 is the larger one
-    __device__ __forceinline__ void set(const float* y, float a) {
-        const uint32_t LH = pack_bf16x2(__fmul_rn(y[0], a), __fmul_rn(y[1], a));
-        const uint32_t L = LH & 0xFFFFu, H = LH >> 16, lo = min(L, H);
-        base = lo * 0x10001u; d = max(L, H) - lo; f = (L > H) ? 0x10001u : 0u;
-    }
-    // elements 16 q .. 16 q + 15 of the block, two per word
-    __device__ __forceinline__ void expand16(const Codes<1>& c, int q, uint32_t (&o)[8]) const {
-        const uint32_t h = (q & 1) ? (c.w[q >> 1] >> 16) : (c.w[q >> 1] & 0xFFFFu);
-        const uint32_t z = h | (h << 15);
+template <int B>
+__device__ __forceinline__ void load_levels(float (&y)[1 << B], const float* row) {
+    if (B == 1) {
+        const float2 v = __ldg(reinterpret_cast<const float2*>(row));
+        y[0] = v.x; y[1] = v.y;
+    } else {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) o[i] = (((z >> (2 * i)) & 0x10001u) ^ f) * d + base;
-    }
-};
-template <> struct Scaled<2> {
-    uint32_t e01, e23;
-    __device__ __forceinline__ void set(const float* y, float a) {
-        e01 = pack_bf16x2(__fmul_rn(y[0], a), __fmul_rn(y[1], a));
-        e23 = pack_bf16x2(__fmul_rn(y[2], a), __fmul_rn(y[3], a));
-    }
-    __device__ __forceinline__ void expand16(const Codes<2>& c, int q, uint32_t (&o)[8]) const {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const uint32_t y = c.w[q] >> (4 * i);
-            const uint32_t s = (y & 3u) | ((y << 6) & 0x300u);
-            o[i] = __byte_perm(e01, e23, s * 0x22u + 0x1010u);
+        for (int i = 0; i < (1 << B) / 4; ++i) {
+            const float4 v = __ldg(reinterpret_cast<const float4*>(row) + i);
+            y[4 * i] = v.x; y[4 * i + 1] = v.y; y[4 * i + 2] = v.z; y[4 * i + 3] = v.w;
         }
     }
-};
-template <> struct Scaled<4> {
-    uint32_t lo[4], hi[4];   // low and high bytes of the sixteen patterns
-    __device__ __forceinline__ void set(const float* y, float a) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const float4 f = __ldg(reinterpret_cast<const float4*>(y) + i);
-            const uint32_t p = pack_bf16x2(__fmul_rn(f.x, a), __fmul_rn(f.y, a)), r = pack_bf16x2(__fmul_rn(f.z, a), __fmul_rn(f.w, a));
-            lo[i] = __byte_perm(p, r, 0x6420u);
-            hi[i] = __byte_perm(p, r, 0x7531u);
-        }
-    }
-    // four codes at a time: a byte permute looks up the low three bits of each in either half of the table, the fourth bits
-    // choose between the halves
-    __device__ __forceinline__ void expand16(const Codes<4>& c, int q, uint32_t (&o)[8]) const {
-#pragma unroll
-        for (int h = 0; h < 4; ++h) {
-            const uint32_t x = c.w[2 * q + (h >> 1)] >> (16 * (h & 1));
-            const uint32_t sel = x & 0x7777u;
-            const uint32_t upper = __byte_perm(0x0000FF00u, 0u, (x >> 3) & 0x1111u);   // 0xFF where the code is 8 or more
-            const uint32_t l = (__byte_perm(lo[0], lo[1], sel) & ~upper) | (__byte_perm(lo[2], lo[3], sel) & upper);
-            const uint32_t u = (__byte_perm(hi[0], hi[1], sel) & ~upper) | (__byte_perm(hi[2], hi[3], sel) & upper);
-            o[2 * h] = __byte_perm(l, u, 0x5140u);
-            o[2 * h + 1] = __byte_perm(l, u, 0x7362u);
-        }
-    }
-};
+}
 
 // Where 16-byte piece j (0 .. 7) of block t of token row m lies in a staged [tokens][256] tile: the pieces of a block are
 // exchanged among themselves so that the eight lanes of a shared-memory wavefront read eight different columns.
@@ -291,26 +247,33 @@ __device__ __forceinline__ void multiply_rows(const SmallParams& P, const SmallM
     };
     fetch(b0);
     stage(b0);
-    float ya[4], yb[4];
+    float ya[1 << B], yb[1 << B];
     if (B <= 2) {
-#pragma unroll
-        for (int i = 0; i < 2 * B; ++i) { ya[i] = __ldg(y0 + i); yb[i] = __ldg(y1 + i); }
+        load_levels<B>(ya, y0);
+        load_levels<B>(yb, y1);
     }
     for (int b = b0; b < b1; ++b) {
         const Codes<B> c0 = n0, c1 = n1;
         fetch(b + 1);
         stage(b + 1);
         Scaled<B> s0, s1;
-        s0.set(B <= 2 ? ya : y0, c0.a);
-        s1.set(B <= 2 ? yb : y1, c1.a);
+        if (B == 4) {   // (sixteen levels of two rows are too many registers to keep: read again, from L1)
+            load_levels<B>(ya, y0);
+            s0.set(ya, c0.a);
+            load_levels<B>(ya, y1);
+            s1.set(ya, c1.a);
+        } else {
+            s0.set(ya, c0.a);
+            s1.set(yb, c1.a);
+        }
         ptx::cp_async_wait<1>();
         ptx::named_barrier_sync(1 + half, 128);
         const uint32_t xs = x_smem + (uint32_t)((b - b0) & 1) * kStep;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {   // sixteen elements of the block
             uint32_t o0[8], o1[8];
-            s0.expand16(c0, q, o0);
-            s1.expand16(c1, q, o1);
+            s0.expand16(c0.w, q, o0);
+            s1.expand16(c1.w, q, o1);
 #pragma unroll
             for (int nt = 0; nt < NT8; ++nt) {
                 const uint4 xl = ld_shared_v4(xs + token_piece(nt * 8 + g, t, 2 * q)), xh = ld_shared_v4(xs + token_piece(nt * 8 + g, t, 2 * q + 1));

@@ -32,11 +32,6 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
     asm volatile("{ .reg .b64 st; mbarrier.arrive.shared::cta.b64 st, [%0]; }" ::"r"(smem_u32(bar)) : "memory");
 }
 
-__device__ __forceinline__ void mbar_arrive_n(uint64_t* bar, uint32_t count) {
-    asm volatile("{ .reg .b64 st; mbarrier.arrive.shared::cta.b64 st, [%0], %1; }" ::"r"(smem_u32(bar)), "r"(count)
-                 : "memory");
-}
-
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t bytes) {
     asm volatile("{ .reg .b64 st; mbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1; }" ::"r"(smem_u32(bar)),
                  "r"(bytes)
@@ -104,6 +99,22 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, v
     return __shfl_sync(0xffffffffu, ok, 0) != 0u;
 }
 
+// The same with every lane looking (all get the same answer): saves the shuffle, a trip through the shared-memory pipe that
+// costs a few hundred cycles while the tensor core is busy.
+__device__ __forceinline__ bool mbar_wait_lanes(uint64_t* bar, uint32_t parity, volatile uint32_t* abort, uint64_t limit_ns) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    const uint64_t t0 = globaltimer_ns();
+#pragma unroll 1
+    for (;;) {
+#pragma unroll 1
+        for (int i = 0; i < 64; ++i) {
+            if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+            __nanosleep(20);
+        }
+        if (__any_sync(0xffffffffu, *abort != 0u || globaltimer_ns() - t0 > limit_ns)) return false;
+    }
+}
+
 // ---------------------------------------------------------------------------------- fences
 __device__ __forceinline__ void fence_proxy_async_smem() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -135,12 +146,6 @@ __device__ __forceinline__ bool flag_wait(const uint32_t* flag, uint32_t want, v
     }
 }
 
-__device__ __forceinline__ uint32_t atom_add_acq_rel_shared(uint32_t* p, uint32_t v) {
-    uint32_t old;
-    asm volatile("atom.acq_rel.cta.shared::cta.add.u32 %0, [%1], %2;" : "=r"(old) : "r"(smem_u32(p)), "r"(v) : "memory");
-    return old;
-}
-
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
@@ -157,6 +162,42 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, i
         ::"r"(smem_u32(dst)),
         "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(x), "r"(y)
         : "memory");
+}
+
+// The same into the shared memory of this CTA of a pair, the bytes counted on a barrier of either CTA of the pair
+// (`cbar`: a shared::cluster address).
+__device__ __forceinline__ void tma_load_2d_pair(void* dst, const CUtensorMap* map, int x, int y, uint32_t cbar) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
+        ::"r"(smem_u32(dst)),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(cbar), "r"(x), "r"(y)
+        : "memory");
+}
+
+// ---------------------------------------------------------------------------------- tcgen05, CTA pairs
+// One MMA works on the 256 x N tile of two neighbouring CTAs of a cluster: each CTA's shared memory holds 128 rows of A and
+// N / 2 rows of B (at the same offsets in both), each CTA's tensor memory receives its 128 rows of D.  The MMAs are
+// issued by one thread of the CTA of even rank; allocation and release are done by a warp of both CTAs.
+__device__ __forceinline__ void tmem_alloc_pair(uint32_t* dst, uint32_t ncols) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(dst)), "r"(ncols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
+}
+__device__ __forceinline__ void umma_bf16_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                               uint32_t accumulate) {
+    asm volatile(
+        "{ .reg .pred p; setp.ne.b32 p, %4, 0; tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p; }" ::"r"(d_tmem),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+// Arrives on the barrier at this shared-memory offset in BOTH CTAs once every MMA issued so far by this thread has completed.
+__device__ __forceinline__ void umma_commit_pair(uint64_t* bar) {
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(smem_u32(bar)),
+                 "h"((uint16_t)3)
+                 : "memory");
 }
 
 // ---------------------------------------------------------------------------------- tcgen05
@@ -231,21 +272,14 @@ __device__ __forceinline__ void tmem_ld_32x32(uint32_t taddr, uint32_t (&v)[32])
         : "memory");
 }
 
-// Inverse of tmem_ld_32x32: thread t of the warp writes v[0..31] to lane (base + t), columns [col, col + 32).
-__device__ __forceinline__ void tmem_st_32x32(uint32_t taddr, const uint32_t (&v)[32]) {
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
-        "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
-        "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};" ::"r"(taddr),
-        "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]), "r"(v[9]),
-        "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]), "r"(v[16]), "r"(v[17]), "r"(v[18]),
-        "r"(v[19]), "r"(v[20]), "r"(v[21]), "r"(v[22]), "r"(v[23]), "r"(v[24]), "r"(v[25]), "r"(v[26]), "r"(v[27]),
-        "r"(v[28]), "r"(v[29]), "r"(v[30]), "r"(v[31])
-        : "memory");
-}
-__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
+// One lane of a converged warp (the same one every time).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{ .reg .pred q; elect.sync _|q, 0xffffffff; selp.u32 %0, 1, 0, q; }" : "=r"(p));
+    return p != 0u;
+}
 
 // ---------------------------------------------------------------------------------- thread-block cluster
 __device__ __forceinline__ uint32_t cluster_ctarank() {
@@ -262,11 +296,6 @@ __device__ __forceinline__ uint32_t map_to_cta(uint32_t saddr, uint32_t rank) {
 __device__ __forceinline__ void st_relaxed_cluster(uint32_t caddr, uint32_t v) {
     asm volatile("st.relaxed.cluster.shared::cluster.u32 [%0], %1;" ::"r"(caddr), "r"(v) : "memory");
 }
-__device__ __forceinline__ uint32_t ld_relaxed_cluster(const uint32_t* p) {   // own shared memory, written by a peer CTA
-    uint32_t v;
-    asm volatile("ld.relaxed.cluster.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
-    return v;
-}
 // Plain loads from the shared memory of any CTA of the cluster (address from map_to_cta); ordered by the
 // cluster barrier around them.
 __device__ __forceinline__ float4 ld_cluster_f4(uint32_t caddr) {
@@ -274,20 +303,9 @@ __device__ __forceinline__ float4 ld_cluster_f4(uint32_t caddr) {
     asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(caddr) : "memory");
     return v;
 }
-// Arrive (count times) on an mbarrier of any CTA of the cluster.  Relaxed: it orders nothing by itself (the data
-// it announces travels as bulk copies that the same barrier counts in bytes).
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t caddr, uint32_t count) {
-    asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0], %1;" ::"r"(caddr), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx_cluster(uint32_t caddr, uint32_t bytes) {
-    asm volatile("mbarrier.expect_tx.relaxed.cluster.shared::cluster.b64 [%0], %1;" ::"r"(caddr), "r"(bytes) : "memory");
-}
-// Asynchronous copy of `bytes` (a multiple of 16) from this CTA's shared memory into a peer CTA's; the bytes are
-// counted on the peer's mbarrier `cbar`.  Both addresses 16-byte aligned; dst and cbar are shared::cluster addresses.
-__device__ __forceinline__ void bulk_copy_to_cta(uint32_t cdst, uint32_t src, uint32_t bytes, uint32_t cbar) {
-    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(cdst), "r"(src), "r"(bytes), "r"(cbar)
-                 : "memory");
+// Arrive once on an mbarrier of any CTA of the cluster.
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t caddr) {
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(caddr) : "memory");
 }
 // Asynchronous copy of `bytes` (a multiple of 16) from global memory into this CTA's shared memory, counted in bytes
 // on an mbarrier of this CTA.  Both addresses 16-byte aligned.
@@ -311,13 +329,12 @@ __device__ __forceinline__ void st_shared_v4(uint32_t saddr, uint4 v) {
                  : "memory");
 }
 
-__device__ __forceinline__ void st_shared_f32(uint32_t saddr, float v) {
-    asm volatile("st.shared.f32 [%0], %1;" ::"r"(saddr), "f"(v) : "memory");
+__device__ __forceinline__ void st_global_v8(void* p, const uint32_t* v) {   // 32-byte aligned
+    asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]),
+                 "r"(v[5]), "r"(v[6]), "r"(v[7])
+                 : "memory");
 }
 
-__device__ __forceinline__ void cp_async_4(uint32_t saddr, const void* gptr) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(saddr), "l"(gptr) : "memory");
-}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() {
