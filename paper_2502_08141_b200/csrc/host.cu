@@ -1,6 +1,7 @@
 // Host side of the C ABI: status strings, the storage planner and argument validation.
 #include <string.h>
 
+#include <atomic>
 #include <mutex>
 
 #include "lowra_common.cuh"
@@ -28,12 +29,17 @@ lowra_status check_layout(const lowra_layout* L) {
 }
 
 lowra_status check_device() {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return LOWRA_ERR_CUDA;
-    int major = 0;
-    if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess)
-        return LOWRA_ERR_CUDA;
-    return major == 10 ? LOWRA_OK : LOWRA_ERR_ARCH;
+    static std::atomic<signed char> seen[kMaxDevices];   // per device: 0 not asked yet, 1 compute capability 10.x, -1 another
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return LOWRA_ERR_CUDA;
+    signed char known = seen[dev].load(std::memory_order_relaxed);
+    if (known == 0) {
+        int major = 0;
+        if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess) return LOWRA_ERR_CUDA;
+        known = major == 10 ? 1 : -1;
+        seen[dev].store(known, std::memory_order_relaxed);
+    }
+    return known == 1 ? LOWRA_OK : LOWRA_ERR_ARCH;
 }
 
 lowra_status ensure_smem_limit(const void* kernel, size_t bytes, SmemLimit* state) {
