@@ -39,18 +39,21 @@ struct SkinnyBarriers {
 static_assert(sizeof(SkinnyBarriers) <= 256, "barrier block");
 
 __global__ void __launch_bounds__(kSkinnyThreads, 2)
-skinny_kernel(const SkinnyArgs P, const int S, const __grid_constant__ CUtensorMap tmP, const __grid_constant__ CUtensorMap tmQ) {
+skinny_kernel(const __grid_constant__ SkinnyPair A, const int S) {
     extern __shared__ __align__(1024) unsigned char skinny_smem[];
     unsigned char* base = skinny_smem;
     SkinnyBarriers* bars = reinterpret_cast<SkinnyBarriers*>(base + kSkinnyRing);
     volatile uint32_t* abort_flag = &bars->abort;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int r0 = blockIdx.x * 128;
+    const bool second = (int)blockIdx.x >= A.tiles0;
+    const SkinnyProduct& P = A.p[second ? 1 : 0];
+    const int rp = A.rp;
+    const int r0 = ((int)blockIdx.x - (second ? A.tiles0 : 0)) * 128;
     const uint32_t crank = ptx::cluster_ctarank();            // which slice of the contraction
     const int n_blocks = (P.C + 63) / 64;
     const int kb0 = (int)((long long)crank * n_blocks / S), kb1 = (int)((long long)(crank + 1) * n_blocks / S);
     const int n_my = kb1 - kb0;
-    const uint32_t stage_bytes = kSkinnySmemP + (uint32_t)P.rp * 128u;   // 24 or 32 KB
+    const uint32_t stage_bytes = kSkinnySmemP + (uint32_t)rp * 128u;   // 24 or 32 KB
     const int stages = (int)(kSkinnyRing / stage_bytes);                  // 4 or 3
     const uint32_t tmem_cols = 128;                                       // >= rp, a power of two
     const bool aligned = (ptx::smem_u32(skinny_smem) & 1023u) == 0u;
@@ -60,8 +63,8 @@ skinny_kernel(const SkinnyArgs P, const int S, const __grid_constant__ CUtensorM
         ptx::mbar_init(&bars->tmem_full, 1);
         bars->abort = aligned ? 0u : 1u;
         ptx::fence_barrier_init();
-        ptx::prefetch_tensormap(&tmP);
-        ptx::prefetch_tensormap(&tmQ);
+        ptx::prefetch_tensormap(&P.tmP);
+        ptx::prefetch_tensormap(&P.tmQ);
     }
     if (warp == 1) ptx::tmem_alloc(&bars->tmem_base, tmem_cols);
     ptx::tc_fence_before();
@@ -69,11 +72,12 @@ skinny_kernel(const SkinnyArgs P, const int S, const __grid_constant__ CUtensorM
     ptx::tc_fence_after();
     const uint32_t tmem_base = bars->tmem_base;
     pdl_enter();   // the operands may come from the kernels launched before this one
+    if (A.clear_status && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *A.status = 0u;
     bool failed = !aligned;
 
     // fp32 partial tile [128 rows][rp + 4]: the padding spreads the rows of a warp over the banks
     float* part = reinterpret_cast<float*>(base);
-    const int pstride = P.rp + 4;
+    const int pstride = rp + 4;
 
     if (failed) {
         // shared memory not aligned as the swizzled tiles need: nothing is loaded or multiplied
@@ -82,21 +86,21 @@ skinny_kernel(const SkinnyArgs P, const int S, const __grid_constant__ CUtensorM
             int issued = 0;
             for (int i = 0; i < n_my; ++i) {
                 const int s = i % stages, kb = kb0 + i;
-                if (!ptx::mbar_wait(&bars->empty[s], ((i / stages) & 1u) ^ 1u, abort_flag, P.wait_ns)) { failed = true; bars->abort = 1u; break; }
+                if (!ptx::mbar_wait(&bars->empty[s], ((i / stages) & 1u) ^ 1u, abort_flag, A.wait_ns)) { failed = true; bars->abort = 1u; break; }
                 unsigned char* p_s = base + s * stage_bytes;
                 unsigned char* q_s = p_s + kSkinnySmemP;
                 ptx::mbar_arrive_expect_tx(&bars->full[s], stage_bytes);
                 // rows, columns and contraction indices past the end of a matrix read as zero
                 if (P.a_mn) {
-                    ptx::tma_load_2d(p_s, &tmP, r0, kb * 64, &bars->full[s]);
-                    ptx::tma_load_2d(p_s + 8192, &tmP, r0 + 64, kb * 64, &bars->full[s]);
+                    ptx::tma_load_2d(p_s, &P.tmP, r0, kb * 64, &bars->full[s]);
+                    ptx::tma_load_2d(p_s + 8192, &P.tmP, r0 + 64, kb * 64, &bars->full[s]);
                 } else {
-                    ptx::tma_load_2d(p_s, &tmP, kb * 64, r0, &bars->full[s]);
+                    ptx::tma_load_2d(p_s, &P.tmP, kb * 64, r0, &bars->full[s]);
                 }
                 if (P.b_mn) {
-                    for (int h = 0; h < P.rp / 64; ++h) ptx::tma_load_2d(q_s + h * 8192, &tmQ, h * 64, kb * 64, &bars->full[s]);
+                    for (int h = 0; h < rp / 64; ++h) ptx::tma_load_2d(q_s + h * 8192, &P.tmQ, h * 64, kb * 64, &bars->full[s]);
                 } else {
-                    ptx::tma_load_2d(q_s, &tmQ, kb * 64, 0, &bars->full[s]);
+                    ptx::tma_load_2d(q_s, &P.tmQ, kb * 64, 0, &bars->full[s]);
                 }
                 issued = i + 1;
             }
@@ -107,11 +111,11 @@ skinny_kernel(const SkinnyArgs P, const int S, const __grid_constant__ CUtensorM
         }
     } else if (warp == 1) {
         if (lane == 0) {
-            const uint32_t idesc = ptx::umma_idesc_bf16(128, P.rp) | (P.a_mn ? (1u << 15) : 0u) | (P.b_mn ? (1u << 16) : 0u);
+            const uint32_t idesc = ptx::umma_idesc_bf16(128, rp) | (P.a_mn ? (1u << 15) : 0u) | (P.b_mn ? (1u << 16) : 0u);
             const uint32_t a_step = P.a_mn ? 128u : 2u, b_step = P.b_mn ? 128u : 2u;   // 16 contraction indices further
             for (int i = 0; i < n_my; ++i) {
                 const int s = i % stages;
-                if (!ptx::mbar_wait(&bars->full[s], (i / stages) & 1u, abort_flag, P.wait_ns)) { failed = true; bars->abort = 1u; break; }
+                if (!ptx::mbar_wait(&bars->full[s], (i / stages) & 1u, abort_flag, A.wait_ns)) { failed = true; bars->abort = 1u; break; }
                 ptx::tc_fence_after();
                 const uint32_t p_addr = ptx::smem_u32(base + s * stage_bytes);
                 const uint32_t q_addr = p_addr + kSkinnySmemP;
@@ -128,10 +132,10 @@ skinny_kernel(const SkinnyArgs P, const int S, const __grid_constant__ CUtensorM
         // ------------------------------------------------------------------ TMEM -> fp32 partial tile in shared memory
         const int q = warp & 3;
         const int row = q * 32 + lane;
-        if (n_my > 0 && !ptx::mbar_wait_warp(&bars->tmem_full, 0u, abort_flag, P.wait_ns)) { failed = true; bars->abort = 1u; }
+        if (n_my > 0 && !ptx::mbar_wait_warp(&bars->tmem_full, 0u, abort_flag, A.wait_ns)) { failed = true; bars->abort = 1u; }
         if (!failed) {
             ptx::tc_fence_after();
-            for (int c0 = 0; c0 < P.rp; c0 += 32) {
+            for (int c0 = 0; c0 < rp; c0 += 32) {
                 uint32_t v[32];
                 if (n_my > 0) {
                     ptx::tmem_ld_32x32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, v);
@@ -149,7 +153,7 @@ skinny_kernel(const SkinnyArgs P, const int S, const __grid_constant__ CUtensorM
             ptx::tc_fence_before();
         }
     }
-    if (failed) atomicExch(P.status, aligned ? (uint32_t)LOWRA_ERR_TIMEOUT : (uint32_t)LOWRA_ERR_CUDA);
+    if (failed) atomicExch(A.status, aligned ? (uint32_t)LOWRA_ERR_TIMEOUT : (uint32_t)LOWRA_ERR_CUDA);
     __syncwarp();
     ptx::cluster_sync();   // every partial tile of the cluster is in place
 
@@ -160,7 +164,7 @@ skinny_kernel(const SkinnyArgs P, const int S, const __grid_constant__ CUtensorM
         const uint32_t part_addr = ptx::smem_u32(part);
         if (!P.transposed) {
             // out [R, ld_out]: four neighbouring columns per thread
-            const int c4n = P.rp / 4;
+            const int c4n = rp / 4;
             for (int u = t; u < rows_per * c4n; u += 128) {
                 const int row = row_base + u / c4n, col = (u % c4n) * 4;
                 const uint32_t addr = part_addr + (uint32_t)(row * pstride + col) * 4u;
@@ -180,7 +184,7 @@ skinny_kernel(const SkinnyArgs P, const int S, const __grid_constant__ CUtensorM
         } else {
             // out [n_cols, ld_out] = D^T.  A warp takes 8 rows x 16 columns of D: its loads read whole 64-byte runs of
             // a row, its stores write 8 neighbouring elements (rows of D) of 16 rows of out.
-            const int c4n = P.rp / 4;
+            const int c4n = rp / 4;
             const int lane_row = lane & 7, lane_c4 = lane >> 3;
             const int units = (rows_per / 8) * (c4n / 4);          // 8 x 16 patches of this CTA's rows
             for (int u = warp - 2; u < units; u += 4) {
@@ -212,11 +216,14 @@ skinny_kernel(const SkinnyArgs P, const int S, const __grid_constant__ CUtensorM
 
 }  // namespace
 
-// tmP: box of [64 c][64 rows] (a_mn) or [128 rows][64 c]; tmQ: box of [64 c][64 columns] (b_mn) or [rp columns][64 c].
-lowra_status launch_skinny(const CUtensorMap& tmP, const CUtensorMap& tmQ, const SkinnyArgs& a, cudaStream_t stream) {
+// The two gradients of a module, or its two down-projections, as one launch: their tiles share the SMs (a 4096-row product
+// alone has 32 tiles) and one fill and drain of the GPU.
+lowra_status launch_skinny(SkinnyPair& pair, cudaStream_t stream) {
     static SmemLimit limit = {};
     if (ensure_smem_limit(reinterpret_cast<const void*>(skinny_kernel), kSkinnySmemBytes, &limit) != LOWRA_OK) return LOWRA_ERR_CUDA;
-    const int tiles = (a.R + 127) / 128, n_blocks = (a.C + 63) / 64;
+    pair.tiles0 = (pair.p[0].R + 127) / 128;
+    const int tiles = pair.tiles0 + (pair.p[1].R + 127) / 128;
+    const int n0 = (pair.p[0].C + 63) / 64, n1 = (pair.p[1].C + 63) / 64, n_blocks = n0 > n1 ? n0 : n1;
     // split of the contraction: the one with the shortest estimated run = waves of CTAs x (blocks per CTA + a fixed
     // cost of set-up, pipeline fill and reduction, about six blocks' worth); every slice keeps four blocks or more
     int S = 1;
@@ -240,7 +247,7 @@ lowra_status launch_skinny(const CUtensorMap& tmP, const CUtensorMap& tmQ, const
     cfg.stream = stream;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, skinny_kernel, a, S, tmP, tmQ) == cudaSuccess ? LOWRA_OK : LOWRA_ERR_CUDA;
+    return cudaLaunchKernelEx(&cfg, skinny_kernel, pair, S) == cudaSuccess ? LOWRA_OK : LOWRA_ERR_CUDA;
 }
 
 }  // namespace lowra

@@ -283,8 +283,7 @@ lowra_status run_members(bool backward, const MemberArgs* mem, int count, int32_
 // Forward pass of members of few tokens each (any number of them, one shape): two launches for every kSmallMembers.
 // Their arguments have been checked as run_members does.  T_of: where member i's down-projected tokens go.
 lowra_status run_small(const MemberArgs* mem, uint16_t* const* T_of, int count, int32_t r, float s, void* workspace, cudaStream_t stream) {
-    SmallParams P;
-    memset(&P, 0, sizeof(P));
+    SmallParams<kSmallMembers> P;
     P.N = mem[0].layout->N;
     P.K = mem[0].layout->K;
     P.r = r;
@@ -585,54 +584,36 @@ lowra_status run_adapters(const uint16_t* X_dev, const uint16_t* dY_dev, int32_t
     uint32_t* status = reinterpret_cast<uint32_t*>(ws);
     const uint16_t* T = reuse ? T_in : reinterpret_cast<uint16_t*>(ws + w.off_T);
     const uint16_t* U = reuse ? U_in : reinterpret_cast<uint16_t*>(ws + w.off_U);
-    clear_status_kernel<<<1, 1, 0, stream>>>(status);
     const int rp = w.rp;
-    CUtensorMap tmX, tmXt, tmdY, tmdYt, tmA, tmB, tmT, tmU;
-    if (!make_map(&tmXt, X_dev, (uint64_t)M, (uint64_t)K, (uint64_t)K, 64) ||      // 64 tokens x 64 features (MN-major)
-        !make_map(&tmdYt, dY_dev, (uint64_t)M, (uint64_t)N, (uint64_t)N, 64) ||
-        !make_map(&tmT, T, (uint64_t)M, (uint64_t)rp, (uint64_t)rp, 64) ||
-        !make_map(&tmU, U, (uint64_t)M, (uint64_t)rp, (uint64_t)rp, 64))
-        return LOWRA_ERR_CUDA;
-    if (!reuse &&
-        (!make_map(&tmX, X_dev, (uint64_t)M, (uint64_t)K, (uint64_t)K, 128) ||      // rows of 64 features (K-major)
-         !make_map(&tmdY, dY_dev, (uint64_t)M, (uint64_t)N, (uint64_t)N, 128) ||
-         !make_map(&tmA, A_dev, (uint64_t)K, (uint64_t)r, (uint64_t)r, 64) ||       // 64 features x 64 ranks (MN-major)
-         !make_map(&tmB, B_dev, (uint64_t)r, (uint64_t)N, (uint64_t)N, (uint32_t)rp)))   // ranks x 64 channels (K-major)
-        return LOWRA_ERR_CUDA;
-    SkinnyArgs a;
+    SkinnyPair a;
     memset(&a, 0, sizeof(a));
     a.status = status;
     a.wait_ns = wait_limit_ns();
     a.rp = rp;
-    // Four skinny products; X and dY are each needed by two of them.  The two uses of the larger operand run back to
-    // back, so that its second reading can come from L2, and the smaller operand is read first and last: T, U, dB, dA
-    // when dY is the larger one, U, T, dA, dB otherwise.  With the caller's T and U only the two gradients are left.
-    auto down_T = [&]() {   // T = s X A: rows = tokens, contraction over the K input features
-        a.out = const_cast<uint16_t*>(T); a.R = M; a.C = K; a.n_cols = rp; a.ld_out = rp; a.a_mn = 0; a.b_mn = 1; a.transposed = 0; a.scale = s;
-        return launch_skinny(tmX, tmA, a, stream);
-    };
-    auto down_U = [&]() {   // U = s dY B^T: rows = tokens, contraction over the N output channels
-        a.out = const_cast<uint16_t*>(U); a.R = M; a.C = N; a.n_cols = rp; a.ld_out = rp; a.a_mn = 0; a.b_mn = 0; a.transposed = 0; a.scale = s;
-        return launch_skinny(tmdY, tmB, a, stream);
-    };
-    auto grad_A = [&]() {   // dA = X^T U: rows = input features, contraction over the tokens
-        a.out = dA_dev; a.R = K; a.C = M; a.n_cols = r; a.ld_out = r; a.a_mn = 1; a.b_mn = 1; a.transposed = 0; a.scale = 1.0f;
-        return launch_skinny(tmXt, tmU, a, stream);
-    };
-    auto grad_B = [&]() {   // dB = (dY^T T)^T: rows = output channels, written transposed
-        a.out = dB_dev; a.R = N; a.C = M; a.n_cols = r; a.ld_out = N; a.a_mn = 1; a.b_mn = 1; a.transposed = 1; a.scale = 1.0f;
-        return launch_skinny(tmdYt, tmT, a, stream);
-    };
-    if (reuse) {
-        if ((st = grad_A()) != LOWRA_OK) return st;
-        return grad_B();
+    a.clear_status = 1;
+    // T = s X A and U = s dY B^T: rows = tokens, contraction over the input features, resp. the output channels
+    if (!reuse) {
+        SkinnyProduct &t = a.p[0], &u = a.p[1];
+        if (!make_map(&t.tmP, X_dev, (uint64_t)M, (uint64_t)K, (uint64_t)K, 128) ||      // rows of 64 features (K-major)
+            !make_map(&t.tmQ, A_dev, (uint64_t)K, (uint64_t)r, (uint64_t)r, 64) ||       // 64 features x 64 ranks (MN-major)
+            !make_map(&u.tmP, dY_dev, (uint64_t)M, (uint64_t)N, (uint64_t)N, 128) ||
+            !make_map(&u.tmQ, B_dev, (uint64_t)r, (uint64_t)N, (uint64_t)N, (uint32_t)rp))   // ranks x 64 channels (K-major)
+            return LOWRA_ERR_CUDA;
+        t.out = const_cast<uint16_t*>(T); t.R = M; t.C = K; t.n_cols = t.ld_out = rp; t.a_mn = 0; t.b_mn = 1; t.transposed = 0; t.scale = s;
+        u.out = const_cast<uint16_t*>(U); u.R = M; u.C = N; u.n_cols = u.ld_out = rp; u.a_mn = 0; u.b_mn = 0; u.transposed = 0; u.scale = s;
+        if ((st = launch_skinny(a, stream)) != LOWRA_OK) return st;
+        a.clear_status = 0;
     }
-    if (N > K) {
-        if ((st = down_T()) != LOWRA_OK || (st = down_U()) != LOWRA_OK || (st = grad_B()) != LOWRA_OK) return st;
-        return grad_A();
-    }
-    if ((st = down_U()) != LOWRA_OK || (st = down_T()) != LOWRA_OK || (st = grad_A()) != LOWRA_OK) return st;
-    return grad_B();
+    // dA = X^T U: rows = input features, contraction over the tokens; dB = (dY^T T)^T: rows = output channels, written transposed
+    SkinnyProduct &ga = a.p[0], &gb = a.p[1];
+    if (!make_map(&ga.tmP, X_dev, (uint64_t)M, (uint64_t)K, (uint64_t)K, 64) ||      // 64 tokens x 64 features (MN-major)
+        !make_map(&ga.tmQ, U, (uint64_t)M, (uint64_t)rp, (uint64_t)rp, 64) ||
+        !make_map(&gb.tmP, dY_dev, (uint64_t)M, (uint64_t)N, (uint64_t)N, 64) ||
+        !make_map(&gb.tmQ, T, (uint64_t)M, (uint64_t)rp, (uint64_t)rp, 64))
+        return LOWRA_ERR_CUDA;
+    ga.out = dA_dev; ga.R = K; ga.C = M; ga.n_cols = r; ga.ld_out = r; ga.a_mn = 1; ga.b_mn = 1; ga.transposed = 0; ga.scale = 1.0f;
+    gb.out = dB_dev; gb.R = N; gb.C = M; gb.n_cols = r; gb.ld_out = N; gb.a_mn = 1; gb.b_mn = 1; gb.transposed = 1; gb.scale = 1.0f;
+    return launch_skinny(a, stream);
 }
 }  // namespace
 }  // namespace lowra

@@ -154,30 +154,39 @@ struct SmallMember {
     uint16_t *Y, *T;          // T [M, rp]: s X A, as the fused calls leave it
     int M;
 };
+template <int NB>   // members the kernel's parameters have room for
 struct SmallParams {
-    SmallMember m[kSmallMembers];
+    SmallMember m[NB];
     int count, N, K, r, rp;
     float s;
     uint32_t* status;
     int clear_status;         // the call brings no deal: its status word starts from zero
 };
-lowra_status launch_small(const SmallParams& P, cudaStream_t stream);
+lowra_status launch_small(const SmallParams<kSmallMembers>& P, cudaStream_t stream);
 
 // One skinny product D [R, rp] = P . Q (see gemm_grad.cu), written in bf16 as out [R, ld_out] or, transposed,
 // as out [n_cols, ld_out].
-struct SkinnyArgs {
+struct SkinnyProduct {
+    CUtensorMap tmP;  // box of [64 c][64 rows] (a_mn) or [128 rows][64 c]
+    CUtensorMap tmQ;  // box of [64 c][64 columns] (b_mn) or [rp columns][64 c]
     uint16_t* out;
-    uint32_t* status;
     int R;            // rows of D
     int C;            // length of the contraction
-    int rp;           // columns of D (64 or 128)
     int n_cols;       // columns of D that are written (a multiple of 16)
     int ld_out;
     int a_mn, b_mn;   // 1: the row (column) index of P (Q) is the contiguous one in memory
     int transposed;
     float scale;
+};
+// Two products that share nothing but a launch.
+struct SkinnyPair {
+    SkinnyProduct p[2];
+    uint32_t* status;
+    int rp;           // columns of D (64 or 128), of both
+    int tiles0;       // row tiles of the first product (set by the launcher)
+    int clear_status; // the status word starts from zero here
     unsigned long long wait_ns;   // limit of every device-side wait
 };
-lowra_status launch_skinny(const CUtensorMap& tmP, const CUtensorMap& tmQ, const SkinnyArgs& a, cudaStream_t stream);
+lowra_status launch_skinny(SkinnyPair& pair, cudaStream_t stream);
 
 }  // namespace lowra

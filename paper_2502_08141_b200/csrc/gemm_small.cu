@@ -30,9 +30,10 @@ constexpr int kSmallSpan = 256;         // contraction indices per step of a war
 constexpr int kPartPitch = kSmallRows + 4;   // fp32 words: neighbouring tokens of a partial tile 4 banks apart
 
 struct Unit { int member, m0; };        // up to 8 NT8 tokens of one member
-__device__ __forceinline__ Unit unit_at(const SmallParams& P, int u, int tokens) {
+template <int NB>
+__device__ __forceinline__ Unit unit_at(const SmallParams<NB>& P, int u, int tokens) {
     Unit r = {0, 0};
-    for (int i = 0; i + 1 < P.count; ++i) {
+    for (int i = 0; NB > 1 && i + 1 < P.count; ++i) {
         const int n = (P.m[i].M + tokens - 1) / tokens;
         if (u < n) break;
         u -= n;
@@ -65,7 +66,8 @@ __device__ __forceinline__ float ld_cluster_f32(uint32_t caddr) {
 constexpr int kProjectBatch = 4;        // steps of 16 contraction indices a warp fetches at a time
 
 // Grid: (slices of the contraction = cluster, tiles of 16 tokens of all members).
-__global__ void __launch_bounds__(kSmallThreads) project_kernel(const __grid_constant__ SmallParams P) {
+template <int NB>
+__global__ void __launch_bounds__(kSmallThreads) project_kernel(const __grid_constant__ SmallParams<NB> P) {
     extern __shared__ __align__(16) unsigned char project_smem[];
     asm volatile("griddepcontrol.wait;" ::: "memory");
     // the next kernel reads its operands right away, so it may start only now that everything before this kernel is complete
@@ -209,11 +211,11 @@ __device__ __forceinline__ uint32_t token_piece(int m, int t, int j) {
 }
 
 template <int B, int NT8>
-__device__ __forceinline__ void multiply_rows(const SmallParams& P, const SmallMember& W, int m0, int p0, int p_end, int slot, int slots,
+__device__ __forceinline__ void multiply_rows(int K, const SmallMember& W, int m0, int p0, int p_end, int slot, int slots,
                                               uint32_t x_smem, int half, float (&acc)[NT8][4]) {
     constexpr int c = B >> 1;
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const int n_span = (P.K + kSmallSpan - 1) / kSmallSpan, nb = P.K / kBlock;
+    const int n_span = (K + kSmallSpan - 1) / kSmallSpan, nb = K / kBlock;
     const int b0 = (int)((long long)slot * n_span / slots), b1 = (int)((long long)(slot + 1) * n_span / slots);
     // rows g and g + 8 of the warp's sixteen
     const bool live0 = p0 + g < p_end, live1 = p0 + g + 8 < p_end;
@@ -233,8 +235,8 @@ __device__ __forceinline__ void multiply_rows(const SmallParams& P, const SmallM
             const uint32_t dst = x_smem + (uint32_t)((b - b0) & 1) * kStep;
             for (int i = th; i < 8 * NT8 * 32; i += 128) {
                 const int m = i >> 5, t2 = (i >> 3) & 3, j = i & 7, k = b * kSmallSpan + t2 * 64 + j * 8;
-                const bool ok = m0 + m < W.M && k < P.K;
-                cp_async_16_zfill(dst + token_piece(m, t2, j), ok ? W.X + (size_t)(m0 + m) * P.K + k : W.X, ok);
+                const bool ok = m0 + m < W.M && k < K;
+                cp_async_16_zfill(dst + token_piece(m, t2, j), ok ? W.X + (size_t)(m0 + m) * K + k : W.X, ok);
             }
         }
         ptx::cp_async_commit();
@@ -288,8 +290,8 @@ __device__ __forceinline__ void multiply_rows(const SmallParams& P, const SmallM
 }
 
 // Grid: (row groups x slices of the contraction = cluster, token tiles of all members).
-template <int NT8>
-__global__ void __launch_bounds__(kSmallThreads, 2) small_kernel(const __grid_constant__ SmallParams P, const int slices) {
+template <int NT8, int NB>
+__global__ void __launch_bounds__(kSmallThreads, 2) small_kernel(const __grid_constant__ SmallParams<NB> P, const int slices) {
     extern __shared__ __align__(16) unsigned char small_smem[];
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     constexpr int kTokens = 8 * NT8;
@@ -334,9 +336,9 @@ __global__ void __launch_bounds__(kSmallThreads, 2) small_kernel(const __grid_co
     }
     if (any) {
         const uint32_t xs = ptx::smem_u32(small_smem) + (uint32_t)half * kTokenBytes;
-        if (c == 0) multiply_rows<1, NT8>(P, W, un.m0, p0, p_end, slot, slots, xs, half, acc);
-        else if (c == 1) multiply_rows<2, NT8>(P, W, un.m0, p0, p_end, slot, slots, xs, half, acc);
-        else multiply_rows<4, NT8>(P, W, un.m0, p0, p_end, slot, slots, xs, half, acc);
+        if (c == 0) multiply_rows<1, NT8>(P.K, W, un.m0, p0, p_end, slot, slots, xs, half, acc);
+        else if (c == 1) multiply_rows<2, NT8>(P.K, W, un.m0, p0, p_end, slot, slots, xs, half, acc);
+        else multiply_rows<4, NT8>(P.K, W, un.m0, p0, p_end, slot, slots, xs, half, acc);
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");                   // T is in place
 #pragma unroll
@@ -377,11 +379,11 @@ __global__ void __launch_bounds__(kSmallThreads, 2) small_kernel(const __grid_co
     ptx::cluster_sync();   // nobody leaves while a peer still reads its sums
 }
 
-template <int NT8>
-lowra_status launch_product(const SmallParams& P, int groups, int units, int slices, cudaStream_t stream) {
+template <int NT8, int NB>
+lowra_status launch_product(const SmallParams<NB>& P, int groups, int units, int slices, cudaStream_t stream) {
     constexpr size_t smem = 4u * (8 * NT8) * kSmallSpan * 2u + 2u * (8 * NT8) * kPartPitch * 4u;
     static SmemLimit limit = {};
-    if (ensure_smem_limit(reinterpret_cast<const void*>(small_kernel<NT8>), smem, &limit) != LOWRA_OK) return LOWRA_ERR_CUDA;
+    if (ensure_smem_limit(reinterpret_cast<const void*>(small_kernel<NT8, NB>), smem, &limit) != LOWRA_OK) return LOWRA_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -395,12 +397,11 @@ lowra_status launch_product(const SmallParams& P, int groups, int units, int sli
     cfg.stream = stream;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, small_kernel<NT8>, P, slices) == cudaSuccess ? LOWRA_OK : LOWRA_ERR_CUDA;
+    return cudaLaunchKernelEx(&cfg, small_kernel<NT8, NB>, P, slices) == cudaSuccess ? LOWRA_OK : LOWRA_ERR_CUDA;
 }
 
-}  // namespace
-
-lowra_status launch_small(const SmallParams& P, cudaStream_t stream) {
+template <int NB>
+lowra_status launch_members(const SmallParams<NB>& P, cudaStream_t stream) {
     int m16 = 0, groups = 0, most = 0;
     for (int i = 0; i < P.count; ++i) {
         const SmallMember& m = P.m[i];
@@ -417,7 +418,7 @@ lowra_status launch_small(const SmallParams& P, cudaStream_t stream) {
         const size_t fetch = (size_t)8 * kProjectBatch * 16 * (P.r * 2 + 16), sums = (size_t)(8 + 1) * 16 * P.r * 4;
         const size_t smem = fetch > sums ? fetch : sums;
         static SmemLimit limit = {};
-        if (ensure_smem_limit(reinterpret_cast<const void*>(project_kernel), smem, &limit) != LOWRA_OK) return LOWRA_ERR_CUDA;
+        if (ensure_smem_limit(reinterpret_cast<const void*>(project_kernel<NB>), smem, &limit) != LOWRA_OK) return LOWRA_ERR_CUDA;
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute attr[2];
         attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -431,7 +432,7 @@ lowra_status launch_small(const SmallParams& P, cudaStream_t stream) {
         cfg.stream = stream;
         cfg.attrs = attr;
         cfg.numAttrs = 2;
-        if (cudaLaunchKernelEx(&cfg, project_kernel, P) != cudaSuccess) return LOWRA_ERR_CUDA;
+        if (cudaLaunchKernelEx(&cfg, project_kernel<NB>, P) != cudaSuccess) return LOWRA_ERR_CUDA;
     }
     // ---- the product: slices of the contraction until the grid is about three CTAs per two places, as long as every warp keeps
     // a step of 256.  The choice depends on the weight's shape alone, so that a member's result does not depend on its company.
@@ -441,9 +442,20 @@ lowra_status launch_small(const SmallParams& P, cudaStream_t stream) {
     const int nt8 = most <= 8 ? 1 : most <= 16 ? 2 : 4;
     int units = 0;
     for (int i = 0; i < P.count; ++i) units += (P.m[i].M + 8 * nt8 - 1) / (8 * nt8);
-    if (nt8 == 1) return launch_product<1>(P, groups, units, slices, stream);
-    if (nt8 == 2) return launch_product<2>(P, groups, units, slices, stream);
-    return launch_product<4>(P, groups, units, slices, stream);
+    if (nt8 == 1) return launch_product<1, NB>(P, groups, units, slices, stream);
+    if (nt8 == 2) return launch_product<2, NB>(P, groups, units, slices, stream);
+    return launch_product<4, NB>(P, groups, units, slices, stream);
+}
+
+}  // namespace
+
+// (A call with one member carries 0.3 KB of kernel parameters instead of 1.5 KB, which its launches show.)
+lowra_status launch_small(const SmallParams<kSmallMembers>& P, cudaStream_t stream) {
+    if (P.count > 1) return launch_members<kSmallMembers>(P, stream);
+    SmallParams<1> Q;
+    Q.m[0] = P.m[0];
+    Q.count = 1; Q.N = P.N; Q.K = P.K; Q.r = P.r; Q.rp = P.rp; Q.s = P.s; Q.status = P.status; Q.clear_status = P.clear_status;
+    return launch_members<1>(Q, stream);
 }
 
 }  // namespace lowra
