@@ -415,16 +415,18 @@ lowra_status lowra_lora_forward_static(const lowra_layout* layout, const uint8_t
  *     assign:  bucket of n = number of current thresholds <= n
  *     levels:  y_j <- sum(w n) / sum(w) over bucket j   (an empty bucket keeps its level)
  *     thresholds: t_j <- (y_j + y_{j+1}) / 2
- * in fp64.  Output tables, fp32 [N, 16], original row order: maps = (float) y (unused entries 0),
+ * in fp64, the sums in 64-bit fixed point (multiples of 2^-46 of the channel's largest weight or, in buckets lighter
+ * than a quarter of that, of the bucket's).  Output tables, fp32 [N, 16], original row order: maps = (float) y (unused entries 0),
  * thresholds[j] = (float)(((double) maps[j] + (double) maps[j+1]) / 2) (unused entries +infinity) - directly
  * usable by lowra_encode / lowra_decode.
  *   W_dev                 fp32 [N, K] row-major, original row order                      (in)
  *   init_levels_host      fp64 [3][16] HOST: starting levels for 1-, 2-, 4-bit rows      (in; the appendix
  *   init_thresholds_host  fp64 [3][16] HOST: starting thresholds                          on initialisation)
  *   iterations            0 .. 1000 (the paper runs 2)
- * The sums are formed by a fixed parallel tree, not in index order: results are reproducible from run to run
- * and agree with a serial fp64 implementation to rounding.  K * 4 bytes must fit in shared memory
- * (K <= 40960), else LOWRA_ERR_SHAPE.  Uses layout->precs_dev only (perm / offsets are not needed).
+ * The sums do not depend on the order of the additions: results are reproducible from run to run, the same whatever
+ * else the matrix holds, and agree with a serial fp64 implementation to rounding.  A channel that holds a NaN or an
+ * infinity gets NaN levels (if iterations > 0).  K * 4 bytes must fit in shared memory
+ * (K <= 40960), else LOWRA_ERR_SHAPE.  Uses counts, precs_dev and perm_dev of the layout (the offsets are not needed).
  */
 lowra_status lowra_learn_codebooks(const lowra_layout* layout, const float* W_dev, const double* init_levels_host,
                                    const double* init_thresholds_host, int32_t iterations, float* maps_dev,

@@ -6,26 +6,19 @@
 // absmax normalisation exactly as in lowra_encode), each weighted by the absmax of its block; starting from the
 // given levels y and thresholds t, T times: assign every value to its bucket (number of thresholds <= n),
 // replace every level by the weighted mean of its bucket (an empty bucket keeps its level), set the thresholds
-// to the midpoints of neighbouring levels.  All of that in fp64.  Output: the levels rounded to fp32 and the
+// to the midpoints of neighbouring levels.  Levels and thresholds in fp64, sums in 64-bit fixed point.  Output: the levels rounded to fp32 and the
 // midpoints of those fp32 levels (computed in fp64, rounded to fp32), in [N, 16] tables.
 //
-// One CTA per row (as many CTAs as rows): the row is read from HBM once (4 bytes per element, the
-// kernel's only traffic), normalised on its way into shared memory; the T passes run out of shared memory.
-// Every thread keeps private fp64 sums per bucket: in registers for 1 and 2 bits, in a bank-conflict-free
-// slice of shared memory for 4 bits; the block's weight enters once per sixteen elements (they are added up exactly
-// first); a fixed reduction tree adds the threads' sums up (a halving exchange inside a warp, then across warps), so
-// results are reproducible from run to run - but the order of the fp64 operations is not the index order of a
-// serial loop, so sums agree with a serial implementation to rounding only.  One barrier per round; every warp forms
-// the new levels and thresholds itself; a row whose thresholds have settled (as fp32 numbers) skips its remaining rounds.
+// Two kernels.  learn_kernel adds the whole row up in every round.  sorted_learn_kernel brings the row's values into order once and
+// then needs a few hundred of them per round; it takes over where the rounds are many or expensive enough (sorted_pays).
+#include <float.h>
+#include <math.h>
 #include <string.h>
 
 #include "lowra_common.cuh"
 
 namespace lowra {
 
-constexpr int kLearnThreads = 128;
-constexpr int kLearnWarps = kLearnThreads / 32;
-constexpr int kLoadsInFlight = 8;   // 128-bit loads a thread issues before it looks at the first one (a 4096-element row in one go)
 
 struct LearnParams {
     RowLayout L;
@@ -34,29 +27,97 @@ struct LearnParams {
     float* thresholds;    // likewise
     int iterations;
     int N, K;             // the three-precision form has no layout: every row is learnt at 1, 2 and 4 bits
+    int row0;             // this launch's rows: stored rows row0 .. row0 + grid - 1
+    int turn;             // see enter()
+    int bins;             // sorted rows: cells
     double init_y[3][16];  // initial levels per class (1, 2, 4 bits)
     double init_t[3][16];  // initial thresholds per class
 };
+
+// The rows of one call may go to two launches, which know nothing of each other's rows.  turn 1, the first of two, lets the second
+// begin once everything before the call is complete; turn 2 does not wait for the first before it begins but before it ends, so that
+// what comes after it may rely on both.  turn 0: a launch by itself.
+__device__ __forceinline__ void enter(int turn) {
+    if (turn != 2) asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void leave(int turn) {
+    if (turn == 2) asm volatile("griddepcontrol.wait;" ::: "memory");
+}
 
 // NV sums per lane (NV = 4, 8 or 16) added up over the warp: instead of NV butterflies over all 32 lanes, every step
 // hands half of a lane's values to its partner and adds the partner's other half to its own, so that the number of
 // values halves with the distance; once a lane holds one value the remaining steps are plain butterflies.  Afterwards
 // the lanes whose low bits are zero hold the totals: value number lane / (32 / NV) in v[0].  A fixed order of additions.
 template <int NV>
-__device__ __forceinline__ void warp_sums(double (&v)[NV], int lane) {
+__device__ __forceinline__ void warp_sums(long long (&v)[NV], int lane) {
     int d = 16;
 #pragma unroll
     for (int n = NV; n > 1; n >>= 1, d >>= 1) {
         const bool upper = (lane & d) != 0;
 #pragma unroll
         for (int k = 0; k < n / 2; ++k) {
-            const double send = upper ? v[k] : v[k + n / 2];
-            const double keep = upper ? v[k + n / 2] : v[k];
+            const long long send = upper ? v[k] : v[k + n / 2];
+            const long long keep = upper ? v[k + n / 2] : v[k];
             v[k] = keep + __shfl_xor_sync(0xffffffffu, send, d);
         }
     }
 #pragma unroll
     for (; d >= 1; d >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], d);
+}
+
+// ---------------------------------------------------------------------------------------------------------------------------------
+// The arithmetic of both kernels.  A bucket's sums of w and of w * n are formed on a grid, so that they do not depend on the order
+// of the additions: results are reproducible, and the same whichever kernel takes the row.  Let the row's largest weight be below
+// 2^e.  fp64 numbers from 64 * 2^e to 128 * 2^e are multiples of u = 2^(e - 46), and adding to g = 96 * 2^e takes w (to nearest) and w * n
+// (down) to that grid: s + w * n, one fused multiply-add rounding down, is s plus w * n taken down, whatever s is, so that a
+// run of sixteen elements is a chain of these.  The sums are whole numbers of u, added up in 64-bit integers.  Where a bucket weighs a quarter of the largest weight or more its level is right to its number of
+// elements * 2^-43 (usually: to 2^-44); otherwise - few or light elements, or none - it is added up again on a grid of its own.
+constexpr long long kLight = 1ll << 44;   // u
+__device__ __forceinline__ double grid_of(float most) {   // g
+    return 96.0 * (most > 0.0f && most < INFINITY ? ldexp(1.0, ilogbf(most) + 1) : 1.0);
+}
+__device__ __forceinline__ unsigned long long grid_bits(double x) { return (unsigned long long)__double_as_longlong(x); }
+__device__ __forceinline__ long long grid_product(double n, double w, double g) { return (long long)(grid_bits(__fma_rd(n, w, g)) - grid_bits(g)); }
+__device__ __forceinline__ long long grid_weight(double w, double g) { return (long long)(grid_bits(w + g) - grid_bits(g)); }
+// A block's weight in multiples of 2^e (for the grid 96), where that is kept instead of the absmax; what is positive stays positive.
+constexpr double kGrid = 96.0;
+__device__ __forceinline__ float scaled_weight(float m, float row_most) {
+    return m > 0.0f && row_most < INFINITY ? fmaxf((float)ldexp((double)m, -ilogbf(row_most) - 1), FLT_MIN) : 0.0f;
+}
+// the larger one; NaN if one is NaN (a row that holds a NaN, an infinity or a block whose reciprocal overflows has no mean: its
+// levels come out as NaN)
+__device__ __forceinline__ float max_nan(float a, float b) {
+    float m;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(m) : "f"(a), "f"(b));
+    return m;
+}
+
+// The mean of a light bucket's elements [t_lo, t_hi) on a grid of its own (by a whole warp), or `keep` if they weigh nothing.
+// element(p): value and weight number p of p0 .. p1 - 1, which hold the bucket.
+template <typename F>
+__device__ __forceinline__ double light_mean(F element, int p0, int p1, float t_lo, float t_hi, double keep) {
+    const int lane = threadIdx.x & 31;
+    float most = 0.0f;
+    for (int p = p0 + lane; p < p1; p += 32) {
+        const float2 e = element(p);
+        if (t_lo <= e.x && e.x < t_hi) most = fmaxf(most, e.y);
+    }
+#pragma unroll
+    for (int d = 16; d >= 1; d >>= 1) most = fmaxf(most, __shfl_xor_sync(0xffffffffu, most, d));
+    if (!(most > 0.0f)) return keep;
+    const double g = grid_of(most);
+    long long wn = 0, w = 0;
+    for (int p = p0 + lane; p < p1; p += 32) {
+        const float2 e = element(p);
+        if (t_lo <= e.x && e.x < t_hi) {
+            wn += grid_product((double)e.x, (double)e.y, g);
+            w += grid_weight((double)e.y, g);
+        }
+    }
+#pragma unroll
+    for (int d = 16; d >= 1; d >>= 1) { wn += __shfl_xor_sync(0xffffffffu, wn, d); w += __shfl_xor_sync(0xffffffffu, w, d); }
+    return (double)wn / (double)w;
 }
 
 // number of thresholds <= x among t[0 .. L-2] (sorted): branch-free binary search, L = 2, 4 or 16.
@@ -82,45 +143,107 @@ __device__ __forceinline__ int bucket_of(float x, const float* tf) {
 // wavefront fall into eight different 16-byte columns, in the rounds' reads and in the loader's writes alike.
 __device__ __forceinline__ int quad_slot(int q) { return q ^ ((q >> 3) & 3); }
 
-// The row: coalesced 128-bit loads (all of a thread's loads in flight together); sixteen neighbouring lanes hold one
-// 64-element block between them, so the block's absmax is four shuffles away and the values go to shared memory
-// already normalised (as in lowra_encode: reciprocal rounded to nearest, one multiplication).  Ends with a barrier.
-__device__ void load_row(const LearnParams& P, int r, float* xs, float* ws) {
+// The row: asynchronous coalesced 128-bit copies, all of them in flight together; then every thread normalises sixteen elements at a
+// time where they lie (as in lowra_encode: reciprocal rounded to nearest, one multiplication): the four lanes that hold a
+// 64-element block between them find its absmax in two shuffles.  Returns the row's largest absmax.  Ends with a barrier.
+template <int THREADS>
+__device__ float load_row(const LearnParams& P, int r, float* xs, float* ws, float* most_of) {
     const int K = P.K;
     const int tid = threadIdx.x;
     const float* wrow = P.W + (size_t)r * K;
-    for (int i0 = 0; i0 < K; i0 += 4 * kLoadsInFlight * kLearnThreads) {
-        float4 v[kLoadsInFlight];
+    for (int i = 4 * tid; i < K; i += 4 * THREADS)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(xs + 4 * quad_slot(i >> 2))), "l"(wrow + i) : "memory");
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    float most = 0.0f;
+    for (int run = tid; run < (K / 16 + 31) / 32 * 32; run += THREADS) {   // (a warp stays together)
+        float4 v[4];
+        float m = 0.0f;
 #pragma unroll
-        for (int u = 0; u < kLoadsInFlight; ++u) {
-            const int i = i0 + 4 * (u * kLearnThreads + tid);
-            v[u] = (i < K) ? ld_stream_f4(wrow + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int q = 0; q < 4; ++q) {
+            v[q] = run < K / 16 ? *reinterpret_cast<const float4*>(xs + 4 * quad_slot(4 * run + q)) : make_float4(0.f, 0.f, 0.f, 0.f);
+            m = max_nan(max_nan(m, max_nan(fabsf(v[q].x), fabsf(v[q].y))), max_nan(fabsf(v[q].z), fabsf(v[q].w)));
         }
+        m = max_nan(m, __shfl_xor_sync(0xffffffffu, m, 1));
+        m = max_nan(m, __shfl_xor_sync(0xffffffffu, m, 2));
+        const float inv = (m == 0.0f) ? 0.0f : __frcp_rn(m);
+        most = max_nan(max_nan(most, m), __fmul_rn(inv, 0.0f));
+        if (run < K / 16) {
 #pragma unroll
-        for (int u = 0; u < kLoadsInFlight; ++u) {
-            const int i = i0 + 4 * (u * kLearnThreads + tid);   // K is a multiple of 128: a warp is in or out as a whole
-            float m = fmaxf(fmaxf(fabsf(v[u].x), fabsf(v[u].y)), fmaxf(fabsf(v[u].z), fabsf(v[u].w)));
-#pragma unroll
-            for (int d = 8; d >= 1; d >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, d));
-            const float inv = (m == 0.0f) ? 0.0f : __frcp_rn(m);
-            if (i < K) {
-                *reinterpret_cast<float4*>(xs + 4 * quad_slot(i >> 2)) =
-                    make_float4(__fmul_rn(v[u].x, inv), __fmul_rn(v[u].y, inv), __fmul_rn(v[u].z, inv), __fmul_rn(v[u].w, inv));
-                if ((tid & 15) == 0) ws[i / kBlock] = m;
-            }
+            for (int q = 0; q < 4; ++q)
+                *reinterpret_cast<float4*>(xs + 4 * quad_slot(4 * run + q)) =
+                    make_float4(__fmul_rn(v[q].x, inv), __fmul_rn(v[q].y, inv), __fmul_rn(v[q].z, inv), __fmul_rn(v[q].w, inv));
+            if ((run & 3) == 0) ws[run >> 2] = m;
         }
     }
+#pragma unroll
+    for (int d = 4; d < 32; d <<= 1) most = max_nan(most, __shfl_xor_sync(0xffffffffu, most, d));
+    if ((tid & 31) == 0) most_of[tid >> 5] = most;
     __syncthreads();
+#pragma unroll
+    for (int w = 0; w < THREADS / 32; ++w) most = max_nan(most, most_of[w]);
+    return most;
+}
+
+// learn_kernel.  One CTA per row: the row is read from HBM once, normalised on its way into shared memory; the T passes run out of
+// shared memory.  Every thread keeps private sums per bucket: in registers for 1 and 2 bits, in a bank-conflict-free
+// slice of shared memory for 4 bits; they are added up by a halving exchange inside a warp, then across warps.  One barrier
+// per round; every warp forms the new levels and thresholds itself; a row whose thresholds have settled (as fp32 numbers) skips its
+// remaining rounds.
+//
+__device__ __noinline__ double light_mean_row(const float* xs, const float* ws, float row_most, int K, float t_lo, float t_hi, double keep) {
+    return light_mean([&](int p) { return make_float2(xs[4 * quad_slot(p >> 2) + (p & 3)], scaled_weight(ws[p / kBlock], row_most)); }, 0, K,
+                      t_lo, t_hi, keep);
+}
+
+// One pass at 1 or 2 bits: this thread's sums over the elements at or above threshold j - 1 (j >= 1) and, if ALL, over all (j = 0).
+template <int B, int THREADS, bool ALL>
+__device__ __forceinline__ void few_buckets(const float* xs, const float* ws, int K, double g, const float* th, unsigned long long* cn, long long* cw) {
+    constexpr int Lv = 1 << B, j0 = ALL ? 0 : 1;
+#pragma unroll
+    for (int j = j0; j < Lv; ++j) { cn[j] = 0ull; cw[j] = 0; }
+    for (int run = threadIdx.x; run < K / 16; run += THREADS) {   // elements 16 run .. 16 run + 15, all in block run / 4
+        const float4 xa = *reinterpret_cast<const float4*>(xs + 4 * quad_slot(4 * run));
+        const float4 xb = *reinterpret_cast<const float4*>(xs + 4 * quad_slot(4 * run + 1));
+        const float4 xc = *reinterpret_cast<const float4*>(xs + 4 * quad_slot(4 * run + 2));
+        const float4 xd = *reinterpret_cast<const float4*>(xs + 4 * quad_slot(4 * run + 3));
+        const double w = (double)ws[run >> 2];
+        const float xf[16] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y, xb.z, xb.w, xc.x, xc.y, xc.z, xc.w, xd.x, xd.y, xd.z, xd.w};
+        double s[Lv];
+        int cq[Lv];
+#pragma unroll
+        for (int j = j0; j < Lv; ++j) { s[j] = g; cq[j] = 0; }
+#pragma unroll
+        for (int u = 0; u < 16; ++u) {
+            const double x = (double)xf[u];
+            if (ALL) s[0] = __fma_rd(x, w, s[0]);
+#pragma unroll
+            for (int j = 1; j < Lv; ++j) {
+                int hi;
+                asm("{\n\t.reg .pred p;\n\tsetp.le.f32 p, %2, %3;\n\tselp.b32 %0, %4, 0, p;\n\t@p add.s32 %1, %1, 1;\n\t}"
+                    : "=r"(hi), "+r"(cq[j]) : "f"(th[j - 1]), "f"(xf[u]), "r"(__double2hiint(x)));
+                s[j] = __fma_rd(__hiloint2double(hi, __double2loint(x)), w, s[j]);
+            }
+        }
+        const long long wg = grid_weight(w, g);
+        if (ALL) cq[0] = 16;
+#pragma unroll
+        for (int j = j0; j < Lv; ++j) {
+            cn[j] += grid_bits(s[j]) - grid_bits(g);
+            cw[j] += cq[j] * wg;
+        }
+    }
 }
 
 // T rounds on the row parked in shared memory, at B bits; tables to maps_out / thr_out ([16] each).
 // One barrier per round: the warps leave their partial sums in shared memory (two buffers, used in turn), meet once, and
 // then EVERY warp forms the new levels and thresholds for itself - lane j holds level j and threshold j in registers, the
-// same numbers in every warp since they come from the same partial sums in the same order - so nobody waits for a
-// first warp to publish them.
-template <int B>
-__device__ void learn_row(const LearnParams& P, const float* xs, const float* ws, double* acc, double* red2, float* tfw_all,
-                          float* maps_out, float* thr_out) {
+// same numbers in every warp since they come from the same sums - so nobody waits for a first warp to publish them.
+template <int B, int THREADS>
+__device__ void learn_row(const LearnParams& P, const float* xs, const float* ws, float row_most, long long* acc, long long* red2,
+                          float* tfw_all, int iterations, float* maps_out, float* thr_out) {
+    constexpr int kLearnThreads = THREADS, kLearnWarps = THREADS / 32;
     constexpr int Lv = 1 << B;      // levels
     constexpr int c = B >> 1;       // class index
     const int K = P.K;
@@ -133,84 +256,70 @@ __device__ void learn_row(const LearnParams& P, const float* xs, const float* ws
 #pragma unroll
         for (int j = 0; j < Lv - 1; ++j) th[j] = __double2float_ru(P.init_t[c][j]);
     } else {
+        __syncthreads();   // (a row's first tenant of this space was its absmax)
         if (lane < 16) tf[lane] = tlane;
         __syncwarp();
     }
 
-    for (int it = 0; it < P.iterations; ++it) {
-        double* red = red2 + (it & 1) * (2 * 16 * kLearnWarps);
+    unsigned long long all_n = 0ull;
+    long long all_w = 0;
+    const double g = grid_of(row_most);
+    const bool bad = !(row_most < INFINITY) && iterations > 0;
+    for (int it = 0; it < iterations; ++it) {
+        long long* red = red2 + (it & 1) * (2 * 16 * kLearnWarps);
         // ---- one pass: private sums of w * n and w per bucket.  The weight is the same for the sixteen elements a thread
-        // takes at a time (a quarter of a 64-element block), so the elements themselves are added up per bucket first
-        // (exactly: sixteen fp32 values in fp64) and counted, and the weight enters once per sixteen elements and bucket.
+        // takes at a time (a quarter of a 64-element block): the elements are counted per bucket, and the weight's sum follows.
         if (B <= 2) {
-            // Few buckets: no bucket index at all.  cn[0] / cd[0] take the elements below the first threshold, cn[j] /
-            // cd[j] (j >= 1) everything at or above threshold j - 1 - predicated adds - and a bucket's sums are the
-            // difference of two neighbours (which were added up over the same elements in the same order wherever the
-            // bucket is empty, so that an empty bucket has exactly zero weight).
-            double cn[Lv], cd[Lv];
-#pragma unroll
-            for (int j = 0; j < Lv; ++j) cn[j] = cd[j] = 0.0;
-            for (int run = tid; run < K / 16; run += kLearnThreads) {   // elements 16 run .. 16 run + 15, all in block run / 4
-                const float4 xa = *reinterpret_cast<const float4*>(xs + 4 * quad_slot(4 * run));
-                const float4 xb = *reinterpret_cast<const float4*>(xs + 4 * quad_slot(4 * run + 1));
-                const float4 xc = *reinterpret_cast<const float4*>(xs + 4 * quad_slot(4 * run + 2));
-                const float4 xd = *reinterpret_cast<const float4*>(xs + 4 * quad_slot(4 * run + 3));
-                const double w = (double)ws[run >> 2];
-                const float xf[16] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y, xb.z, xb.w, xc.x, xc.y, xc.z, xc.w, xd.x, xd.y, xd.z, xd.w};
-                double sq[Lv];
-                int cq[Lv];
-#pragma unroll
-                for (int j = 0; j < Lv; ++j) { sq[j] = 0.0; cq[j] = 0; }
-#pragma unroll
-                for (int u = 0; u < 16; ++u) {
-                    const double x = (double)xf[u];
-                    if (th[0] <= xf[u]) { sq[1] += x; ++cq[1]; } else { sq[0] += x; ++cq[0]; }
-#pragma unroll
-                    for (int j = 2; j < Lv; ++j)
-                        if (th[j - 1] <= xf[u]) { sq[j] += x; ++cq[j]; }
-                }
-#pragma unroll
-                for (int j = 0; j < Lv; ++j) {
-                    cn[j] = fma(w, sq[j], cn[j]);
-                    cd[j] = fma(w, (double)cq[j], cd[j]);
-                }
-            }
-            double v[2 * Lv];
+            // Few buckets: no bucket index at all.  cn[0] / cw[0] take all elements, cn[j] / cw[j] (j >= 1) those at or above
+            // threshold j - 1, and a bucket's sums are the difference of two neighbours.  An element that is out becomes
+            // a tiny positive number (the upper half of the fp64 number zero), which rounding down leaves without effect: one
+            // selection, where the predicated addition comes out of the compiler as two of the sum (1 bit, 4096 x 4096: 8.2 against
+            // 10 us a round).
+            // (The first round forms cn[0] for all.)
+            unsigned long long cn[Lv];
+            long long cw[Lv];
+            if (it == 0) few_buckets<B, THREADS, true>(xs, ws, K, g, th, cn, cw);
+            else few_buckets<B, THREADS, false>(xs, ws, K, g, th, cn, cw);
+            if (it == 0) { all_n = cn[0]; all_w = cw[0]; }
+            cn[0] = all_n;
+            cw[0] = all_w;
+            long long v[2 * Lv];
 #pragma unroll
             for (int j = 0; j < Lv; ++j) {
-                v[2 * j] = (j == 0 || j == Lv - 1) ? cn[j] : cn[j] - cn[j + 1];
-                v[2 * j + 1] = (j == 0 || j == Lv - 1) ? cd[j] : cd[j] - cd[j + 1];
+                v[2 * j] = (long long)(j == Lv - 1 ? cn[j] : cn[j] - cn[j + 1]);
+                v[2 * j + 1] = j == Lv - 1 ? cw[j] : cw[j] - cw[j + 1];
             }
             warp_sums<2 * Lv>(v, lane);
             if ((lane & (32 / (2 * Lv) - 1)) == 0) red[(lane / (32 / (2 * Lv))) * kLearnWarps + warp] = v[0];
         } else {
             // 16 buckets: the sums live in shared memory, one (w n, w) pair per thread and bucket; eight elements at a
             // time, their bucket searches side by side
-            double2* acc2 = reinterpret_cast<double2*>(acc);
+            longlong2* acc2 = reinterpret_cast<longlong2*>(acc);
 #pragma unroll
-            for (int j = 0; j < Lv; ++j) acc2[j * kLearnThreads + tid] = make_double2(0.0, 0.0);
+            for (int j = 0; j < Lv; ++j) acc2[j * kLearnThreads + tid] = make_longlong2(0, 0);
             for (int run = tid; run < K / 8; run += kLearnThreads) {
                 const float4 xa = *reinterpret_cast<const float4*>(xs + 4 * quad_slot(2 * run));
                 const float4 xb = *reinterpret_cast<const float4*>(xs + 4 * quad_slot(2 * run + 1));
                 const double w = (double)ws[run >> 3];
+                const long long wg = grid_weight(w, g);
                 const float xf[8] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y, xb.z, xb.w};
                 int b[8];
 #pragma unroll
                 for (int u = 0; u < 8; ++u) b[u] = bucket_of<B>(xf[u], tf);
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
-                    double2 a = acc2[b[u] * kLearnThreads + tid];
-                    a.x = fma(w, (double)xf[u], a.x);
-                    a.y += w;
+                    longlong2 a = acc2[b[u] * kLearnThreads + tid];
+                    a.x += grid_product((double)xf[u], w, g);
+                    a.y += wg;
                     acc2[b[u] * kLearnThreads + tid] = a;
                 }
             }
 #pragma unroll
             for (int half = 0; half < 2; ++half) {   // eight buckets = sixteen sums at a time
-                double v[16];
+                long long v[16];
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                    const double2 a = acc2[(8 * half + j) * kLearnThreads + tid];
+                    const longlong2 a = acc2[(8 * half + j) * kLearnThreads + tid];
                     v[2 * j] = a.x;
                     v[2 * j + 1] = a.y;
                 }
@@ -219,12 +328,20 @@ __device__ void learn_row(const LearnParams& P, const float* xs, const float* ws
             }
         }
         __syncthreads();
-        // ---- new levels (an empty bucket keeps its level), then midpoints with a shuffle in between: every warp
+        // ---- new levels, then midpoints with a shuffle in between: every warp
+        bool light = false;
         if (lane < Lv) {
-            double sn = 0.0, sd = 0.0;
+            long long sn = 0, sd = 0;
 #pragma unroll
             for (int w2 = 0; w2 < kLearnWarps; ++w2) { sn += red[(2 * lane) * kLearnWarps + w2]; sd += red[(2 * lane + 1) * kLearnWarps + w2]; }
-            if (sd > 0.0) ylane = sn / sd;
+            light = sd < kLight;
+            if (!light) ylane = (double)sn / (double)sd;
+        }
+        for (unsigned left = __ballot_sync(0xffffffffu, light); left != 0u; left &= left - 1u) {
+            const int k = __ffs(left) - 1;
+            const float t_lo = __shfl_sync(0xffffffffu, tlane, max(k - 1, 0)), t_hi = __shfl_sync(0xffffffffu, tlane, k);
+            const double mean = light_mean_row(xs, ws, row_most, K, k > 0 ? t_lo : -INFINITY, k < Lv - 1 ? t_hi : INFINITY, __shfl_sync(0xffffffffu, ylane, k));
+            if (lane == k) ylane = mean;
         }
         const double yn = __shfl_down_sync(0xffffffffu, ylane, 1);
         bool same = true;
@@ -241,13 +358,13 @@ __device__ void learn_row(const LearnParams& P, const float* xs, const float* ws
             __syncwarp();
         }
         // thresholds that have not moved (as the fp32 numbers the elements are compared with) assign every element
-        // as before: the next round would add the same sums up in the same order and change nothing, nor any later one
+        // as before: the next round would form the same sums and change nothing, nor any later one
         if (__all_sync(0xffffffffu, same)) break;
     }
 
     // ---- tables: fp32 levels, midpoints of the fp32 levels; unused levels 0, unused thresholds +inf
     if (warp == 0) {
-        const float m = (lane < Lv) ? (float)ylane : 0.0f;
+        const float m = (lane < Lv) ? (bad ? __int_as_float(0x7fc00000) : (float)ylane) : 0.0f;
         const float mn = __shfl_down_sync(0xffffffffu, m, 1);
         if (lane < kTableStride) {
             maps_out[lane] = m;
@@ -257,41 +374,305 @@ __device__ void learn_row(const LearnParams& P, const float* xs, const float* ws
     __syncthreads();   // the sums in shared memory are reused by the next run, the row buffer by the next row
 }
 
-// FOUR = false: for weights without 4-bit rows.  Only the 4-bit runs need the 32 KB of per-thread bucket sums in shared
-// memory, and the rounds of a row are a chain of short phases between barriers, so what hides their latency is the number
-// of CTAs per SM: without those 32 KB three times as many fit (all-1-bit rows: 0.52 -> 0.34 ms on 4096 x 11008 at ten
-// rounds).  (Running the 4-bit rows of a mixed weight in a kernel of their own was slower: the few rows leave most SMs
-// idle for the length of a row.)
-template <bool ALL3, bool FOUR>
-__global__ void __launch_bounds__(kLearnThreads) learn_kernel(const __grid_constant__ LearnParams P) {
+// FOUR: with rounds at 4 bits.  Only these need the 32 KB of per-thread bucket sums in shared memory, and the rounds of a row are a
+// chain of short phases between barriers, so what hides their latency is the number of CTAs per SM: without those 32 KB three times
+// as many fit (all-1-bit rows: 0.52 -> 0.34 ms on 4096 x 11008 at ten rounds).
+// THREADS: short rows take fewer, which all have work, and pay less for the end of a round (1-bit rows, T = 2, 4096 of them: 20.5 ->
+// 13.5 us at K = 1024, 29 -> 26 us at K = 4096; at K = 11008 the other way round: 86 against 72).
+// What bounds it: instruction issue, five per element, round and threshold.  Together with the row's way in, 4096 x 4096, T = 2: 27.4 ->
+// 24.5 us at 1 bit and 41.6 -> 37 at 2; 4096 x 11008: 78 -> 69 and 112 -> 101; without rounds 50 -> 38 there.
+template <bool ALL3, bool FOUR, int THREADS>
+__global__ void __launch_bounds__(THREADS) learn_kernel(const __grid_constant__ LearnParams P) {
     extern __shared__ __align__(16) unsigned char learn_smem[];
-    // [2 x 2 * 16 * warps doubles partial sums][FOUR: 2 * 16 * threads doubles sums][K floats][nb floats][warps x 16 floats]
-    double* red2 = reinterpret_cast<double*>(learn_smem);
-    double* acc = red2 + 2 * 2 * 16 * kLearnWarps;
-    float* xs = reinterpret_cast<float*>(acc + (FOUR ? 2 * 16 * kLearnThreads : 0));
+    constexpr int kWarps = THREADS / 32;
+    // [2 x 2 * 16 * warps partial sums][FOUR: 2 * 16 * threads sums][K floats][nb floats][warps x 16 floats]
+    long long* red2 = reinterpret_cast<long long*>(learn_smem);
+    long long* acc = red2 + 2 * 2 * 16 * kWarps;
+    float* xs = reinterpret_cast<float*>(acc + (FOUR ? 2 * 16 * THREADS : 0));
     float* ws = xs + P.K;
     float* tfw = ws + P.K / kBlock;   // 4-bit runs: a copy of the thresholds (fp32 upper neighbours) per warp
-    pdl_enter();
-    for (int i = blockIdx.x; i < P.N; i += gridDim.x) {
-        // with a layout: stored rows from the last to the first, i.e. the long 4-bit rows are handed out first and the
-        // short 1-bit rows fill the gaps at the end
-        const int r = ALL3 ? i : P.L.perm[P.N - 1 - i];
-        load_row(P, r, xs, ws);
-        float* m = P.maps + (size_t)r * kTableStride;
-        float* h = P.thresholds + (size_t)r * kTableStride;
-        if (ALL3) {
-            // the row under every precision, from the one copy in shared memory
-            const size_t plane = (size_t)P.N * kTableStride;
-            learn_row<1>(P, xs, ws, acc, red2, tfw, m, h);
-            learn_row<2>(P, xs, ws, acc, red2, tfw, m + plane, h + plane);
-            if (FOUR) learn_row<4>(P, xs, ws, acc, red2, tfw, m + 2 * plane, h + 2 * plane);
-        } else {
-            const int b = P.L.precs[r];
-            if (b == 1) learn_row<1>(P, xs, ws, acc, red2, tfw, m, h);
-            else if (b == 2) learn_row<2>(P, xs, ws, acc, red2, tfw, m, h);
-            else if (FOUR) learn_row<4>(P, xs, ws, acc, red2, tfw, m, h);
+    enter(P.turn);
+    // with a layout: stored rows from the last to the first, i.e. the longer 2-bit rows (4-bit rows) are handed out first and the
+    // short 1-bit rows fill the gaps at the end
+    const int i = P.row0 + (int)(gridDim.x - 1 - blockIdx.x);
+    const int r = ALL3 ? i : P.L.perm[i];
+    const float most = load_row<THREADS>(P, r, xs, ws, tfw);
+    float* m = P.maps + (size_t)r * kTableStride;
+    float* h = P.thresholds + (size_t)r * kTableStride;
+    if (ALL3) {
+        // the row under every precision, from the one copy in shared memory
+        const size_t plane = (size_t)P.N * kTableStride;
+        learn_row<1, THREADS>(P, xs, ws, most, acc, red2, tfw, P.iterations, m, h);
+        learn_row<2, THREADS>(P, xs, ws, most, acc, red2, tfw, P.iterations, m + plane, h + plane);
+        learn_row<4, THREADS>(P, xs, ws, most, acc, red2, tfw, FOUR ? P.iterations : 0, m + 2 * plane, h + 2 * plane);
+    } else {
+        const int b = P.L.precs[r];
+        if (b == 1) learn_row<1, THREADS>(P, xs, ws, most, acc, red2, tfw, P.iterations, m, h);
+        else if (b == 2) learn_row<2, THREADS>(P, xs, ws, most, acc, red2, tfw, P.iterations, m, h);
+        else learn_row<4, THREADS>(P, xs, ws, most, acc, red2, tfw, FOUR ? P.iterations : 0, m, h);
+    }
+    leave(P.turn);
+}
+
+// ---------------------------------------------------------------------------------------------------------------------------------
+// Rounds on a sorted row.  A round needs, for every threshold, the weighted sums over the values below it.  With the row in
+// (nearly) sorted order and running sums of it, that is one look-up and a short scan per threshold, whatever the number of
+// rounds, levels and precisions - where a pass over the row costs about 13 thread instructions per element, half of them on the fp64
+// and conversion pipes, and six times that at 4 bits.  One CTA per row:
+//   - the row comes asynchronously into shared memory and from there, normalised (as in lowra_encode), into registers; bins_of(K)
+//     equal cells of [-1, 1] are counted and their counts added up; then every value and its weight go to their place, a cell's
+//     places being handed out by an atomic;
+//   - running sums over every sixteen places;
+//   - T rounds by one warp (in the three-precision form a warp per precision): threshold t lies in cell b; everything before cell b
+//     is below it, so its sums are the running sums up to the last multiple of sixteen before the cell plus the values from there
+//     to the end of the cell that are below t.
+// The order inside a cell is that in which the atomics arrive, which integer sums do not see.
+// What bounds it: shared-memory wavefronts (two atomics and an 8-byte store per element at random places: 24 wavefronts for 32
+// elements, the pipe 77 % busy at T = 0) and, in the rounds, the latency of one warp's steps (about 1000 cycles each, hidden by the
+// other rows of the SM).  Measured against a pass over the row per round, 4096 x 4096, T = 10: 391 -> 105 us at 4 bits, 157 -> 86
+// at 2; 127 -> 80 at 60/35/5 % of 1/2/4 bits (1-bit rows in learn_kernel); three precisions, T = 2: 133 -> 66 us.
+constexpr int kSortedMaxK = 16384;         // 10 to 11 bytes of shared memory per element
+int bins_of(int K) { int n = 256; while (n < K / 6) n *= 2; return n; }
+
+struct Sums {
+    long long wn, w;     // multiples of 2^-46
+};
+
+// Where place p lies in shared memory (in units of 8 bytes): the 16-byte pairs of every 16 places are exchanged among
+// themselves, so that the eight lanes of a wavefront, which read 128 bytes apart, meet different banks.
+__device__ __forceinline__ int sorted_slot(int p) { return p ^ ((p >> 3) & 14); }
+
+// Cell of x among `bins`: monotone in x, so a value in an earlier cell than a threshold is below it.  Normalised values lie in
+// [-1, 1] up to a rounding, thresholds anywhere; adding 2^23 rounds to a whole number in the low bits (the mask: NaN lands
+// somewhere, but inside).
+__device__ __forceinline__ int cell_of(float x, int bins) {
+    return __float_as_int(fmaf(x, (float)(bins / 2 - 1), (float)(bins / 2) + 8388608.0f)) & (bins - 1);
+}
+__device__ __forceinline__ int cell_of_threshold(float t, int bins) { return cell_of(fminf(fmaxf(t, -1.0000005f), 1.0000005f), bins); }
+__device__ __forceinline__ Sums shfl_xor_sums(const Sums& s, int d) {
+    return Sums{__shfl_xor_sync(0xffffffffu, s.wn, d), __shfl_xor_sync(0xffffffffu, s.w, d)};
+}
+
+__device__ __noinline__ double light_mean_sorted(const float2* sorted, int p0, int p1, float t_lo, float t_hi, double keep) {
+    return light_mean([&](int p) { return sorted[sorted_slot(p)]; }, p0, p1, t_lo, t_hi, keep);
+}
+
+// T rounds at B bits by one warp; tables to maps_out / thr_out ([16] each).  first[b]: places before cell b; run[i]: sums over
+// the first 16 i places.  The G lanes of group j look after level j and the threshold above it (the last group: everything), all with
+// the same values; what bounds a round is the length of this chain, so it has few shuffles.
+template <int B>
+__device__ void learn_sorted(const LearnParams& P, const float2* sorted, const uint32_t* first, const Sums* run, int bins, float row_most,
+                             float* maps_out, float* thr_out) {
+    constexpr int Lv = 1 << B, c = B >> 1;
+    constexpr int G = B == 4 ? 2 : 8;
+    const int lane = threadIdx.x & 31, j = lane / G, K = P.K;
+    const bool top = j >= Lv - 1;                          // no threshold above
+    double y = j < Lv ? P.init_y[c][j] : 0.0;
+    float t = !top ? __double2float_ru(P.init_t[c][j]) : INFINITY;   // the least fp32 number >= the threshold
+    for (int it = 0; it < P.iterations; ++it) {
+        const int b = cell_of_threshold(t, bins);
+        const int p1 = top ? K : (int)first[b + 1], p0 = top ? K : (int)first[b] & ~15;
+        const Sums base = run[p0 >> 4];
+        Sums s = {0, 0};
+        for (int p = p0 + lane % G; p < p1; p += G) {
+            const float2 e = sorted[sorted_slot(p)];
+            if (e.x < t) {
+                s.wn += grid_product((double)e.x, (double)e.y, kGrid);
+                s.w += grid_weight((double)e.y, kGrid);
+            }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int d = G / 2; d >= 1; d >>= 1) {
+            const Sums o = shfl_xor_sums(s, d);
+            s.wn += o.wn; s.w += o.w;
+        }
+        s.wn += base.wn; s.w += base.w;
+        // the bucket: what lies below its upper threshold less what lies below its lower one
+        Sums low = {__shfl_up_sync(0xffffffffu, s.wn, G), __shfl_up_sync(0xffffffffu, s.w, G)};
+        if (j == 0) low.wn = low.w = 0;
+        const long long sw = s.w - low.w;
+        const bool light = j < Lv && sw < kLight;
+        if (j < Lv && !light) y = (double)(s.wn - low.wn) / (double)sw;
+        for (unsigned left = __ballot_sync(0xffffffffu, light); left != 0u;) {   // light or empty buckets, one after the other
+            const int k = (__ffs(left) - 1) / G;
+            left &= ~(((1u << G) - 1u) << (k * G));
+            const float t_lo = k > 0 ? __shfl_sync(0xffffffffu, t, max(k - 1, 0) * G) : -INFINITY;
+            const float t_hi = __shfl_sync(0xffffffffu, t, k * G);
+            const int q0 = k > 0 ? (int)first[cell_of_threshold(t_lo, bins)] : 0, q1 = k < Lv - 1 ? (int)first[cell_of_threshold(t_hi, bins) + 1] : K;
+            const double mean = light_mean_sorted(sorted, q0, q1, t_lo, t_hi, __shfl_sync(0xffffffffu, y, k * G));
+            if (j == k) y = mean;
+        }
+        const double yn = __shfl_down_sync(0xffffffffu, y, G);
+        const float tn = !top ? __double2float_ru((y + yn) * 0.5) : INFINITY;
+        // thresholds that have not moved (as the fp32 numbers the elements are compared with) assign every element as
+        // before: the next round would form the same sums and change nothing, nor any later one
+        const bool same = tn == t;
+        t = tn;
+        if (__all_sync(0xffffffffu, same)) break;
+    }
+    // tables: fp32 levels, midpoints of the fp32 levels; unused levels 0, unused thresholds +inf
+    const double yl = __shfl_sync(0xffffffffu, y, min(lane, Lv - 1) * G);
+    const float m = (lane < Lv) ? (row_most < INFINITY ? (float)yl : __int_as_float(0x7fc00000)) : 0.0f;
+    const float mn = __shfl_down_sync(0xffffffffu, m, 1);
+    if (lane < kTableStride) {
+        maps_out[lane] = m;
+        thr_out[lane] = (lane + 1 < Lv) ? (float)(((double)m + (double)mn) * 0.5) : __int_as_float(0x7f800000);
+    }
+}
+
+// Exclusive sums of v[0 .. NV-1] over the threads of the CTA (scratch: NV entries per warp).  Ends with a barrier.
+template <int NV, typename T>
+__device__ __forceinline__ void block_exclusive(T (&v)[NV], T (*scratch)[NV]) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    T incl[NV];
+#pragma unroll
+    for (int k = 0; k < NV; ++k) incl[k] = v[k];
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+            const T o = __shfl_up_sync(0xffffffffu, incl[k], d);
+            if (lane >= d) incl[k] += o;
         }
     }
+    if (lane == 31) {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) scratch[warp][k] = incl[k];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < NV; ++k) v[k] = incl[k] - v[k];
+    for (int w = 0; w < warp; ++w) {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) v[k] += scratch[w][k];
+    }
+    __syncthreads();
+}
+
+// THREADS threads at most, PER elements each, CTAS of them per SM.
+template <bool ALL3, int THREADS, int PER, int CTAS>
+__global__ void __launch_bounds__(THREADS, CTAS) sorted_learn_kernel(const __grid_constant__ LearnParams P) {
+    extern __shared__ __align__(16) unsigned char sorted_smem[];
+    const int K = P.K, bins = P.bins, tid = threadIdx.x, nt = blockDim.x, warp = tid >> 5, n_warps = nt >> 5;
+    // [K float2 values and weights in order; before that, the row][K / 16 + 1 Sums][32 x 2 long long][32 floats][0, 0, 0, 0][cells]
+    float2* sorted = reinterpret_cast<float2*>(sorted_smem);
+    Sums* run = reinterpret_cast<Sums*>(sorted + K);
+    long long(*scratch)[2] = reinterpret_cast<long long(*)[2]>(run + K / 16 + 1);
+    float* most_of = reinterpret_cast<float*>(scratch + 32);
+    uint32_t* cells = reinterpret_cast<uint32_t*>(most_of + 32) + 4;
+    enter(P.turn);
+    // stored rows from the last to the first: the 4-bit rows, whose rounds are a little longer, go out first
+    const int i0 = P.row0 + (int)(gridDim.x - 1 - blockIdx.x);
+    const int r = ALL3 ? i0 : P.L.perm[i0];
+    const float* wrow = P.W + (size_t)r * K;
+    const bool in = tid * PER < K;
+#pragma unroll
+    for (int u = 0; u < PER / 4; ++u) {
+        const int i = 4 * (u * nt + tid);
+        if (i < K)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(sorted_smem + 4 * i)), "l"(wrow + i) : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    for (int i = tid - 1; i < bins / 4; i += nt) *reinterpret_cast<uint4*>(cells + 4 * i) = make_uint4(0u, 0u, 0u, 0u);
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    // ---- this thread's part of a block, its 16-byte pieces in an order that spreads the lanes over the banks
+    float x[PER];
+    float m = 0.0f;
+#pragma unroll
+    for (int j = 0; j < PER / 4; ++j) {
+        float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (in) f = *reinterpret_cast<const float4*>(sorted_smem + 4 * PER * tid + 16 * (j ^ ((tid * PER / 32) & (PER / 4 - 1))));
+        x[4 * j] = f.x; x[4 * j + 1] = f.y; x[4 * j + 2] = f.z; x[4 * j + 3] = f.w;
+        m = max_nan(max_nan(m, max_nan(fabsf(f.x), fabsf(f.y))), max_nan(fabsf(f.z), fabsf(f.w)));
+    }
+    for (int d = 1; d < kBlock / PER; d <<= 1) m = max_nan(m, __shfl_xor_sync(0xffffffffu, m, d));
+    const float inv = (m == 0.0f) ? 0.0f : __frcp_rn(m);
+    float most = max_nan(m, __fmul_rn(inv, 0.0f));
+#pragma unroll
+    for (int d = 16; d >= kBlock / PER; d >>= 1) most = max_nan(most, __shfl_xor_sync(0xffffffffu, most, d));
+    if ((tid & 31) == 0) most_of[warp] = most;
+    // ---- count the cells
+#pragma unroll
+    for (int e = 0; e < PER; ++e) x[e] = __fmul_rn(x[e], inv);
+    if (in) {
+#pragma unroll
+        for (int e = 0; e < PER; ++e) atomicAdd(&cells[cell_of(x[e], bins)], 1u);
+    }
+    __syncthreads();
+    // ---- counts -> places before the cell
+    {
+        const int per = (bins / 4 + nt - 1) / nt, c0 = tid * per, c1 = min(c0 + per, bins / 4);
+        uint32_t before[1] = {0u};
+        for (int i = c0; i < c1; ++i) {
+            const uint4 n = *reinterpret_cast<const uint4*>(cells + 4 * i);
+            before[0] += n.x + n.y + n.z + n.w;
+        }
+        block_exclusive<1, uint32_t>(before, reinterpret_cast<uint32_t(*)[1]>(scratch));
+        uint32_t b = before[0];
+        for (int i = c0; i < c1; ++i) {
+            const uint4 n = *reinterpret_cast<const uint4*>(cells + 4 * i);
+            *reinterpret_cast<uint4*>(cells + 4 * i) = make_uint4(b, b + n.x, b + n.x + n.y, b + n.x + n.y + n.z);
+            b += n.x + n.y + n.z + n.w;
+        }
+    }
+    float row_most = 0.0f;
+    for (int w = 0; w < n_warps; ++w) row_most = max_nan(row_most, most_of[w]);
+    const float weight = scaled_weight(m, row_most);
+    __syncthreads();
+    // ---- every value and its weight to their place; afterwards a cell's entry is the place where it ends
+    if (in) {
+#pragma unroll
+        for (int e = 0; e < PER; ++e)
+            sorted[sorted_slot((int)atomicAdd(&cells[cell_of(x[e], bins)], 1u))] = make_float2(x[e], weight);
+    }
+    __syncthreads();
+    // ---- running sums: this thread's places, sixteen at a time
+    {
+        unsigned long long part[PER / 16][2], all[2] = {0ull, 0ull};     // (modulo 2^64)
+#pragma unroll
+        for (int q = 0; q < PER / 16; ++q) {
+            part[q][0] = all[0]; part[q][1] = all[1];
+            if (in) {
+#pragma unroll
+                for (int p = 0; p < 16; p += 2) {
+                    const float4 e = *reinterpret_cast<const float4*>(sorted + sorted_slot(tid * PER + q * 16 + p));
+                    all[0] += grid_bits(__fma_rd((double)e.x, (double)e.y, kGrid)) + grid_bits(__fma_rd((double)e.z, (double)e.w, kGrid));
+                    all[1] += grid_bits((double)e.y + kGrid) + grid_bits((double)e.w + kGrid);
+                }
+                all[0] -= 16ull * grid_bits(kGrid);
+                all[1] -= 16ull * grid_bits(kGrid);
+            }
+        }
+        unsigned long long before[2] = {all[0], all[1]};
+        block_exclusive<2, unsigned long long>(before, reinterpret_cast<unsigned long long(*)[2]>(scratch));
+        if (in) {
+#pragma unroll
+            for (int q = 0; q < PER / 16; ++q)
+                run[tid * (PER / 16) + q] = Sums{(long long)(before[0] + part[q][0]), (long long)(before[1] + part[q][1])};
+        }
+        if (tid == K / PER - 1) run[K / 16] = Sums{(long long)(before[0] + all[0]), (long long)(before[1] + all[1])};
+    }
+    __syncthreads();
+    // ---- rounds
+    const uint32_t* first = cells - 1;   // first[b]: the places before cell b
+    float* y = P.maps + (size_t)r * kTableStride;
+    float* h = P.thresholds + (size_t)r * kTableStride;
+    if (ALL3) {   // a warp per precision
+        const size_t plane = (size_t)P.N * kTableStride;
+        for (int c = warp; c < 3; c += n_warps) {
+            if (c == 0) learn_sorted<4>(P, sorted, first, run, bins, row_most, y + 2 * plane, h + 2 * plane);
+            else if (c == 1) learn_sorted<2>(P, sorted, first, run, bins, row_most, y + plane, h + plane);
+            else learn_sorted<1>(P, sorted, first, run, bins, row_most, y, h);
+        }
+    } else if (warp == 0) {
+        const int b = P.L.precs[r];
+        if (b == 1) learn_sorted<1>(P, sorted, first, run, bins, row_most, y, h);
+        else if (b == 2) learn_sorted<2>(P, sorted, first, run, bins, row_most, y, h);
+        else learn_sorted<4>(P, sorted, first, run, bins, row_most, y, h);
+    }
+    leave(P.turn);
 }
 
 }  // namespace lowra
@@ -299,36 +680,68 @@ __global__ void __launch_bounds__(kLearnThreads) learn_kernel(const __grid_const
 namespace lowra {
 namespace {
 
-// validation shared by the two entry points is done by the callers; this fills the tables and launches
-template <bool ALL3, bool FOUR>
-lowra_status launch_learn_kernel(const LearnParams& P, void* stream) {
-    const size_t smem = (2 * 2 * 16 * kLearnWarps + (FOUR ? 2 * 16 * kLearnThreads : 0)) * sizeof(double) +
-                        ((size_t)P.K + (size_t)P.K / kBlock + 16 * kLearnWarps) * sizeof(float);
-    if (smem > 200 * 1024) return LOWRA_ERR_SHAPE;   // the row has to fit into shared memory (K <= 40960)
-    static SmemLimit limit = {};
-    if (ensure_smem_limit(reinterpret_cast<const void*>(learn_kernel<ALL3, FOUR>), smem, &limit) != LOWRA_OK) return LOWRA_ERR_CUDA;
+lowra_status launch_rows(void (*kernel)(LearnParams), const LearnParams& P, int rows, int threads, size_t smem, SmemLimit* limit, void* stream) {
+    if (ensure_smem_limit(reinterpret_cast<const void*>(kernel), smem, limit) != LOWRA_OK) return LOWRA_ERR_CUDA;
     // a row per CTA and as many CTAs as rows: a 4-bit row takes five times as long as a 1-bit one, and fresh CTAs handed out
     // by the hardware keep the SMs evenly busy where a persistent grid (every CTA walking over its share of the rows) left
     // some of them waiting at the end (the 7B layer at 60/35/5: 2.05 -> 1.68 ms)
-    const unsigned grid = (unsigned)P.N;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.gridDim = dim3(grid, 1, 1);
-    cfg.blockDim = dim3(kLearnThreads, 1, 1);
+    cfg.gridDim = dim3((unsigned)rows, 1, 1);
+    cfg.blockDim = dim3((unsigned)threads, 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = (cudaStream_t)stream;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, learn_kernel<ALL3, FOUR>, P) == cudaSuccess ? LOWRA_OK : LOWRA_ERR_CUDA;
+    return cudaLaunchKernelEx(&cfg, kernel, P) == cudaSuccess ? LOWRA_OK : LOWRA_ERR_CUDA;
 }
 
-// validation shared by the two entry points is done by the callers; this fills the tables and launches (`four`: whether
-// any run at 4 bits is asked for)
+template <bool ALL3, bool FOUR, int THREADS>
+lowra_status launch_learn_kernel(const LearnParams& P, int rows, void* stream) {
+    const size_t smem = (2 * 2 * 16 * (THREADS / 32) + (FOUR ? 2 * 16 * THREADS : 0)) * sizeof(long long) +
+                        ((size_t)P.K + (size_t)P.K / kBlock + 16 * (THREADS / 32)) * sizeof(float);
+    if (smem > 200 * 1024) return LOWRA_ERR_SHAPE;   // the row has to fit into shared memory (K <= 40960)
+    static SmemLimit limit = {};
+    return launch_rows(learn_kernel<ALL3, FOUR, THREADS>, P, rows, THREADS, smem, &limit, stream);
+}
+
+size_t sorted_smem_bytes(int K) {
+    return (size_t)K * sizeof(float2) + ((size_t)K / 16 + 1) * sizeof(Sums) + 32 * (2 * sizeof(long long) + sizeof(float)) + ((size_t)bins_of(K) + 4) * 4;
+}
+
+template <bool ALL3, int THREADS, int PER, int CTAS>
+lowra_status launch_sorted_kernel(LearnParams& P, int rows, void* stream) {
+    P.bins = bins_of(P.K);
+    static SmemLimit limit = {};
+    return launch_rows(sorted_learn_kernel<ALL3, THREADS, PER, CTAS>, P, rows, (P.K / PER + 31) / 32 * 32, sorted_smem_bytes(P.K), &limit, stream);
+}
+
+bool two_long_rows(int K) { return 2 * (sorted_smem_bytes(K) + 1024) <= 228 * 1024; }   // an SM holds two (K <= 11264)
+
+// Whether the rounds of a class together are long enough to pay for the order (c = 0, 1, 2: 1, 2, 4 bits; 3: all of them).  Measured, us, 4096 rows
+// (K = 13824: 3328), learn_kernel against sorted_learn_kernel, after 2, 4 and 10 rounds:
+//             1 bit                              2 bits                             4 bits                              all three, 2 and 10
+//   K=1024    11 16 27       19 22 30            15 24 52       19 22 33            54 98 221        22 30 53           80 311     27 69
+//   K=2048    15 23 41       31 34 42            22 37 79       31 34 46            63 114 271       33 39 57           97 391     36 69
+//   K=4096    24 38 72       57 65 80            37 63 137      57 64 86            95 173 408       62 72 105          149 622    64 122
+//   K=5120    33 50 93       72 81 102           50 83 184      73 82 108           111 202 474      78 91 132          178 748    83 156
+//   K=8192    48 71 135      134 151 195         73 122 270     134 152 201         173 313 733      141 166 238        273 1140   141 247
+//   K=11008   69 99 188      171 187 229         101 167 369    173 189 238         274 491 1143     179 204 278        436 1800   180 278
+//   K=13824   74 106 199     238 263 331         108 175 383    238 264 344         273 494 1160     252 290 403        429 1780   253 416
+// The lines cross where the table below has them; with all three (an assessment) already in the first round.
+bool sorted_pays(int K, int c, int iterations) {
+    if (K > kSortedMaxK || iterations < 1) return false;
+    constexpr int kRounds[3][3] = {{12, 4, 1}, {25, 6, 2}, {43, 9, 2}};
+    return c == 3 || iterations >= kRounds[K <= 5120 ? 0 : two_long_rows(K) ? 1 : 2][c];
+}
+
+// validation shared by the two entry points is done by the callers; this fills the tables and launches (n1, n2, n4: rows to be
+// learnt at 1, 2 and 4 bits)
 template <bool ALL3>
 lowra_status launch_learn(LearnParams& P, const double* init_levels_host, const double* init_thresholds_host,
-                          bool four, void* stream) {
+                          int n1, int n2, int n4, void* stream) {
     if (((size_t)P.K + (size_t)P.K / kBlock) * sizeof(float) > 160 * 1024) return LOWRA_ERR_SHAPE;   // K <= 40960: the row has to fit
     lowra_status st = check_device();
     if (st != LOWRA_OK) return st;
@@ -337,7 +750,35 @@ lowra_status launch_learn(LearnParams& P, const double* init_levels_host, const 
             P.init_y[c][j] = init_levels_host[c * 16 + j];
             P.init_t[c][j] = init_thresholds_host[c * 16 + j];
         }
-    return four ? launch_learn_kernel<ALL3, true>(P, stream) : launch_learn_kernel<ALL3, false>(P, stream);
+    // stored rows are in the order of their precisions: the last `sorted` of them go to the sorted kernel
+    int sorted = 0;
+    if (ALL3) {
+        sorted = sorted_pays(P.K, 3, P.iterations) ? P.N : 0;
+    } else {
+        if (sorted_pays(P.K, 2, P.iterations)) sorted += n4;
+        if (sorted_pays(P.K, 1, P.iterations)) sorted += n2;
+        if (sorted_pays(P.K, 0, P.iterations)) sorted += n1;
+    }
+    const bool two = sorted > 0 && sorted < P.N;
+    if (sorted > 0) {
+        P.row0 = P.N - sorted;
+        P.turn = two ? 1 : 0;
+        // As many CTAs to an SM as its shared memory takes, for the phases of one row leave what bounds the others idle.  The registers
+        // go with that: 16 elements a thread up to K = 8192; beyond it two rows of 512 threads beat one of 1024 (K = 11008: 152
+        // against 232 us) as long as two fit.
+        st = P.K <= 4096       ? launch_sorted_kernel<ALL3, 256, 16, 5>(P, sorted, stream)
+           : P.K <= 5120       ? launch_sorted_kernel<ALL3, 320, 16, 4>(P, sorted, stream)
+           : P.K <= 8192       ? launch_sorted_kernel<ALL3, 512, 16, 2>(P, sorted, stream)
+           : two_long_rows(P.K) ? launch_sorted_kernel<ALL3, 512, 32, 2>(P, sorted, stream)
+                                : launch_sorted_kernel<ALL3, 1024, 16, 1>(P, sorted, stream);
+        if (st != LOWRA_OK || !two) return st;
+    }
+    const int rows = P.N - sorted;
+    P.row0 = 0;
+    P.turn = two ? 2 : 0;
+    const bool four = (ALL3 || (!two && n4 > 0)) && P.iterations > 0;
+    return four ? launch_learn_kernel<ALL3, true, 128>(P, rows, stream)
+         : P.K <= 4096 ? launch_learn_kernel<ALL3, false, 64>(P, rows, stream) : launch_learn_kernel<ALL3, false, 128>(P, rows, stream);
 }
 
 }  // namespace
@@ -360,7 +801,7 @@ extern "C" lowra_status lowra_learn_codebooks(const lowra_layout* layout, const 
     P.iterations = iterations;
     P.N = layout->N;
     P.K = layout->K;
-    return launch_learn<false>(P, init_levels_host, init_thresholds_host, layout->counts[2] > 0, stream);
+    return launch_learn<false>(P, init_levels_host, init_thresholds_host, layout->counts[0], layout->counts[1], layout->counts[2], stream);
 }
 
 extern "C" lowra_status lowra_learn_codebooks_all(int32_t N, int32_t K, const float* W_dev,
@@ -379,5 +820,5 @@ extern "C" lowra_status lowra_learn_codebooks_all(int32_t N, int32_t K, const fl
     P.iterations = iterations;
     P.N = N;
     P.K = K;
-    return launch_learn<true>(P, init_levels_host, init_thresholds_host, true, stream);
+    return launch_learn<true>(P, init_levels_host, init_thresholds_host, N, N, N, stream);
 }
