@@ -13,17 +13,21 @@
 // so SSE agrees with the exact sum to 2^-21 relative at worst (residual rounded to fp32: 2^-23; a square and two
 // additions in fp32: 3 * 2^-24 more), typically far closer.
 //
-// One warp per row at a time (grid-stride, no block-wide synchronisation); sixteen lanes with one float4 each cover
-// a 64-element absmax block, so the block maximum is four shuffles.  Traffic: 4 bytes per element read (+ 4 written with the residual).
-#include "lowra_common.cuh"
+// Traffic: 4 bytes per element read (+ 4 written with the residual), streamed as row_stream.cuh says: a lane works on half an absmax block at a
+// time.  At 1 and 2 bits the two or four values w_hat are formed once per half block and picked by comparison; at 4 bits
+// a branch-free binary search finds the level.  The residual is written over the weights in shared memory and leaves in one bulk copy
+// per chunk.
+// What bounds it: memory at 1 and 2 bits (5120 x 5120 at 85/15 % with the residual 44.6 -> 37.3 us, 85 % of the copy rate; without it 26.2 ->
+// 20.7), the half-rate pipe for comparisons, selections and address arithmetic at 4 bits and for all three precisions at once (4096 x 4096: 29.1 ->
+// 21.1 and 40.7 -> 31 us).
+#include "row_stream.cuh"
 
 namespace lowra {
 
 namespace {
 
-constexpr int kErrThreads = 256;
-constexpr int kErrWarps = kErrThreads / 32;
-constexpr int kErrBatch = 4;   // float4 loads per thread and batch; two batches in flight
+constexpr int kErrThreads = 32 * kRowWarps;
+constexpr int kErrRows = 16;   // rows of a CTA between two barriers (their sums per warp are kept in shared memory)
 
 struct ErrParams {
     RowLayout L;
@@ -34,109 +38,208 @@ struct ErrParams {
     float* residual;          // [N, K] or null
 };
 
-// level of the bucket of n: the number of thresholds <= n picks the level (thresholds sorted, as the encoder assumes).
-// 4 bits: levels at tab[0 .. 15], thresholds at tab[16 .. 30] of the warp's table in shared memory; branch-free binary
-// search, four look-ups by index (the same search as lowra_encode's).
-template <int B>
-__device__ __forceinline__ float level_of(float n, const float (&t)[3], const float (&y)[4], const float* tab) {
-    if (B == 1) return t[0] <= n ? y[1] : y[0];
-    if (B == 2) {
-        const bool hi = t[1] <= n;
-        const bool lo = (hi ? t[2] : t[0]) <= n;
-        return hi ? (lo ? y[3] : y[2]) : (lo ? y[1] : y[0]);
-    }
-    const float* ts = tab + 16;
-    int k = ts[7] <= n ? 8 : 0;
-    k += ts[k + 3] <= n ? 4 : 0;
-    k += ts[k + 1] <= n ? 2 : 0;
-    k += ts[k] <= n ? 1 : 0;
-    return tab[k];
+__device__ __forceinline__ float lds_f32(uint32_t at) {
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(at));
+    return v;
 }
 
-template <int B>
-__device__ void error_row(const ErrParams& P, int r, float* y_warp) {
-    const int lane = threadIdx.x & 31;
-    const int K = P.L.K;
-    const float* wrow = P.W + (size_t)r * K;
-    float* rrow = P.residual ? P.residual + (size_t)r * K : nullptr;
-    const float* trow = P.thresholds + (size_t)r * kTableStride;
-    const float* yrow = P.maps + (size_t)r * kTableStride;
-    float t[3] = {0.f, 0.f, 0.f}, y[4] = {0.f, 0.f, 0.f, 0.f};
-    if (B == 1) {
-        t[0] = __ldg(trow); y[0] = __ldg(yrow); y[1] = __ldg(yrow + 1);
-    } else if (B == 2) {
-        t[0] = __ldg(trow); t[1] = __ldg(trow + 1); t[2] = __ldg(trow + 2);
-        y[0] = __ldg(yrow); y[1] = __ldg(yrow + 1); y[2] = __ldg(yrow + 2); y[3] = __ldg(yrow + 3);
-    } else {
-        __syncwarp();   // the previous row's look-ups are over
-        if (lane < 16) { y_warp[lane] = __ldg(yrow + lane); y_warp[16 + lane] = __ldg(trow + lane); }
-        __syncwarp();
-    }
-
+// Error of a lane's part of a block at B bits (inv: what normalises it; m: the block's absmax; y: the row's levels in shared memory, its
+// thresholds behind them); with RES the residuals take the weights' places.  The number of thresholds <= n picks the level
+// (thresholds sorted, as the encoder assumes).
+template <int B, bool RES, int PER>
+__device__ __forceinline__ double half_block_error(float (&x)[PER], float inv, float m, const float* y) {
+    const float* t = y + kTableStride;
     double acc = 0.0;
-    const int n4 = K / 4;   // float4 pieces of the row (a multiple of 32); lane l takes pieces l, l + 32, ...
-    // the loads of the next batch are under way while this one is worked on
-    float4 nxt[kErrBatch];
+    float wh[B == 4 ? 1 : 1 << B], th[B == 4 ? 1 : (1 << B) - 1];
+    if (B <= 2) {
 #pragma unroll
-    for (int u = 0; u < kErrBatch; ++u) {
-        const int i = lane + u * 32;
-        nxt[u] = (i < n4) ? ld_stream_f4(wrow + (size_t)i * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int k = 0; k < (1 << B); ++k) wh[k] = __uint_as_float(pack_bf16x2(0.0f, __fmul_rn(y[k], m)) & 0xFFFF0000u);
+#pragma unroll
+        for (int k = 0; k + 1 < (1 << B); ++k) th[k] = t[k];
     }
-    for (int base = lane; base < n4; base += 32 * kErrBatch) {
-        float4 x[kErrBatch];
+    const float t7 = t[7];
+    const uint32_t t_at = (uint32_t)__cvta_generic_to_shared(t);
 #pragma unroll
-        for (int u = 0; u < kErrBatch; ++u) {
-            x[u] = nxt[u];
-            const int i = base + 32 * kErrBatch + u * 32;
-            nxt[u] = (i < n4) ? ld_stream_f4(wrow + (size_t)i * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int q = 0; q < PER / 4; ++q) {
+        float res[4];
+#pragma unroll
+        for (int e = 0; e < 4; e += 2) {
+            const float n0 = __fmul_rn(x[4 * q + e], inv), n1 = __fmul_rn(x[4 * q + e + 1], inv);
+            float w0, w1;
+            if (B <= 2) {
+                auto pick = [&](float n) {
+                    if (B == 1) return th[0] <= n ? wh[1] : wh[0];
+                    const bool hi = th[B == 2 ? 1 : 0] <= n;
+                    const bool lo = (hi ? th[B == 2 ? 2 : 0] : th[0]) <= n;
+                    const float a = hi ? wh[B == 2 ? 2 : 0] : wh[0], b = hi ? wh[B == 2 ? 3 : 0] : wh[1];
+                    return lo ? b : a;
+                };
+                w0 = pick(n0);
+                w1 = pick(n1);
+            } else {
+                // binary search on shared-memory addresses: the thresholds lie behind the levels
+                auto level = [&](float n) {
+                    uint32_t a = t7 <= n ? t_at + 32u : t_at;
+                    a += lds_f32(a + 12u) <= n ? 16u : 0u;
+                    a += lds_f32(a + 4u) <= n ? 8u : 0u;
+                    a += lds_f32(a) <= n ? 4u : 0u;
+                    return lds_f32(a - 4u * kTableStride);
+                };
+                const uint32_t h = pack_bf16x2(__fmul_rn(level(n0), m), __fmul_rn(level(n1), m));
+                w0 = __uint_as_float(h << 16);
+                w1 = __uint_as_float(h & 0xFFFF0000u);
+            }
+            res[e] = __fsub_rn(x[4 * q + e], w0);
+            res[e + 1] = __fsub_rn(x[4 * q + e + 1], w1);
         }
+        // four squares in fp32, then into the fp64 sum
+        acc += (double)__fadd_rn(__fmaf_rn(res[0], res[0], __fmul_rn(res[1], res[1])), __fmaf_rn(res[2], res[2], __fmul_rn(res[3], res[3])));
+        if (RES) { x[4 * q] = res[0]; x[4 * q + 1] = res[1]; x[4 * q + 2] = res[2]; x[4 * q + 3] = res[3]; }
+    }
+    return acc;
+}
+
+// sum over the warp, in a fixed order
+__device__ __forceinline__ double warp_total(double v) {
 #pragma unroll
-        for (int u = 0; u < kErrBatch; ++u) {
-            const int i = base + u * 32;
-            // sixteen neighbouring lanes hold one absmax block
-            float m = fmaxf(fmaxf(fabsf(x[u].x), fabsf(x[u].y)), fmaxf(fabsf(x[u].z), fabsf(x[u].w)));
+    for (int d = 16; d >= 1; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+    return v;
+}
+
+// NP = 1: the error at the rows' own precisions, rows in stored order; NP = 3: at all three.  PER: elements per lane; AHEAD: chunks on
+// their way in.
+template <int NP, bool RES, int PER, int AHEAD, typename Params>
+__device__ __forceinline__ void error_rows(const Params& P, int N, int K) {
+    constexpr int kTables = NP * 2 * kTableStride * (int)sizeof(float);
+    constexpr int kChunk = 32 * PER;
+    constexpr int kBuffer = kChunk * (int)sizeof(float) + kTables;
+    extern __shared__ __align__(128) unsigned char smem[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double* part = reinterpret_cast<double*>(smem + kRowWarps * kRowDepth * kBuffer);   // [kErrRows][kRowWarps][NP]
+    int* row_ids = reinterpret_cast<int*>(part + kErrRows * kRowWarps * NP);            // [kErrRows]
+    unsigned char* mine = smem + warp * kRowDepth * kBuffer;
+    for (int i = threadIdx.x; i < kErrRows * kRowWarps * NP; i += kErrThreads) part[i] = 0.0;
+    __syncthreads();
+    pdl_enter();
+    const uint64_t once = once_policy();
+    const int rows = (N - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
+    // stored rows from the last to the first; original row of the CTA's row i
+    auto row_of = [&](int i) {
+        const int p = (int)blockIdx.x + i * (int)gridDim.x;
+        if constexpr (NP == 3) return p;
+        else return i < rows ? (int)__ldg(P.L.perm + (N - 1 - p)) : 0;
+    };
+    const RowWalk walk(K, kChunk);
+    RowPlace at = walk.start(warp), ahead = at;
+    int r_of[AHEAD + 1];                      // rows of the chunks under way and of the one after them
+    {
+        RowPlace a = at;
 #pragma unroll
-            for (int d = 8; d >= 1; d >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, d));
-            const float inv = (m == 0.0f) ? 0.0f : __frcp_rn(m);
-            // w_hat of the four elements, rounded to bf16 two at a time
-            const float l0 = __fmul_rn(level_of<B>(__fmul_rn(x[u].x, inv), t, y, y_warp), m);
-            const float l1 = __fmul_rn(level_of<B>(__fmul_rn(x[u].y, inv), t, y, y_warp), m);
-            const float l2 = __fmul_rn(level_of<B>(__fmul_rn(x[u].z, inv), t, y, y_warp), m);
-            const float l3 = __fmul_rn(level_of<B>(__fmul_rn(x[u].w, inv), t, y, y_warp), m);
-            const uint32_t h01 = pack_bf16x2(l0, l1), h23 = pack_bf16x2(l2, l3);
-            float4 res;
-            res.x = __fsub_rn(x[u].x, __uint_as_float(h01 << 16));
-            res.y = __fsub_rn(x[u].y, __uint_as_float(h01 & 0xFFFF0000u));
-            res.z = __fsub_rn(x[u].z, __uint_as_float(h23 << 16));
-            res.w = __fsub_rn(x[u].w, __uint_as_float(h23 & 0xFFFF0000u));
-            if (i < n4) {
-                // four squares in fp32 (three roundings of the partial sum), then into the fp64 sum
-                const float q = __fadd_rn(__fadd_rn(__fmul_rn(res.x, res.x), __fmul_rn(res.y, res.y)),
-                                          __fadd_rn(__fmul_rn(res.z, res.z), __fmul_rn(res.w, res.w)));
-                acc += (double)q;
-                if (rrow) __stcs(reinterpret_cast<float4*>(rrow + (size_t)i * 4), res);
+        for (int d = 0; d <= AHEAD; ++d) { r_of[d] = row_of(a.i); walk.next(a); }
+    }
+    auto copy_ahead = [&](int buffer, int r) {
+        const RowPlace a = ahead;
+        walk.next(ahead);
+        if (a.i < rows) {
+            unsigned char* buf = mine + buffer * kBuffer;
+            chunk_copy<PER>(buf, P.W + (size_t)r * K + (size_t)a.j * kChunk, min(K - a.j * kChunk, kChunk), lane, once);
+            if (lane < 8 * NP) {   // per precision 64 bytes of levels, 64 of thresholds
+                const size_t plane = NP == 3 ? (size_t)(lane >> 3) * N * kTableStride : 0;
+                const float* src = ((lane & 4) ? P.thresholds : P.maps) + plane + (size_t)r * kTableStride + 4 * (lane & 3);
+                copy16_async(buf + kChunk * sizeof(float) + 16 * lane, src);
             }
         }
-    }
-    // fixed tree over the lanes
+        copies_commit();
+    };
 #pragma unroll
-    for (int d = 16; d >= 1; d >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, d);
-    if (lane == 0) P.sse[r] = acc;
+    for (int d = 0; d < AHEAD; ++d) copy_ahead(d, r_of[d]);
+    int buffer = 0;
+    double acc[NP] = {};
+    for (int i0 = 0; i0 < rows; i0 += kErrRows) {
+        const int i1 = min(i0 + kErrRows, rows);
+        while (at.i < i1) {
+            copies_wait<AHEAD - 1>();
+            __syncwarp();
+            unsigned char* buf = mine + buffer * kBuffer;
+            const int r = r_of[0], valid = min(K - at.j * kChunk, kChunk);
+            const float* tables = reinterpret_cast<const float*>(buf + kChunk * sizeof(float));
+            float x[PER];
+            float m = 0.0f;
+            const bool in = PER * lane < valid;
+#pragma unroll
+            for (int t = 0; t < PER / 4; ++t) {
+                float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (in) f = *reinterpret_cast<const float4*>(buf + piece_at<PER>(t, lane));
+                x[4 * t] = f.x; x[4 * t + 1] = f.y; x[4 * t + 2] = f.z; x[4 * t + 3] = f.w;
+                m = fmaxf(fmaxf(m, fmaxf(fabsf(f.x), fabsf(f.y))), fmaxf(fabsf(f.z), fabsf(f.w)));
+            }
+            for (int d = 1; d < kBlock / PER; d <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, d));
+            const float inv = (m == 0.0f) ? 0.0f : __frcp_rn(m);
+            if (in) {
+                if constexpr (NP == 3) {
+                    acc[0] += half_block_error<1, false, PER>(x, inv, m, tables);
+                    acc[1] += half_block_error<2, false, PER>(x, inv, m, tables + 32);
+                    acc[2] += half_block_error<4, false, PER>(x, inv, m, tables + 64);
+                } else {
+                    const int p = N - 1 - ((int)blockIdx.x + at.i * (int)gridDim.x);
+                    if (p < P.L.class_start[1]) acc[0] += half_block_error<1, RES, PER>(x, inv, m, tables);
+                    else if (p < P.L.class_start[2]) acc[0] += half_block_error<2, RES, PER>(x, inv, m, tables);
+                    else acc[0] += half_block_error<4, RES, PER>(x, inv, m, tables);
+                }
+            }
+            if constexpr (RES) {
+                if (in) {
+#pragma unroll
+                    for (int t = 0; t < PER / 4; ++t) *reinterpret_cast<float4*>(buf + piece_at<PER>(t, lane)) = make_float4(x[4 * t], x[4 * t + 1], x[4 * t + 2], x[4 * t + 3]);
+                }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) {
+                    asm volatile("cp.async.bulk.global.shared::cta.bulk_group.L2::cache_hint [%0], [%1], %2, %3;" ::"l"(P.residual + (size_t)r * K + (size_t)at.j * kChunk),
+                                 "r"((uint32_t)__cvta_generic_to_shared(buf)), "r"((uint32_t)valid * 4u), "l"(once) : "memory");
+                    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                    asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(kRowDepth - AHEAD) : "memory");   // the buffer that is filled next has been read
+                }
+            }
+            __syncwarp();
+            if (lane == 0 && at.j == 0) row_ids[at.i - i0] = r;
+            const RowPlace was = at;
+            walk.next(at);
+            if (at.i != was.i) {
+#pragma unroll
+                for (int k = 0; k < NP; ++k) {
+                    const double v = warp_total(acc[k]);
+                    if (lane == 0) part[((was.i - i0) * kRowWarps + warp) * NP + k] = v;
+                    acc[k] = 0.0;
+                }
+            }
+#pragma unroll
+            for (int d = 0; d < AHEAD; ++d) r_of[d] = r_of[d + 1];
+            copy_ahead(buffer + AHEAD < kRowDepth ? buffer + AHEAD : buffer + AHEAD - kRowDepth, r_of[AHEAD - 1]);
+            r_of[AHEAD] = row_of(ahead.i);
+            buffer = buffer + 1 == kRowDepth ? 0 : buffer + 1;
+        }
+        __syncthreads();
+        for (int s = threadIdx.x; s < (i1 - i0) * NP; s += kErrThreads) {
+            double v = 0.0;
+#pragma unroll
+            for (int w = 0; w < kRowWarps; ++w) {
+                double& slot = part[((s / NP) * kRowWarps + w) * NP + s % NP];
+                v += slot;
+                slot = 0.0;
+            }
+            P.sse[(size_t)row_ids[s / NP] * NP + s % NP] = v;
+        }
+        __syncthreads();
+    }
+    copies_wait<0>();
+    if (RES && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
-__global__ void __launch_bounds__(kErrThreads) error_kernel(const ErrParams P) {
-    __shared__ float y_smem[kErrWarps][32];   // per warp: the 16 levels and 15 thresholds of a 4-bit row
-    pdl_enter();
-    const int warp = threadIdx.x >> 5;
-    float* y_warp = y_smem[warp];
-    // one warp per row at a time
-    for (int i = blockIdx.x * kErrWarps + warp; i < P.L.N; i += gridDim.x * kErrWarps) {
-        const int r = P.L.perm[P.L.N - 1 - i];   // stored rows from the last to the first: the dear 4-bit rows go out first
-        const int b = P.L.precs[r];
-        if (b == 1) error_row<1>(P, r, y_warp);
-        else if (b == 2) error_row<2>(P, r, y_warp);
-        else error_row<4>(P, r, y_warp);
-    }
+template <bool RES, int PER, int AHEAD>
+__global__ void __launch_bounds__(kErrThreads, row_ctas(PER)) error_kernel(const __grid_constant__ ErrParams P) {
+    error_rows<1, RES, PER, AHEAD>(P, P.L.N, P.L.K);
 }
 
 // ---- all three precisions in one pass (the assigner's input: every channel's error under 1, 2 and 4 bits) ----
@@ -148,72 +251,26 @@ struct Err3Params {
     int N, K;
 };
 
-__global__ void __launch_bounds__(kErrThreads) error3_kernel(const Err3Params P) {
-    __shared__ float y_smem[kErrWarps][32];   // per warp: the 16 levels and 15 thresholds of the row's 4-bit codebook
-    pdl_enter();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float* y_warp = y_smem[warp];
-    const int K = P.K, n4 = K / 4;
-    const size_t plane = (size_t)P.N * kTableStride;
-    for (int r = blockIdx.x * kErrWarps + warp; r < P.N; r += gridDim.x * kErrWarps) {
-        const float* wrow = P.W + (size_t)r * K;
-        const float* t1 = P.thresholds + (size_t)r * kTableStride;
-        const float* y1 = P.maps + (size_t)r * kTableStride;
-        const float ta[3] = {__ldg(t1), 0.f, 0.f};
-        const float ya[4] = {__ldg(y1), __ldg(y1 + 1), 0.f, 0.f};
-        const float tb[3] = {__ldg(t1 + plane), __ldg(t1 + plane + 1), __ldg(t1 + plane + 2)};
-        const float yb[4] = {__ldg(y1 + plane), __ldg(y1 + plane + 1), __ldg(y1 + plane + 2), __ldg(y1 + plane + 3)};
-        __syncwarp();   // the previous row's look-ups are over
-        if (lane < 16) { y_warp[lane] = __ldg(y1 + 2 * plane + lane); y_warp[16 + lane] = __ldg(t1 + 2 * plane + lane); }
-        __syncwarp();
-        double acc1 = 0.0, acc2 = 0.0, acc4 = 0.0;
-        float4 nxt[kErrBatch];
-#pragma unroll
-        for (int u = 0; u < kErrBatch; ++u) {
-            const int i = lane + u * 32;
-            nxt[u] = (i < n4) ? ld_stream_f4(wrow + (size_t)i * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-        for (int base = lane; base < n4; base += 32 * kErrBatch) {
-            float4 x[kErrBatch];
-#pragma unroll
-            for (int u = 0; u < kErrBatch; ++u) {
-                x[u] = nxt[u];
-                const int i = base + 32 * kErrBatch + u * 32;
-                nxt[u] = (i < n4) ? ld_stream_f4(wrow + (size_t)i * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-#pragma unroll
-            for (int u = 0; u < kErrBatch; ++u) {
-                const int i = base + u * 32;
-                float m = fmaxf(fmaxf(fabsf(x[u].x), fabsf(x[u].y)), fmaxf(fabsf(x[u].z), fabsf(x[u].w)));
-#pragma unroll
-                for (int d = 8; d >= 1; d >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, d));
-                const float inv = (m == 0.0f) ? 0.0f : __frcp_rn(m);
-                const float xs[4] = {x[u].x, x[u].y, x[u].z, x[u].w};
-                float n[4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e) n[e] = __fmul_rn(xs[e], inv);
-                // squared residuals of the four elements at one precision, added in fp32
-                auto group = [&](auto level) -> float {
-                    const uint32_t h01 = pack_bf16x2(__fmul_rn(level(n[0]), m), __fmul_rn(level(n[1]), m));
-                    const uint32_t h23 = pack_bf16x2(__fmul_rn(level(n[2]), m), __fmul_rn(level(n[3]), m));
-                    const float r0 = __fsub_rn(xs[0], __uint_as_float(h01 << 16)), r1 = __fsub_rn(xs[1], __uint_as_float(h01 & 0xFFFF0000u));
-                    const float r2 = __fsub_rn(xs[2], __uint_as_float(h23 << 16)), r3 = __fsub_rn(xs[3], __uint_as_float(h23 & 0xFFFF0000u));
-                    return __fadd_rn(__fadd_rn(__fmul_rn(r0, r0), __fmul_rn(r1, r1)), __fadd_rn(__fmul_rn(r2, r2), __fmul_rn(r3, r3)));
-                };
-                const float q1 = group([&](float v) { return level_of<1>(v, ta, ya, y_warp); });
-                const float q2 = group([&](float v) { return level_of<2>(v, tb, yb, y_warp); });
-                const float q4 = group([&](float v) { return level_of<4>(v, tb, yb, y_warp); });
-                if (i < n4) { acc1 += (double)q1; acc2 += (double)q2; acc4 += (double)q4; }
-            }
-        }
-#pragma unroll
-        for (int d = 16; d >= 1; d >>= 1) {
-            acc1 += __shfl_xor_sync(0xffffffffu, acc1, d);
-            acc2 += __shfl_xor_sync(0xffffffffu, acc2, d);
-            acc4 += __shfl_xor_sync(0xffffffffu, acc4, d);
-        }
-        if (lane == 0) { P.sse[(size_t)r * 3] = acc1; P.sse[(size_t)r * 3 + 1] = acc2; P.sse[(size_t)r * 3 + 2] = acc4; }
-    }
+template <int PER>
+__global__ void __launch_bounds__(kErrThreads, row_ctas(PER)) error3_kernel(const __grid_constant__ Err3Params P) {
+    error_rows<3, false, PER, kRowDepth - 1>(P, P.N, P.K);
+}
+
+template <int NP, int PER, typename Params>
+lowra_status launch_errors(void (*kernel)(Params), const Params& P, int N, SmemLimit* limit, void* stream) {
+    const size_t smem = kRowWarps * kRowDepth * (32 * PER * sizeof(float) + NP * 2 * kTableStride * sizeof(float)) + kErrRows * (kRowWarps * NP * sizeof(double) + sizeof(int));
+    if (ensure_smem_limit(reinterpret_cast<const void*>(kernel), smem, limit) != LOWRA_OK) return LOWRA_ERR_CUDA;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3((unsigned)(N < row_ctas(PER) * kNumSMs ? N : row_ctas(PER) * kNumSMs), 1, 1);
+    cfg.blockDim = dim3(kErrThreads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = (cudaStream_t)stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P) == cudaSuccess ? LOWRA_OK : LOWRA_ERR_CUDA;
 }
 
 }  // namespace
@@ -238,10 +295,17 @@ extern "C" lowra_status lowra_quant_error(const lowra_layout* layout, const floa
     P.thresholds = thresholds_dev;
     P.sse = sse_dev;
     P.residual = residual_dev;
-    // a row per warp and as many CTAs as that takes: rows differ in cost with their precision, and fresh CTAs handed out
-    // by the hardware keep the SMs more evenly busy than a persistent grid did (+12 to 23 %)
-    const unsigned grid = (unsigned)((layout->N + kErrWarps - 1) / kErrWarps);
-    return launch_pdl(error_kernel, grid, kErrThreads, (cudaStream_t)stream, P) == cudaSuccess ? LOWRA_OK : LOWRA_ERR_CUDA;
+    static SmemLimit limits[5] = {};
+    if (row_per_lane(layout->K) == 16)
+        return residual_dev ? launch_errors<1, 16>(error_kernel<true, 16, 2>, P, layout->N, &limits[0], stream)
+                            : launch_errors<1, 16>(error_kernel<false, 16, 2>, P, layout->N, &limits[1], stream);
+    if (!residual_dev) return launch_errors<1, 32>(error_kernel<false, 32, 2>, P, layout->N, &limits[2], stream);
+    // Where weights and residuals do not fit into L2 twice over and most rows are cheap ones, memory is the better for fewer reads between
+    // the writes: one chunk ahead against two, 11008 x 4096 at 60/35/5 %: 60.8 against 63.1 us; but 4096 x 4096 22.5 against 20.7 us, and
+    // 11008 x 4096 at 4 bits 66.9 against 61.4.
+    const bool writes_wait = 8ull * layout->N * layout->K > 2ull * 126 * 1024 * 1024 && layout->counts[2] < layout->N / 2;
+    return writes_wait ? launch_errors<1, 32>(error_kernel<true, 32, 1>, P, layout->N, &limits[3], stream)
+                       : launch_errors<1, 32>(error_kernel<true, 32, 2>, P, layout->N, &limits[4], stream);
 }
 
 extern "C" lowra_status lowra_channel_errors(int32_t N, int32_t K, const float* W_dev, const float* maps3_dev,
@@ -260,6 +324,7 @@ extern "C" lowra_status lowra_channel_errors(int32_t N, int32_t K, const float* 
     P.sse = sse3_dev;
     P.N = N;
     P.K = K;
-    const unsigned grid = (unsigned)((N + kErrWarps - 1) / kErrWarps);   // a row per warp, as above
-    return launch_pdl(error3_kernel, grid, kErrThreads, (cudaStream_t)stream, P) == cudaSuccess ? LOWRA_OK : LOWRA_ERR_CUDA;
+    static SmemLimit limits[2] = {};
+    return row_per_lane(K) == 16 ? launch_errors<3, 16>(error3_kernel<16>, P, N, &limits[0], stream)
+                                 : launch_errors<3, 32>(error3_kernel<32>, P, N, &limits[1], stream);
 }
