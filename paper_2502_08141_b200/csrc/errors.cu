@@ -38,12 +38,6 @@ struct ErrParams {
     float* residual;          // [N, K] or null
 };
 
-__device__ __forceinline__ float lds_f32(uint32_t at) {
-    float v;
-    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(at));
-    return v;
-}
-
 // Error of a lane's part of a block at B bits (inv: what normalises it; m: the block's absmax; y: the row's levels in shared memory, its
 // thresholds behind them); with RES the residuals take the weights' places.  The number of thresholds <= n picks the level
 // (thresholds sorted, as the encoder assumes).

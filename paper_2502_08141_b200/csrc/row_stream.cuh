@@ -44,21 +44,23 @@ __device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_
 template <int N>
 __device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// the chunk at src (valid elements, a multiple of 128) on its way into buf
 // L2 policy of what is read or written once
 __device__ __forceinline__ uint64_t once_policy() {
     uint64_t p;
     asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
     return p;
 }
+__device__ __forceinline__ void copy16_once(void* dst, const void* src, uint64_t policy) {
+    asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "l"(policy) : "memory");
+}
+
+// the chunk at src (valid elements, a multiple of 128) on its way into buf
 template <int PER>
 __device__ __forceinline__ void chunk_copy(unsigned char* buf, const float* src, int valid, int lane, uint64_t policy) {
 #pragma unroll
     for (int u = 0; u < PER / 4; ++u) {
         const int e = 4 * (32 * u + lane);
-        if (e < valid)
-            asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(buf + 4 * e)), "l"(src + e),
-                         "l"(policy) : "memory");
+        if (e < valid) copy16_once(buf + 4 * e, src + e, policy);
     }
 }
 // byte offset of 16-byte piece t of this lane's elements: all of them for every lane, in an order of its own
