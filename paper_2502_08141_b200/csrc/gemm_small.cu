@@ -26,8 +26,8 @@ namespace {
 
 constexpr int kSmallThreads = 256;
 constexpr int kSmallRows = 64;          // stored rows per CTA
+constexpr int kMergedPitch = kSmallRows + 4;   // fp32 words: neighbouring tokens of a tile of sums 4 banks apart
 constexpr int kSmallSpan = 256;         // contraction indices per step of a warp: one absmax block for each of four lanes
-constexpr int kPartPitch = kSmallRows + 4;   // fp32 words: neighbouring tokens of a partial tile 4 banks apart
 
 struct Unit { int member, m0; };        // up to 8 NT8 tokens of one member
 template <int NB>
@@ -44,7 +44,7 @@ __device__ __forceinline__ Unit unit_at(const SmallParams<NB>& P, int u, int tok
 }
 
 __device__ __forceinline__ void mma_bf16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
                  : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
                  : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
@@ -53,17 +53,18 @@ __device__ __forceinline__ void cp_async_16_zfill(uint32_t saddr, const void* gp
 }
 __device__ __forceinline__ uint4 ld_shared_v4(uint32_t saddr) {
     uint4 v;
-    asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(saddr) : "memory");
+    asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(saddr));
     return v;
 }
-__device__ __forceinline__ float ld_cluster_f32(uint32_t caddr) {
-    float v;
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(caddr) : "memory");
-    return v;
-}
+__device__ __forceinline__ void st_cluster_f32(uint32_t caddr, float v) { asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(caddr), "f"(v) : "memory"); }
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
 // ------------------------------------------------------------------------------------------------ T = bf16(s X A)
 constexpr int kProjectBatch = 4;        // steps of 16 contraction indices a warp fetches at a time
+
+// bytes of A a CTA fetches at a time (more than its warps' sums, 512 r, which later take the same place)
+__host__ __device__ constexpr size_t project_fetch_bytes(int r) { return (size_t)(kSmallThreads / 32) * kProjectBatch * 16 * (r * 2 + 16); }
 
 // Grid: (slices of the contraction = cluster, tiles of 16 tokens of all members).
 template <int NB>
@@ -72,6 +73,7 @@ __global__ void __launch_bounds__(kSmallThreads) project_kernel(const __grid_con
     asm volatile("griddepcontrol.wait;" ::: "memory");
     // the next kernel reads its operands right away, so it may start only now that everything before this kernel is complete
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    cluster_arrive();   // "this CTA runs": waited for before its shared memory is written from elsewhere
     if (P.clear_status && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *P.status = 0u;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const int slices = (int)gridDim.x, slice = (int)blockIdx.x;
@@ -135,30 +137,32 @@ __global__ void __launch_bounds__(kSmallThreads) project_kernel(const __grid_con
         d[8 * P.r] = acc[j][2]; d[8 * P.r + 1] = acc[j][3];
     }
     __syncthreads();
-    float* part = red + kWarps * 16 * P.r;                            // [16][r]
+    // every CTA of the cluster owns a share of the sums: its own sums of a share go into the owner's shared memory
+    const int share = 16 * P.r / slices;
+    float* sums = reinterpret_cast<float*>(project_smem + project_fetch_bytes(P.r));   // [slices][share]: behind what this CTA may still be reading
+    const uint32_t recv = ptx::smem_u32(sums);
+    cluster_wait();
     for (int i = threadIdx.x; i < 16 * P.r; i += kSmallThreads) {
         float sum = 0.0f;
 #pragma unroll
         for (int w = 0; w < kWarps; ++w) sum += red[w * 16 * P.r + i];
-        part[i] = sum;
+        const int owner = i / share;
+        st_cluster_f32(ptx::map_to_cta(recv + (uint32_t)(slice * share + i - owner * share) * 4u, (uint32_t)owner), sum);
     }
     ptx::cluster_sync();
-    const uint32_t part_addr = ptx::smem_u32(part);
-    // pairs of neighbouring ranks; columns between the rank and its padded width are zero
-    for (int i = slice * kSmallThreads + (int)threadIdx.x; i < 16 * P.rp / 2; i += slices * kSmallThreads) {
-        const int row = i / (P.rp / 2), col = (i - row * (P.rp / 2)) * 2;
+    for (int i = 2 * (int)threadIdx.x; i < share; i += 2 * kSmallThreads) {   // pairs of neighbouring ranks
+        const int e = slice * share + i, row = e / P.r, col = e - row * P.r;
         if (un.m0 + row >= W.M) continue;
         float a = 0.0f, b = 0.0f;
-        if (col < P.r) {
-            for (int c = 0; c < slices; ++c) {
-                const uint32_t addr = ptx::map_to_cta(part_addr + (uint32_t)(row * P.r + col) * 4u, (uint32_t)c);
-                a += ld_cluster_f32(addr);
-                b += ld_cluster_f32(addr + 4u);
-            }
-        }
+        for (int c = 0; c < slices; ++c) { a += sums[c * share + i]; b += sums[c * share + i + 1]; }
         *reinterpret_cast<uint32_t*>(W.T + (size_t)(un.m0 + row) * P.rp + col) = pack_bf16x2(P.s * a, P.s * b);
     }
-    ptx::cluster_sync();   // nobody leaves while a peer still reads its sums
+    // columns between the rank and its padded width are zero
+    const int pad = P.rp - P.r;
+    for (int i = slice * kSmallThreads + (int)threadIdx.x; i < 16 * pad; i += slices * kSmallThreads) {
+        const int row = i / pad;
+        if (un.m0 + row < W.M) W.T[(size_t)(un.m0 + row) * P.rp + P.r + (i - row * pad)] = 0;
+    }
 }
 
 // ------------------------------------------------------------------------------------------------ the product
@@ -210,13 +214,16 @@ __device__ __forceinline__ uint32_t token_piece(int m, int t, int j) {
     return (uint32_t)(m * (kSmallSpan * 2) + (t * 8 + (j ^ (t | ((m & 1) << 2)))) * 16);
 }
 
-template <int B, int NT8>
-__device__ __forceinline__ void multiply_rows(int K, const SmallMember& W, int m0, int p0, int p_end, int slot, int slots,
-                                              uint32_t x_smem, int half, float (&acc)[NT8][4]) {
+// A warp's sixteen rows times the tokens, over the contraction's slots slot0 .. slot1 - 1 of `slots` (neighbouring ranges of it); before and
+// after each one's steps begin(slot) and end(slot, acc).
+template <int B, int NT8, typename Begin, typename End>
+__device__ __forceinline__ void multiply_rows(int K, const SmallMember& W, int m0, int p0, int p_end, int slot0, int slot1, int slots,
+                                              uint32_t x_smem, int half, Begin begin, End end) {
     constexpr int c = B >> 1;
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const int n_span = (K + kSmallSpan - 1) / kSmallSpan, nb = K / kBlock;
-    const int b0 = (int)((long long)slot * n_span / slots), b1 = (int)((long long)(slot + 1) * n_span / slots);
+    auto bound = [&](int slot) { return (int)((long long)slot * n_span / slots); };
+    const int b0 = bound(slot0), b1 = bound(slot1);
     // rows g and g + 8 of the warp's sixteen
     const bool live0 = p0 + g < p_end, live1 = p0 + g + 8 < p_end;
     const int q0 = live0 ? p0 + g : p_end - 1, q1 = live1 ? p0 + g + 8 : p_end - 1;
@@ -229,15 +236,18 @@ __device__ __forceinline__ void multiply_rows(int K, const SmallMember& W, int m
     const float* y1 = W.maps + (size_t)r1 * kTableStride;
     // tokens of one step: fetched by the four warps that share it, two steps in flight
     constexpr uint32_t kStep = 8u * NT8 * kSmallSpan * 2u;
-    const int th = threadIdx.x & 127;
+    const int warp4 = (threadIdx.x >> 5) & 3;
+    const uint32_t stage_at = x_smem + token_piece(warp4, lane >> 3, lane & 7);
+    const uint32_t read_at = x_smem + token_piece(g, t, 0);          // piece j of its block: read_at ^ 16 j
     auto stage = [&](int b) {
         if (b < b1) {
-            const uint32_t dst = x_smem + (uint32_t)((b - b0) & 1) * kStep;
-            for (int i = th; i < 8 * NT8 * 32; i += 128) {
-                const int m = i >> 5, t2 = (i >> 3) & 3, j = i & 7, k = b * kSmallSpan + t2 * 64 + j * 8;
-                const bool ok = m0 + m < W.M && k < K;
-                cp_async_16_zfill(dst + token_piece(m, t2, j), ok ? W.X + (size_t)(m0 + m) * K + k : W.X, ok);
-            }
+            // a warp to every fourth token, a lane to a 16-byte piece of its 512 bytes
+            const int k = b * kSmallSpan + lane * 8, left = k < K ? W.M - m0 - warp4 : 0;
+            const uint16_t* src = W.X + (size_t)(m0 + warp4) * K + k;
+            const uint32_t dst = stage_at + (uint32_t)((b - b0) & 1) * kStep;
+#pragma unroll
+            for (int i = 0; i < 2 * NT8; ++i)
+                cp_async_16_zfill(dst + (uint32_t)(4 * i * kSmallSpan * 2), 4 * i < left ? src + (size_t)(4 * i) * K : W.X, 4 * i < left);
         }
         ptx::cp_async_commit();
     };
@@ -254,52 +264,66 @@ __device__ __forceinline__ void multiply_rows(int K, const SmallMember& W, int m
         load_levels<B>(ya, y0);
         load_levels<B>(yb, y1);
     }
-    for (int b = b0; b < b1; ++b) {
-        const Codes<B> c0 = n0, c1 = n1;
-        fetch(b + 1);
-        stage(b + 1);
-        Scaled<B> s0, s1;
-        if (B == 4) {   // (sixteen levels of two rows are too many registers to keep: read again, from L1)
-            load_levels<B>(ya, y0);
-            s0.set(ya, c0.a);
-            load_levels<B>(ya, y1);
-            s1.set(ya, c1.a);
-        } else {
-            s0.set(ya, c0.a);
-            s1.set(yb, c1.a);
-        }
-        ptx::cp_async_wait<1>();
-        ptx::named_barrier_sync(1 + half, 128);
-        const uint32_t xs = x_smem + (uint32_t)((b - b0) & 1) * kStep;
+    int b = b0;
+    for (int slot = slot0; slot < slot1; ++slot) {
+        begin(slot);
+        float acc[NT8][4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {   // sixteen elements of the block
-            uint32_t o0[8], o1[8];
-            s0.expand16(c0.w, q, o0);
-            s1.expand16(c1.w, q, o1);
-#pragma unroll
-            for (int nt = 0; nt < NT8; ++nt) {
-                const uint4 xl = ld_shared_v4(xs + token_piece(nt * 8 + g, t, 2 * q)), xh = ld_shared_v4(xs + token_piece(nt * 8 + g, t, 2 * q + 1));
-                mma_bf16(acc[nt], o0[0], o1[0], o0[1], o1[1], xl.x, xl.y);
-                mma_bf16(acc[nt], o0[2], o1[2], o0[3], o1[3], xl.z, xl.w);
-                mma_bf16(acc[nt], o0[4], o1[4], o0[5], o1[5], xh.x, xh.y);
-                mma_bf16(acc[nt], o0[6], o1[6], o0[7], o1[7], xh.z, xh.w);
+        for (int i = 0; i < NT8; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.0f;
+        for (const int slot_end = bound(slot + 1); b < slot_end; ++b) {
+            const Codes<B> c0 = n0, c1 = n1;
+            fetch(b + 1);
+            stage(b + 1);
+            Scaled<B> s0, s1;
+            if (B == 4) {   // (sixteen levels of two rows are too many registers to keep: read again, from L1)
+                load_levels<B>(ya, y0);
+                s0.set(ya, c0.a);
+                load_levels<B>(ya, y1);
+                s1.set(ya, c1.a);
+            } else {
+                s0.set(ya, c0.a);
+                s1.set(yb, c1.a);
             }
+            ptx::cp_async_wait<1>();
+            ptx::named_barrier_sync(1 + half, 128);
+            const uint32_t xs = read_at + (uint32_t)((b - b0) & 1) * kStep;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {   // sixteen elements of the block
+                uint32_t o0[8], o1[8];
+                s0.expand16(c0.w, q, o0);
+                s1.expand16(c1.w, q, o1);
+#pragma unroll
+                for (int nt = 0; nt < NT8; ++nt) {
+                    const uint4 xl = ld_shared_v4((xs ^ (32u * q)) + (uint32_t)(nt * 8 * kSmallSpan * 2)), xh = ld_shared_v4((xs ^ (32u * q + 16u)) + (uint32_t)(nt * 8 * kSmallSpan * 2));
+                    mma_bf16(acc[nt], o0[0], o1[0], o0[1], o1[1], xl.x, xl.y);
+                    mma_bf16(acc[nt], o0[2], o1[2], o0[3], o1[3], xl.z, xl.w);
+                    mma_bf16(acc[nt], o0[4], o1[4], o0[5], o1[5], xh.x, xh.y);
+                    mma_bf16(acc[nt], o0[6], o1[6], o0[7], o1[7], xh.z, xh.w);
+                }
+            }
+            if (b + 2 < b1) ptx::named_barrier_sync(1 + half, 128);   // the tokens have been read: the buffer may be filled again
         }
-        ptx::named_barrier_sync(1 + half, 128);   // the tokens have been read: the buffer may be filled again
+        end(slot, acc);
     }
 }
 
-// Grid: (row groups x slices of the contraction = cluster, token tiles of all members).
-template <int NT8, int NB>
+// Grid: (row groups, for each the slices of the contraction; token tiles of all members).  Every slice has two slots, whose sums are added up
+// first, then the slices' sums one after the other; where that happens does not change the result:
+//   spread: a slice per CTA, a slot per half of its warps; the slices of a group are a cluster, and every CTA of it adds up a share of the rows,
+//           which the others' warps write into its shared memory;
+//   MERGED: one CTA does all slices of a group, each half of its warps every other half of them.  For grids of several waves: a CTA costs
+//           about 4 us beside its steps (its launch in a cluster, the way from a row's number to its codes, a barrier of the cluster).
+template <int NT8, int NB, bool MERGED>
 __global__ void __launch_bounds__(kSmallThreads, 2) small_kernel(const __grid_constant__ SmallParams<NB> P, const int slices) {
-    extern __shared__ __align__(16) unsigned char small_smem[];
+    extern __shared__ __align__(128) unsigned char small_smem[];
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (!MERGED) cluster_arrive();   // "this CTA runs": waited for before its shared memory is written from elsewhere
     constexpr int kTokens = 8 * NT8;
     constexpr uint32_t kTokenBytes = 2u * kTokens * kSmallSpan * 2u;     // two steps of one half of the warps
-    float* part = reinterpret_cast<float*>(small_smem + 2 * kTokenBytes);   // [2][tokens][kPartPitch]
+    float* sums = reinterpret_cast<float*>(small_smem + 2 * kTokenBytes);   // spread: [slots][tokens][share of the rows]; MERGED: see end()
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const int rank = (int)ptx::cluster_ctarank();
-    int grp = (int)blockIdx.x / slices;
+    const int rank = MERGED ? 0 : (int)ptx::cluster_ctarank();
+    int grp = MERGED ? (int)blockIdx.x : (int)blockIdx.x / slices;
     const Unit un = unit_at(P, (int)blockIdx.y, kTokens);
     const SmallMember& W = P.m[un.member];
     // the group's rows: 64 neighbouring stored rows of one precision class
@@ -311,93 +335,126 @@ __global__ void __launch_bounds__(kSmallThreads, 2) small_kernel(const __grid_co
     }
     const int p_first = W.L.class_start[c] + grp * kSmallRows, p_end = W.L.class_start[c + 1];
     const bool any = p_first < p_end;                                    // (members with other class counts have fewer groups)
+    if (MERGED && !any) return;
     const int tile = warp & 3, half = warp >> 2;
     const int p0 = p_first + tile * 16;
-    const int slot = rank * 2 + half, slots = slices * 2;
-    float acc[NT8][4];
-#pragma unroll
-    for (int i = 0; i < NT8; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.0f;
-    // the up-projection's fragments for this warp's rows: steps of 16 ranks, dealt to the slots
-    const int q0 = min(p0 + g, p_end - 1), q1 = min(p0 + g + 8, p_end - 1);
-    uint32_t up[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int j0 = (slot + i * slots) * 16 + 2 * t;
-        up[i][0] = up[i][1] = up[i][2] = up[i][3] = 0u;
-        if (any && (slot + i * slots) * 16 < P.r) {
-            const uint16_t* b0 = W.B + __ldg(W.L.perm + q0);
-            const uint16_t* b1 = W.B + __ldg(W.L.perm + q1);
-            const size_t N = (size_t)P.N;
-            up[i][0] = (uint32_t)__ldg(b0 + j0 * N) | ((uint32_t)__ldg(b0 + (j0 + 1) * N) << 16);
-            up[i][1] = (uint32_t)__ldg(b1 + j0 * N) | ((uint32_t)__ldg(b1 + (j0 + 1) * N) << 16);
-            up[i][2] = (uint32_t)__ldg(b0 + (j0 + 8) * N) | ((uint32_t)__ldg(b0 + (j0 + 9) * N) << 16);
-            up[i][3] = (uint32_t)__ldg(b1 + (j0 + 8) * N) | ((uint32_t)__ldg(b1 + (j0 + 9) * N) << 16);
-        }
+    const int slots = slices * 2, slot0 = MERGED ? half * slices : rank * 2 + half, slot1 = MERGED ? slot0 + slices : slot0 + 1;
+    const int share_log = 6 - (31 - __clz(slices)), share = 1 << share_log;
+    // the up-projection's fragments for this warp's rows: steps of 16 ranks, dealt to the slots; a slot's first one is fetched
+    // before its steps and put together when it is needed
+    const uint16_t *u0 = W.B, *u1 = W.B;
+    if (any && slot0 * 16 < P.r) {
+        u0 += __ldg(W.L.perm + min(p0 + g, p_end - 1));
+        u1 += __ldg(W.L.perm + min(p0 + g + 8, p_end - 1));
     }
+    const size_t N = (size_t)P.N;
+    uint32_t raw[8];
+    auto fetch_up = [&](int step) {
+        const size_t j = (size_t)(step * 16 + 2 * t) * N;
+        raw[0] = __ldg(u0 + j); raw[1] = __ldg(u0 + j + N); raw[2] = __ldg(u0 + j + 8 * N); raw[3] = __ldg(u0 + j + 9 * N);
+        raw[4] = __ldg(u1 + j); raw[5] = __ldg(u1 + j + N); raw[6] = __ldg(u1 + j + 8 * N); raw[7] = __ldg(u1 + j + 9 * N);
+    };
+    auto begin = [&](int slot) {
+        if (slot * 16 < P.r) fetch_up(slot);
+    };
+    auto end = [&](int slot, float (&acc)[NT8][4]) {
+        asm volatile("griddepcontrol.wait;" ::: "memory");               // T is in place
+        for (int i = slot; i * 16 < P.r; i += slots) {
+            if (i != slot) fetch_up(i);
+            const uint32_t a0 = raw[0] | (raw[1] << 16), a1 = raw[4] | (raw[5] << 16), a2 = raw[2] | (raw[3] << 16), a3 = raw[6] | (raw[7] << 16);
+#pragma unroll
+            for (int nt = 0; nt < NT8; ++nt) {
+                const int m = un.m0 + nt * 8 + g;
+                uint32_t b0 = 0u, b1 = 0u;
+                if (m < W.M) {
+                    const uint32_t* tr = reinterpret_cast<const uint32_t*>(W.T + (size_t)m * P.rp + i * 16) + t;
+                    b0 = __ldcg(tr);
+                    b1 = __ldcg(tr + 4);
+                }
+                mma_bf16(acc[nt], a0, a1, a2, a3, b0, b1);
+            }
+        }
+        if (MERGED) {
+            // Tiles of sums: 0 that of the first half's slices so far, 1 its slot that waits for the slice's other one, 2 + i the
+            // second half's slice i.  Every thread reads and writes its own places.
+            const int i = (slot - slot0) >> 1;
+            const bool odd = (slot & 1) != 0;
+            float* at = sums + (half == 0 ? (i == 0 ? 0 : 1) : 2 + i) * (kTokens * kMergedPitch) + 2 * t * kMergedPitch + tile * 16 + g;
+            float* first = sums + 2 * t * kMergedPitch + tile * 16 + g;
+#pragma unroll
+            for (int nt = 0; nt < NT8; ++nt) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const int o = (nt * 8 + (e & 1)) * kMergedPitch + (e >> 1) * 8;
+                    const float sum = odd ? at[o] + acc[nt][e] : acc[nt][e];
+                    if (half == 0 && odd && i > 0) first[o] += sum;
+                    else at[o] = sum;
+                }
+            }
+        } else {
+            const uint32_t to = ptx::smem_u32(sums) + (uint32_t)((slot * kTokens + 2 * t) << share_log) * 4u;
+            cluster_wait();
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int row = tile * 16 + 8 * h + g;
+                const uint32_t at = ptx::map_to_cta(to + (uint32_t)(row & (share - 1)) * 4u, (uint32_t)(row >> share_log));
+#pragma unroll
+                for (int nt = 0; nt < NT8; ++nt) {
+                    st_cluster_f32(at + (uint32_t)((nt * 8) << share_log) * 4u, acc[nt][2 * h]);
+                    st_cluster_f32(at + (uint32_t)((nt * 8 + 1) << share_log) * 4u, acc[nt][2 * h + 1]);
+                }
+            }
+        }
+    };
     if (any) {
         const uint32_t xs = ptx::smem_u32(small_smem) + (uint32_t)half * kTokenBytes;
-        if (c == 0) multiply_rows<1, NT8>(P.K, W, un.m0, p0, p_end, slot, slots, xs, half, acc);
-        else if (c == 1) multiply_rows<2, NT8>(P.K, W, un.m0, p0, p_end, slot, slots, xs, half, acc);
-        else multiply_rows<4, NT8>(P.K, W, un.m0, p0, p_end, slot, slots, xs, half, acc);
+        if (c == 0) multiply_rows<1, NT8>(P.K, W, un.m0, p0, p_end, slot0, slot1, slots, xs, half, begin, end);
+        else if (c == 1) multiply_rows<2, NT8>(P.K, W, un.m0, p0, p_end, slot0, slot1, slots, xs, half, begin, end);
+        else multiply_rows<4, NT8>(P.K, W, un.m0, p0, p_end, slot0, slot1, slots, xs, half, begin, end);
+    } else {
+        cluster_wait();
     }
-    asm volatile("griddepcontrol.wait;" ::: "memory");                   // T is in place
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        if (!any || (slot + i * slots) * 16 >= P.r) break;
-#pragma unroll
-        for (int nt = 0; nt < NT8; ++nt) {
-            const int m = un.m0 + nt * 8 + g;
-            uint32_t b0 = 0u, b1 = 0u;
-            if (m < W.M) {
-                const uint32_t* tr = reinterpret_cast<const uint32_t*>(W.T + (size_t)m * P.rp + (slot + i * slots) * 16) + t;
-                b0 = __ldcg(tr);
-                b1 = __ldcg(tr + 4);
-            }
-            mma_bf16(acc[nt], up[i][0], up[i][1], up[i][2], up[i][3], b0, b1);
+    if (MERGED) {
+        __syncthreads();
+        for (int i = threadIdx.x; i < kTokens * kSmallRows; i += kSmallThreads) {
+            const int m = i / kSmallRows, row = i % kSmallRows;
+            if (un.m0 + m >= W.M || p_first + row >= p_end) continue;
+            const float* from = sums + m * kMergedPitch + row;
+            float sum = from[0];
+            for (int s = 0; s < slices / 2; ++s) sum += from[(2 + s) * (kTokens * kMergedPitch)];
+            W.Y[(size_t)(un.m0 + m) * P.N + __ldg(W.L.perm + p_first + row)] = (uint16_t)pack_bf16x2(sum, 0.0f);
         }
-    }
-#pragma unroll
-    for (int nt = 0; nt < NT8; ++nt) {
-        float* d = part + (half * kTokens + nt * 8 + 2 * t) * kPartPitch + tile * 16 + g;
-        d[0] = acc[nt][0]; d[kPartPitch] = acc[nt][1];
-        d[8] = acc[nt][2]; d[kPartPitch + 8] = acc[nt][3];
+        return;
     }
     ptx::cluster_sync();
-    // every CTA of the cluster adds up its share of the rows over the slices, in a fixed order
-    const int share = kSmallRows / slices;
-    const uint32_t part_addr = ptx::smem_u32(part);
-    for (int i = threadIdx.x; any && i < share * kTokens; i += kSmallThreads) {
-        const int m = i / share, row = rank * share + (i - m * share);
+    for (int i = threadIdx.x; any && i < (kTokens << share_log); i += kSmallThreads) {
+        const int m = i >> share_log, row = (rank << share_log) + (i & (share - 1));
         if (un.m0 + m >= W.M || p_first + row >= p_end) continue;
         float sum = 0.0f;
-        for (int s = 0; s < slices; ++s) {
-            const uint32_t addr = ptx::map_to_cta(part_addr + (uint32_t)(m * kPartPitch + row) * 4u, (uint32_t)s);
-            sum += ld_cluster_f32(addr) + ld_cluster_f32(addr + (uint32_t)(kTokens * kPartPitch) * 4u);
-        }
+        for (int s = 0; s < slices; ++s) sum += sums[((2 * s * kTokens) << share_log) + i] + sums[(((2 * s + 1) * kTokens) << share_log) + i];
         W.Y[(size_t)(un.m0 + m) * P.N + __ldg(W.L.perm + p_first + row)] = (uint16_t)pack_bf16x2(sum, 0.0f);
     }
-    ptx::cluster_sync();   // nobody leaves while a peer still reads its sums
 }
 
-template <int NT8, int NB>
+template <int NT8, int NB, bool MERGED>
 lowra_status launch_product(const SmallParams<NB>& P, int groups, int units, int slices, cudaStream_t stream) {
-    constexpr size_t smem = 4u * (8 * NT8) * kSmallSpan * 2u + 2u * (8 * NT8) * kPartPitch * 4u;
+    const size_t smem = 4u * (8 * NT8) * kSmallSpan * 2u + (MERGED ? (2 + slices / 2) * (8 * NT8) * kMergedPitch * 4u : 2u * (8 * NT8) * kSmallRows * 4u);
     static SmemLimit limit = {};
-    if (ensure_smem_limit(reinterpret_cast<const void*>(small_kernel<NT8, NB>), smem, &limit) != LOWRA_OK) return LOWRA_ERR_CUDA;
+    if (ensure_smem_limit(reinterpret_cast<const void*>(small_kernel<NT8, NB, MERGED>), smem, &limit) != LOWRA_OK) return LOWRA_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)slices;
-    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.gridDim = dim3((unsigned)(groups * slices), (unsigned)units, 1);
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)slices;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)(MERGED ? groups : groups * slices), (unsigned)units, 1);
     cfg.blockDim = dim3(kSmallThreads, 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cfg.attrs = attr;
-    cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, small_kernel<NT8, NB>, P, slices) == cudaSuccess ? LOWRA_OK : LOWRA_ERR_CUDA;
+    cfg.numAttrs = MERGED ? 1 : 2;
+    return cudaLaunchKernelEx(&cfg, small_kernel<NT8, NB, MERGED>, P, slices) == cudaSuccess ? LOWRA_OK : LOWRA_ERR_CUDA;
 }
 
 template <int NB>
@@ -415,8 +472,7 @@ lowra_status launch_members(const SmallParams<NB>& P, cudaStream_t stream) {
     {
         int slices = 1;
         while (slices < 8 && P.K >= 256 * slices) slices *= 2;
-        const size_t fetch = (size_t)8 * kProjectBatch * 16 * (P.r * 2 + 16), sums = (size_t)(8 + 1) * 16 * P.r * 4;
-        const size_t smem = fetch > sums ? fetch : sums;
+        const size_t smem = project_fetch_bytes(P.r) + (size_t)16 * P.r * 4;
         static SmemLimit limit = {};
         if (ensure_smem_limit(reinterpret_cast<const void*>(project_kernel<NB>), smem, &limit) != LOWRA_OK) return LOWRA_ERR_CUDA;
         cudaLaunchConfig_t cfg = {};
@@ -439,12 +495,20 @@ lowra_status launch_members(const SmallParams<NB>& P, cudaStream_t stream) {
     const int n_span = (P.K + kSmallSpan - 1) / kSmallSpan, by_shape = (P.N + kSmallRows - 1) / kSmallRows;
     int slices = 1;
     while (slices < 8 && 4 * slices <= n_span && 2 * slices * by_shape <= 3 * kNumSMs) slices *= 2;
-    const int nt8 = most <= 8 ? 1 : most <= 16 ? 2 : 4;
+    const int nt8 = most <= 8 ? 1 : most <= 16 ? 2 : most <= 24 ? 3 : 4;
     int units = 0;
     for (int i = 0; i < P.count; ++i) units += (P.m[i].M + 8 * nt8 - 1) / (8 * nt8);
-    if (nt8 == 1) return launch_product<1, NB>(P, groups, units, slices, stream);
-    if (nt8 == 2) return launch_product<2, NB>(P, groups, units, slices, stream);
-    return launch_product<4, NB>(P, groups, units, slices, stream);
+    // Merged where a CTA's own cost outweighs its steps: slots of one or two steps, few tokens, more CTAs than run at a time.  (Groups of
+    // adapters on 4096 x 4096 at 30/50/20 %: 8 tokens in 4 groups 26.0 against 34.6 us spread, 16 in 8 48.5 against 60.0; but with up to 32
+    // tokens a group 64 in 2 38.5 against 34.8; on 4096 x 11008 - slots of five steps - 6 in 3 54.5 against 46.1; one group 18.8 against 10.6.)
+    if constexpr (NB > 1) {
+        if (slices > 1 && nt8 <= 2 && n_span <= 2 * (2 * slices) && groups * slices * units > 2 * kNumSMs)
+            return nt8 == 1 ? launch_product<1, NB, true>(P, groups, units, slices, stream) : launch_product<2, NB, true>(P, groups, units, slices, stream);
+    }
+    if (nt8 == 1) return launch_product<1, NB, false>(P, groups, units, slices, stream);
+    if (nt8 == 2) return launch_product<2, NB, false>(P, groups, units, slices, stream);
+    if (nt8 == 3) return launch_product<3, NB, false>(P, groups, units, slices, stream);
+    return launch_product<4, NB, false>(P, groups, units, slices, stream);
 }
 
 }  // namespace
