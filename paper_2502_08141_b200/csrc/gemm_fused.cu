@@ -821,16 +821,19 @@ static int plan_schedule(GemmParams& Q, bool may_cut, int max_clusters) {
         }
         if (!may_cut || Q.sk_part == nullptr || n_t > max_clusters || blocks < 2 * kMinRange) continue;
         if ((long long)n * blocks * max_clusters >= (1ll << 31)) continue;     // (32-bit arithmetic in the kernel)
-        // fewer pieces than clusters: s clusters per weight tile, the clusters left over share the T tiles
+        // Fewer pieces than clusters: s clusters per weight tile, the clusters left over share the T tiles.  Short runs have estimates of
+        // their own: a shared T tile takes 0.3 per block and 7.5 + 0.5 per 256 tokens and contributor around them, a 256-token
+        // tile 0.55 per block, and collecting starts 3.2 later than at the end of a range, for the contributors end together.  (With the
+        // ranges' figures, which have T twice as late: 4096 x 4096, 256 tokens, weight tiles cut in two 41.4 us, in four 32.0.)
         for (int s = 1; s < kMaxContributors && n_w * s + n_t <= max_clusters && blocks / s >= shortest; ++s) {
             int ts = (max_clusters - n_w * s) / n_t;
             if (ts > kMaxContributors) ts = kMaxContributors;
             if (ts > Q.main_blocks / kMinRange) ts = Q.main_blocks / kMinRange;
             if (ts < 2) ts = 1;
             if (ts == 1 && s == 1) continue;
-            const float t_done = ts == 1 ? t_us : ramp + t_pace * Q.main_blocks / ts + 2.4f + 4.5f + 1.2f * halves * ts;
-            const float w_done = ramp + pace * blocks / s;
-            const float us = (t_done > w_done ? t_done : w_done) + (s == 1 ? drain : drain + collect(s - 1));
+            const float t_done = ts == 1 ? t_us : 7.5f + 0.3f * Q.main_blocks / ts + 0.5f * halves * ts;
+            const float w_done = ramp + (halves == 1 ? 0.55f : 0.8f) * blocks / s;
+            const float us = (t_done > w_done ? t_done : w_done) + (s == 1 ? drain : drain + collect(s - 1) + 3.2f);
             offer({us, halves, n_t * ts + n_w * s, 1, 0, n_t * ts, 0, ts, n_w * blocks});
         }
         // Ranges for the last row of pieces, or for the last two.  The clusters' sweeps over the contraction fall out of step
