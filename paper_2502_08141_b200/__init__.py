@@ -173,11 +173,16 @@ def _stream(stream) -> int:
     return torch.cuda.current_stream().cuda_stream
 
 
+_BF16 = torch.bfloat16
+
+
 def _ptr(t: Optional[torch.Tensor]) -> int:
     return 0 if t is None else t.data_ptr()
 
 
 def _dev(t: torch.Tensor, dtype, name: str) -> torch.Tensor:
+    if t.is_cuda and t.dtype is dtype and t.is_contiguous():
+        return t
     if not t.is_cuda:
         raise ValueError(f"{name} must be a CUDA tensor")
     if t.dtype != dtype:
@@ -231,6 +236,7 @@ class Layout:
         c.natural_offsets_dev = None
         self.c = c
         self.ref = ctypes.byref(c)
+        self.last_size = (0, 0, 0)
         self.deal = None
         self.natural_offsets = None
         if natural:
@@ -399,9 +405,14 @@ def lowra_workspace_bytes(layout: Layout, M: int, r: int) -> int:
 
 
 def _workspace(layout: Layout, M: int, r: int, device) -> torch.Tensor:
-    n = lowra_workspace_bytes(layout, M, r)
-    if n == 0:
-        raise LowraError(LOWRA_ERR_SHAPE, "lowra_workspace_bytes")
+    last = layout.last_size           # the size follows from the shape, M and r: asked for once for calls of one size
+    if last[0] == M and last[1] == r:
+        n = last[2]
+    else:
+        n = lowra_workspace_bytes(layout, M, r)
+        if n == 0:
+            raise LowraError(LOWRA_ERR_SHAPE, "lowra_workspace_bytes")
+        layout.last_size = (M, r, n)
     ws = torch.empty(n, dtype=torch.uint8, device=device)
     if layout.deal is not None:   # no prologue launch will clear it
         lowra_workspace_init(ws)
@@ -419,19 +430,20 @@ def lowra_lora_forward(layout: Layout, packed, absmax, maps, X, A, B, s: float,
                        Y: Optional[torch.Tensor] = None, workspace: Optional[torch.Tensor] = None,
                        stream=None) -> torch.Tensor:
     """Y = X . deq(Wq)^T + s (X . A) . B ; X bf16 [M,K], A bf16 [K,r], B bf16 [r,N] -> Y bf16 [M,N]."""
-    for t, n in ((X, "X"), (A, "A"), (B, "B")):
-        _dev(t, torch.bfloat16, n)
-    M, r = int(X.shape[0]), int(A.shape[1])
-    if tuple(X.shape) != (M, layout.K) or tuple(A.shape) != (layout.K, r) or tuple(B.shape) != (r, layout.N):
+    _dev(X, _BF16, "X")
+    _dev(A, _BF16, "A")
+    _dev(B, _BF16, "B")
+    M, r = X.shape[0], A.shape[1]
+    if X.shape != (M, layout.K) or A.shape != (layout.K, r) or B.shape != (r, layout.N):
         raise ValueError("shape mismatch")
     if Y is None:
         Y = X.new_empty((M, layout.N))
     if workspace is None:
         workspace = _workspace(layout, M, r, X.device)
-    code = lib().lowra_lora_forward(layout.ref, _ptr(packed), _ptr(absmax), _ptr(maps), _ptr(X), M, _ptr(A),
-                                    _ptr(B), r, s, _ptr(Y), _ptr(workspace),
-                                    workspace.numel(), _stream(stream))
-    _check(code, "lowra_lora_forward")
+    code = (_lib or lib()).lowra_lora_forward(layout.ref, _ptr(packed), _ptr(absmax), _ptr(maps), X.data_ptr(), M, A.data_ptr(),
+                                              B.data_ptr(), r, s, Y.data_ptr(), workspace.data_ptr(), workspace.numel(), _stream(stream))
+    if code:
+        _check(code, "lowra_lora_forward")
     return Y
 
 
