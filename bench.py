@@ -180,10 +180,10 @@ def host_matrix(cfg, mat, rank: int, per_rank: int):
 
 # DRAM traffic of one fused_kernel launch measured with ncu (dram__bytes_read.sum + dram__bytes_write.sum) on a
 # launch of workload 3: the backward-input pass of gate_proj (dX [4096, 4096] from dY [4096, 11008];
-# profiles/fused_backward_input_11008x4096_m4096_streamk.md): 169.0 MB read + 26.9 MB written.  The bytes the call
-# has to read and write once are 137 MB (the output is partly still in L2 when the kernel ends; the stream-K partial
-# tiles add 19 MB each way).  Scaled to the step's average launch in proportion to those input + output bytes.
-NCU_CASE = dict(N=4096, K=11008, M=4096, r=64, bits=1.5, dram_bytes=169.0e6 + 26.9e6)
+# profiles/fused_backward_input_11008x4096_m4096_streamk.md): 193.7 MB read + 50.6 MB written.  The bytes the call
+# has to read and write once are 137 MB (the output is partly still in L2 when the kernel ends; the partial tiles of
+# the cut last row add up to 38 MB each way).  Scaled to the step's average launch in proportion to those input + output bytes.
+NCU_CASE = dict(N=4096, K=11008, M=4096, r=64, bits=1.5, dram_bytes=193.7e6 + 50.6e6)
 
 
 def fused_io_bytes(N, K, M, r, bits):
@@ -985,7 +985,7 @@ CASES = ("forward", "backward", "forward4096", "backward_gate", "forward_4bit", 
 
 def run_case(case: str) -> None:
     """forward / backward: fused calls, N = K = 4096, 2048 tokens, rank 64 (config-3 mix; *_4bit, *_1bit: every row
-    at that precision); forward4096: 4096 tokens (264 pieces: tiles cut between SMs, partial tiles preloaded);
+    at that precision); forward4096: 4096 tokens (136 pieces: tiles cut between SMs);
     backward_gate: 11008 x 4096 at 4096 tokens (last row of tiles cut); codec: decode + encode of an 11008 x 4096
     matrix; decode_layer: the seven decodes of a Llama-7B layer back to back; learn: codebook learner, 4096 x 4096,
     10 rounds; adapters: gradients of the low-rank factors, 4096 x 11008, 4096 tokens (adapters_reuse: from given projections); errors: per-channel
