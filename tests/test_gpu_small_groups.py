@@ -1,6 +1,6 @@
 """Several adapters' small token groups where their product changes its form: one CTA for all slices of 64 rows (many groups of up to 16
 tokens, slots of one or two steps) or a cluster for them.  Every group's result is bit for bit that of a call of its own, which
-takes the other form."""
+takes the other form, and leaves the projection that the gradients read."""
 import pytest
 import torch
 
@@ -16,6 +16,9 @@ pytestmark = pytest.mark.gpu
     (704, 4096, 48, (8, 8, 8, 8, 8, 8, 8)),             # eight slices
     (4096, 4096, 64, (12, 16)),
     (4096, 4224, 64, (2, 2)),                           # slots of three steps: a cluster after all
+    (512, 512, 16, (16, 1, 33)),
+    (136, 128, 128, (9, 32)),                           # a contraction of half a step
+    (264, 640, 16, (2, 25)),                            # steps that do not come out even
 ])
 def test_groups_equal_calls_of_their_own(N, K, r, counts):
     import paper_2502_08141_b200 as lw
@@ -35,3 +38,8 @@ def test_groups_equal_calls_of_their_own(N, K, r, counts):
         rows = slice(start[a], start[a + 1])
         own = lw.lowra_lora_forward(layout, packed, absmax, tables[a].contiguous(), X[rows].contiguous(), A[a].contiguous(), B[a].contiguous(), 2.0)
         assert torch.equal(Y[rows], own), a
+        T = 2.0 * (X[rows].float() @ A[a].float())      # what the call leaves for the gradients: bf16 of that, ranks padded to 64 with zeros
+        ws = torch.zeros(lw.lowra_workspace_bytes(layout, counts[a], r), dtype=torch.uint8, device="cuda")
+        lw.lowra_lora_forward(layout, packed, absmax, tables[a].contiguous(), X[rows].contiguous(), A[a].contiguous(), B[a].contiguous(), 2.0, workspace=ws)
+        left = lw.lowra_workspace_projection(ws, counts[a], r).float()
+        assert bool(((left[:, :r] - T).abs() <= 2.0 ** -8 * T.abs() + 2.0 ** -16 * K ** 0.5).all()) and not bool(left[:, r:].any()), a
