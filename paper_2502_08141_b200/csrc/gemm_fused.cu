@@ -800,7 +800,7 @@ fused_kernel(const __grid_constant__ KParams<NB> P, const __grid_constant__ KMap
 //   4.5 until the first MMA; 0.6 / 0.8 per contraction block of a 256- / 512-token tile (the smaller one paced by dequantisation,
 //   the larger one by the tensor core); 0.5 / 0.7 of a T tile (paced by its loads); 2.4 per 256 tokens to write a partial tile or to
 //   drain the last accumulator; to collect partial tiles 4.5 and, per 256 tokens, four steps of 1.1 or 0.6 per contributor.
-static int plan_schedule(GemmParams& Q, bool may_cut, int max_clusters) {
+static int plan_schedule(GemmParams& Q, bool may_cut, int max_clusters, float* estimate = nullptr) {
     const int blocks = Q.main_blocks + Q.lora_blocks;
     struct Choice { float us; int halves, clusters, cut, first, c0, extra, t_split, num; } best = {};
     best.us = -1.0f;
@@ -873,7 +873,26 @@ static int plan_schedule(GemmParams& Q, bool may_cut, int max_clusters) {
     Q.sk_extra = best.extra;
     Q.sk_num = best.num;
     Q.t_split = best.t_split;
+    if (estimate != nullptr) *estimate = best.us;
     return best.clusters;
+}
+
+// The estimate for a forward call of M tokens by itself on a whole GPU.  Weights that mix 4-bit channels with others take longer than the choice
+// of a schedule counts for (13824 x 13824, a quarter of 4 bits, 64 tokens, 158 us for 126; 11008 x 1024, 4 % of 4 bits, 20.0 for 17.9;
+// 4096 x 4096, 64 tokens: 29.5 with 5 % of 4 bits, 27.0 with 4 bits alone): what lies above a tile's start and drain counts so much more.
+float fused_estimate(int N, int K, int M, int r) {
+    GemmParams Q;
+    memset(&Q, 0, sizeof(Q));
+    float some = 0.0f, us = 0.0f;
+    Q.count = 1;
+    Q.mem[0].M = Q.M = M;
+    Q.C = K;
+    Q.main_blocks = (K + kTileC - 1) / kTileC;
+    Q.lora_blocks = (r + 63) / 64 * 64 / kTileC;
+    Q.tiles_r = (N + kPairR - 1) / kPairR;
+    Q.sk_part = &some;   // (tiles may be cut)
+    plan_schedule(Q, true, kNumSMs / kCluster, &us);
+    return us + (Q.sk ? 0.35f : 0.12f) * (us - 7.0f);
 }
 
 template <int MODE, int NB>

@@ -141,9 +141,10 @@ constexpr uint32_t kGemmSmemBytes = kSmemRing + kSmemBarriers;
 static_assert(kGemmSmemBytes <= 232448, "227 KB of shared memory per CTA");
 
 lowra_status launch_fused(int mode, const GemmParams& G, const BatchMaps& TM, cudaStream_t stream);
+float fused_estimate(int N, int K, int M, int r);
 
 // ---- forward pass for few tokens (gemm_small.cu) --------------------------------------------
-constexpr int kSmallTokens = 64;    // members of up to so many tokens take it
+constexpr int kSmallTokens = 64;    // members of up to so many tokens may take it, of 16 and fewer do
 constexpr int kSmallMembers = 8;    // per launch
 struct SmallMember {
     RowLayout L;
@@ -154,6 +155,7 @@ struct SmallMember {
     uint16_t *Y, *T;          // T [M, rp]: s X A, as the fused calls leave it
     int M;
 };
+float small_estimate(int N, int K, int M);
 template <int NB>   // members the kernel's parameters have room for
 struct SmallParams {
     SmallMember m[NB];
