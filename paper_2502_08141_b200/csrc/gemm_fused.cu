@@ -880,9 +880,9 @@ static int plan_schedule(GemmParams& Q, bool may_cut, int max_clusters, float* e
     return best.clusters;
 }
 
-// The estimate for a forward call of M tokens by itself on a whole GPU.  Weights that mix 4-bit channels with others take longer than the choice
-// of a schedule counts for (13824 x 13824, a quarter of 4 bits, 64 tokens, 158 us for 126; 11008 x 1024, 4 % of 4 bits, 20.0 for 17.9;
-// 4096 x 4096, 64 tokens: 29.5 with 5 % of 4 bits, 27.0 with 4 bits alone): what lies above a tile's start and drain counts so much more.
+// The estimate for a forward call of M tokens by itself on a whole GPU.  Where tiles are cut, weights that mix 4-bit channels with others take
+// longer than the choice of a schedule counts for (13824 x 5120 at 60/35/5, 65 tokens, 56.5 us for 51.5; with 1 and 2 bits 46.7): what
+// lies above a tile's start and drain counts a quarter more, so that the tiles are chosen where they win for every mix.
 float fused_estimate(int N, int K, int M, int r) {
     GemmParams Q;
     memset(&Q, 0, sizeof(Q));
@@ -895,7 +895,7 @@ float fused_estimate(int N, int K, int M, int r) {
     Q.tiles_r = (N + kPairR - 1) / kPairR;
     Q.sk_part = &some;   // (tiles may be cut)
     plan_schedule(Q, true, kNumSMs / kCluster, &us);
-    return us + (Q.sk ? 0.35f : 0.12f) * (us - 7.0f);
+    return Q.sk ? us + 0.26f * (us - 7.0f) : us;
 }
 
 template <int MODE, int NB>

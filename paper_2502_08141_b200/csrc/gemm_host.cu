@@ -163,11 +163,10 @@ lowra_status run_small(const MemberArgs* mem, uint16_t* const* T_of, int count, 
 // The diagnostic lowra_diag_drop_t_flags is about flags, which the path for few tokens has none of: it leaves that path out.  Otherwise the
 // choice follows from the weight's shape and the member's tokens alone, so that a member's result does not depend on its company.
 // From 33 tokens on that path dequantises every weight twice, which weights with many channels and short contractions do not repay (64 tokens,
-// forward, few-token path against tensor-core tiles, us: 2048 x 2048 13.5 against 31, 4096 x 4096 27.0 against 29.5, 8192 x 8192 54 against
-// 64; but 8192 x 512 16.6 against 14.1, 11008 x 1024 32 against 20, 13824 x 512 28 against 13, 13824 x 2560 44 against 38).  The
-// choice leans to the few-token path where the weight's precisions decide: 5120 x 13824, all of 4 bits, keeps it at 72 against 54.
-// At 17 to 32 tokens only the shortest contractions of many channels leave it (13824 x 256, 32 tokens, 18.0 against 11.0; 13824 x 512
-// 17.8 against 13.1), up to 16 tokens none.
+// forward, few-token path against tensor-core tiles, us: 2048 x 2048 13.7 against 26, 4096 x 4096 and 8192 x 8192 alike; but 8192 x 512 16.9
+// against 13.1, 11008 x 1024 32 against 18, 13824 x 512 28.7 against 13.3, 13824 x 2560 44 against 33).  The choice leans to the few-token
+// path where the weight's precisions decide: 5120 x 13824, all of 4 bits, keeps it at 72 against 54.  At 17 to 32 tokens only
+// the shortest contractions of many channels leave it (32 tokens, 13824 x 256 18.0 against 11.0; 13824 x 512 17.8 against 13.1).
 bool takes_small_path(bool backward, int N, int K, int M, int r) {
     if (backward || M > kSmallTokens || g_drop_t_flags.load(std::memory_order_relaxed) != 0) return false;
     return M <= 16 || small_estimate(N, K, M) < fused_estimate(N, K, M, r);
