@@ -815,7 +815,7 @@ static int plan_schedule(GemmParams& Q, bool may_cut, int max_clusters, float* e
     auto offer = [&](const Choice& c) { if (best.us < 0.0f || c.us < best.us) best = c; };
     // every range keeps a sixth of a tile, so that a tile has at most kMaxContributors contributors
     const int sixth = (blocks + kMaxContributors - 2) / (kMaxContributors - 1), shortest = sixth > kMinRange ? sixth : kMinRange;
-    for (int halves = 1; halves <= (Q.M > kHalfT ? 2 : 1); ++halves) {
+    for (int halves = Q.wide_only ? 2 : 1; halves <= (Q.M > kHalfT ? 2 : 1); ++halves) {
         const float pace = halves == 1 ? 0.6f : 0.8f, t_pace = halves == 1 ? 0.5f : 0.7f;
         const float ramp = 4.5f, drain = 2.4f * halves;
         auto collect = [&](int nc) { return 4.5f + 4.0f * halves * (0.6f * nc > 1.1f ? 0.6f * nc : 1.1f); };

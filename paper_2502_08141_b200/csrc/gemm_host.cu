@@ -25,14 +25,22 @@ namespace {
 constexpr size_t kStatusBytes = 256;   // status word at byte 0, then the two words that number the calls:
 constexpr size_t kEpochOffset = 64;    //   number of the last call that ran on this workspace
 constexpr size_t kExitsOffset = 128;   //   CTAs of the running call that have left
+// The flags of the fused calls ("partial tile ready", one per CTA, then "T ready") follow at a place that does not depend on the call.
+// Nothing else is ever written there, so a flag word holds zero or the number of an earlier call on this workspace.  (Behind T they moved
+// with the number of tokens, and "up" - equal to the call's number - could be read out of old T values.)
+constexpr size_t kFlagsOffset = kStatusBytes;
+constexpr size_t kHeaderBytes = 4096;  // status word, numbering, flags
+constexpr int kHeaderFlags = (int)((kHeaderBytes - kFlagsOffset) / 4), kSkFlags = kMaxClusters * kCluster;
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 struct Workspace {
     size_t off_T[kMaxBatch];      // per member: its down-projected activations
-    int flag0[kMaxBatch];         // per member: index of its first "T ready" flag
-    size_t off_flags, off_items, off_part, total;
-    int rp, n_flags, sk_flag0;
+    int flag0[kMaxBatch];         // per member: index of its first "T ready" flag, counted from off_t_flags
+    size_t off_t_flags;
+    size_t t_flag_bytes;          // 0: they lie in the header; else behind T, and every call clears them
+    size_t off_items, off_part, total;
+    int rp, n_flags;              // flags of the header that the call uses
 };
 
 bool rank_ok(int r) { return r >= 16 && r <= 128 && r % 16 == 0; }
@@ -59,18 +67,24 @@ Workspace plan_workspace(int N, int K, const int* Ms, int count, int r, bool str
     Workspace w;
     memset(&w, 0, sizeof(w));
     w.rp = (r + 63) / 64 * 64;
-    size_t off = kStatusBytes;
+    // "T ready" flags: one per CTA and token tile of 256.  A call with so many tokens that they do not fit into the header (100 000 tokens)
+    // brings them along, one per CTA and token tile of 512, which such a call always takes.
+    int tiles = 0;
+    for (int i = 0; i < count; ++i) tiles += (Ms[i] + kHalfT - 1) / kHalfT;
+    const bool in_header = tiles <= (kHeaderFlags - kSkFlags) / kCluster;
+    const int per_tile = in_header ? kHalfT : kTileT;
+    size_t off = kHeaderBytes;
     int flags = 0;
     for (int i = 0; i < count; ++i) {
         w.off_T[i] = off;
         off += align256((size_t)Ms[i] * w.rp * 2);
-        w.flag0[i] = flags;          // the member's "T ready" flags: one per CTA and token tile
-        flags += (Ms[i] + kHalfT - 1) / kHalfT * kCluster;
+        w.flag0[i] = flags;
+        flags += (Ms[i] + per_tile - 1) / per_tile * kCluster;
     }
-    w.off_flags = off;
-    w.sk_flag0 = flags;                                  // then one "partial tile ready" flag per CTA
-    w.n_flags = flags + kMaxClusters * kCluster;
-    w.off_items = w.off_flags + align256((size_t)w.n_flags * 4);
+    w.off_t_flags = in_header ? kFlagsOffset + kSkFlags * 4 : off;
+    w.t_flag_bytes = in_header ? 0 : (size_t)flags * 4;
+    w.n_flags = kSkFlags + (in_header ? flags : 0);
+    w.off_items = off + align256(w.t_flag_bytes);
     // room for the deal of one direction, rebuilt by every call that brings none
     const size_t fwd = deal_forward_bytes(N), bwd = deal_backward_bytes(N);
     w.off_part = w.off_items + align256(fwd > bwd ? fwd : bwd);
@@ -189,13 +203,15 @@ lowra_status run_members(bool backward, const MemberArgs* mem, int count, int32_
 
     unsigned char* ws = static_cast<unsigned char*>(workspace);
     uint32_t* status = reinterpret_cast<uint32_t*>(ws);
-    uint32_t* flags = reinterpret_cast<uint32_t*>(ws + w.off_flags);
+    uint32_t* flags = reinterpret_cast<uint32_t*>(ws + kFlagsOffset);
+    uint32_t* t_flags = reinterpret_cast<uint32_t*>(ws + w.off_t_flags);
 
     if (takes_small_path(backward, N, K, M, r)) {   // (M: the largest member's tokens)
         uint16_t* T_of[kMaxBatch];
         for (int i = 0; i < count; ++i) T_of[i] = reinterpret_cast<uint16_t*>(ws + w.off_T[i]);
         return run_small(mem, T_of, count, r, s, workspace, stream);
     }
+    if (w.t_flag_bytes > 0 && cudaMemsetAsync(t_flags, 0, w.t_flag_bytes, stream) != cudaSuccess) return LOWRA_ERR_CUDA;
 
     GemmParams G;
     memset(&G, 0, sizeof(G));
@@ -211,7 +227,7 @@ lowra_status run_members(bool backward, const MemberArgs* mem, int count, int32_
         g.maps = m.maps;
         g.out = m.out;
         g.T = reinterpret_cast<uint16_t*>(ws + w.off_T[i]);
-        g.flags = flags + w.flag0[i];
+        g.flags = t_flags + w.flag0[i];
         g.M = m.M;
         if (m.layout->deal_dev != nullptr) {
             // the rows were dealt once for this weight (lowra_deal_build) and the workspace numbers its calls
@@ -246,7 +262,8 @@ lowra_status run_members(bool backward, const MemberArgs* mem, int count, int32_
     G.status = status;
     G.epoch = reinterpret_cast<uint32_t*>(ws + kEpochOffset);
     G.exits = reinterpret_cast<uint32_t*>(ws + kExitsOffset);
-    G.n_flags = w.n_flags;
+    G.n_flags = kHeaderFlags;
+    G.wide_only = w.t_flag_bytes > 0;
     G.s = s;
     G.rp = w.rp;
     G.r = r;
@@ -264,7 +281,7 @@ lowra_status run_members(bool backward, const MemberArgs* mem, int count, int32_
         if (!seen) G.operand_bytes += (long long)mem[i].M * G.C * 2;
     }
     G.sk_part = stream_k ? reinterpret_cast<float*>(ws + w.off_part) : nullptr;   // null: whole tiles only
-    G.sk_flags = flags + w.sk_flag0;
+    G.sk_flags = flags;
     G.wait_ns = wait_limit_ns();
     {   // diagnostic, armed by lowra_diag_drop_t_flags: take one of the calls it asked for
         int left = g_drop_t_flags.load(std::memory_order_relaxed);
@@ -478,7 +495,7 @@ extern "C" lowra_status lowra_lora_forward_adapters(const lowra_layout* layout, 
     for (int a = 0; a <= n_adapters; ++a) {
         if (a < n_adapters && group_start_host[a + 1] > group_start_host[a] && is_small(a)) {
             if (n_few == 0 && (st = check_members(&(few[0] = member(a)), 1, r, workspace_dev, workspace_bytes, true)) != LOWRA_OK) return st;
-            few_T[n_few] = reinterpret_cast<uint16_t*>(static_cast<unsigned char*>(workspace_dev) + kStatusBytes) +
+            few_T[n_few] = reinterpret_cast<uint16_t*>(static_cast<unsigned char*>(workspace_dev) + kHeaderBytes) +
                            (size_t)group_start_host[a] * (size_t)((r + 63) / 64 * 64);
             few[n_few++] = member(a);
         }
@@ -648,7 +665,7 @@ extern "C" const uint16_t* lowra_workspace_projection(const void* workspace_dev,
     using namespace lowra;
     if (!workspace_dev || member < 0 || member >= kMaxBatch || M < 1 || !rank_ok(r)) return nullptr;
     const size_t t_bytes = align256((size_t)M * (size_t)((r + 63) / 64 * 64) * 2);   // as plan_workspace lays equal members out
-    return reinterpret_cast<const uint16_t*>(static_cast<const unsigned char*>(workspace_dev) + kStatusBytes + (size_t)member * t_bytes);
+    return reinterpret_cast<const uint16_t*>(static_cast<const unsigned char*>(workspace_dev) + kHeaderBytes + (size_t)member * t_bytes);
 }
 
 extern "C" lowra_status lowra_device_status(const void* workspace_dev, void* stream) {

@@ -87,14 +87,15 @@ using BatchMaps = KMaps<kMaxBatch>;
 // plain call then carries 0.7 KB of kernel parameters instead of 2.8 KB, which its launch latency shows.)
 struct GemmCommon {
     int count;              // members (1 for the plain calls); all of one shape
-    uint32_t* flags;        // all flags of the workspace (the members' T flags, then the partial-tile flags)
+    uint32_t* flags;        // the flags that stay in the workspace from call to call
     uint32_t* status;
     // Calls on one workspace are numbered: `epoch` holds the number of the last call that ran on it, a call's own
     // number is that + 1, and a flag is up when it holds the call's number - so flags left over from earlier calls
     // never need clearing.  The last CTA to leave (counted in `exits`) writes the call's number back.
     uint32_t* epoch;
     uint32_t* exits;
-    int n_flags;            // all flags of the workspace (T ready + partial tile ready), for the wrap of the numbering
+    int n_flags;            // their number, for the wrap of the numbering
+    int wide_only;          // (host) token tiles of 512 only: the call's flags are counted for those
     float s;
     int rp;                 // LoRA rank rounded up to 64
     int r;                  // LoRA rank

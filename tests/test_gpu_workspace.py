@@ -1,0 +1,100 @@
+"""What a workspace carries from call to call: the flags of the fused calls, which are "up" when they hold the number of the call,
+must never lie where another call leaves its down-projected tokens (whose bits can be any number); and calls of so many tokens
+that their flags do not fit beside the others.
+"""
+import numpy as np
+import pytest
+import torch
+
+import synth_inputs as si
+from helpers import FRO_TOL, MAX_TOL, gemm_errors
+
+pytestmark = pytest.mark.gpu
+
+
+class _Problem:
+    def __init__(self, N, K, r, dealt=True, adapters=1):
+        import paper_2502_08141_b200 as lw
+
+        self.lw, self.N, self.K, self.r = lw, N, K, r
+        self.gen = torch.Generator(device="cuda").manual_seed(N + K + r)
+        precs = si.precisions(N, {1: 0.3, 2: 0.5, 4: 0.2}, matrix_id=7)
+        self.layout = lw.Layout(precs, K)
+        if dealt:
+            self.layout.build_deal()
+        maps, thr = (torch.from_numpy(t).cuda() for t in si.standin_codebooks(precs))
+        self.maps = maps
+        self.packed, self.absmax = lw.lowra_encode(self.layout, self.draw(N, K).float(), thr)
+        self.A, self.B = self.draw(K, r) * 0.05, self.draw(r, N) * 0.05
+
+    def draw(self, *shape):
+        return torch.randn(*shape, device="cuda", generator=self.gen).bfloat16()
+
+    def call(self, backward, act, ws):
+        f = self.lw.lowra_lora_backward_input if backward else self.lw.lowra_lora_forward
+        return f(self.layout, self.packed, self.absmax, self.maps, act, self.A, self.B, 2.0, workspace=ws)
+
+    def right(self, backward, act, out, rows):
+        W = self.lw.lowra_decode(self.layout, self.packed, self.absmax, self.maps).double()
+        a, A, B = act[rows].double(), self.A.double(), self.B.double()
+        ref = a @ W + 2.0 * (a @ B.T) @ A.T if backward else a @ W.T + 2.0 * (a @ A) @ B
+        emax, efro = gemm_errors(out[rows].float().cpu().numpy(), ref.cpu().numpy())
+        return emax <= MAX_TOL and efro <= FRO_TOL
+
+
+@pytest.mark.parametrize("backward", [False, True])
+@pytest.mark.parametrize("M", [70, 300, 1000])
+def test_no_flag_is_read_from_old_projections(backward, M):
+    """A call whose "T ready" flags are withheld has to run out of time, also where an earlier call of more tokens has left
+    T values with the bits of this call's number."""
+    p = _Problem(512, 640, 64)
+    lw = p.lw
+    ws = lw.lowra_workspace_init(torch.empty(lw.lowra_workspace_bytes(p.layout, 2000, p.r), dtype=torch.uint8, device="cuda"))
+    act = p.draw(M, p.N if backward else p.K)
+    lw.lowra_workspace_projection(ws, 2000, p.r).view(torch.int32).fill_(1)     # the first call's number
+    lw.lowra_set_wait_limit(2_000_000)
+    try:
+        lw.lowra_diag_drop_t_flags(1)
+        p.call(backward, act, ws)
+        assert lw.lowra_device_status(ws) == lw.LOWRA_ERR_TIMEOUT
+    finally:
+        lw.lowra_diag_drop_t_flags(0)
+        lw.lowra_set_wait_limit(0)
+    lw.lowra_workspace_init(ws)
+    assert p.right(backward, act, p.call(backward, act, ws), slice(None))
+    assert lw.lowra_device_status(ws) == lw.LOWRA_OK
+
+
+def test_groups_of_few_and_of_many_tokens_keep_apart():
+    """Several adapters, one of them with a few tokens: its projection (at its tokens' rows) is written before the larger
+    group's launch raises its flags."""
+    p = _Problem(512, 640, 64)
+    lw, M = p.lw, 316
+    X = p.draw(M, p.K)
+    two = lambda t: torch.stack([t, t])
+    ws = lw.lowra_workspace_init(torch.empty(lw.lowra_batch_workspace_bytes(p.layout, 4, M, p.r), dtype=torch.uint8, device="cuda"))
+    Y = lw.lowra_lora_forward_adapters(p.layout, p.packed, p.absmax, two(p.maps), X, [0, 300, M], two(p.A), two(p.B), 2.0, workspace=ws)
+    left = lw.lowra_workspace_projection(ws, M, p.r)[300:].clone()
+    assert lw.lowra_device_status(ws) == lw.LOWRA_OK and p.right(False, X, Y, slice(None))
+    own = lw.lowra_workspace_init(torch.empty_like(ws))
+    p.call(False, X[300:].contiguous(), own)
+    assert torch.equal(left.view(torch.int16), lw.lowra_workspace_projection(own, M - 300, p.r).view(torch.int16))
+
+
+@pytest.mark.parametrize("dealt", [False, True])
+def test_more_tokens_than_the_flags_have_room_for(dealt):
+    """From about 104 000 tokens on the "T ready" flags lie behind T and are cleared by every call."""
+    p = _Problem(136, 128, 16, dealt)
+    lw = p.lw
+    counts = [103_900, 300, 120_001, 120_001, 104_100]
+    ws = torch.empty(lw.lowra_workspace_bytes(p.layout, max(counts), p.r), dtype=torch.uint8, device="cuda").fill_(0xA5)
+    if dealt:
+        lw.lowra_workspace_init(ws)
+    acts = [p.draw(max(counts), p.K), p.draw(max(counts), p.N)]
+    for M in counts:
+        rows = torch.from_numpy(np.unique(np.linspace(0, M - 1, 4000).astype(np.int64))).cuda()
+        for backward in (False, True):
+            act = acts[backward][:M]
+            out = p.call(backward, act, ws)
+            assert lw.lowra_device_status(ws) == lw.LOWRA_OK
+            assert p.right(backward, act, out, rows), (M, backward)
