@@ -174,15 +174,16 @@ int out_alignment(const MemberArgs* mem, int count, int R) {
 }
 
 lowra_status run_small(const MemberArgs* mem, uint16_t* const* T_of, int count, int32_t r, float s, void* workspace, cudaStream_t stream);
-// The diagnostic lowra_diag_drop_t_flags is about flags, which the path for few tokens has none of: it leaves that path out.  Otherwise the
-// choice follows from the weight's shape and the member's tokens alone, so that a member's result does not depend on its company.
+// The diagnostic lowra_diag_drop_t_flags is about flags, which the path for few tokens has none of: it leaves that path out.
+bool dropping_flags() { return g_drop_t_flags.load(std::memory_order_relaxed) != 0; }
+// The choice follows from the weight's shape and the member's tokens alone, so that a member's result does not depend on its company.
 // From 33 tokens on that path dequantises every weight twice, which weights with many channels and short contractions do not repay (64 tokens,
 // forward, few-token path against tensor-core tiles, us: 2048 x 2048 13.7 against 26, 4096 x 4096 and 8192 x 8192 alike; but 8192 x 512 16.9
 // against 13.1, 11008 x 1024 32 against 18, 13824 x 512 28.7 against 13.3, 13824 x 2560 44 against 33).  The choice leans to the few-token
 // path where the weight's precisions decide: 5120 x 13824, all of 4 bits, keeps it at 72 against 54.  At 17 to 32 tokens only
 // the shortest contractions of many channels leave it (32 tokens, 13824 x 256 18.0 against 11.0; 13824 x 512 17.8 against 13.1).
 bool takes_small_path(bool backward, int N, int K, int M, int r) {
-    if (backward || M > kSmallTokens || g_drop_t_flags.load(std::memory_order_relaxed) != 0) return false;
+    if (backward || M > kSmallTokens) return false;
     return M <= 16 || small_estimate(N, K, M) < fused_estimate(N, K, M, r);
 }
 
@@ -206,7 +207,7 @@ lowra_status run_members(bool backward, const MemberArgs* mem, int count, int32_
     uint32_t* flags = reinterpret_cast<uint32_t*>(ws + kFlagsOffset);
     uint32_t* t_flags = reinterpret_cast<uint32_t*>(ws + w.off_t_flags);
 
-    if (takes_small_path(backward, N, K, M, r)) {   // (M: the largest member's tokens)
+    if (!dropping_flags() && takes_small_path(backward, N, K, M, r)) {   // (M: the largest member's tokens)
         uint16_t* T_of[kMaxBatch];
         for (int i = 0; i < count; ++i) T_of[i] = reinterpret_cast<uint16_t*>(ws + w.off_T[i]);
         return run_small(mem, T_of, count, r, s, workspace, stream);
@@ -488,7 +489,8 @@ extern "C" lowra_status lowra_lora_forward_adapters(const lowra_layout* layout, 
                           A_dev + (size_t)a * K * (size_t)r, B_dev + (size_t)a * (size_t)r * N, Y_dev + (size_t)m0 * N,
                           group_start_host[a + 1] - m0};
     };
-    auto is_small = [&](int a) { return takes_small_path(false, N, layout->K, group_start_host[a + 1] - group_start_host[a], r); };
+    const bool dropping = dropping_flags();   // (asked once: the launches below use the diagnostic's calls up)
+    auto is_small = [&](int a) { return !dropping && takes_small_path(false, N, layout->K, group_start_host[a + 1] - group_start_host[a], r); };
     MemberArgs mem[kMaxBatch], few[kSmallMembers];
     uint16_t* few_T[kSmallMembers];
     int n = 0, n_few = 0;

@@ -81,6 +81,26 @@ def test_groups_of_few_and_of_many_tokens_keep_apart():
     assert torch.equal(left.view(torch.int16), lw.lowra_workspace_projection(own, M - 300, p.r).view(torch.int16))
 
 
+def test_every_group_is_served_while_flags_are_withheld():
+    """The diagnostic keeps the few-token groups on the tensor-core tiles; the first group's launch uses it up, and the
+    second group must not fall between the two paths."""
+    p = _Problem(512, 640, 64, dealt=False)
+    lw, M = p.lw, 308
+    X = p.draw(M, p.K)
+    two = lambda t: torch.stack([t, t])
+    ws = torch.empty(lw.lowra_workspace_bytes(p.layout, M, p.r), dtype=torch.uint8, device="cuda")
+    Y = torch.full((M, p.N), float("nan"), dtype=torch.bfloat16, device="cuda")
+    lw.lowra_set_wait_limit(2_000_000)
+    try:
+        lw.lowra_diag_drop_t_flags(1)
+        lw.lowra_lora_forward_adapters(p.layout, p.packed, p.absmax, two(p.maps), X, [0, 300, M], two(p.A), two(p.B), 2.0, Y=Y, workspace=ws)
+        assert p.right(False, X, Y, slice(300, M))
+    finally:
+        torch.cuda.synchronize()
+        lw.lowra_diag_drop_t_flags(0)
+        lw.lowra_set_wait_limit(0)
+
+
 @pytest.mark.parametrize("dealt", [False, True])
 def test_more_tokens_than_the_flags_have_room_for(dealt):
     """From about 104 000 tokens on the "T ready" flags lie behind T and are cleared by every call."""
