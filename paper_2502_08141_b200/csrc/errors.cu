@@ -9,7 +9,7 @@
 // or W_hat - then
 //     residual = fl32(x - w_hat)            one fp32 subtraction per element (optional output)
 //     SSE_row  = sum of residual^2          four neighbouring squares are added in fp32, those partial sums in fp64,
-//                                           fixed reduction tree (reproducible)
+//                                           fixed reduction tree (reproducible, the same for a row wherever it stands)
 // so SSE agrees with the exact sum to 2^-21 relative at worst (residual rounded to fp32: 2^-23; a square and two
 // additions in fp32: 3 * 2^-24 more), typically far closer.
 //
@@ -217,9 +217,11 @@ __device__ __forceinline__ void error_rows(const Params& P, int N, int K) {
         __syncthreads();
         for (int s = threadIdx.x; s < (i1 - i0) * NP; s += kErrThreads) {
             double v = 0.0;
+            // from the warp that had the row's first chunk: a row's sum does not depend on its place
+            const int first = (i0 + s / NP) * walk.per_row;
 #pragma unroll
             for (int w = 0; w < kRowWarps; ++w) {
-                double& slot = part[((s / NP) * kRowWarps + w) * NP + s % NP];
+                double& slot = part[((s / NP) * kRowWarps + (first + w) % kRowWarps) * NP + s % NP];
                 v += slot;
                 slot = 0.0;
             }

@@ -37,3 +37,24 @@ def test_split_of_the_rows(N, K):
     rows = torch.arange(N, device="cuda")
     maps3[plane, rows], thr3[plane, rows] = maps, thr
     assert torch.equal(lw.lowra_channel_errors(W, maps3, thr3)[rows, plane], sse)
+
+
+@pytest.mark.parametrize("N,K", [(3000, 640), (2000, 2176), (1500, 4224), (1000, 9216), (1000, 11008)])
+def test_a_rows_error_does_not_depend_on_its_place(N, K):
+    """One row over and over, its block maxima spread over six decades, so that fp64 sums show the order of the additions."""
+    import paper_2502_08141_b200 as lw
+
+    gen = torch.Generator(device="cuda").manual_seed(K)
+    scale = 10.0 ** (-6.0 * torch.rand(K // 64, device="cuda", generator=gen)).repeat_interleave(64)
+    W = (torch.randn(K, device="cuda", generator=gen) * scale).expand(N, K).contiguous()
+    precs = si.precisions(N, {1: 0.5, 2: 0.35, 4: 0.15}, matrix_id=K % 61)
+    plane = torch.from_numpy(precs).cuda().long() // 2
+    maps3, thr3 = (torch.empty(3, N, 16, device="cuda") for _ in range(2))
+    for c in range(3):
+        m, t = si.standin_codebooks(precs[:1] * 0 + (1 << c))
+        maps3[c], thr3[c] = torch.from_numpy(m[0]).cuda(), torch.from_numpy(t[0]).cuda()
+    sse3 = lw.lowra_channel_errors(W, maps3, thr3)
+    assert torch.equal(sse3, sse3[:1].expand(N, 3))
+    rows = torch.arange(N, device="cuda")
+    sse, _ = lw.lowra_quant_error(lw.Layout(precs, K), W, maps3[plane, rows].contiguous(), thr3[plane, rows].contiguous())
+    assert torch.equal(sse, sse3[0, plane])
