@@ -30,6 +30,7 @@ struct LearnParams {
     int row0;             // this launch's rows: stored rows row0 .. row0 + grid - 1
     int turn;             // see enter()
     int bins;             // sorted rows: cells
+    unsigned near_zero;   // see too_coarse
     double init_y[3][16];  // initial levels per class (1, 2, 4 bits)
     double init_t[3][16];  // initial thresholds per class
 };
@@ -71,9 +72,9 @@ __device__ __forceinline__ void warp_sums(long long (&v)[NV], int lane) {
 // of the additions: results are reproducible, and the same whichever kernel takes the row.  Let the row's largest weight be below
 // 2^e.  fp64 numbers from 64 * 2^e to 128 * 2^e are multiples of u = 2^(e - 46), and adding to g = 96 * 2^e takes w (to nearest) and w * n
 // (down) to that grid: s + w * n, one fused multiply-add rounding down, is s plus w * n taken down, whatever s is, so that a
-// run of sixteen elements is a chain of these.  The sums are whole numbers of u, added up in 64-bit integers.  Where a bucket weighs a quarter of the largest weight or more its level is right to its number of
-// elements * 2^-43 (usually: to 2^-44); otherwise - few or light elements, or none - it is added up again on a grid of its own.
-constexpr long long kLight = 1ll << 44;   // u
+// run of sixteen elements is a chain of these.  The sums are whole numbers of u, added up in 64-bit integers.  An element of a bucket costs its
+// sum less than u, K of them less than 2^-24 of a sum of 2^24 K u, a rounding to fp32.  A bucket whose sum is nearer to zero (light elements only,
+// or a mean next to zero) is added up again with what the grid leaves over.
 __device__ __forceinline__ double grid_of(float most) {   // g
     return 96.0 * (most > 0.0f && most < INFINITY ? ldexp(1.0, ilogbf(most) + 1) : 1.0);
 }
@@ -82,9 +83,10 @@ __device__ __forceinline__ long long grid_product(double n, double w, double g) 
 __device__ __forceinline__ long long grid_weight(double w, double g) { return (long long)(grid_bits(w + g) - grid_bits(g)); }
 // A block's weight in multiples of 2^e (for the grid 96), where that is kept instead of the absmax; what is positive stays positive.
 constexpr double kGrid = 96.0;
-__device__ __forceinline__ float scaled_weight(float m, float row_most) {
-    return m > 0.0f && row_most < INFINITY ? fmaxf((float)ldexp((double)m, -ilogbf(row_most) - 1), FLT_MIN) : 0.0f;
+__device__ __forceinline__ float weight_scale(float row_most) {
+    return row_most > 0.0f && row_most < INFINITY ? (float)ldexp(1.0, -ilogbf(row_most) - 1) : 0.0f;
 }
+__device__ __forceinline__ float scaled_weight(float m, float scale) { return m > 0.0f && scale > 0.0f ? fmaxf(__fmul_rn(m, scale), FLT_MIN) : 0.0f; }
 // the larger one; NaN if one is NaN (a row that holds a NaN, an infinity or a block whose reciprocal overflows has no mean: its
 // levels come out as NaN)
 __device__ __forceinline__ float max_nan(float a, float b) {
@@ -93,31 +95,55 @@ __device__ __forceinline__ float max_nan(float a, float b) {
     return m;
 }
 
-// The mean of a light bucket's elements [t_lo, t_hi) on a grid of its own (by a whole warp), or `keep` if they weigh nothing.
-// element(p): value and weight number p of p0 .. p1 - 1, which hold the bucket.
+// Whether a bucket's sum of w n is not enough: below 2^24 K u (near_zero: the upper half of that as an fp64 number, K rounded down to a power of two).  Exactly zero is
+// the sum of zeros.  But an empty bucket and one of weights below u look alike: rows that have such weights (zero_too = 1) are looked through for
+// them.  (Rows of a few different values have many empty buckets, and took up to 40 times as long when all were looked through for them.)
+__device__ __forceinline__ bool too_coarse(double sn, unsigned near_zero, unsigned zero_too) {
+    return ((unsigned)__double2hiint(sn) & 0x7fffffffu) - 1u + zero_too < near_zero;
+}
+constexpr float kVanishing = 0x1p-44f;   // scaled weights from here on are above u
+// A bucket added up again, by all threads that call this (element(p): value and scaled weight number p of p0, p0 + step, ... below p1): on the grid
+// kGrid, or, where its weights vanish there, on one of its own.  wn and w in multiples of u, the others in multiples of 2^-46 u.
+struct Fine {
+    long long wn, wn_lo, w, w_lo;
+};
+template <int UNROLL, typename F>
+__device__ __forceinline__ Fine fine_sums(F element, int p0, int p1, int step, float t_lo, float t_hi, double g) {
+    const double g2 = g * 0x1p-46;
+    Fine f = {0, 0, 0, 0};
+#pragma unroll UNROLL
+    for (int p = p0; p < p1; p += step) {
+        const float2 e = element(p);
+        const bool in = t_lo <= e.x && e.x < t_hi;
+        const double n = in ? (double)e.x : 0.0, w = in ? (double)e.y : 0.0;
+        const double a = __fma_rd(n, w, g), b = __dadd_rn(w, g);           // what they leave over is exact
+        f.wn += (long long)(grid_bits(a) - grid_bits(g));
+        f.w += (long long)(grid_bits(b) - grid_bits(g));
+        f.wn_lo += (long long)(grid_bits(__dadd_rd(__fma_rn(n, w, -__dsub_rn(a, g)), g2)) - grid_bits(g2));
+        f.w_lo += (long long)(grid_bits(__dadd_rn(__dsub_rn(w, __dsub_rn(b, g)), g2)) - grid_bits(g2));
+    }
+#pragma unroll
+    for (int d = 16; d >= 1; d >>= 1) {
+        f.wn += __shfl_xor_sync(0xffffffffu, f.wn, d);
+        f.wn_lo += __shfl_xor_sync(0xffffffffu, f.wn_lo, d);
+        f.w += __shfl_xor_sync(0xffffffffu, f.w, d);
+        f.w_lo += __shfl_xor_sync(0xffffffffu, f.w_lo, d);
+    }
+    return f;
+}
 template <typename F>
-__device__ __forceinline__ double light_mean(F element, int p0, int p1, float t_lo, float t_hi, double keep) {
-    const int lane = threadIdx.x & 31;
+__device__ __forceinline__ float largest_weight(F element, int p0, int p1, int step, float t_lo, float t_hi) {
     float most = 0.0f;
-    for (int p = p0 + lane; p < p1; p += 32) {
+    for (int p = p0; p < p1; p += step) {
         const float2 e = element(p);
         if (t_lo <= e.x && e.x < t_hi) most = fmaxf(most, e.y);
     }
 #pragma unroll
     for (int d = 16; d >= 1; d >>= 1) most = fmaxf(most, __shfl_xor_sync(0xffffffffu, most, d));
-    if (!(most > 0.0f)) return keep;
-    const double g = grid_of(most);
-    long long wn = 0, w = 0;
-    for (int p = p0 + lane; p < p1; p += 32) {
-        const float2 e = element(p);
-        if (t_lo <= e.x && e.x < t_hi) {
-            wn += grid_product((double)e.x, (double)e.y, g);
-            w += grid_weight((double)e.y, g);
-        }
-    }
-#pragma unroll
-    for (int d = 16; d >= 1; d >>= 1) { wn += __shfl_xor_sync(0xffffffffu, wn, d); w += __shfl_xor_sync(0xffffffffu, w, d); }
-    return (double)wn / (double)w;
+    return most;
+}
+__device__ __forceinline__ double fine_mean(const Fine& f) {
+    return ((double)f.wn + 0x1p-46 * (double)f.wn_lo) / ((double)f.w + 0x1p-46 * (double)f.w_lo);
 }
 
 // number of thresholds <= x among t[0 .. L-2] (sorted): branch-free binary search, L = 2, 4 or 16.
@@ -145,9 +171,10 @@ __device__ __forceinline__ int quad_slot(int q) { return q ^ ((q >> 3) & 3); }
 
 // The row: asynchronous coalesced 128-bit copies, all of them in flight together; then every thread normalises sixteen elements at a
 // time where they lie (as in lowra_encode: reciprocal rounded to nearest, one multiplication): the four lanes that hold a
-// 64-element block between them find its absmax in two shuffles.  Returns the row's largest absmax.  Ends with a barrier.
+// 64-element block between them find its absmax in two shuffles.  Returns the row's largest absmax and its smallest but zero.  Ends with a
+// barrier.
 template <int THREADS>
-__device__ float load_row(const LearnParams& P, int r, float* xs, float* ws, float* most_of) {
+__device__ float2 load_row(const LearnParams& P, int r, float* xs, float* ws, float* most_of) {
     const int K = P.K;
     const int tid = threadIdx.x;
     const float* wrow = P.W + (size_t)r * K;
@@ -156,7 +183,7 @@ __device__ float load_row(const LearnParams& P, int r, float* xs, float* ws, flo
     asm volatile("cp.async.commit_group;" ::: "memory");
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
-    float most = 0.0f;
+    float most = 0.0f, least = INFINITY;
     for (int run = tid; run < (K / 16 + 31) / 32 * 32; run += THREADS) {   // (a warp stays together)
         float4 v[4];
         float m = 0.0f;
@@ -169,6 +196,7 @@ __device__ float load_row(const LearnParams& P, int r, float* xs, float* ws, flo
         m = max_nan(m, __shfl_xor_sync(0xffffffffu, m, 2));
         const float inv = (m == 0.0f) ? 0.0f : __frcp_rn(m);
         most = max_nan(max_nan(most, m), __fmul_rn(inv, 0.0f));
+        if (m > 0.0f) least = fminf(least, m);
         if (run < K / 16) {
 #pragma unroll
             for (int q = 0; q < 4; ++q)
@@ -178,12 +206,15 @@ __device__ float load_row(const LearnParams& P, int r, float* xs, float* ws, flo
         }
     }
 #pragma unroll
-    for (int d = 4; d < 32; d <<= 1) most = max_nan(most, __shfl_xor_sync(0xffffffffu, most, d));
-    if ((tid & 31) == 0) most_of[tid >> 5] = most;
+    for (int d = 4; d < 32; d <<= 1) {
+        most = max_nan(most, __shfl_xor_sync(0xffffffffu, most, d));
+        least = fminf(least, __shfl_xor_sync(0xffffffffu, least, d));
+    }
+    if ((tid & 31) == 0) { most_of[2 * (tid >> 5)] = most; most_of[2 * (tid >> 5) + 1] = least; }
     __syncthreads();
 #pragma unroll
-    for (int w = 0; w < THREADS / 32; ++w) most = max_nan(most, most_of[w]);
-    return most;
+    for (int w = 0; w < THREADS / 32; ++w) { most = max_nan(most, most_of[2 * w]); least = fminf(least, most_of[2 * w + 1]); }
+    return make_float2(most, least);
 }
 
 // learn_kernel.  One CTA per row: the row is read from HBM once, normalised on its way into shared memory; the T passes run out of
@@ -192,9 +223,35 @@ __device__ float load_row(const LearnParams& P, int r, float* xs, float* ws, flo
 // per round; every warp forms the new levels and thresholds itself; a row whose thresholds have settled (as fp32 numbers) skips its
 // remaining rounds.
 //
-__device__ __noinline__ double light_mean_row(const float* xs, const float* ws, float row_most, int K, float t_lo, float t_hi, double keep) {
-    return light_mean([&](int p) { return make_float2(xs[4 * quad_slot(p >> 2) + (p & 3)], scaled_weight(ws[p / kBlock], row_most)); }, 0, K,
-                      t_lo, t_hi, keep);
+// The mean of the bucket [t_lo, t_hi) by the whole CTA; y if it weighs nothing (vanished: nothing on the row's grid).  scratch: five words per warp
+// that nobody reads, free again at the end.
+template <int THREADS>
+__device__ __noinline__ double fine_mean_row(const float* xs, const float* ws, float row_most, int K, float t_lo, float t_hi, bool vanished,
+                                             double y, long long* scratch) {
+    constexpr int kWarps = THREADS / 32;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const float scale = weight_scale(row_most);
+    auto element = [&](int p) { return make_float2(xs[4 * quad_slot(p >> 2) + (p & 3)], scaled_weight(ws[p / kBlock], scale)); };
+    double g = kGrid;
+    if (vanished) {
+        float* most_of = reinterpret_cast<float*>(scratch + 4 * kWarps);
+        float most = largest_weight(element, tid, K, THREADS, t_lo, t_hi);
+        if (lane == 0) most_of[warp] = most;
+        __syncthreads();
+        for (int w = 0; w < kWarps; ++w) most = fmaxf(most, most_of[w]);
+        g = grid_of(most);
+        if (!(most > 0.0f)) {
+            __syncthreads();
+            return y;
+        }
+    }
+    Fine f = fine_sums<2>(element, tid, K, THREADS, t_lo, t_hi, g);
+    if (lane == 0) { scratch[4 * warp] = f.wn; scratch[4 * warp + 1] = f.wn_lo; scratch[4 * warp + 2] = f.w; scratch[4 * warp + 3] = f.w_lo; }
+    __syncthreads();
+    f = Fine{0, 0, 0, 0};
+    for (int w = 0; w < kWarps; ++w) { f.wn += scratch[4 * w]; f.wn_lo += scratch[4 * w + 1]; f.w += scratch[4 * w + 2]; f.w_lo += scratch[4 * w + 3]; }
+    __syncthreads();
+    return fine_mean(f);
 }
 
 // One pass at 1 or 2 bits: this thread's sums over the elements at or above threshold j - 1 (j >= 1) and, if ALL, over all (j = 0).
@@ -241,7 +298,7 @@ __device__ __forceinline__ void few_buckets(const float* xs, const float* ws, in
 // then EVERY warp forms the new levels and thresholds for itself - lane j holds level j and threshold j in registers, the
 // same numbers in every warp since they come from the same sums - so nobody waits for a first warp to publish them.
 template <int B, int THREADS>
-__device__ void learn_row(const LearnParams& P, const float* xs, const float* ws, float row_most, long long* acc, long long* red2,
+__device__ void learn_row(const LearnParams& P, const float* xs, const float* ws, float row_most, unsigned zero_too, long long* acc, long long* red2,
                           float* tfw_all, int iterations, float* maps_out, float* thr_out) {
     constexpr int kLearnThreads = THREADS, kLearnWarps = THREADS / 32;
     constexpr int Lv = 1 << B;      // levels
@@ -329,18 +386,21 @@ __device__ void learn_row(const LearnParams& P, const float* xs, const float* ws
         }
         __syncthreads();
         // ---- new levels, then midpoints with a shuffle in between: every warp
-        bool light = false;
+        bool coarse = false, vanished = false;
         if (lane < Lv) {
             long long sn = 0, sd = 0;
 #pragma unroll
             for (int w2 = 0; w2 < kLearnWarps; ++w2) { sn += red[(2 * lane) * kLearnWarps + w2]; sd += red[(2 * lane + 1) * kLearnWarps + w2]; }
-            light = sd < kLight;
-            if (!light) ylane = (double)sn / (double)sd;
+            vanished = sd <= 0;
+            coarse = too_coarse((double)sn, P.near_zero, zero_too);
+            if (!vanished) ylane = (double)sn / (double)sd;
         }
-        for (unsigned left = __ballot_sync(0xffffffffu, light); left != 0u; left &= left - 1u) {
+        for (unsigned left = __ballot_sync(0xffffffffu, coarse); left != 0u; left &= left - 1u) {     // (the same in every warp)
             const int k = __ffs(left) - 1;
             const float t_lo = __shfl_sync(0xffffffffu, tlane, max(k - 1, 0)), t_hi = __shfl_sync(0xffffffffu, tlane, k);
-            const double mean = light_mean_row(xs, ws, row_most, K, k > 0 ? t_lo : -INFINITY, k < Lv - 1 ? t_hi : INFINITY, __shfl_sync(0xffffffffu, ylane, k));
+            const double mean = fine_mean_row<THREADS>(xs, ws, row_most, K, k > 0 ? t_lo : -INFINITY, k < Lv - 1 ? t_hi : INFINITY,
+                                                       __shfl_sync(0xffffffffu, (int)vanished, k) != 0, __shfl_sync(0xffffffffu, ylane, k),
+                                                       red2 + ((it & 1) ^ 1) * (2 * 16 * kLearnWarps));
             if (lane == k) ylane = mean;
         }
         const double yn = __shfl_down_sync(0xffffffffu, ylane, 1);
@@ -396,20 +456,23 @@ __global__ void __launch_bounds__(THREADS) learn_kernel(const __grid_constant__ 
     // short 1-bit rows fill the gaps at the end
     const int i = P.row0 + (int)(gridDim.x - 1 - blockIdx.x);
     const int r = ALL3 ? i : P.L.perm[i];
-    const float most = load_row<THREADS>(P, r, xs, ws, tfw);
+    const float2 scale = load_row<THREADS>(P, r, xs, ws, tfw);
+    const float most = scale.x;
+    // (scaled_weight of the smallest against kVanishing, without the scaling: the largest lies between this power of two and the next)
+    const unsigned zero_too = scale.y < __uint_as_float(__float_as_uint(most) & 0x7f800000u) * (2.0f * kVanishing) ? 1u : 0u;
     float* m = P.maps + (size_t)r * kTableStride;
     float* h = P.thresholds + (size_t)r * kTableStride;
     if (ALL3) {
         // the row under every precision, from the one copy in shared memory
         const size_t plane = (size_t)P.N * kTableStride;
-        learn_row<1, THREADS>(P, xs, ws, most, acc, red2, tfw, P.iterations, m, h);
-        learn_row<2, THREADS>(P, xs, ws, most, acc, red2, tfw, P.iterations, m + plane, h + plane);
-        learn_row<4, THREADS>(P, xs, ws, most, acc, red2, tfw, FOUR ? P.iterations : 0, m + 2 * plane, h + 2 * plane);
+        learn_row<1, THREADS>(P, xs, ws, most, zero_too, acc, red2, tfw, P.iterations, m, h);
+        learn_row<2, THREADS>(P, xs, ws, most, zero_too, acc, red2, tfw, P.iterations, m + plane, h + plane);
+        learn_row<4, THREADS>(P, xs, ws, most, zero_too, acc, red2, tfw, FOUR ? P.iterations : 0, m + 2 * plane, h + 2 * plane);
     } else {
         const int b = P.L.precs[r];
-        if (b == 1) learn_row<1, THREADS>(P, xs, ws, most, acc, red2, tfw, P.iterations, m, h);
-        else if (b == 2) learn_row<2, THREADS>(P, xs, ws, most, acc, red2, tfw, P.iterations, m, h);
-        else learn_row<4, THREADS>(P, xs, ws, most, acc, red2, tfw, FOUR ? P.iterations : 0, m, h);
+        if (b == 1) learn_row<1, THREADS>(P, xs, ws, most, zero_too, acc, red2, tfw, P.iterations, m, h);
+        else if (b == 2) learn_row<2, THREADS>(P, xs, ws, most, zero_too, acc, red2, tfw, P.iterations, m, h);
+        else learn_row<4, THREADS>(P, xs, ws, most, zero_too, acc, red2, tfw, FOUR ? P.iterations : 0, m, h);
     }
     leave(P.turn);
 }
@@ -453,8 +516,17 @@ __device__ __forceinline__ Sums shfl_xor_sums(const Sums& s, int d) {
     return Sums{__shfl_xor_sync(0xffffffffu, s.wn, d), __shfl_xor_sync(0xffffffffu, s.w, d)};
 }
 
-__device__ __noinline__ double light_mean_sorted(const float2* sorted, int p0, int p1, float t_lo, float t_hi, double keep) {
-    return light_mean([&](int p) { return sorted[sorted_slot(p)]; }, p0, p1, t_lo, t_hi, keep);
+// The same by a warp; the bucket lies somewhere in places p0 .. p1 - 1.
+__device__ __noinline__ double fine_mean_sorted(const float2* sorted, int p0, int p1, float t_lo, float t_hi, bool vanished, double y) {
+    const int lane = threadIdx.x & 31;
+    auto element = [&](int p) { return sorted[sorted_slot(p)]; };
+    double g = kGrid;
+    if (vanished) {
+        const float most = largest_weight(element, p0 + lane, p1, 32, t_lo, t_hi);
+        if (!(most > 0.0f)) return y;
+        g = grid_of(most);
+    }
+    return fine_mean(fine_sums<1>(element, p0 + lane, p1, 32, t_lo, t_hi, g));
 }
 
 // T rounds at B bits by one warp; tables to maps_out / thr_out ([16] each).  first[b]: places before cell b; run[i]: sums over
@@ -470,6 +542,7 @@ __device__ void learn_sorted(const LearnParams& P, const float2* sorted, const u
     double y = j < Lv ? P.init_y[c][j] : 0.0;
     float t = !top ? __double2float_ru(P.init_t[c][j]) : INFINITY;   // the least fp32 number >= the threshold
     for (int it = 0; it < P.iterations; ++it) {
+        const unsigned zero_too = *reinterpret_cast<const volatile uint32_t*>(first - 1);     // (not worth a register)
         const int b = cell_of_threshold(t, bins);
         const int p1 = top ? K : (int)first[b + 1], p0 = top ? K : (int)first[b] & ~15;
         const Sums base = run[p0 >> 4];
@@ -491,16 +564,17 @@ __device__ void learn_sorted(const LearnParams& P, const float2* sorted, const u
         // the bucket: what lies below its upper threshold less what lies below its lower one
         Sums low = {__shfl_up_sync(0xffffffffu, s.wn, G), __shfl_up_sync(0xffffffffu, s.w, G)};
         if (j == 0) low.wn = low.w = 0;
+        const double sn = (double)(s.wn - low.wn);
         const long long sw = s.w - low.w;
-        const bool light = j < Lv && sw < kLight;
-        if (j < Lv && !light) y = (double)(s.wn - low.wn) / (double)sw;
-        for (unsigned left = __ballot_sync(0xffffffffu, light); left != 0u;) {   // light or empty buckets, one after the other
+        if (j < Lv && sw > 0) y = sn / (double)sw;
+        for (unsigned left = __ballot_sync(0xffffffffu, j < Lv && too_coarse(sn, P.near_zero, zero_too)); left != 0u;) {
             const int k = (__ffs(left) - 1) / G;
             left &= ~(((1u << G) - 1u) << (k * G));
             const float t_lo = k > 0 ? __shfl_sync(0xffffffffu, t, max(k - 1, 0) * G) : -INFINITY;
             const float t_hi = __shfl_sync(0xffffffffu, t, k * G);
             const int q0 = k > 0 ? (int)first[cell_of_threshold(t_lo, bins)] : 0, q1 = k < Lv - 1 ? (int)first[cell_of_threshold(t_hi, bins) + 1] : K;
-            const double mean = light_mean_sorted(sorted, q0, q1, t_lo, t_hi, __shfl_sync(0xffffffffu, y, k * G));
+            const double mean = fine_mean_sorted(sorted, q0, q1, t_lo, t_hi, __shfl_sync(0xffffffffu, (int)(sw <= 0), k * G) != 0,
+                                                 __shfl_sync(0xffffffffu, y, k * G));
             if (j == k) y = mean;
         }
         const double yn = __shfl_down_sync(0xffffffffu, y, G);
@@ -555,7 +629,7 @@ template <bool ALL3, int THREADS, int PER, int CTAS>
 __global__ void __launch_bounds__(THREADS, CTAS) sorted_learn_kernel(const __grid_constant__ LearnParams P) {
     extern __shared__ __align__(16) unsigned char sorted_smem[];
     const int K = P.K, bins = P.bins, tid = threadIdx.x, nt = blockDim.x, warp = tid >> 5, n_warps = nt >> 5;
-    // [K float2 values and weights in order; before that, the row][K / 16 + 1 Sums][32 x 2 long long][32 floats][0, 0, 0, 0][cells]
+    // [K float2 values and weights in order; before that, the row][K / 16 + 1 Sums][32 x 2 long long][32 floats][0, 0, zero_too, 0][cells]
     float2* sorted = reinterpret_cast<float2*>(sorted_smem);
     Sums* run = reinterpret_cast<Sums*>(sorted + K);
     long long(*scratch)[2] = reinterpret_cast<long long(*)[2]>(run + K / 16 + 1);
@@ -619,7 +693,8 @@ __global__ void __launch_bounds__(THREADS, CTAS) sorted_learn_kernel(const __gri
     }
     float row_most = 0.0f;
     for (int w = 0; w < n_warps; ++w) row_most = max_nan(row_most, most_of[w]);
-    const float weight = scaled_weight(m, row_most);
+    const float weight = scaled_weight(m, weight_scale(row_most));
+    if (weight > 0.0f && weight < kVanishing) cells[-2] = 1u;
     __syncthreads();
     // ---- every value and its weight to their place; afterwards a cell's entry is the place where it ends
     if (in) {
@@ -745,6 +820,9 @@ lowra_status launch_learn(LearnParams& P, const double* init_levels_host, const 
     if (((size_t)P.K + (size_t)P.K / kBlock) * sizeof(float) > 160 * 1024) return LOWRA_ERR_SHAPE;   // K <= 40960: the row has to fit
     lowra_status st = check_device();
     if (st != LOWRA_OK) return st;
+    int log_k = 0;
+    while ((2 << log_k) <= P.K) ++log_k;
+    P.near_zero = (unsigned)(1023 + 24 + log_k) << 20;
     for (int c = 0; c < 3; ++c)
         for (int j = 0; j < 16; ++j) {
             P.init_y[c][j] = init_levels_host[c * 16 + j];
