@@ -529,11 +529,41 @@ __device__ __noinline__ double fine_mean_sorted(const float2* sorted, int p0, in
     return fine_mean(fine_sums<1>(element, p0 + lane, p1, 32, t_lo, t_hi, g));
 }
 
+constexpr int kMany = 32 * 4;
+// Sums of places p0 .. p1 - 1 whose values are below t, by a warp.
+__device__ __noinline__ Sums sums_below(const float2* sorted, int p0, int p1, float t) {
+    Sums s = {0, 0};
+#pragma unroll 4
+    for (int p = p0 + (int)(threadIdx.x & 31); p < p1; p += 32) {
+        const float2 e = sorted[sorted_slot(p)];
+        const double n = e.x < t ? (double)e.x : 0.0, w = e.x < t ? (double)e.y : 0.0;
+        s.wn += grid_product(n, w, kGrid);
+        s.w += grid_weight(w, kGrid);
+    }
+#pragma unroll
+    for (int d = 16; d >= 1; d >>= 1) {
+        const Sums o = shfl_xor_sums(s, d);
+        s.wn += o.wn; s.w += o.w;
+    }
+    return s;
+}
+
+// One more value in cell c for every lane that is in; the lanes that share a cell add together, for one by one their additions wait for one another
+// (not so where nobody asks for the place: the hardware adds up ones).  Returns the lane's place.
+__device__ __forceinline__ int add_to_cell(uint32_t* cells, int c, bool in) {
+    const int lane = threadIdx.x & 31;
+    const unsigned peers = __match_any_sync(0xffffffffu, in ? c : -1 - lane);
+    const int leader = __ffs(peers) - 1;
+    uint32_t before = 0u;
+    if (in && lane == leader) before = atomicAdd(&cells[c], (uint32_t)__popc(peers));
+    return (int)__shfl_sync(0xffffffffu, before, leader) + __popc(peers & ((1u << lane) - 1u));
+}
+
 // T rounds at B bits by one warp; tables to maps_out / thr_out ([16] each).  first[b]: places before cell b; run[i]: sums over
 // the first 16 i places.  The G lanes of group j look after level j and the threshold above it (the last group: everything), all with
 // the same values; what bounds a round is the length of this chain, so it has few shuffles.
-template <int B>
-__device__ void learn_sorted(const LearnParams& P, const float2* sorted, const uint32_t* first, const Sums* run, int bins, float row_most,
+template <int B, bool CROWDED>
+__device__ __forceinline__ void learn_sorted(const LearnParams& P, const float2* sorted, const uint32_t* first, const Sums* run, int bins, float row_most,
                              float* maps_out, float* thr_out) {
     constexpr int Lv = 1 << B, c = B >> 1;
     constexpr int G = B == 4 ? 2 : 8;
@@ -547,7 +577,8 @@ __device__ void learn_sorted(const LearnParams& P, const float2* sorted, const u
         const int p1 = top ? K : (int)first[b + 1], p0 = top ? K : (int)first[b] & ~15;
         const Sums base = run[p0 >> 4];
         Sums s = {0, 0};
-        for (int p = p0 + lane % G; p < p1; p += G) {
+        // (crowded rows: a cell of many places is the whole warp's work, below)
+        for (int p = p0 + lane % G, end = CROWDED && p1 - p0 > kMany ? p0 : p1; p < end; p += G) {
             const float2 e = sorted[sorted_slot(p)];
             if (e.x < t) {
                 s.wn += grid_product((double)e.x, (double)e.y, kGrid);
@@ -559,6 +590,14 @@ __device__ void learn_sorted(const LearnParams& P, const float2* sorted, const u
         for (int d = G / 2; d >= 1; d >>= 1) {
             const Sums o = shfl_xor_sums(s, d);
             s.wn += o.wn; s.w += o.w;
+        }
+        if (CROWDED) {
+            for (unsigned left = __ballot_sync(0xffffffffu, p1 - p0 > kMany); left != 0u;) {
+                const int k = (__ffs(left) - 1) / G;
+                left &= ~(((1u << G) - 1u) << (k * G));
+                const Sums all = sums_below(sorted, __shfl_sync(0xffffffffu, p0, k * G), __shfl_sync(0xffffffffu, p1, k * G), __shfl_sync(0xffffffffu, t, k * G));
+                if (j == k) s = all;
+            }
         }
         s.wn += base.wn; s.w += base.w;
         // the bucket: what lies below its upper threshold less what lies below its lower one
@@ -595,6 +634,31 @@ __device__ void learn_sorted(const LearnParams& P, const float2* sorted, const u
     }
 }
 
+// All rounds of row r.  Crowded rows by a function of their own, which leaves the others' registers alone.
+template <bool ALL3, bool CROWDED>
+__device__ __forceinline__ void learn_rounds(const LearnParams& P, const float2* sorted, const uint32_t* first, const Sums* run, float row_most, int r) {
+    const int warp = threadIdx.x >> 5, bins = P.bins;
+    float* y = P.maps + (size_t)r * kTableStride;
+    float* h = P.thresholds + (size_t)r * kTableStride;
+    if (ALL3) {   // a warp per precision
+        const size_t plane = (size_t)P.N * kTableStride;
+        for (int c = warp; c < 3; c += blockDim.x >> 5) {
+            if (c == 0) learn_sorted<4, CROWDED>(P, sorted, first, run, bins, row_most, y + 2 * plane, h + 2 * plane);
+            else if (c == 1) learn_sorted<2, CROWDED>(P, sorted, first, run, bins, row_most, y + plane, h + plane);
+            else learn_sorted<1, CROWDED>(P, sorted, first, run, bins, row_most, y, h);
+        }
+    } else if (warp == 0) {
+        const int b = P.L.precs[r];
+        if (b == 1) learn_sorted<1, CROWDED>(P, sorted, first, run, bins, row_most, y, h);
+        else if (b == 2) learn_sorted<2, CROWDED>(P, sorted, first, run, bins, row_most, y, h);
+        else learn_sorted<4, CROWDED>(P, sorted, first, run, bins, row_most, y, h);
+    }
+}
+template <bool ALL3>
+__device__ __noinline__ void learn_rounds_crowded(const LearnParams& P, const float2* sorted, const uint32_t* first, const Sums* run, float row_most, int r) {
+    learn_rounds<ALL3, true>(P, sorted, first, run, row_most, r);
+}
+
 // Exclusive sums of v[0 .. NV-1] over the threads of the CTA (scratch: NV entries per warp).  Ends with a barrier.
 template <int NV, typename T>
 __device__ __forceinline__ void block_exclusive(T (&v)[NV], T (*scratch)[NV]) {
@@ -629,7 +693,7 @@ template <bool ALL3, int THREADS, int PER, int CTAS>
 __global__ void __launch_bounds__(THREADS, CTAS) sorted_learn_kernel(const __grid_constant__ LearnParams P) {
     extern __shared__ __align__(16) unsigned char sorted_smem[];
     const int K = P.K, bins = P.bins, tid = threadIdx.x, nt = blockDim.x, warp = tid >> 5, n_warps = nt >> 5;
-    // [K float2 values and weights in order; before that, the row][K / 16 + 1 Sums][32 x 2 long long][32 floats][0, 0, zero_too, 0][cells]
+    // [K float2 values and weights in order; before that, the row][K / 16 + 1 Sums][32 x 2 long long][32 floats][0, crowded, zero_too, 0][cells]
     float2* sorted = reinterpret_cast<float2*>(sorted_smem);
     Sums* run = reinterpret_cast<Sums*>(sorted + K);
     long long(*scratch)[2] = reinterpret_cast<long long(*)[2]>(run + K / 16 + 1);
@@ -670,6 +734,9 @@ __global__ void __launch_bounds__(THREADS, CTAS) sorted_learn_kernel(const __gri
     // ---- count the cells
 #pragma unroll
     for (int e = 0; e < PER; ++e) x[e] = __fmul_rn(x[e], inv);
+    // Crowded (for a warp): neighbours are equal in one lane of eight - a row of a few different values.
+    const bool crowded = __popc(__ballot_sync(0xffffffffu, in && x[0] == x[1])) >= 4;
+    if (crowded) cells[-3] = 1u;
     if (in) {
 #pragma unroll
         for (int e = 0; e < PER; ++e) atomicAdd(&cells[cell_of(x[e], bins)], 1u);
@@ -697,7 +764,13 @@ __global__ void __launch_bounds__(THREADS, CTAS) sorted_learn_kernel(const __gri
     if (weight > 0.0f && weight < kVanishing) cells[-2] = 1u;
     __syncthreads();
     // ---- every value and its weight to their place; afterwards a cell's entry is the place where it ends
-    if (in) {
+    if (crowded) {
+#pragma unroll
+        for (int e = 0; e < PER; ++e) {
+            const int place = add_to_cell(cells, cell_of(x[e], bins), in);
+            if (in) sorted[sorted_slot(place)] = make_float2(x[e], weight);
+        }
+    } else if (in) {
 #pragma unroll
         for (int e = 0; e < PER; ++e)
             sorted[sorted_slot((int)atomicAdd(&cells[cell_of(x[e], bins)], 1u))] = make_float2(x[e], weight);
@@ -732,21 +805,8 @@ __global__ void __launch_bounds__(THREADS, CTAS) sorted_learn_kernel(const __gri
     __syncthreads();
     // ---- rounds
     const uint32_t* first = cells - 1;   // first[b]: the places before cell b
-    float* y = P.maps + (size_t)r * kTableStride;
-    float* h = P.thresholds + (size_t)r * kTableStride;
-    if (ALL3) {   // a warp per precision
-        const size_t plane = (size_t)P.N * kTableStride;
-        for (int c = warp; c < 3; c += n_warps) {
-            if (c == 0) learn_sorted<4>(P, sorted, first, run, bins, row_most, y + 2 * plane, h + 2 * plane);
-            else if (c == 1) learn_sorted<2>(P, sorted, first, run, bins, row_most, y + plane, h + plane);
-            else learn_sorted<1>(P, sorted, first, run, bins, row_most, y, h);
-        }
-    } else if (warp == 0) {
-        const int b = P.L.precs[r];
-        if (b == 1) learn_sorted<1>(P, sorted, first, run, bins, row_most, y, h);
-        else if (b == 2) learn_sorted<2>(P, sorted, first, run, bins, row_most, y, h);
-        else learn_sorted<4>(P, sorted, first, run, bins, row_most, y, h);
-    }
+    if (first[-2] != 0u) learn_rounds_crowded<ALL3>(P, sorted, first, run, row_most, r);
+    else learn_rounds<ALL3, false>(P, sorted, first, run, row_most, r);
     leave(P.turn);
 }
 

@@ -105,3 +105,36 @@ def _few_values(bits, T, K, factor):
 def test_rows_of_few_values_looked_through(K, bits, T):
     """Empty buckets are not looked for (the longest took 40 times the usual)."""
     _few_values(bits, T, K, 2.0)
+
+
+@pytest.mark.parametrize("K,factor", [(4096, 2.5), (8192, 3.2)])
+def test_rows_of_few_values_sorted(K, factor):
+    """Values that share a cell are placed together, and a threshold in a cell of many is the whole warp's work (the pruned rows took
+    3.1 and 4.2 times the usual)."""
+    _few_values(0, 2, K, factor)
+
+
+@pytest.mark.parametrize("K", [256, 1024, 4096, 5120, 8192, 11008, 16384])
+def test_crowded_rows_give_the_same_tables(K):
+    """Rows of a few values, ordinary ones and rows that are half of either, in the sorted form and (through a layout, one round) in the
+    form that looks through the row: one set of tables, the oracle's."""
+    import paper_2502_08141_b200 as lw
+
+    rng = np.random.default_rng(K)
+    W = rng.standard_normal((12, K)).astype(np.float32) * 0.02
+    W[0:3] = np.sign(W[0:3]) * (np.abs(W[0:3]) > 0.012)
+    W[3:6] *= rng.random((3, K)) < 0.1
+    W[6:8] = np.round(W[6:8] / np.abs(W[6:8]).max() * 7)
+    W[8, : K // 2] = 0.02
+    W[9, K // 2:] = 0.0
+    W[10] = 0.0
+    y0, t0 = _start()
+    Wd = torch.from_numpy(W).cuda()
+    for T in (1, 2, 5):
+        maps3, thr3 = lw.lowra_learn_codebooks_all(Wd, y0, t0, T)
+        for c, b in enumerate((1, 2, 4)):
+            precs = np.full(12, b, np.uint8)
+            maps, thr = lw.lowra_learn_codebooks(lw.Layout(precs, K), Wd, y0, t0, T)
+            assert torch.equal(maps, maps3[c]) and torch.equal(thr, thr3[c]), (T, b)
+            ref, _ = oracle.lloyd_max(W, precs, T=T)
+            assert np.all(np.abs(maps.cpu().numpy().astype(np.float64) - ref) <= 2.4e-7), (T, b)
