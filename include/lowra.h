@@ -191,8 +191,8 @@ lowra_status lowra_channel_errors(int32_t N, int32_t K, const float* W_dev, cons
                                   const float* thresholds3_dev, double* sse3_dev, void* stream);
 
 /* Bytes of device scratch that lowra_lora_forward / lowra_lora_backward_input need for M tokens and
- * LoRA rank r (0 if the arguments are invalid).  The first 256 bytes hold the device status word; the
- * rest: the down-projected activations, flags, the deal of the rows to the dequant warps and 39 MB for
+ * LoRA rank r (0 if the arguments are invalid).  The first 4 KB hold the device status word and flags; the
+ * rest: the down-projected activations, the deal of the rows to the dequant warps and 39 MB for
  * the fp32 partial tiles that tiles cut between SMs are handed over in (about 41 MB for a 4096 x 11008
  * matrix at 4096 tokens). */
 size_t lowra_workspace_bytes(const lowra_layout* layout, int32_t M, int32_t r);
@@ -212,7 +212,8 @@ size_t lowra_workspace_bytes(const lowra_layout* layout, int32_t M, int32_t r);
  *                      forward and the backward-input call; reads layout->precs_dev / inv_perm_dev and
  *                      ignores layout->deal_dev.  The buffer is read-only afterwards and may serve any
  *                      number of calls, streams and workspaces.
- *   lowra_workspace_init   zero-fills the workspace (status word, call numbering, flags).
+ *   lowra_workspace_init   clears what the calls rely on (status word, call numbering, flags: the first 4 KB); the rest of
+ *                      the workspace needs no initial value and is left alone.
  * Errors: as lowra_lora_forward; LOWRA_ERR_WORKSPACE for a buffer that is too small or not 256-byte aligned
  * (lowra_deal_build: LOWRA_ERR_ALIGN for the alignment).
  */

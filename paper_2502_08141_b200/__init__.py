@@ -420,7 +420,7 @@ def _workspace(layout: Layout, M: int, r: int, device) -> torch.Tensor:
 
 
 def lowra_workspace_init(workspace: torch.Tensor, stream=None) -> torch.Tensor:
-    """Zero-fill a workspace: needed once before calls on a layout that carries a deal (Layout.build_deal)."""
+    """Clear the status word and the flags of a workspace: needed once before calls on a layout that carries a deal (Layout.build_deal)."""
     _dev(workspace, torch.uint8, "workspace")
     _check(lib().lowra_workspace_init(_ptr(workspace), workspace.numel(), _stream(stream)), "lowra_workspace_init")
     return workspace

@@ -101,6 +101,21 @@ def test_every_group_is_served_while_flags_are_withheld():
         lw.lowra_set_wait_limit(0)
 
 
+def test_initialising_touches_the_header_only():
+    """A call that brings no workspace pays for one each time: what is cleared does not grow with the workspace, and what is not cleared
+    is not relied on."""
+    p = _Problem(512, 640, 64)
+    lw = p.lw
+    ws = torch.empty(lw.lowra_workspace_bytes(p.layout, 600, p.r), dtype=torch.uint8, device="cuda").fill_(0xA5)
+    lw.lowra_workspace_init(ws)
+    assert not bool(ws[:4096].any()) and bool((ws[4096:] == 0xA5).all())
+    for M in (600, 300, 10, 600):
+        for backward in (False, True):
+            act = p.draw(M, p.N if backward else p.K)
+            assert p.right(backward, act, p.call(backward, act, ws), slice(None))
+    assert lw.lowra_device_status(ws) == lw.LOWRA_OK
+
+
 @pytest.mark.parametrize("dealt", [False, True])
 def test_more_tokens_than_the_flags_have_room_for(dealt):
     """From about 104 000 tokens on the "T ready" flags lie behind T and are cleared by every call."""
