@@ -192,9 +192,11 @@ lowra_status lowra_channel_errors(int32_t N, int32_t K, const float* W_dev, cons
 
 /* Bytes of device scratch that lowra_lora_forward / lowra_lora_backward_input need for M tokens and
  * LoRA rank r (0 if the arguments are invalid).  The first 4 KB hold the device status word and flags; the
- * rest: the down-projected activations, the deal of the rows to the dequant warps and 39 MB for
- * the fp32 partial tiles that tiles cut between SMs are handed over in (about 41 MB for a 4096 x 11008
- * matrix at 4096 tokens). */
+ * rest: the down-projected activations, the deal of the rows to the dequant warps and 38 MB for
+ * the fp32 partial tiles that tiles cut between SMs are handed over in (about 40 MB for a 4096 x 11008
+ * matrix at 4096 tokens).  The last LOWRA_WORKSPACE_OPTIONAL of these bytes may be missing, here and in
+ * lowra_batch_workspace_bytes: a call then cuts no tile of 512 tokens, which some sizes are slower for. */
+#define LOWRA_WORKSPACE_OPTIONAL ((size_t)73 * 256 * 1024)
 size_t lowra_workspace_bytes(const lowra_layout* layout, int32_t M, int32_t r);
 
 /*

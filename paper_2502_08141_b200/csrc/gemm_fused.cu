@@ -500,7 +500,7 @@ fused_kernel(const __grid_constant__ KParams<NB> P, const __grid_constant__ KMap
             const int cols = t.is_t ? P.rp : min(kPairR, P.R - r0);   // rows of the tile that exist
             // the columns c0, c0 + 32, ... that this warp takes: half of the tile's; a T tile has few
             const int c_first = t.is_t ? ch * 32 : ch * 128, c_step = t.is_t ? 64 : 32, c_last = t.is_t ? cols : min(cols, ch * 128 + 128);
-            float* part = P.sk_part + ((size_t)cid * CL + crank) * kSkCtaFloats + my_tok;
+            float* part = P.sk_part + (size_t)(cid * CL + (int)crank - CL) * (P.halves * kSkHalfFloats) + my_tok;
             // 32 rows of one token: rounded and stored
             auto put = [&](uint16_t* dst, int left, uint32_t (&v)[32]) {
 #pragma unroll
@@ -559,7 +559,7 @@ fused_kernel(const __grid_constant__ KParams<NB> P, const __grid_constant__ KMap
                     const int h = s / per_half, c0 = (s - h * per_half) * 32;
                     ptx::mbar_arrive_expect_tx(bar, (uint32_t)pieces * kSmemSlot);
                     for (int k = 0; k < pieces; ++k) {
-                        const float* src = P.sk_part + ((size_t)(cid + 1 + k / wide) * CL + crank) * kSkCtaFloats +
+                        const float* src = P.sk_part + (size_t)((cid + k / wide) * CL + (int)crank) * (P.halves * kSkHalfFloats) +
                                            (size_t)(h * kPairR + (k % wide) * 128 + c0) * 128;
                         ptx::bulk_copy_g2s(ptx::smem_u32(x_ring) + (uint32_t)((s % ahead) * pieces + k) * kSmemSlot, src, kSmemSlot, bar);
                     }
@@ -826,7 +826,7 @@ static int plan_schedule(GemmParams& Q, bool may_cut, int max_clusters, float* e
             const float w_us = ramp + pace * blocks * rows;
             offer({(rows == 1 && n_t > 0 && t_us > w_us ? t_us : w_us) + drain, halves, clusters, 0, 0, 0, 0, 1, 0});
         }
-        if (!may_cut || Q.sk_part == nullptr || n_t > max_clusters || blocks < 2 * kMinRange) continue;
+        if (!may_cut || halves > Q.part_halves || n_t > max_clusters || blocks < 2 * kMinRange) continue;
         if ((long long)n * blocks * max_clusters >= (1ll << 31)) continue;     // (32-bit arithmetic in the kernel)
         // Fewer pieces than clusters: s clusters per weight tile, the clusters left over share the T tiles.  Short runs have estimates of
         // their own: a shared T tile takes 0.3 per block and 7.5 + 0.5 per 256 tokens and contributor around them, a 256-token
@@ -886,14 +886,14 @@ static int plan_schedule(GemmParams& Q, bool may_cut, int max_clusters, float* e
 float fused_estimate(int N, int K, int M, int r) {
     GemmParams Q;
     memset(&Q, 0, sizeof(Q));
-    float some = 0.0f, us = 0.0f;
+    float us = 0.0f;
     Q.count = 1;
     Q.mem[0].M = Q.M = M;
     Q.C = K;
     Q.main_blocks = (K + kTileC - 1) / kTileC;
     Q.lora_blocks = (r + 63) / 64 * 64 / kTileC;
     Q.tiles_r = (N + kPairR - 1) / kPairR;
-    Q.sk_part = &some;   // (tiles may be cut)
+    Q.part_halves = 2;   // (tiles may be cut)
     plan_schedule(Q, true, kNumSMs / kCluster, &us);
     return Q.sk ? us + 0.26f * (us - 7.0f) : us;
 }

@@ -39,7 +39,8 @@ struct Workspace {
     int flag0[kMaxBatch];         // per member: index of its first "T ready" flag, counted from off_t_flags
     size_t off_t_flags;
     size_t t_flag_bytes;          // 0: they lie in the header; else behind T, and every call clears them
-    size_t off_items, off_part, total;
+    size_t off_items, off_part;
+    size_t least, total;          // with room for partial tiles of 256 tokens, of 512
     int rp, n_flags;              // flags of the header that the call uses
 };
 
@@ -88,7 +89,8 @@ Workspace plan_workspace(int N, int K, const int* Ms, int count, int r, bool str
     // room for the deal of one direction, rebuilt by every call that brings none
     const size_t fwd = deal_forward_bytes(N), bwd = deal_backward_bytes(N);
     w.off_part = w.off_items + align256(fwd > bwd ? fwd : bwd);
-    w.total = w.off_part + (stream_k ? align256((size_t)kMaxClusters * kSkSlotFloats * 4) : 0);   // stream-K partial tiles
+    w.least = w.off_part + (stream_k ? kSkHalfBytes : 0);
+    w.total = w.off_part + (stream_k ? 2 * kSkHalfBytes : 0);
     return w;
 }
 Workspace plan_workspace(int N, int K, int M, int r, bool stream_k, int count = 1) {
@@ -162,7 +164,7 @@ lowra_status check_members(const MemberArgs* mem, int count, int32_t r, const vo
             return LOWRA_ERR_ALIGN;
     }
     const Workspace w = plan_workspace(N, K, Ms, count, r, stream_k);
-    if (workspace_bytes < w.total || (reinterpret_cast<uintptr_t>(workspace) & 255u) != 0) return LOWRA_ERR_WORKSPACE;
+    if (workspace_bytes < w.least || (reinterpret_cast<uintptr_t>(workspace) & 255u) != 0) return LOWRA_ERR_WORKSPACE;
     return check_device();
 }
 
@@ -282,6 +284,7 @@ lowra_status run_members(bool backward, const MemberArgs* mem, int count, int32_
         if (!seen) G.operand_bytes += (long long)mem[i].M * G.C * 2;
     }
     G.sk_part = stream_k ? reinterpret_cast<float*>(ws + w.off_part) : nullptr;   // null: whole tiles only
+    G.part_halves = !stream_k ? 0 : workspace_bytes >= w.total ? 2 : 1;
     G.sk_flags = flags;
     G.wait_ns = wait_limit_ns();
     {   // diagnostic, armed by lowra_diag_drop_t_flags: take one of the calls it asked for
@@ -476,12 +479,12 @@ extern "C" lowra_status lowra_lora_forward_adapters(const lowra_layout* layout, 
     for (int a = 0; a < n_adapters; ++a)
         if (group_start_host[a + 1] < group_start_host[a]) return LOWRA_ERR_SHAPE;
     const size_t N = (size_t)layout->N, K = (size_t)layout->K;
-    if (workspace_bytes < lowra_workspace_bytes(layout, M, r)) return LOWRA_ERR_WORKSPACE;
+    if (workspace_bytes < plan_workspace(layout->N, layout->K, M, r, true).least) return LOWRA_ERR_WORKSPACE;
     // Up to kMaxBatch token groups go into one launch (one member per group: the same packed weight, the group's
     // mappings, factors and token rows) when the layout carries a deal and the workspace has room for it; otherwise
     // every group is a launch of its own.
     const bool together = layout->deal_dev != nullptr &&
-                          workspace_bytes >= plan_workspace(layout->N, layout->K, M, r, true, kMaxBatch).total;
+                          workspace_bytes >= plan_workspace(layout->N, layout->K, M, r, true, kMaxBatch).least;
     // Groups of few tokens take the path for those, all of them together and first; their T lies where the tokens' own
     // rows lie in the T of a call for all M tokens.
     auto member = [&](int a) {

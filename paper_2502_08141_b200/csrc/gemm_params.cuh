@@ -110,7 +110,8 @@ struct GemmCommon {
     int tiles_r;            // tiles of 256 operand rows of a member (all members have one shape)
     long long operand_bytes;   // token operands of the call, each distinct one counted once (host: schedule choice)
     // schedule of the tiles that are cut between clusters (set by the launcher; sk == 0: whole tiles, dealt round-robin)
-    float* sk_part;         // fp32 partial tiles, one [kCluster][2 halves][256 rows][128 tokens] slot per cluster
+    float* sk_part;         // fp32 partial tiles, one [kCluster][halves][256 rows][128 tokens] slot per cluster but the first, which starts its tiles
+    int part_halves;        // (host) halves of a token tile that the slots have room for: 2, or 1, or 0 (no tile is cut)
     uint32_t* sk_flags;     // [clusters][kCluster] raised when a CTA's partial tile is complete
     int halves;             // token tiles of 256 (1) or 512 tokens (2)
     int t_split;            // > 1: every T tile is cut between so many clusters, which do nothing else
@@ -130,8 +131,8 @@ struct KParams : GemmCommon {
 using GemmParams = KParams<kMaxBatch>;
 unsigned long long wait_limit_ns();   // the process-wide limit, 1 s unless lowra_set_wait_limit changed it
 constexpr int kMaxClusters = kNumSMs / kCluster;
-constexpr size_t kSkCtaFloats = (size_t)kTileT / kCluster * kPairR;   // a CTA's partial tile: its 256 tokens x 256 rows
-constexpr size_t kSkSlotFloats = (size_t)kCluster * kSkCtaFloats;
+constexpr size_t kSkHalfFloats = (size_t)kHalfT / kCluster * kPairR;   // a CTA's partial tile for every 256 tokens: its 128 of them x 256 rows
+constexpr size_t kSkHalfBytes = (size_t)(kMaxClusters - 1) * kCluster * kSkHalfFloats * 4;   // of all slots
 
 constexpr uint32_t kSmemSlot = 128 * kTileC * 2;   // 16 KB: 128 operand rows or tokens of a stage
 constexpr uint32_t kSmemRing = (kSlotsW + kSlotsX) * kSmemSlot;

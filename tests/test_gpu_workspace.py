@@ -116,6 +116,36 @@ def test_initialising_touches_the_header_only():
     assert lw.lowra_device_status(ws) == lw.LOWRA_OK
 
 
+OPTIONAL = 73 * 256 * 1024     # LOWRA_WORKSPACE_OPTIONAL
+
+
+@pytest.mark.parametrize("dealt", [False, True])
+@pytest.mark.parametrize("N,K,M", [(512, 640, 300), (1800, 2304, 777), (2304, 1792, 2500), (1800, 2304, 7500)])
+def test_a_workspace_of_half_the_partial_tiles(N, K, M, dealt):
+    """As large as it had to be while partial tiles held 256 tokens: still accepted, and nothing behind its end is written."""
+    p = _Problem(N, K, 80, dealt)
+    lw = p.lw
+    least = lw.lowra_workspace_bytes(p.layout, M, p.r) - OPTIONAL
+    # what was asked for then: status, T, one flag per 256 tokens and CTA, about 32 bytes a channel for the deal, 74 slots of 256 KB
+    entries = 2 * (4 * ((N + 127) // 128) + 40)
+    up = lambda x: (x + 255) // 256 * 256
+    assert least <= 256 + up(M * 128 * 2) + up(((M + 255) // 256 + 2 + 148) * 4) + up(entries * 512) + up(entries * 4) + 74 * 262144
+    whole = torch.empty(least + OPTIONAL, dtype=torch.uint8, device="cuda").fill_(0xA5)
+    ws = whole[:least]
+    if dealt:
+        lw.lowra_workspace_init(ws)
+    rows = torch.from_numpy(np.unique(np.linspace(0, M - 1, 500).astype(np.int64))).cuda()
+    for backward in (False, True):
+        act = p.draw(M, p.N if backward else p.K)
+        for _ in range(2):
+            out = p.call(backward, act, ws)
+            assert lw.lowra_device_status(ws) == lw.LOWRA_OK and p.right(backward, act, out, rows)
+        with pytest.raises(lw.LowraError) as e:
+            p.call(backward, act, whole[:least - 1])
+        assert e.value.code == lw.LOWRA_ERR_WORKSPACE
+    assert bool((whole[least:] == 0xA5).all())
+
+
 @pytest.mark.parametrize("dealt", [False, True])
 def test_more_tokens_than_the_flags_have_room_for(dealt):
     """From about 104 000 tokens on the "T ready" flags lie behind T and are cleared by every call."""
