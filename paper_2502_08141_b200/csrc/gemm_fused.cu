@@ -500,7 +500,7 @@ fused_kernel(const __grid_constant__ KParams<NB> P, const __grid_constant__ KMap
             const int cols = t.is_t ? P.rp : min(kPairR, P.R - r0);   // rows of the tile that exist
             // the columns c0, c0 + 32, ... that this warp takes: half of the tile's; a T tile has few
             const int c_first = t.is_t ? ch * 32 : ch * 128, c_step = t.is_t ? 64 : 32, c_last = t.is_t ? cols : min(cols, ch * 128 + 128);
-            float* part = P.sk_part + (size_t)(cid * CL + (int)crank - CL) * (P.halves * kSkHalfFloats) + my_tok;
+            float* part = P.sk_part + ((size_t)cid * CL + crank) * kSkHalfFloats + my_tok;
             // 32 rows of one token: rounded and stored
             auto put = [&](uint16_t* dst, int left, uint32_t (&v)[32]) {
 #pragma unroll
@@ -559,8 +559,8 @@ fused_kernel(const __grid_constant__ KParams<NB> P, const __grid_constant__ KMap
                     const int h = s / per_half, c0 = (s - h * per_half) * 32;
                     ptx::mbar_arrive_expect_tx(bar, (uint32_t)pieces * kSmemSlot);
                     for (int k = 0; k < pieces; ++k) {
-                        const float* src = P.sk_part + (size_t)((cid + k / wide) * CL + (int)crank) * (P.halves * kSkHalfFloats) +
-                                           (size_t)(h * kPairR + (k % wide) * 128 + c0) * 128;
+                        const float* src = P.sk_part + ((size_t)(cid + 1 + k / wide) * CL + crank) * kSkHalfFloats +
+                                           (size_t)h * kSkAllFloats + (size_t)((k % wide) * 128 + c0) * 128;
                         ptx::bulk_copy_g2s(ptx::smem_u32(x_ring) + (uint32_t)((s % ahead) * pieces + k) * kSmemSlot, src, kSmemSlot, bar);
                     }
                 };
@@ -615,7 +615,7 @@ fused_kernel(const __grid_constant__ KParams<NB> P, const __grid_constant__ KMap
                     if (t.part) {
                         // fp32 sums of a slice: [row][token], so that a warp writes 128 consecutive bytes
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) __stcg(part + ((size_t)h * kPairR + c0 + j) * 128, __uint_as_float(v[j]));
+                        for (int j = 0; j < 32; ++j) __stcg(part + (size_t)h * kSkAllFloats + (size_t)(c0 + j) * 128, __uint_as_float(v[j]));
                     } else if (tok < M) {
                         if (t.is_t) put_t(tok, c0, v);
                         else put(P.mem[t.prob].out + (size_t)tok * P.ld_out + r0 + c0, cols - c0, v);

@@ -283,7 +283,7 @@ lowra_status run_members(bool backward, const MemberArgs* mem, int count, int32_
         for (int j = 0; j < i; ++j) seen = seen || mem[j].act == mem[i].act;
         if (!seen) G.operand_bytes += (long long)mem[i].M * G.C * 2;
     }
-    G.sk_part = stream_k ? reinterpret_cast<float*>(ws + w.off_part) : nullptr;   // null: whole tiles only
+    G.sk_part = stream_k ? reinterpret_cast<float*>(ws + w.off_part) - kCluster * kSkHalfFloats : nullptr;   // null: whole tiles only
     G.part_halves = !stream_k ? 0 : workspace_bytes >= w.total ? 2 : 1;
     G.sk_flags = flags;
     G.wait_ns = wait_limit_ns();

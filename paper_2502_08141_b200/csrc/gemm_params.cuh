@@ -110,7 +110,8 @@ struct GemmCommon {
     int tiles_r;            // tiles of 256 operand rows of a member (all members have one shape)
     long long operand_bytes;   // token operands of the call, each distinct one counted once (host: schedule choice)
     // schedule of the tiles that are cut between clusters (set by the launcher; sk == 0: whole tiles, dealt round-robin)
-    float* sk_part;         // fp32 partial tiles, one [kCluster][halves][256 rows][128 tokens] slot per cluster but the first, which starts its tiles
+    float* sk_part;         // fp32 partial tiles: for either half of the tokens, [kCluster][256 rows][128 tokens] per cluster.  Points in front of them by
+                            // the slot of the first cluster, which starts its tiles and has none.
     int part_halves;        // (host) halves of a token tile that the slots have room for: 2, or 1, or 0 (no tile is cut)
     uint32_t* sk_flags;     // [clusters][kCluster] raised when a CTA's partial tile is complete
     int halves;             // token tiles of 256 (1) or 512 tokens (2)
@@ -132,7 +133,7 @@ using GemmParams = KParams<kMaxBatch>;
 unsigned long long wait_limit_ns();   // the process-wide limit, 1 s unless lowra_set_wait_limit changed it
 constexpr int kMaxClusters = kNumSMs / kCluster;
 constexpr size_t kSkHalfFloats = (size_t)kHalfT / kCluster * kPairR;   // a CTA's partial tile for every 256 tokens: its 128 of them x 256 rows
-constexpr size_t kSkHalfBytes = (size_t)(kMaxClusters - 1) * kCluster * kSkHalfFloats * 4;   // of all slots
+constexpr size_t kSkAllFloats = (size_t)(kMaxClusters - 1) * kCluster * kSkHalfFloats, kSkHalfBytes = kSkAllFloats * 4;   // of all clusters
 
 constexpr uint32_t kSmemSlot = 128 * kTileC * 2;   // 16 KB: 128 operand rows or tokens of a stage
 constexpr uint32_t kSmemRing = (kSlotsW + kSlotsX) * kSmemSlot;
