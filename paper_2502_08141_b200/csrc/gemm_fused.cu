@@ -880,22 +880,24 @@ static int plan_schedule(GemmParams& Q, bool may_cut, int max_clusters, float* e
     return best.clusters;
 }
 
-// The estimate for a forward call of M tokens by itself on a whole GPU.  Where tiles are cut, weights that mix 4-bit channels with others take
-// longer than the choice of a schedule counts for (13824 x 5120 at 60/35/5, 65 tokens, 56.5 us for 51.5; with 1 and 2 bits 46.7): what
-// lies above a tile's start and drain counts a quarter more, so that the tiles are chosen where they win for every mix.
-float fused_estimate(int N, int K, int M, int r) {
+// The estimate for a forward call of `count` members of M tokens each on a whole GPU.  Where tiles are cut, weights that mix 4-bit channels with
+// others (mixed) take longer than the choice of a schedule counts for (13824 x 5120 at 60/35/5, 65 tokens, 56.5 us for 51.5; with 1 and 2 bits
+// 46.7, all 4 bits 48): what lies above a tile's start and drain counts a quarter more for them.
+float fused_estimate(int N, int K, int M, int r, bool mixed, int count) {
     GemmParams Q;
     memset(&Q, 0, sizeof(Q));
     float us = 0.0f;
-    Q.count = 1;
-    Q.mem[0].M = Q.M = M;
+    Q.count = count < kMaxBatch ? count : kMaxBatch;
+    for (int i = 0; i < Q.count; ++i) Q.mem[i].M = M;
+    Q.M = M;
     Q.C = K;
     Q.main_blocks = (K + kTileC - 1) / kTileC;
     Q.lora_blocks = (r + 63) / 64 * 64 / kTileC;
     Q.tiles_r = (N + kPairR - 1) / kPairR;
     Q.part_halves = 2;   // (tiles may be cut)
     plan_schedule(Q, true, kNumSMs / kCluster, &us);
-    return Q.sk ? us + 0.26f * (us - 7.0f) : us;
+    if (Q.sk && mixed) us += 0.26f * (us - 7.0f);
+    return us * (float)((count + kMaxBatch - 1) / kMaxBatch);
 }
 
 template <int MODE, int NB>

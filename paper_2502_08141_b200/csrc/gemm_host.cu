@@ -178,21 +178,21 @@ int out_alignment(const MemberArgs* mem, int count, int R) {
 lowra_status run_small(const MemberArgs* mem, uint16_t* const* T_of, int count, int32_t r, float s, void* workspace, cudaStream_t stream);
 // The diagnostic lowra_diag_drop_t_flags is about flags, which the path for few tokens has none of: it leaves that path out.
 bool dropping_flags() { return g_drop_t_flags.load(std::memory_order_relaxed) != 0; }
-// The choice follows from the weight's shape and the member's tokens alone, so that a member's result does not depend on its company.
-// From 33 tokens on that path dequantises every weight twice, which weights with many channels and short contractions do not repay (64 tokens,
-// forward, few-token path against tensor-core tiles, us: 2048 x 2048 13.7 against 26, 4096 x 4096 and 8192 x 8192 alike; but 8192 x 512 16.9
-// against 13.1, 11008 x 1024 32 against 18, 13824 x 512 28.7 against 13.3, 13824 x 2560 44 against 33).  The choice leans to the few-token
-// path where the weight's precisions decide: 5120 x 13824, all of 4 bits, keeps it at 72 against 54.  At 17 to 32 tokens only
-// the shortest contractions of many channels leave it (32 tokens, 13824 x 256 18.0 against 11.0; 13824 x 512 17.8 against 13.1).
-bool takes_small_path(bool backward, int N, int K, int M, int r) {
+// Up to 16 tokens it is always taken.  From 33 on it dequantises every weight twice, which many channels with short contractions do not repay, and
+// the two estimates decide (64 tokens, forward, few-token path against tensor-core tiles, us: 2048 x 2048 12 - 13.5 against 21 - 25, 4096 x 4096
+// 23 - 26 against 26 - 27; but 8192 x 512 16.9 against 13.1, 13824 x 512 28.7 against 13.3, 6144 x 2048 of 1 and 2 bits 26.6 against 21.9, 5120 x 5120
+// 34 against 29, 5120 x 13824 of 4 bits 70 against 52).  Weights that mix 4-bit channels with others are slower on cut tiles and lean to the
+// few-token path.  At 17 to 32 tokens only the shortest contractions of many channels leave it (32 tokens, 13824 x 256 18.0 against 11.0).
+bool mixes_4_bits(const lowra_layout* L) { return L->counts[2] > 0 && L->counts[2] < L->N; }
+bool takes_small_path(bool backward, int N, int K, int M, int r, bool mixed) {
     if (backward || M > kSmallTokens) return false;
-    return M <= 16 || small_estimate(N, K, M) < fused_estimate(N, K, M, r);
+    return M <= 16 || small_estimate(N, K, M) < fused_estimate(N, K, M, r, mixed);
 }
 
 // Forward / backward-input for `count` weights of one shape in one launch (count == 1: the plain calls).  The members
-// may have different token counts (several adapters on one weight: one member per token group).
+// may have different token counts (several adapters on one weight: one member per token group).  few_tokens: the path for few tokens is open.
 lowra_status run_members(bool backward, const MemberArgs* mem, int count, int32_t r, float s, void* workspace,
-                         size_t workspace_bytes, void* stream_v, bool stream_k = true) {
+                         size_t workspace_bytes, void* stream_v, bool stream_k = true, bool few_tokens = true) {
     lowra_status st = check_members(mem, count, r, workspace, workspace_bytes, stream_k);
     if (st != LOWRA_OK) return st;
     const int N = mem[0].layout->N, K = mem[0].layout->K;
@@ -209,7 +209,9 @@ lowra_status run_members(bool backward, const MemberArgs* mem, int count, int32_
     uint32_t* flags = reinterpret_cast<uint32_t*>(ws + kFlagsOffset);
     uint32_t* t_flags = reinterpret_cast<uint32_t*>(ws + w.off_t_flags);
 
-    if (!dropping_flags() && takes_small_path(backward, N, K, M, r)) {   // (M: the largest member's tokens)
+    bool mixed = false;
+    for (int i = 0; i < count; ++i) mixed = mixed || mixes_4_bits(mem[i].layout);
+    if (few_tokens && !dropping_flags() && takes_small_path(backward, N, K, M, r, mixed)) {   // (M: the largest member's tokens)
         uint16_t* T_of[kMaxBatch];
         for (int i = 0; i < count; ++i) T_of[i] = reinterpret_cast<uint16_t*>(ws + w.off_T[i]);
         return run_small(mem, T_of, count, r, s, workspace, stream);
@@ -494,7 +496,17 @@ extern "C" lowra_status lowra_lora_forward_adapters(const lowra_layout* layout, 
                           group_start_host[a + 1] - m0};
     };
     const bool dropping = dropping_flags();   // (asked once: the launches below use the diagnostic's calls up)
-    auto is_small = [&](int a) { return !dropping && takes_small_path(false, N, layout->K, group_start_host[a + 1] - group_start_host[a], r); };
+    const bool mixed = mixes_4_bits(layout);
+    auto by_itself = [&](int a) { return !dropping && takes_small_path(false, N, layout->K, group_start_host[a + 1] - group_start_host[a], r, mixed); };
+    // Several groups of 33 to 64 tokens that would take that path each by itself: together they fill the tensor-core tiles' launch, which
+    // dequantises once per group (4096 x 4096 of 4 bits, 64 tokens in each of 2 / 4 / 8 groups, us: 47 / 86 / 164 against 34 / 41 / 80).
+    int few_limit = kSmallTokens;
+    if (together) {
+        int n_mid = 0;
+        for (int a = 0; a < n_adapters; ++a) n_mid += group_start_host[a + 1] - group_start_host[a] > 32 && by_itself(a) ? 1 : 0;
+        if (n_mid > 1 && fused_estimate((int)N, layout->K, kSmallTokens, r, mixed, n_mid) < small_estimate((int)N, layout->K, kSmallTokens, n_mid)) few_limit = 32;
+    }
+    auto is_small = [&](int a) { return group_start_host[a + 1] - group_start_host[a] <= few_limit && by_itself(a); };
     MemberArgs mem[kMaxBatch], few[kSmallMembers];
     uint16_t* few_T[kSmallMembers];
     int n = 0, n_few = 0;
@@ -516,7 +528,7 @@ extern "C" lowra_status lowra_lora_forward_adapters(const lowra_layout* layout, 
             mem[n++] = member(a);
         }
         if (n > 0 && (a == n_adapters || n == (together ? kMaxBatch : 1))) {
-            st = run_members(false, mem, n, r, s, workspace_dev, workspace_bytes, stream);
+            st = run_members(false, mem, n, r, s, workspace_dev, workspace_bytes, stream, true, false);
             if (st != LOWRA_OK) return st;
             n = 0;
         }

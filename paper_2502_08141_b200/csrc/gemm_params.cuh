@@ -144,7 +144,7 @@ constexpr uint32_t kGemmSmemBytes = kSmemRing + kSmemBarriers;
 static_assert(kGemmSmemBytes <= 232448, "227 KB of shared memory per CTA");
 
 lowra_status launch_fused(int mode, const GemmParams& G, const BatchMaps& TM, cudaStream_t stream);
-float fused_estimate(int N, int K, int M, int r);
+float fused_estimate(int N, int K, int M, int r, bool mixed, int count = 1);
 
 // ---- forward pass for few tokens (gemm_small.cu) --------------------------------------------
 constexpr int kSmallTokens = 64;    // members of up to so many tokens may take it, of 16 and fewer do
@@ -158,7 +158,7 @@ struct SmallMember {
     uint16_t *Y, *T;          // T [M, rp]: s X A, as the fused calls leave it
     int M;
 };
-float small_estimate(int N, int K, int M);
+float small_estimate(int N, int K, int M, int count = 1);
 template <int NB>   // members the kernel's parameters have room for
 struct SmallParams {
     SmallMember m[NB];

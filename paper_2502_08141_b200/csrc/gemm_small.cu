@@ -518,13 +518,14 @@ lowra_status launch_members(const SmallParams<NB>& P, cudaStream_t stream) {
 
 }  // namespace
 
-// An estimate of a call's time in microseconds for 17 to 64 tokens, fitted to 40 shapes of 256 to 13824 (within 20 % for most): 6 for the
-// projection and the start; then CTAs that take 1.7, 0.4 for every 8 tokens past 32 (less so many below), 2.7 for every span of a
-// slot and 6 / slices for adding up and storing.  Two share an SM; the last one, if alone on its SM, takes 0.65 of that.
-float small_estimate(int N, int K, int M) {
+// An estimate of a call's time in microseconds for `count` members of 17 to 64 tokens each, fitted to 40 shapes of 256 to 13824 (within 20 % for
+// most): 6 for the projection and the start; then CTAs that take 1.7, 0.4 for every 8 tokens under or over 32 (past 32, where a member has
+// two, 1.2), 2.7 for every span of a slot and 6 / slices for adding up and storing.  Two share an SM; the last one, if alone on its SM,
+// takes 0.65 of that.
+float small_estimate(int N, int K, int M, int count) {
     const int slices = product_slices(N, K), n_span = (K + kSmallSpan - 1) / kSmallSpan;
-    const int ctas = (N / kSmallRows + 2) * slices * ((M + 31) / 32), per_sm = (ctas + kNumSMs - 1) / kNumSMs;
-    const float cta_us = 1.7f + 0.4f * ((M + 7) / 8 - 4) + 2.7f * n_span / (2.0f * slices) + 6.0f / slices;
+    const int ctas = (N / kSmallRows + 2) * slices * ((M + 31) / 32) * count, per_sm = (ctas + kNumSMs - 1) / kNumSMs;
+    const float cta_us = 1.7f + 0.4f * (M > 32 ? 3 : (M + 7) / 8 - 4) + 2.7f * n_span / (2.0f * slices) + 6.0f / slices;
     return 6.0f + cta_us * (per_sm / 2 + (per_sm % 2 != 0 ? 0.65f : 0.0f));
 }
 
