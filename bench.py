@@ -179,8 +179,8 @@ def host_matrix(cfg, mat, rank: int, per_rank: int):
 
 
 # DRAM traffic of one fused_kernel launch measured with ncu (dram__bytes_read.sum + dram__bytes_write.sum) on a
-# launch of workload 3: the backward-input pass of gate_proj (dX [4096, 4096] from dY [4096, 11008];
-# profiles/fused_backward_input_11008x4096_m4096_streamk.md): 193.7 MB read + 50.6 MB written.  The bytes the call
+# launch of workload 3: the backward-input pass of gate_proj (dX [4096, 4096] from dY [4096, 11008]): 193.7 MB
+# read + 50.6 MB written.  The bytes the call
 # has to read and write once are 137 MB (the output is partly still in L2 when the kernel ends; the partial tiles of
 # the cut last row add up to 38 MB each way).  Scaled to the step's average launch in proportion to those input + output bytes.
 NCU_CASE = dict(N=4096, K=11008, M=4096, r=64, bits=1.5, dram_bytes=193.7e6 + 50.6e6)
@@ -593,7 +593,7 @@ def run_gpu(args):
                                               if capped else " (burst figure: the SM clock stayed at its maximum during the timed region)"),
                 "traffic": fused_traffic_per_launch(fused_calls, r, bits),
                 "traffic_source": "ncu dram__bytes_read.sum + dram__bytes_write.sum of the gate_proj backward-input launch of "
-                                  "workload 3 (profiles/fused_backward_input_11008x4096_m4096_streamk.md), scaled by the "
+                                  "workload 3, scaled by the "
                                   "input + output bytes of this step's average launch",
                 "ms_by_step": fused_ms_by_step if args.steps <= 64 else fused_ms_by_step[:32] + fused_ms_by_step[-32:],
                 "before_power_limit": before_limit,

@@ -205,7 +205,8 @@ size_t lowra_workspace_bytes(const lowra_layout* layout, int32_t M, int32_t r);
  * dequantising warps sorted by precision.  With layout->deal_dev == NULL every call works that out again in
  * a small prologue launch, which also clears the status word and the flags in the workspace.  With
  * layout->deal_dev pointing at a buffer filled by lowra_deal_build the fused kernel is the only launch
- * of a call (2-3 us less per call on a B200); the workspace then has to be initialised once with
+ * of a call (2-3 us less per call on a B200; forward calls of up to 64 tokens mostly take another path, of two launches, which needs no
+ * deal); the workspace then has to be initialised once with
  * lowra_workspace_init before its first use, is written by these calls only, and its status word is no
  * longer cleared per call: lowra_device_status reports the first failure since the initialisation.
  *   lowra_deal_bytes   size of the buffer for this layout (0 if the layout is invalid); about 20 bytes per
@@ -264,7 +265,8 @@ lowra_status lowra_lora_backward_input(const lowra_layout* layout, const uint8_t
  * factors, input and output:
  *     forward:         Y_i  = X_i  . deq(Wq_i)^T + s * (X_i . A_i) . B_i
  *     backward-input:  dX_i = dY_i . deq(Wq_i)   + s * (dY_i . B_i^T) . A_i^T          i = 0 .. count - 1
- * The results are bit for bit those of `count` single calls.  What is saved is what a call costs beside its tiles:
+ * The results are bit for bit those of `count` single calls wherever no tile is cut between SMs (where one is, which depends on all
+ * members together, fp32 partial sums are added in another order).  What is saved is what a call costs beside its tiles:
  * the launch, the pipeline's fill and drain, the wait for the first down-projected tile and the ragged last row of
  * tiles are paid once for the group instead of once per weight (on a B200 about 12 us per weight left out; a
  * 4096 x 4096 call at 4096 tokens takes 155 us).  Members may share an input (q, k, v read the same X).
@@ -299,10 +301,12 @@ lowra_status lowra_lora_backward_input_batch(const lowra_member* members_host, i
  * table and its own low-rank factors).  The tokens of the batch are sorted by adapter: adapter a owns the token rows
  * [group_start_host[a], group_start_host[a + 1]) of X and Y, and for those rows
  *     Y = X . deq_a(Wq)^T + s * (X . A_a) . B_a
- * with deq_a the dequantisation through adapter a's mappings.  One call routes every group to its tables.  Up to
- * LOWRA_MAX_BATCH groups run in one fused launch (their tiles dealt to the SMs together, so that small groups fill the
+ * with deq_a the dequantisation through adapter a's mappings.  One call routes every group to its tables.  Groups of few tokens (up to 16
+ * always, up to 64 by the weight's shape and precisions) go first, eight to two launches, with or without a deal.  Of the others up to
+ * LOWRA_MAX_BATCH run in one fused launch (their tiles dealt to the SMs together, so that small groups fill the
  * GPU between them) when the layout carries a deal and the workspace has lowra_batch_workspace_bytes(layout,
- * LOWRA_MAX_BATCH, M, r) bytes; otherwise every group is a launch of its own.  A dequantised weight tile depends on
+ * LOWRA_MAX_BATCH, M, r) bytes; otherwise every group is a launch of its own.  Groups of up to 16 tokens are bit for bit what a call of their
+ * own gives; with larger ones, which path and which cuts they take depends on the other groups.  A dequantised weight tile depends on
  * the adapter's mappings, so groups never share tiles; empty groups are skipped.
  *   maps_dev         fp32 [n_adapters][N][16]
  *   A_dev            bf16 [n_adapters][K][r];   B_dev  bf16 [n_adapters][r][N]
@@ -418,8 +422,9 @@ lowra_status lowra_lora_forward_static(const lowra_layout* layout, const uint8_t
  *     assign:  bucket of n = number of current thresholds <= n
  *     levels:  y_j <- sum(w n) / sum(w) over bucket j   (an empty bucket keeps its level)
  *     thresholds: t_j <- (y_j + y_{j+1}) / 2
- * in fp64, the sums in 64-bit fixed point (multiples of 2^-46 of the channel's largest weight or, in buckets lighter
- * than a quarter of that, of the bucket's).  Output tables, fp32 [N, 16], original row order: maps = (float) y (unused entries 0),
+ * in fp64, the sums in 64-bit fixed point: multiples of u = 2^-46 of the power of two above the channel's largest weight, w to nearest and w n
+ * down, so that a level is less than u / (mean weight of its bucket) below the exact mean.  Where |sum(w n)| < 2^24 K u - levels next to zero, light
+ * buckets - the bucket is added up to 2^-92 instead, so every level is right to 2^-23 of itself before it is rounded to fp32.  Output tables, fp32 [N, 16], original row order: maps = (float) y (unused entries 0),
  * thresholds[j] = (float)(((double) maps[j] + (double) maps[j+1]) / 2) (unused entries +infinity) - directly
  * usable by lowra_encode / lowra_decode.
  *   W_dev                 fp32 [N, K] row-major, original row order                      (in)
