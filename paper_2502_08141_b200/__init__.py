@@ -236,7 +236,7 @@ class Layout:
         c.natural_offsets_dev = None
         self.c = c
         self.ref = ctypes.byref(c)
-        self.last_size = (0, 0, 0)
+        self.last_size = (-1, -1, 0)   # (tokens, rank) of the last workspace made here, and its size
         self.deal = None
         self.natural_offsets = None
         if natural:
@@ -404,7 +404,16 @@ def lowra_workspace_bytes(layout: Layout, M: int, r: int) -> int:
     return int(lib().lowra_workspace_bytes(layout.ref, int(M), int(r)))
 
 
-def _workspace(layout: Layout, M: int, r: int, device) -> torch.Tensor:
+def _scratch(nbytes: int, device, stream=None) -> torch.Tensor:
+    """Scratch of one call, from the memory of the stream that uses it: it is given back as soon as the call has been
+    enqueued, and whoever gets it next on that stream comes after the call."""
+    if stream is None:
+        return torch.empty(nbytes, dtype=torch.uint8, device=device)
+    with torch.cuda.stream(stream):
+        return torch.empty(nbytes, dtype=torch.uint8, device=device)
+
+
+def _workspace(layout: Layout, M: int, r: int, device, stream=None) -> torch.Tensor:
     last = layout.last_size           # the size follows from the shape, M and r: asked for once for calls of one size
     if last[0] == M and last[1] == r:
         n = last[2]
@@ -413,9 +422,9 @@ def _workspace(layout: Layout, M: int, r: int, device) -> torch.Tensor:
         if n == 0:
             raise LowraError(LOWRA_ERR_SHAPE, "lowra_workspace_bytes")
         layout.last_size = (M, r, n)
-    ws = torch.empty(n, dtype=torch.uint8, device=device)
+    ws = _scratch(n, device, stream)
     if layout.deal is not None:   # no prologue launch will clear it
-        lowra_workspace_init(ws)
+        lowra_workspace_init(ws, stream)
     return ws
 
 
@@ -439,7 +448,7 @@ def lowra_lora_forward(layout: Layout, packed, absmax, maps, X, A, B, s: float,
     if Y is None:
         Y = X.new_empty((M, layout.N))
     if workspace is None:
-        workspace = _workspace(layout, M, r, X.device)
+        workspace = _workspace(layout, M, r, X.device, stream)
     code = (_lib or lib()).lowra_lora_forward(layout.ref, _ptr(packed), _ptr(absmax), _ptr(maps), X.data_ptr(), M, A.data_ptr(),
                                               B.data_ptr(), r, s, Y.data_ptr(), workspace.data_ptr(), workspace.numel(), _stream(stream))
     if code:
@@ -503,7 +512,7 @@ def lowra_lora_forward_adapters(layout: Layout, packed, absmax, maps, X, group_s
     if Y is None:
         Y = X.new_empty((M, layout.N))
     if workspace is None:
-        workspace = _workspace(layout, M, r, X.device)
+        workspace = _workspace(layout, M, r, X.device, stream)
     code = lib().lowra_lora_forward_adapters(layout.ref, _ptr(packed), _ptr(absmax), _ptr(maps), n, _ptr(X), M,
                                              gs.ctypes.data_as(ctypes.c_void_p), _ptr(A), _ptr(B), r, s,
                                              _ptr(Y), _ptr(workspace), workspace.numel(), _stream(stream))
@@ -545,7 +554,7 @@ def lowra_lora_backward_input(layout: Layout, packed, absmax, maps, dY, A, B, s:
     if dX is None:
         dX = dY.new_empty((M, layout.K))
     if workspace is None:
-        workspace = _workspace(layout, M, r, dY.device)
+        workspace = _workspace(layout, M, r, dY.device, stream)
     code = lib().lowra_lora_backward_input(layout.ref, _ptr(packed), _ptr(absmax), _ptr(maps), _ptr(dY), M,
                                            _ptr(A), _ptr(B), r, s, _ptr(dX), _ptr(workspace),
                                            workspace.numel(), _stream(stream))
@@ -641,7 +650,7 @@ def lowra_lora_backward_adapters(X, dY, A, B, s: float, dA: Optional[torch.Tenso
         nbytes = lowra_adapter_workspace_bytes(M, r)
         if nbytes == 0:
             raise LowraError(LOWRA_ERR_SHAPE, "lowra_adapter_workspace_bytes")
-        workspace = torch.empty(nbytes, dtype=torch.uint8, device=X.device)
+        workspace = _scratch(nbytes, X.device, stream)
     code = lib().lowra_lora_backward_adapters(_ptr(X), _ptr(dY), M, K, N, _ptr(A), _ptr(B), r, s,
                                               _ptr(dA), _ptr(dB), _ptr(workspace), workspace.numel(),
                                               _stream(stream))
@@ -677,7 +686,7 @@ def lowra_lora_backward_adapters_reuse(X, dY, T, U, r: int, dA: Optional[torch.T
     if dB is None:
         dB = X.new_empty((r, N))
     if workspace is None:
-        workspace = torch.empty(256, dtype=torch.uint8, device=X.device)
+        workspace = _scratch(256, X.device, stream)
     code = lib().lowra_lora_backward_adapters_reuse(_ptr(X), _ptr(dY), M, K, N, _ptr(T), _ptr(U), int(r), _ptr(dA), _ptr(dB),
                                                     _ptr(workspace), workspace.numel(), _stream(stream))
     _check(code, "lowra_lora_backward_adapters_reuse")
@@ -716,7 +725,7 @@ def lowra_dense_nt(P: torch.Tensor, Q: torch.Tensor, C: Optional[torch.Tensor] =
     if C is None:
         C = torch.empty((M, N), dtype=torch.bfloat16, device=P.device)
     if workspace is None:
-        workspace = torch.empty(256, dtype=torch.uint8, device=P.device)
+        workspace = _scratch(256, P.device, stream)
     code = lib().lowra_dense_nt(_ptr(P), _ptr(Q), int(M), int(N), int(K), _ptr(C), _ptr(workspace),
                                 workspace.numel(), _stream(stream))
     _check(code, "lowra_dense_nt")

@@ -116,6 +116,31 @@ def test_initialising_touches_the_header_only():
     assert lw.lowra_device_status(ws) == lw.LOWRA_OK
 
 
+def test_scratch_of_a_call_belongs_to_its_stream(monkeypatch):
+    """A call on a stream of its own, with no workspace passed: cleared on that stream and taken from its memory, not the current one's."""
+    p = _Problem(512, 640, 64)
+    lw = p.lw
+    side = torch.cuda.Stream()
+    X, dY = p.draw(300, p.K), p.draw(300, p.N)
+    torch.cuda.synchronize()
+    seen = []
+    init, empty = lw.lowra_workspace_init, torch.empty
+    monkeypatch.setattr(lw, "lowra_workspace_init", lambda ws, stream=None: (seen.append(stream), init(ws, stream))[1])
+
+    def record(*size, **kw):
+        if kw.get("dtype") is torch.uint8:
+            seen.append(torch.cuda.current_stream())
+        return empty(*size, **kw)
+    monkeypatch.setattr(lw.torch, "empty", record)
+    Y = lw.lowra_lora_forward(p.layout, p.packed, p.absmax, p.maps, X, p.A, p.B, 2.0, stream=side)
+    dX = lw.lowra_lora_backward_input(p.layout, p.packed, p.absmax, p.maps, dY, p.A, p.B, 2.0, stream=side)
+    lw.lowra_lora_backward_adapters(X, dY, p.A, p.B, 2.0, stream=side)
+    monkeypatch.undo()
+    side.synchronize()
+    assert len(seen) == 5 and all(s == side for s in seen)
+    assert p.right(False, X, Y, slice(None)) and p.right(True, dY, dX, slice(None))
+
+
 OPTIONAL = 73 * 256 * 1024     # LOWRA_WORKSPACE_OPTIONAL
 
 
