@@ -271,7 +271,6 @@ lowra_status run_members(bool backward, const MemberArgs* mem, int count, int32_
     G.wide_only = w.t_flag_bytes > 0;
     G.s = s;
     G.rp = w.rp;
-    G.r = r;
     G.M = M;
     G.R = backward ? K : N;
     G.C = backward ? N : K;
@@ -280,11 +279,6 @@ lowra_status run_members(bool backward, const MemberArgs* mem, int count, int32_
     G.main_blocks = (G.C + kTileC - 1) / kTileC;
     G.lora_blocks = w.rp / kTileC;
     G.tiles_r = (G.R + kPairR - 1) / kPairR;
-    for (int i = 0; i < count; ++i) {   // token operands: every distinct one once (q, k, v share X in the forward pass)
-        bool seen = false;
-        for (int j = 0; j < i; ++j) seen = seen || mem[j].act == mem[i].act;
-        if (!seen) G.operand_bytes += (long long)mem[i].M * G.C * 2;
-    }
     G.sk_part = stream_k ? reinterpret_cast<float*>(ws + w.off_part) - kCluster * kSkHalfFloats : nullptr;   // null: whole tiles only
     G.part_halves = !stream_k ? 0 : workspace_bytes >= w.total ? 2 : 1;
     G.sk_flags = flags;

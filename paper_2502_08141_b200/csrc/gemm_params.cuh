@@ -98,7 +98,6 @@ struct GemmCommon {
     int wide_only;          // (host) token tiles of 512 only: the call's flags are counted for those
     float s;
     int rp;                 // LoRA rank rounded up to 64
-    int r;                  // LoRA rank
     int M;                  // tokens of the largest member (host: schedule choice)
     int super_total;        // token tiles of all members
     int R;                  // A-operand rows in total: N (forward, dense) or K (backward)
@@ -108,7 +107,6 @@ struct GemmCommon {
     int main_blocks;        // ceil(C / 64)
     int lora_blocks;        // rp / 64 (0 in dense mode)
     int tiles_r;            // tiles of 256 operand rows of a member (all members have one shape)
-    long long operand_bytes;   // token operands of the call, each distinct one counted once (host: schedule choice)
     // schedule of the tiles that are cut between clusters (set by the launcher; sk == 0: whole tiles, dealt round-robin)
     float* sk_part;         // fp32 partial tiles: for either half of the tokens, [kCluster][256 rows][128 tokens] per cluster.  Points in front of them by
                             // the slot of the first cluster, which starts its tiles and has none.

@@ -330,8 +330,7 @@ __device__ void learn_row(const LearnParams& P, const float* xs, const float* ws
             // Few buckets: no bucket index at all.  cn[0] / cw[0] take all elements, cn[j] / cw[j] (j >= 1) those at or above
             // threshold j - 1, and a bucket's sums are the difference of two neighbours.  An element that is out becomes
             // a tiny positive number (the upper half of the fp64 number zero), which rounding down leaves without effect: one
-            // selection, where the predicated addition comes out of the compiler as two of the sum (1 bit, 4096 x 4096: 8.2 against
-            // 10 us a round).
+            // selection instead of a conditional addition (1 bit, 4096 x 4096: 8.2 against 10 us a round).
             // (The first round forms cn[0] for all.)
             unsigned long long cn[Lv];
             long long cw[Lv];
@@ -853,7 +852,7 @@ lowra_status launch_sorted_kernel(LearnParams& P, int rows, void* stream) {
     return launch_rows(sorted_learn_kernel<ALL3, THREADS, PER, CTAS>, P, rows, (P.K / PER + 31) / 32 * 32, sorted_smem_bytes(P.K), &limit, stream);
 }
 
-bool two_long_rows(int K) { return 2 * (sorted_smem_bytes(K) + 1024) <= 228 * 1024; }   // an SM holds two (K <= 11264)
+bool two_long_rows(int K) { return 2 * (sorted_smem_bytes(K) + 1024) <= 228 * 1024; }   // an SM holds two (K <= 11776)
 
 // Whether the rounds of a class together are long enough to pay for the order (c = 0, 1, 2: 1, 2, 4 bits; 3: all of them).  Measured, us, 4096 rows
 // (K = 13824: 3328), learn_kernel against sorted_learn_kernel, after 2, 4 and 10 rounds:

@@ -38,21 +38,13 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t by
                  : "memory");
 }
 
-template <bool kClusterAcquire = false>
 __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
     uint32_t ok;
-    if (kClusterAcquire)   // also acquires what other CTAs of the cluster wrote before they arrived
-        asm volatile(
-            "{ .reg .pred p; mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
-            : "=r"(ok)
-            : "r"(smem_u32(bar)), "r"(parity)
-            : "memory");
-    else
-        asm volatile(
-            "{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
-            : "=r"(ok)
-            : "r"(smem_u32(bar)), "r"(parity)
-            : "memory");
+    asm volatile(
+        "{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
     return ok != 0;
 }
 
@@ -71,18 +63,17 @@ __device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
 // Waits until the phase with the given parity has completed, or until `limit_ns` has passed, or until
 // *abort (a shared-memory flag set by a role that already gave up; may be null) becomes non-zero.  Returns true
 // only when the phase completed.
-template <bool kClusterAcquire = false>
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile uint32_t* abort,
                                           uint64_t limit_ns) {
 #pragma unroll 1
     for (int i = 0; i < 2048; ++i)
-        if (mbar_try_wait<kClusterAcquire>(bar, parity)) return true;
+        if (mbar_try_wait(bar, parity)) return true;
     const uint64_t t0 = globaltimer_ns();
 #pragma unroll 1
     for (;;) {
 #pragma unroll 1
         for (int i = 0; i < 64; ++i) {
-            if (mbar_try_wait<kClusterAcquire>(bar, parity)) return true;
+            if (mbar_try_wait(bar, parity)) return true;
             __nanosleep(32);
         }
         if (abort != nullptr && *abort != 0u) return false;
@@ -127,11 +118,6 @@ __device__ __forceinline__ void fence_proxy_async_all() { asm volatile("fence.pr
 // Global-memory flag between CTAs: release store / bounded acquire poll.  A flag is up when it holds `want`.
 __device__ __forceinline__ void flag_release(uint32_t* flag, uint32_t value) {
     asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(flag), "r"(value) : "memory");
-}
-__device__ __forceinline__ bool flag_test(const uint32_t* flag, uint32_t want) {   // one look, no waiting
-    uint32_t v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(flag) : "memory");
-    return v == want;
 }
 __device__ __forceinline__ bool flag_wait(const uint32_t* flag, uint32_t want, volatile uint32_t* abort, uint64_t limit_ns) {
     const uint64_t t0 = globaltimer_ns();
