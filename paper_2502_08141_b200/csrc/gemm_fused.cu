@@ -843,6 +843,19 @@ static int plan_schedule(GemmParams& Q, bool may_cut, int max_clusters, float* e
             const float us = (t_done > w_done ? t_done : w_done) + (s == 1 ? drain : drain + collect(s - 1) + 3.2f);
             offer({us, halves, n_t * ts + n_w * s, 1, 0, n_t * ts, 0, ts, n_w * blocks});
         }
+        // T by clusters of its own, each tile by ts of them, and ranges over all weight tiles for the others: for few channels and many tokens, where one
+        // piece in a few is a T tile that the others wait for, and for pieces that come out a little over a row (forward, us, against the
+        // choices around: 1024 x 4096, 4096 / 8192 tokens 60 -> 52 / 92 -> 78; 1024 x 11008, 4096 tokens 137 -> 101; 3072 x 3072, 3000 tokens 75 -> 61;
+        // 6144 x 2048, 1500 tokens 54 -> 46).  Ranges of less than half a tile gain nothing (2048 x 4096, 600 tokens 30.4 -> 33.7); nor
+        // does a choice that is ahead by less than a microsecond or so (1024 x 11008, 6000 tokens 140 -> 152).
+        for (int ts = 1; ts <= kMaxContributors && n_t * ts < max_clusters; ++ts) {
+            if (ts > 1 && ts > Q.main_blocks / kMinRange) break;
+            const int c = max_clusters - n_t * ts;
+            const float range = (float)n_w * blocks / c;
+            if (range < shortest || 2.0f * range < blocks) continue;      // (longer with every ts)
+            const float t_done = ts == 1 ? t_us : 7.5f + 0.3f * Q.main_blocks / ts + 0.5f * halves * ts, w_done = ramp + pace * range;
+            offer({(t_done > w_done ? t_done : w_done) + drain + collect((int)((blocks + range - 1) / range)) + 1.5f, halves, max_clusters, 1, 0, n_t * ts, 0, ts, n_w * blocks});
+        }
         // Ranges for the last row of pieces, or for the last two.  The clusters' sweeps over the contraction fall out of step
         // inside the ranges, so the part of the token operand that is live there has to stay in L2 (ranges over all tiles of a
         // 90 MB operand: 6.5 times the DRAM reads, and no gain).
