@@ -2,15 +2,25 @@
 // A Scaled<B> holds the row's 2^B levels multiplied by the block's absmax and rounded to bf16 (exactly as lowra_decode does),
 // in the form in which expand16 picks them: sixteen elements, two per word (the earlier one in the low half).
 //   1 bit : both patterns differ by d; one multiply-add forms two elements (3 instructions a pair);
-//   2 bits: the low and the high bytes of the four patterns are a word each; a byte permute looks four codes up, further
-//           ones put the bytes of neighbouring elements together (3.6 instructions a pair; picking 16-bit patterns pair by pair, 6);
-//   4 bits: likewise with four words each, the fourth bit of a code choosing between the halves of the table (5.5 instructions a
-//           pair, no memory; a table in shared memory costs 9 and two loads).
+//   2 bits: the four patterns are two words, and one byte permute picks a pair out of them; what that needs - the codes c of
+//           the pair as the nibbles 2 c, 2 c + 1 - comes from two multiplications for every two pairs;
+//   4 bits: the low and the high bytes of the sixteen patterns are four words each; a byte permute looks four codes up, further ones put the
+//           bytes together, the fourth bit of a code choosing between the halves of the table (a table in shared memory costs 9 and two loads).
+// What bounds it: the half-rate pipe that permutes, shifts and logic share, the multiplications being on another.  Cycles of a scheduler for a
+// block of 64 elements of 32 rows: 194 at 1 bit, 201 at 2 (258 with low and high bytes looked up by themselves, as at 4 bits), 438 at 4 (468 with four
+// codes at a time and masked selectors).
 #pragma once
 
 #include "lowra_common.cuh"
 
 namespace lowra {
+
+// PRMT with a selector whose nibbles are known to be below 8 (__byte_perm masks them)
+__device__ __forceinline__ uint32_t pick_bytes(uint32_t a, uint32_t b, uint32_t sel) {
+    uint32_t r;
+    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(sel));
+    return r;
+}
 
 template <int B> struct Scaled;
 template <> struct Scaled<1> {
@@ -29,24 +39,17 @@ template <> struct Scaled<1> {
     }
 };
 template <> struct Scaled<2> {
-    uint32_t lo, hi;         // low and high bytes of the four patterns
+    uint32_t p01, p23;       // the four patterns
     __device__ __forceinline__ void set(const float* y, float a) {
-        const uint32_t p = pack_bf16x2(__fmul_rn(y[0], a), __fmul_rn(y[1], a)), r = pack_bf16x2(__fmul_rn(y[2], a), __fmul_rn(y[3], a));
-        lo = __byte_perm(p, r, 0x6420u);
-        hi = __byte_perm(p, r, 0x7531u);
+        p01 = pack_bf16x2(__fmul_rn(y[0], a), __fmul_rn(y[1], a));
+        p23 = pack_bf16x2(__fmul_rn(y[2], a), __fmul_rn(y[3], a));
     }
     __device__ __forceinline__ void expand16(const uint32_t* w, int q, uint32_t (&o)[8]) const {
-        const uint32_t even = w[q] & 0x33333333u, odd = (w[q] >> 2) & 0x33333333u;   // the codes of every second element, one per nibble
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const uint32_t e = h ? even >> 16 : even, d = h ? odd >> 16 : odd;
-            const uint32_t el = __byte_perm(lo, 0u, e), eh = __byte_perm(hi, 0u, e), dl = __byte_perm(lo, 0u, d), dh = __byte_perm(hi, 0u, d);
-            const uint32_t e01 = __byte_perm(el, eh, 0x5140u), e23 = __byte_perm(el, eh, 0x7362u);
-            const uint32_t d01 = __byte_perm(dl, dh, 0x5140u), d23 = __byte_perm(dl, dh, 0x7362u);
-            o[4 * h] = __byte_perm(e01, d01, 0x5410u);
-            o[4 * h + 1] = __byte_perm(e01, d01, 0x7632u);
-            o[4 * h + 2] = __byte_perm(e23, d23, 0x5410u);
-            o[4 * h + 3] = __byte_perm(e23, d23, 0x7632u);
+        for (int k = 0; k < 4; ++k) {   // pairs k and 4 + k: their codes in a byte each, times 2, and that plus 1 beside it
+            const uint32_t c = (((w[q] >> (4 * k)) & 0x000F000Fu) * 0x41u) & 0x03030303u, sel = c * 0x22u + 0x10101010u;
+            o[k] = pick_bytes(p01, p23, sel);
+            o[4 + k] = pick_bytes(p01, p23, sel >> 16);
         }
     }
 };
@@ -63,14 +66,17 @@ template <> struct Scaled<4> {
     }
     __device__ __forceinline__ void expand16(const uint32_t* w, int q, uint32_t (&o)[8]) const {
 #pragma unroll
-        for (int h = 0; h < 4; ++h) {   // four codes at a time
-            const uint32_t x = w[2 * q + (h >> 1)] >> (16 * (h & 1));
-            const uint32_t sel = x & 0x7777u;
-            const uint32_t upper = __byte_perm(0x0000FF00u, 0u, (x >> 3) & 0x1111u);   // 0xFF where the code is 8 or more
-            const uint32_t l = (__byte_perm(lo[0], lo[1], sel) & ~upper) | (__byte_perm(lo[2], lo[3], sel) & upper);
-            const uint32_t u = (__byte_perm(hi[0], hi[1], sel) & ~upper) | (__byte_perm(hi[2], hi[3], sel) & upper);
-            o[2 * h] = __byte_perm(l, u, 0x5140u);
-            o[2 * h + 1] = __byte_perm(l, u, 0x7362u);
+        for (int h = 0; h < 2; ++h) {   // eight codes at a time
+            const uint32_t x = w[2 * q + h], sel = x & 0x77777777u, top = (x >> 3) & 0x11111111u;
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const uint32_t sl = i ? sel >> 16 : sel;
+                const uint32_t upper = pick_bytes(0x0000FF00u, 0u, i ? top >> 16 : top);   // 0xFF where the code is 8 or more
+                const uint32_t l = (pick_bytes(lo[0], lo[1], sl) & ~upper) | (pick_bytes(lo[2], lo[3], sl) & upper);
+                const uint32_t u = (pick_bytes(hi[0], hi[1], sl) & ~upper) | (pick_bytes(hi[2], hi[3], sl) & upper);
+                o[4 * h + 2 * i] = __byte_perm(l, u, 0x5140u);
+                o[4 * h + 2 * i + 1] = __byte_perm(l, u, 0x7362u);
+            }
         }
     }
 };
