@@ -175,7 +175,7 @@ int out_alignment(const MemberArgs* mem, int count, int R) {
     return wide ? 32 : 16;
 }
 
-lowra_status run_small(const MemberArgs* mem, uint16_t* const* T_of, int count, int32_t r, float s, void* workspace, cudaStream_t stream);
+lowra_status run_small(const MemberArgs* mem, uint16_t* const* T_of, int count, int32_t r, float s, bool one_weight, void* workspace, cudaStream_t stream);
 // The diagnostic lowra_diag_drop_t_flags is about flags, which the path for few tokens has none of: it leaves that path out.
 bool dropping_flags() { return g_drop_t_flags.load(std::memory_order_relaxed) != 0; }
 // Up to 16 tokens it is always taken.  From 33 on it dequantises every weight twice, which many channels with short contractions do not repay, and
@@ -214,7 +214,7 @@ lowra_status run_members(bool backward, const MemberArgs* mem, int count, int32_
     if (few_tokens && !dropping_flags() && takes_small_path(backward, N, K, M, r, mixed)) {   // (M: the largest member's tokens)
         uint16_t* T_of[kMaxBatch];
         for (int i = 0; i < count; ++i) T_of[i] = reinterpret_cast<uint16_t*>(ws + w.off_T[i]);
-        return run_small(mem, T_of, count, r, s, workspace, stream);
+        return run_small(mem, T_of, count, r, s, count == 1, workspace, stream);
     }
     if (w.t_flag_bytes > 0 && cudaMemsetAsync(t_flags, 0, w.t_flag_bytes, stream) != cudaSuccess) return LOWRA_ERR_CUDA;
 
@@ -307,8 +307,9 @@ lowra_status run_members(bool backward, const MemberArgs* mem, int count, int32_
 }
 
 // Forward pass of members of few tokens each (any number of them, one shape): two launches for every kSmallMembers.
-// Their arguments have been checked as run_members does.  T_of: where member i's down-projected tokens go.
-lowra_status run_small(const MemberArgs* mem, uint16_t* const* T_of, int count, int32_t r, float s, void* workspace, cudaStream_t stream) {
+// Their arguments have been checked as run_members does.  T_of: where member i's down-projected tokens go.  one_weight: they share layout, codes
+// and absmax.
+lowra_status run_small(const MemberArgs* mem, uint16_t* const* T_of, int count, int32_t r, float s, bool one_weight, void* workspace, cudaStream_t stream) {
     SmallParams<kSmallMembers> P;
     P.N = mem[0].layout->N;
     P.K = mem[0].layout->K;
@@ -316,6 +317,7 @@ lowra_status run_small(const MemberArgs* mem, uint16_t* const* T_of, int count, 
     P.rp = (r + 63) / 64 * 64;
     P.s = s;
     P.status = static_cast<uint32_t*>(workspace);
+    P.one_weight = one_weight ? 1 : 0;
     for (int first = 0; first < count; first += kSmallMembers) {
         P.count = count - first < kSmallMembers ? count - first : kSmallMembers;
         P.clear_status = first == 0 && mem[0].layout->deal_dev == nullptr;
@@ -512,7 +514,7 @@ extern "C" lowra_status lowra_lora_forward_adapters(const lowra_layout* layout, 
             few[n_few++] = member(a);
         }
         if (n_few > 0 && (a == n_adapters || n_few == kSmallMembers)) {
-            if ((st = run_small(few, few_T, n_few, r, s, workspace_dev, (cudaStream_t)stream)) != LOWRA_OK) return st;
+            if ((st = run_small(few, few_T, n_few, r, s, true, workspace_dev, (cudaStream_t)stream)) != LOWRA_OK) return st;
             n_few = 0;
         }
     }

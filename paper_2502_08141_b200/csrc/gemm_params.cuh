@@ -164,6 +164,7 @@ struct SmallParams {
     float s;
     uint32_t* status;
     int clear_status;         // the call brings no deal: its status word starts from zero
+    int one_weight;           // all members have the same layout, codes and absmax (several adapters)
 };
 lowra_status launch_small(const SmallParams<kSmallMembers>& P, cudaStream_t stream);
 

@@ -16,6 +16,8 @@
 //                    the same accumulation.
 // It starts while project_kernel runs and waits for it only before the low-rank term (programmatic dependent launch).
 // No flags, no waits that need a limit, any number of such calls may share the GPU.
+#include <type_traits>
+
 #include "dequant.cuh"
 #include "gemm_params.cuh"
 #include "ptx.cuh"
@@ -214,6 +216,25 @@ __device__ __forceinline__ uint32_t token_piece(int m, int t, int j) {
     return (uint32_t)(m * (kSmallSpan * 2) + (t * 8 + (j ^ (t | ((m & 1) << 2)))) * 16);
 }
 
+// Sixteen elements of the lane's block of either row, times the tokens (xs: where the block's first piece lies for token g).  A sum's steps wait for
+// one another, so the tokens take turns.
+template <int B, int NT8>
+__device__ __forceinline__ void multiply_16(float (&acc)[NT8][4], const Scaled<B>& s0, const Scaled<B>& s1, const Codes<B>& c0, const Codes<B>& c1, int q, uint32_t xs) {
+    uint32_t o0[8], o1[8];
+    s0.expand16(c0.w, q, o0);
+    s1.expand16(c1.w, q, o1);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        uint4 x[NT8];
+#pragma unroll
+        for (int nt = 0; nt < NT8; ++nt) x[nt] = ld_shared_v4((xs ^ (32u * q + 16u * h)) + (uint32_t)(nt * 8 * kSmallSpan * 2));
+#pragma unroll
+        for (int nt = 0; nt < NT8; ++nt) mma_bf16(acc[nt], o0[4 * h], o1[4 * h], o0[4 * h + 1], o1[4 * h + 1], x[nt].x, x[nt].y);
+#pragma unroll
+        for (int nt = 0; nt < NT8; ++nt) mma_bf16(acc[nt], o0[4 * h + 2], o1[4 * h + 2], o0[4 * h + 3], o1[4 * h + 3], x[nt].z, x[nt].w);
+    }
+}
+
 // A warp's sixteen rows times the tokens, over the contraction's slots slot0 .. slot1 - 1 of `slots` (neighbouring ranges of it); before and
 // after each one's steps begin(slot) and end(slot, acc).
 template <int B, int NT8, typename Begin, typename End>
@@ -288,19 +309,7 @@ __device__ __forceinline__ void multiply_rows(int K, const SmallMember& W, int m
             ptx::named_barrier_sync(1 + half, 128);
             const uint32_t xs = read_at + (uint32_t)((b - b0) & 1) * kStep;
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {   // sixteen elements of the block
-                uint32_t o0[8], o1[8];
-                s0.expand16(c0.w, q, o0);
-                s1.expand16(c1.w, q, o1);
-#pragma unroll
-                for (int nt = 0; nt < NT8; ++nt) {
-                    const uint4 xl = ld_shared_v4((xs ^ (32u * q)) + (uint32_t)(nt * 8 * kSmallSpan * 2)), xh = ld_shared_v4((xs ^ (32u * q + 16u)) + (uint32_t)(nt * 8 * kSmallSpan * 2));
-                    mma_bf16(acc[nt], o0[0], o1[0], o0[1], o1[1], xl.x, xl.y);
-                    mma_bf16(acc[nt], o0[2], o1[2], o0[3], o1[3], xl.z, xl.w);
-                    mma_bf16(acc[nt], o0[4], o1[4], o0[5], o1[5], xh.x, xh.y);
-                    mma_bf16(acc[nt], o0[6], o1[6], o0[7], o1[7], xh.z, xh.w);
-                }
-            }
+            for (int q = 0; q < 4; ++q) multiply_16<B, NT8>(acc, s0, s1, c0, c1, q, xs);
             if (b + 2 < b1) ptx::named_barrier_sync(1 + half, 128);   // the tokens have been read: the buffer may be filled again
         }
         end(slot, acc);
@@ -436,6 +445,225 @@ __global__ void __launch_bounds__(kSmallThreads, 2) small_kernel(const __grid_co
     }
 }
 
+// ------------------------------------------------------------------------------------------------ several units of one weight
+// Token groups of several adapters on one weight, and groups of more than 32 tokens: a CTA takes 64 rows as above and one unit of up to 32 tokens,
+// and does all slices of the contraction.  No cluster, and every unit is as many eights of tokens wide as it has.  The halves of the warps take a
+// slot of every slice each; the second half hands its sums to the first one's threads, which hold the same places, add them up in the
+// order of the other two forms - a group's result does not depend on its company, nor on the kernel - and store them.
+// The CTAs go out in the order of their length: rows of 4 bits first, and a weight's largest unit before its others.
+constexpr int kUnitTokens = 32;
+struct UnitOrder { uint8_t member[2 * kSmallMembers], first[2 * kSmallMembers]; };   // units: member, and its first token in units
+
+__device__ __forceinline__ void barrier_arrive(int id, int threads) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
+
+template <int B, int NT8, int NB>
+__device__ __forceinline__ void unit_rows(const SmallParams<NB>& P, const SmallMember& W, int m0, int p0, int p_end, int slices, unsigned char* smem) {
+    constexpr uint32_t kStep = 8u * NT8 * kSmallSpan * 2u;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, half = warp >> 2;
+    const int K = P.K, n_span = (K + kSmallSpan - 1) / kSmallSpan, nb = K / kBlock, slots = 2 * slices;
+    auto bound = [&](int slot) { return (int)((long long)slot * n_span / slots); };
+    const bool live0 = p0 + g < p_end, live1 = p0 + g + 8 < p_end;
+    const int q0 = live0 ? p0 + g : p_end - 1, q1 = live1 ? p0 + g + 8 : p_end - 1;
+    const int r0 = __ldg(W.L.perm + q0), r1 = __ldg(W.L.perm + q1);
+    const uint8_t* row0 = W.packed + packed_row_offset(W.L, B >> 1, q0, r0) + t * (8 * B);
+    const uint8_t* row1 = W.packed + packed_row_offset(W.L, B >> 1, q1, r1) + t * (8 * B);
+    const float* am0 = W.absmax + (size_t)absmax_row_of(W.L, q0, r0) * nb + t;
+    const float* am1 = W.absmax + (size_t)absmax_row_of(W.L, q1, r1) * nb + t;
+    const float* y0 = W.maps + (size_t)r0 * kTableStride;
+    const float* y1 = W.maps + (size_t)r1 * kTableStride;
+    // tokens of a step: two buffers for either half of the warps; a warp to every fourth token, a lane to a 16-byte piece of its 512 bytes
+    const uint32_t x_smem = ptx::smem_u32(smem) + (uint32_t)half * 2u * kStep;
+    float* handed = reinterpret_cast<float*>(smem + 4u * kStep) + (threadIdx.x & 127);      // two buffers of [4 NT8][128 threads]
+    float* total = handed + 2 * (4 * NT8 * 128);                                            // the slices so far, likewise
+    const int warp4 = warp & 3, tokens = W.M - m0 - warp4;
+    const uint32_t stage_at = x_smem + token_piece(warp4, lane >> 3, lane & 7), read_at = x_smem + token_piece(g, t, 0);
+    const uint16_t* x_src = W.X + (size_t)(m0 + warp4) * K + lane * 8;
+    auto stage = [&](int b, uint32_t turn) {
+        const int k = b * kSmallSpan;
+        const bool in = k + lane * 8 < K;
+        const uint16_t* src = x_src + k;
+#pragma unroll
+        for (int i = 0; i < 2 * NT8; ++i) {
+            const bool valid = in && 4 * i < tokens;
+            cp_async_16_zfill(stage_at + turn * kStep + (uint32_t)(4 * i * kSmallSpan * 2), valid ? src + (size_t)(4 * i) * K : W.X, valid);
+        }
+    };
+    Codes<B> n0, n1;
+    auto fetch = [&](int b) {
+        const bool in = 4 * b + t < nb;
+        fetch_codes<B>(n0, row0, am0, 4 * b, live0 && in);
+        fetch_codes<B>(n1, row1, am1, 4 * b, live1 && in);
+    };
+    uint32_t raw[8];
+    auto fetch_up = [&](int step) {
+        const size_t N = (size_t)P.N, j = (size_t)(step * 16 + 2 * t) * N;
+        const uint16_t *u0 = W.B + r0 + j, *u1 = W.B + r1 + j;
+        raw[0] = __ldg(u0); raw[1] = __ldg(u0 + N); raw[2] = __ldg(u0 + 8 * N); raw[3] = __ldg(u0 + 9 * N);
+        raw[4] = __ldg(u1); raw[5] = __ldg(u1 + N); raw[6] = __ldg(u1 + 8 * N); raw[7] = __ldg(u1 + 9 * N);
+    };
+    float ya[1 << B], yb[1 << B];
+    if (B <= 2) {
+        load_levels<B>(ya, y0);
+        load_levels<B>(yb, y1);
+    }
+    uint32_t turn = 0u;
+    if (bound(half) < bound(half + 1)) {
+        fetch(bound(half));
+        stage(bound(half), 0u);
+    }
+    ptx::cp_async_commit();
+#pragma unroll 1
+    for (int slice = 0; slice < slices; ++slice) {
+        const int slot = 2 * slice + half, b1 = bound(slot + 1), after = slice + 1 < slices ? bound(slot + 2) : -1;
+        float acc[NT8][4];
+#pragma unroll
+        for (int i = 0; i < NT8; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.0f;
+        if (slot * 16 < P.r) fetch_up(slot);
+#pragma unroll 1
+        for (int b = bound(slot); b < b1; ++b) {
+            ptx::cp_async_wait<0>();
+            ptx::named_barrier_sync(1 + half, 128);      // the step's tokens are there, those of the step before have been read
+            const int next = b + 1 < b1 ? b + 1 : after;
+            const Codes<B> c0 = n0, c1 = n1;
+            if (next >= 0) {
+                stage(next, turn ^ 1u);
+                fetch(next);
+            }
+            ptx::cp_async_commit();
+            Scaled<B> s0, s1;
+            if (B == 4) {   // (sixteen levels of two rows are too many registers to keep: read again, from L1)
+                load_levels<B>(ya, y0);
+                s0.set(ya, c0.a);
+                load_levels<B>(ya, y1);
+                s1.set(ya, c1.a);
+            } else {
+                s0.set(ya, c0.a);
+                s1.set(yb, c1.a);
+            }
+            const uint32_t xs = read_at + turn * kStep;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) multiply_16<B, NT8>(acc, s0, s1, c0, c1, q, xs);
+            turn ^= 1u;
+        }
+        asm volatile("griddepcontrol.wait;" ::: "memory");               // T is in place
+        for (int i = slot; i * 16 < P.r; i += slots) {
+            if (i != slot) fetch_up(i);
+            const uint32_t a0 = raw[0] | (raw[1] << 16), a1 = raw[4] | (raw[5] << 16), a2 = raw[2] | (raw[3] << 16), a3 = raw[6] | (raw[7] << 16);
+#pragma unroll
+            for (int nt = 0; nt < NT8; ++nt) {
+                const int m = m0 + nt * 8 + g;
+                uint32_t t0 = 0u, t1 = 0u;
+                if (m < W.M) {
+                    const uint32_t* tr = reinterpret_cast<const uint32_t*>(W.T + (size_t)m * P.rp + i * 16) + t;
+                    t0 = __ldcg(tr);
+                    t1 = __ldcg(tr + 4);
+                }
+                mma_bf16(acc[nt], a0, a1, a2, a3, t0, t1);
+            }
+        }
+        // the slice's two sums: buffer slice mod 2 full (barriers 3, 4), and read (5, 6)
+        float* at = handed + (slice & 1) * (4 * NT8 * 128);
+        if (half == 1) {
+            if (slice >= 2) ptx::named_barrier_sync(5 + (slice & 1), 256);
+#pragma unroll
+            for (int i = 0; i < 4 * NT8; ++i) at[i * 128] = acc[i >> 2][i & 3];
+            barrier_arrive(3 + (slice & 1), 256);
+        } else {
+            ptx::named_barrier_sync(3 + (slice & 1), 256);
+#pragma unroll
+            for (int i = 0; i < 4 * NT8; ++i) acc[i >> 2][i & 3] = (slice > 0 ? total[i * 128] : 0.0f) + (acc[i >> 2][i & 3] + at[i * 128]);
+            if (slice + 2 < slices) barrier_arrive(5 + (slice & 1), 256);
+            if (slice + 1 < slices) {
+#pragma unroll
+                for (int i = 0; i < 4 * NT8; ++i) total[i * 128] = acc[i >> 2][i & 3];
+                continue;
+            }
+#pragma unroll
+            for (int nt = 0; nt < NT8; ++nt) {
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const int m = m0 + nt * 8 + 2 * t + e;
+                    if (m >= W.M) continue;
+                    if (live0) W.Y[(size_t)m * P.N + r0] = (uint16_t)pack_bf16x2(acc[nt][e], 0.0f);
+                    if (live1) W.Y[(size_t)m * P.N + r1] = (uint16_t)pack_bf16x2(acc[nt][2 + e], 0.0f);
+                }
+            }
+        }
+    }
+}
+
+// Grid: (units, row groups).
+template <int NB>
+__global__ void __launch_bounds__(kSmallThreads, 2) units_kernel(const __grid_constant__ SmallParams<NB> P, const __grid_constant__ UnitOrder order, const int slices) {
+    extern __shared__ __align__(128) unsigned char small_smem[];
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const SmallMember& W = P.m[order.member[blockIdx.x]];
+    const int m0 = order.first[blockIdx.x] * kUnitTokens;
+    int grp = (int)(gridDim.y - 1 - blockIdx.y), c = 0;
+    for (; c < 2; ++c) {
+        const int n = (W.L.class_start[c + 1] - W.L.class_start[c] + kSmallRows - 1) / kSmallRows;
+        if (grp < n) break;
+        grp -= n;
+    }
+    const int p0 = W.L.class_start[c] + grp * kSmallRows + (int)((threadIdx.x >> 5) & 3) * 16, p_end = W.L.class_start[c + 1];
+    const int tokens = W.M - m0;
+    auto work = [&](auto bits) {
+        constexpr int B = decltype(bits)::value;
+        if (tokens <= 8) unit_rows<B, 1, NB>(P, W, m0, p0, p_end, slices, small_smem);
+        else if (tokens <= 16) unit_rows<B, 2, NB>(P, W, m0, p0, p_end, slices, small_smem);
+        else if (tokens <= 24) unit_rows<B, 3, NB>(P, W, m0, p0, p_end, slices, small_smem);
+        else unit_rows<B, 4, NB>(P, W, m0, p0, p_end, slices, small_smem);
+    };
+    if (c == 0) work(std::integral_constant<int, 1>());
+    else if (c == 1) work(std::integral_constant<int, 2>());
+    else work(std::integral_constant<int, 4>());
+}
+
+// Whether a CTA for every group of 64 rows and unit beats one for every slice of it.  Both in microseconds, two CTAs to an SM: of the former 3 and
+// 1.2 for every slice, of the latter 5.5; and 2 (1, 2 bits) to 2.6 (4 bits) for a step.  The long ones leave SMs idle at the end, more so where all
+// are alike.  (Against the slices, us: 4096 x 4096 at 30/50/20 %, 101 tokens in 6 groups 66.0 -> 48.6, 64 in 8 72 -> 46, 60 in 3 34.4 -> 29.9, 16 in
+// 8 48.5 -> 38.7; at 4 bits 101 in 6 66.4 -> 55.4.  Not taken: 4 in 2 there 19.3 -> 19.8, 64 in one 26.9 -> 31.5; 4096 x 11008 of 4 bits 60 in 3 71 -> 83.)
+template <int NB>
+bool units_pay(const SmallParams<NB>& P, int groups, int slices) {
+    int units = 0;
+    for (int i = 0; i < P.count; ++i) units += (P.m[i].M + kUnitTokens - 1) / kUnitTokens;
+    if (units < 2) return false;
+    const int* start = P.m[0].L.class_start;
+    const bool alike = start[1] == P.N || (start[1] == 0 && start[2] == P.N) || start[2] == 0;
+    const float step = 2.0f + 0.6f * (float)(start[3] - start[2]) / (float)P.N, steps = 0.5f * (float)((P.K + kSmallSpan - 1) / kSmallSpan);
+    const float waves = (float)(groups * units) / (2 * kNumSMs), spread = waves * slices, whole = waves + (alike ? 0.35f : 0.15f);
+    return (whole > 1.0f ? whole : 1.0f) * (3.0f + 1.2f * slices + step * steps) < (spread > 1.0f ? spread : 1.0f) * (5.5f + step * steps / slices);
+}
+
+template <int NB>
+lowra_status launch_units(const SmallParams<NB>& P, int groups, int slices, cudaStream_t stream) {
+    UnitOrder order;
+    int units = 0, widest = 1;
+    for (int size = kUnitTokens; size > 0; size -= 8)          // 32 to 25 tokens first
+        for (int i = 0; i < P.count; ++i)
+            for (int u = 0; u * kUnitTokens < P.m[i].M; ++u) {
+                const int left = P.m[i].M - u * kUnitTokens, n = left < kUnitTokens ? left : kUnitTokens;
+                if (n > size || n <= size - 8) continue;
+                order.member[units] = (uint8_t)i;
+                order.first[units++] = (uint8_t)u;
+                widest = (n + 7) / 8 > widest ? (n + 7) / 8 : widest;
+            }
+    const size_t smem = 4u * (8 * widest) * kSmallSpan * 2u + 3u * 4 * widest * 128 * 4u;
+    static SmemLimit limit = {};
+    if (ensure_smem_limit(reinterpret_cast<const void*>(units_kernel<NB>), smem, &limit) != LOWRA_OK) return LOWRA_ERR_CUDA;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3((unsigned)units, (unsigned)groups, 1);
+    cfg.blockDim = dim3(kSmallThreads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, units_kernel<NB>, P, order, slices) == cudaSuccess ? LOWRA_OK : LOWRA_ERR_CUDA;
+}
+
 template <int NT8, int NB, bool MERGED>
 lowra_status launch_product(const SmallParams<NB>& P, int groups, int units, int slices, cudaStream_t stream) {
     const size_t smem = 4u * (8 * NT8) * kSmallSpan * 2u + (MERGED ? (2 + slices / 2) * (8 * NT8) * kMergedPitch * 4u : 2u * (8 * NT8) * kSmallRows * 4u);
@@ -501,6 +729,7 @@ lowra_status launch_members(const SmallParams<NB>& P, cudaStream_t stream) {
     // a step of 256.  The choice depends on the weight's shape alone, so that a member's result does not depend on its company.
     const int n_span = (P.K + kSmallSpan - 1) / kSmallSpan, slices = product_slices(P.N, P.K);
     const int nt8 = most <= 8 ? 1 : most <= 16 ? 2 : most <= 24 ? 3 : 4;
+    if (P.one_weight && units_pay(P, groups, slices)) return launch_units<NB>(P, groups, slices, stream);
     int units = 0;
     for (int i = 0; i < P.count; ++i) units += (P.m[i].M + 8 * nt8 - 1) / (8 * nt8);
     // Merged where a CTA's own cost outweighs its steps: slots of one or two steps, few tokens, more CTAs than run at a time.  (Groups of
@@ -534,7 +763,7 @@ lowra_status launch_small(const SmallParams<kSmallMembers>& P, cudaStream_t stre
     if (P.count > 1) return launch_members<kSmallMembers>(P, stream);
     SmallParams<1> Q;
     Q.m[0] = P.m[0];
-    Q.count = 1; Q.N = P.N; Q.K = P.K; Q.r = P.r; Q.rp = P.rp; Q.s = P.s; Q.status = P.status; Q.clear_status = P.clear_status;
+    Q.count = 1; Q.N = P.N; Q.K = P.K; Q.r = P.r; Q.rp = P.rp; Q.s = P.s; Q.status = P.status; Q.clear_status = P.clear_status; Q.one_weight = P.one_weight;
     return launch_members<1>(Q, stream);
 }
 
