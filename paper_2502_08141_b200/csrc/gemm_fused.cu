@@ -44,9 +44,14 @@ namespace {
 
 constexpr uint64_t kGraceNs = 50ull * 1000ull;   // after a failure: time for copies and MMAs still in flight to land
 constexpr int kMinRange = 12;                    // schedule (plan_schedule): the shortest range of contraction blocks
+constexpr int kMinShare = 8;                     // and a cluster's share of a T tile of two such ranges or more
+constexpr int kTFlags = 8;                       // "T ready" flags of a CTA and token tile whose T is shared out
 // Collecting partial tiles: they come in pieces of 32 rows x 128 tokens (16 KB, a ring entry), two rows' worth of pieces - one for
 // either warp of a lane quarter - from every contributor per step.
 constexpr int kPartSlots = kSlotsX + kSlotsW, kMaxContributors = kPartSlots / 2, kPartSteps = kPartSlots / 2;
+// Where they start among the header's flags, behind those of the partial tiles: 32-byte aligned, for they are read together.
+constexpr int kSharedTFlags = (kMaxClusters * kCluster + 7) / 8 * 8;
+static_assert(kMaxContributors <= kTFlags, "a flag for every cluster that shares a T tile");
 constexpr int kRankCols = 128;                   // columns of a T tile: the ranks, padded
 constexpr uint32_t kIdesc = ptx::umma_idesc_bf16(kHalfT, kPairR), kIdescT = ptx::umma_idesc_bf16(kHalfT, kRankCols);
 constexpr uint32_t kIdescBmn = 1u << 16;         // operand B MN-major
@@ -151,11 +156,13 @@ struct Seg {
     int m0;        // the token tile's first token
     int nh;        // halves of the token tile that hold tokens
     int kb0, kb1;  // contraction blocks [kb0, kb1) of the tile
+    int shares;    // > 1: this cluster and its neighbours hold a slice of the tile each, and each of them finishes a share of it
     int tile;      // weight tile index (ranges)
 };
 
-// NB: members the kernel's parameters have room for (1: the plain calls; kMaxBatch: the batch calls).
-template <int MODE, int NB>
+// NB: members the kernel's parameters have room for (1: the plain calls; kMaxBatch: the batch calls).  SHARED: with tiles that several clusters
+// share (t_split or w_split above one), which long calls have none of: their loops pay for the code (512-token tiles by 1.5 to 2 % in the forward pass).
+template <int MODE, int NB, bool SHARED>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 fused_kernel(const __grid_constant__ KParams<NB> P, const __grid_constant__ KMaps<NB> TM) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -203,7 +210,7 @@ fused_kernel(const __grid_constant__ KParams<NB> P, const __grid_constant__ KMap
     const bool sk = MODE != kModeDense && P.sk != 0;
     // Short calls (t_split > 1): the T tiles are what everybody would wait for, so every one of them is cut as well, between
     // the first clusters, and the weight tiles' ranges belong to the others.
-    const int t_cl = MODE != kModeDense && P.t_split > 1 ? n_t_tiles * P.t_split : 0;
+    const int t_cl = SHARED && P.t_split > 1 ? n_t_tiles * P.t_split : 0;
     const int n_whole = sk ? n_t_tiles + P.sk_first : n_t_tiles + P.tiles_r * super_t;   // pieces dealt round-robin
     const int w_whole = t_cl > 0 ? (cid < t_cl ? 1 : 0) : n_whole > cid ? (n_whole - cid + NC - 1) / NC : 0;   // this cluster's
     auto sk_lo = [&](int c) -> int {   // where cluster c's range starts (the launcher keeps the products below 2^31)
@@ -220,6 +227,7 @@ fused_kernel(const __grid_constant__ KParams<NB> P, const __grid_constant__ KMap
         Seg t;
         t.part = t.pre = false;
         t.tile = 0;
+        t.shares = 1;
         if (i < w_whole) {
             const int g = cid + i * NC;
             t.kb0 = 0; t.kb1 = P.main_blocks;
@@ -228,7 +236,7 @@ fused_kernel(const __grid_constant__ KParams<NB> P, const __grid_constant__ KMap
                 member_of(cid / P.t_split, t);
                 t.is_t = true; t.lora = false; t.rt = 0;
                 t.kb0 = P.main_blocks * slice / P.t_split; t.kb1 = P.main_blocks * (slice + 1) / P.t_split;
-                t.part = slice > 0; t.pre = slice == 0;
+                t.shares = P.t_split;
             } else if (g < n_t_tiles) {
                 member_of(g, t);
                 t.is_t = true; t.lora = false; t.rt = 0;
@@ -250,19 +258,26 @@ fused_kernel(const __grid_constant__ KParams<NB> P, const __grid_constant__ KMap
             member_of(gst, t);
             t.is_t = false; t.rt = idx - gst * P.tiles_r;
             t.lora = p0 == 0;
-            t.part = p0 > 0;
-            t.pre = p0 == 0 && p1 < B;
+            if (SHARED && P.w_split > 1) {
+                t.shares = P.w_split;
+            } else {
+                t.part = p0 > 0;
+                t.pre = p0 == 0 && p1 < B;
+            }
         }
         return t;
     };
     // the clusters cid + 1 .. c_end - 1 hold the rest of the tile that this cluster's last piece starts
     auto contributors_end = [&](const Seg& t) {
-        if (t.is_t) return cid + P.t_split;
         const int tile_end = (t.tile + 1) * B;
         int c_end = cid + 1;
         while (c_end < NC && sk_lo(c_end) < tile_end) ++c_end;
         return c_end;
     };
+    // Pieces of a shared tile, 32 columns of a weight tile, 16 of a T tile: cluster k of S finishes those numbered k, k + S, ...; so the first
+    // t_finishers clusters of a shared T tile have some, and raise a flag each.
+    auto t_finishers = [&](const Seg& t) { return SHARED && P.t_split > 1 ? min(P.t_split, t.nh * (P.rp / 16)) : 1; };
+    auto t_flags_of = [&](const Seg& t) { return P.mem[t.prob].flags + (t.mt * CL + (int)crank) * (SHARED && P.t_split > 1 ? kTFlags : 1); };
     // How many stages, from stage st of a piece's n, are worked on half by half before the next ones: see kSkew.
     auto run_of = [&](const Seg& t, int st, int n) { return (t.nh == 2 && (st == 0 || n - st <= kSkew)) ? min(kSkew, n - st) : 1; };
 
@@ -330,9 +345,11 @@ fused_kernel(const __grid_constant__ KParams<NB> P, const __grid_constant__ KMap
                         const bool lora = u >= n_main;
                         const bool w = h == 0 && (lora || w_main);
                         if (lora && !t_ready) {
-                            // T of these tokens is written by the CTA of the same rank in another cluster: wait for its
-                            // flag, then make those generic-proxy writes visible to the TMA (async proxy) reads below
-                            const bool up = ptx::flag_wait(P.mem[t.prob].flags + t.mt * CL + (int)crank, want, abort_flag, wait_ns);
+                            // T of these tokens is written by the CTAs of the same rank in other clusters: wait for their
+                            // flags, then make those generic-proxy writes visible to the TMA (async proxy) reads below
+                            const int n_flags = t_finishers(t);
+                            const bool up = n_flags > 1 ? ptx::flags_wait(t_flags_of(t), n_flags, want, abort_flag, wait_ns)
+                                                        : ptx::flag_wait(t_flags_of(t), want, abort_flag, wait_ns);
                             if (!__all_sync(0xffffffffu, up)) { failed = true; break; }
                             ptx::fence_proxy_async_all();
                             t_ready = true;
@@ -500,7 +517,8 @@ fused_kernel(const __grid_constant__ KParams<NB> P, const __grid_constant__ KMap
             const int cols = t.is_t ? P.rp : min(kPairR, P.R - r0);   // rows of the tile that exist
             // the columns c0, c0 + 32, ... that this warp takes: half of the tile's; a T tile has few
             const int c_first = t.is_t ? ch * 32 : ch * 128, c_step = t.is_t ? 64 : 32, c_last = t.is_t ? cols : min(cols, ch * 128 + 128);
-            float* part = P.sk_part + ((size_t)cid * CL + crank) * kSkHalfFloats + my_tok;
+            auto part_of = [&](int c) { return P.sk_part + ((size_t)(SHARED && c == 0 ? P.sk_slot0 : c) * CL + crank) * kSkHalfFloats; };   // cluster c's place
+            float* const part = part_of(cid) + my_tok;
             // 32 rows of one token: rounded and stored
             auto put = [&](uint16_t* dst, int left, uint32_t (&v)[32]) {
 #pragma unroll
@@ -518,26 +536,120 @@ fused_kernel(const __grid_constant__ KParams<NB> P, const __grid_constant__ KMap
                         if (j < left) dst[j] = (uint16_t)(v[j >> 1] >> (16 * (j & 1)));
                 }
             };
-            // publish this CTA's tokens of T, resp. its half of the cluster's partial tile: every writer fences, then one
-            // thread raises the flag
+            // publish this CTA's tokens of T, resp. its half of the cluster's partial tile: the writers meet, and one thread's
+            // release covers what all of them have written
             auto raise = [&](uint32_t* flag, bool withheld) {
-                __threadfence();
                 ptx::named_barrier_sync(1, kThreads);
                 if (et == 0) {
                     ptx::fence_proxy_async_all();
                     if (!withheld) ptx::flag_release(flag, want);
                 }
             };
-            uint32_t* const t_flag = MODE == kModeDense ? nullptr : P.mem[t.prob].flags + t.mt * CL + (int)crank;
             const bool drop = P.diag_drop_t_flags != 0;     // (diagnostic: the waits for T run out)
-            // 32 ranks of one token of T, scaled by s
-            auto put_t = [&](int tok, int c0, uint32_t (&v)[32]) {
+            // the first ranks of one token of T among v (16 or 32), scaled by s
+            auto put_t = [&](int tok, int c0, int ranks, uint32_t (&v)[32]) {
                 uint16_t* dst = P.mem[t.prob].T + (size_t)tok * P.rp + c0;
 #pragma unroll
                 for (int j = 0; j < 16; ++j) v[j] = pack_bf16x2(P.s * __uint_as_float(v[2 * j]), P.s * __uint_as_float(v[2 * j + 1]));
 #pragma unroll
-                for (int j = 0; j < 4; ++j) *reinterpret_cast<uint4*>(dst + 8 * j) = make_uint4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+                for (int j = 0; j < 4; ++j)
+                    if (8 * j < ranks) *reinterpret_cast<uint4*>(dst + 8 * j) = make_uint4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
             };
+            if (SHARED && t.shares > 1) {
+                // Every cluster of a few consecutive ones has a slice of this tile, and no other piece.  Either CTA's part of the tile is
+                // pieces of 32 columns (a T tile: 16) x 128 tokens; cluster k of S finishes those numbered k, k + S, ...: the others' sums of them
+                // come through the scratch and the operand ring, idle by now, and are added to its own in the order of the slices.
+                // What bounds it: two trips through L2 with a flag (3 us) and the SM's L2 port; with S = 4 a CTA writes 96 KB and reads 96 for every
+                // 256 tokens, where the cluster of the first slice alone read 384 and the others wrote 128.  (4096 x 4096 at 128 tokens, S = 4 and T between
+                // seven: 28.7 -> 26.0 us.)
+                const int S = t.shares, k = t.is_t ? cid % S : (cid - P.sk_c0) % S, first = cid - k;
+                const int width = t.is_t ? 16 : 32, per_half = (cols + width - 1) / width, pieces = t.nh * per_half;
+                for (int h = 0; h < t.nh; ++h) {
+                    const uint32_t acc = (hc + (uint32_t)h) & 1u;
+                    if (!ptx::mbar_wait_warp(&bars->tmem_full[acc], ((hc + (uint32_t)h) >> 1) & 1u, abort_flag, wait_ns)) bars->abort = 1u;
+                    if (agree_abort()) { failed = true; break; }
+                    ptx::tc_fence_after();
+                    if (t.m0 + h * kHalfT + (int)crank * 128 + my_tok - lane >= M) continue;      // (nobody in this warp has a token)
+#pragma unroll 1
+                    for (int c0 = c_first; c0 < c_last; c0 += c_step) {
+                        const int u = h * per_half + c0 / width;
+                        const bool lower = u % S != k, upper = (t.is_t ? u + 1 : u) % S != k;      // sixteen columns each
+                        if (!lower && !upper) continue;
+                        uint32_t v[32];
+                        ptx::tmem_ld_32x32(tmem_lane + acc * (uint32_t)kPairR + (uint32_t)c0, v);
+                        ptx::tmem_ld_wait();
+                        float* to = part + (size_t)h * kSkAllFloats + (size_t)c0 * 128;
+                        if (lower) {
+#pragma unroll
+                            for (int j = 0; j < 16; ++j) __stcg(to + j * 128, __uint_as_float(v[j]));
+                        }
+                        if (upper) {
+#pragma unroll
+                            for (int j = 16; j < 32; ++j) __stcg(to + j * 128, __uint_as_float(v[j]));
+                        }
+                    }
+                }
+                if (failed) break;
+                raise(P.sk_flags + cid * CL + (int)crank, false);
+                const int mine = k < pieces ? (pieces - k + S - 1) / S : 0;
+                if (t.m0 + (int)crank * 128 < M && mine > 0) {            // (a CTA without tokens has nothing to finish)
+                    if (lane < S && !ptx::flag_wait(P.sk_flags + (first + lane) * CL + (int)crank, want, abort_flag, wait_ns)) bars->abort = 1u;
+                    if (agree_abort()) { failed = true; break; }
+                    // a step: two pieces, one for either warp of a lane quarter, from every other cluster
+                    const int steps = (mine + 1) / 2, ahead = min(kPartSlots / (2 * (S - 1)), kPartSteps);
+                    auto fetch = [&](int st) {      // one thread
+                        if (st >= steps) return;
+                        uint64_t* bar = &bars->part_full[st % kPartSteps];
+                        const int wide = min(2, mine - 2 * st);
+                        ptx::mbar_arrive_expect_tx(bar, (uint32_t)(wide * (S - 1) * width) * 512u);
+                        for (int w = 0; w < wide; ++w) {
+                            const int u = k + (2 * st + w) * S, h = u / per_half, c0 = (u - h * per_half) * width;
+                            uint32_t to = ptx::smem_u32(x_ring) + (uint32_t)(((st % ahead) * 2 + w) * (S - 1)) * kSmemSlot;
+                            for (int c = 0; c < S; ++c) {
+                                if (c == k) continue;
+                                ptx::bulk_copy_g2s(to, part_of(first + c) + (size_t)h * kSkAllFloats + (size_t)c0 * 128, (uint32_t)width * 512u, bar);
+                                to += kSmemSlot;
+                            }
+                        }
+                    };
+                    if (et < 32) {                  // (as for the other cut tiles, below)
+                        ptx::fence_proxy_async_all();
+                        __syncwarp();
+                        if (et == 0)
+                            for (int st = 0; st < ahead; ++st) fetch(st);
+                    }
+                    for (int st = 0; st < steps && !failed; ++st) {
+                        if (!ptx::mbar_wait_warp(&bars->part_full[st % kPartSteps], (uint32_t)(st / kPartSteps) & 1u, abort_flag, wait_ns)) bars->abort = 1u;
+                        if (2 * st + ch < mine) {
+                            const int u = k + (2 * st + ch) * S, h = u / per_half, c0 = (u - h * per_half) * width;
+                            const int tok = t.m0 + h * kHalfT + (int)crank * 128 + my_tok;
+                            const float* ring = reinterpret_cast<const float*>(x_ring) + (size_t)(((st % ahead) * 2 + ch) * (S - 1)) * (kSmemSlot / 4) + my_tok;
+                            uint32_t v[32];
+                            ptx::tmem_ld_32x32(tmem_lane + ((hc + (uint32_t)h) & 1u) * (uint32_t)kPairR + (uint32_t)c0, v);
+                            ptx::tmem_ld_wait();
+                            for (int c = 1; c < S; ++c, ring += kSmemSlot / 4) {
+#pragma unroll
+                                for (int j = 0; j < 16; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) + ring[j * 128]);
+                                if (width == 32) {
+#pragma unroll
+                                    for (int j = 16; j < 32; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) + ring[j * 128]);
+                                }
+                            }
+                            if (tok < M) {
+                                if (t.is_t) put_t(tok, c0, 16, v);
+                                else put(P.mem[t.prob].out + (size_t)tok * P.ld_out + r0 + c0, cols - c0, v);
+                            }
+                        }
+                        if (st + ahead < steps) {
+                            if (agree_abort()) { failed = true; break; }     // everybody has read the step's pieces: their place is filled again
+                            if (et == 0) fetch(st + ahead);
+                        }
+                    }
+                    if (!failed && agree_abort()) failed = true;
+                }
+                if (t.is_t && !failed && mine > 0) raise(t_flags_of(t) + k, drop);
+                break;                          // (the only piece)
+            }
             if (t.pre) {
                 // A piece that starts a tile which other clusters finish: their partial tiles are added here.  The piece is
                 // this cluster's last one; once its MMAs are complete the operand ring is idle, and the partial tiles are
@@ -550,17 +662,14 @@ fused_kernel(const __grid_constant__ KParams<NB> P, const __grid_constant__ KMap
                 if (lane < nc && !ptx::flag_wait(P.sk_flags + (cid + 1 + lane) * CL + (int)crank, want, abort_flag, wait_ns)) bars->abort = 1u;
                 if (agree_abort()) { failed = true; break; }
                 ptx::tc_fence_after();
-                const int per_half = t.is_t ? cols / 32 : 4, steps = t.nh * per_half;
-                const int wide = t.is_t ? 1 : 2;          // column halves per step: both, but a T tile's all lie in the first
-                const int pieces = wide * nc, ahead = min(kPartSlots / pieces, kPartSteps);
+                const int steps = 4 * t.nh, pieces = 2 * nc, ahead = min(kPartSlots / pieces, kPartSteps);
                 auto fetch = [&](int s) {       // one thread
                     if (s >= steps) return;
                     uint64_t* bar = &bars->part_full[s % kPartSteps];
-                    const int h = s / per_half, c0 = (s - h * per_half) * 32;
+                    const int h = s / 4, c0 = (s & 3) * 32;
                     ptx::mbar_arrive_expect_tx(bar, (uint32_t)pieces * kSmemSlot);
                     for (int k = 0; k < pieces; ++k) {
-                        const float* src = P.sk_part + ((size_t)(cid + 1 + k / wide) * CL + crank) * kSkHalfFloats +
-                                           (size_t)h * kSkAllFloats + (size_t)((k % wide) * 128 + c0) * 128;
+                        const float* src = part_of(cid + 1 + k / 2) + (size_t)h * kSkAllFloats + (size_t)((k % 2) * 128 + c0) * 128;
                         ptx::bulk_copy_g2s(ptx::smem_u32(x_ring) + (uint32_t)((s % ahead) * pieces + k) * kSmemSlot, src, kSmemSlot, bar);
                     }
                 };
@@ -573,30 +682,24 @@ fused_kernel(const __grid_constant__ KParams<NB> P, const __grid_constant__ KMap
                         for (int s = 0; s < ahead; ++s) fetch(s);
                 }
                 for (int s = 0; s < steps && !failed; ++s) {
-                    const int h = s / per_half, c0 = (t.is_t ? 0 : ch * 128) + (s - h * per_half) * 32;
+                    const int h = s / 4, c0 = ch * 128 + (s & 3) * 32;
                     const int tok = t.m0 + h * kHalfT + (int)crank * 128 + my_tok;
                     if (!ptx::mbar_wait_warp(&bars->part_full[s % kPartSteps], (uint32_t)(s / kPartSteps) & 1u, abort_flag, wait_ns)) bars->abort = 1u;
-                    if (ch < wide) {
-                        uint32_t v[32];
-                        ptx::tmem_ld_32x32(tmem_lane + ((hc + (uint32_t)h) & 1u) * (uint32_t)kPairR + (uint32_t)c0, v);
-                        ptx::tmem_ld_wait();
-                        const float* ring = reinterpret_cast<const float*>(x_ring) + (size_t)((s % ahead) * pieces + ch) * (kSmemSlot / 4) + my_tok;
-                        for (int c = 0; c < nc; ++c) {
+                    uint32_t v[32];
+                    ptx::tmem_ld_32x32(tmem_lane + ((hc + (uint32_t)h) & 1u) * (uint32_t)kPairR + (uint32_t)c0, v);
+                    ptx::tmem_ld_wait();
+                    const float* ring = reinterpret_cast<const float*>(x_ring) + (size_t)((s % ahead) * pieces + ch) * (kSmemSlot / 4) + my_tok;
+                    for (int c = 0; c < nc; ++c) {
 #pragma unroll
-                            for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) + ring[(size_t)(c * wide) * (kSmemSlot / 4) + j * 128]);
-                        }
-                        if (tok < M) {
-                            if (t.is_t) put_t(tok, c0, v);
-                            else if (c0 < cols) put(P.mem[t.prob].out + (size_t)tok * P.ld_out + r0 + c0, cols - c0, v);
-                        }
+                        for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) + ring[(size_t)(2 * c) * (kSmemSlot / 4) + j * 128]);
                     }
+                    if (tok < M && c0 < cols) put(P.mem[t.prob].out + (size_t)tok * P.ld_out + r0 + c0, cols - c0, v);
                     if (s + ahead < steps) {
                         if (agree_abort()) { failed = true; break; }     // everybody has read the step's pieces: their place is filled again
                         if (et == 0) fetch(s + ahead);
                     }
                 }
                 if (!failed && agree_abort()) failed = true;
-                if (t.is_t && !failed) raise(t_flag, drop);
                 break;                          // (the last piece; its accumulators are not handed on)
             }
             for (int h = 0; h < t.nh; ++h, ++hc) {
@@ -617,7 +720,7 @@ fused_kernel(const __grid_constant__ KParams<NB> P, const __grid_constant__ KMap
 #pragma unroll
                         for (int j = 0; j < 32; ++j) __stcg(part + (size_t)h * kSkAllFloats + (size_t)(c0 + j) * 128, __uint_as_float(v[j]));
                     } else if (tok < M) {
-                        if (t.is_t) put_t(tok, c0, v);
+                        if (t.is_t) put_t(tok, c0, 32, v);
                         else put(P.mem[t.prob].out + (size_t)tok * P.ld_out + r0 + c0, cols - c0, v);
                     }
                 }
@@ -625,7 +728,7 @@ fused_kernel(const __grid_constant__ KParams<NB> P, const __grid_constant__ KMap
             }
             if (failed) break;
             if (t.part) raise(P.sk_flags + cid * CL + (int)crank, false);
-            else if (t.is_t) raise(t_flag, drop);
+            else if (t.is_t) raise(t_flags_of(t), drop);
         }
     } else if (MODE != kModeDense) {
         // ================================================================== dequant producers
@@ -805,7 +908,7 @@ fused_kernel(const __grid_constant__ KParams<NB> P, const __grid_constant__ KMap
 //   drain the last accumulator; to collect partial tiles 4.5 and, per 256 tokens, four steps of 1.1 or 0.6 per contributor.
 static int plan_schedule(GemmParams& Q, bool may_cut, int max_clusters, float* estimate = nullptr) {
     const int blocks = Q.main_blocks + Q.lora_blocks;
-    struct Choice { float us; int halves, clusters, cut, first, c0, extra, t_split, num; } best = {};
+    struct Choice { float us; int halves, clusters, cut, first, c0, extra, t_split, num, w_split; } best = {};
     best.us = -1.0f;
     auto tiles_of = [&](int halves) {
         int n = 0;
@@ -820,28 +923,29 @@ static int plan_schedule(GemmParams& Q, bool may_cut, int max_clusters, float* e
         const float ramp = 4.5f, drain = 2.4f * halves;
         auto collect = [&](int nc) { return 4.5f + 4.0f * halves * (0.6f * nc > 1.1f ? 0.6f * nc : 1.1f); };
         const int super_t = tiles_of(halves), n_t = may_cut ? super_t : 0, n_w = Q.tiles_r * super_t, n = n_w + n_t;
-        const float t_us = ramp + t_pace * Q.main_blocks + 3.0f;               // when whole T tiles are there
+        // when whole T tiles are there (256 tokens: device timestamps of 1800 x 2304, 777 tokens)
+        const float t_us = halves == 1 ? 8.2f + 0.4f * Q.main_blocks : ramp + t_pace * Q.main_blocks + 3.0f;
+        auto short_us = [&](float n) { return 5.0f + (halves == 1 ? 0.52f : 0.8f) * n; };      // MMAs of a cluster's only piece
         {   // whole tiles
             const int clusters = n < max_clusters ? n : max_clusters, rows = (n + clusters - 1) / clusters;
-            const float w_us = ramp + pace * blocks * rows;
-            offer({(rows == 1 && n_t > 0 && t_us > w_us ? t_us : w_us) + drain, halves, clusters, 0, 0, 0, 0, 1, 0});
+            const float w_us = rows == 1 ? short_us(blocks) : ramp + pace * blocks * rows;
+            offer({(rows == 1 && n_t > 0 && t_us > w_us ? t_us : w_us) + drain, halves, clusters, 0, 0, 0, 0, 1, 0, 1});
         }
         if (!may_cut || halves > Q.part_halves || n_t > max_clusters || blocks < 2 * kMinRange) continue;
         if ((long long)n * blocks * max_clusters >= (1ll << 31)) continue;     // (32-bit arithmetic in the kernel)
-        // Fewer pieces than clusters: s clusters per weight tile, the clusters left over share the T tiles.  Short runs have estimates of
-        // their own: a shared T tile takes 0.3 per block and 7.5 + 0.5 per 256 tokens and contributor around them, a 256-token
-        // tile 0.55 per block, and collecting starts 3.2 later than at the end of a range, for the contributors end together.  (With the
-        // ranges' figures, which have T twice as late: 4096 x 4096, 256 tokens, weight tiles cut in two 41.4 us, in four 32.0.)
+        // Fewer pieces than clusters: s clusters share every weight tile, and those left over the T tiles.  From the end of a shared tile's MMAs to that of its
+        // stores it takes 4.5 and 3.5 for every 256 tokens; a shared T tile 0.42 per block, 9.2 around them and 1.5 for the low-rank blocks behind
+        // it, 1.5 more for its second half.
+        auto shared_t = [&](int ts) { return 10.7f + 1.5f * halves + 0.42f * Q.main_blocks / ts; };
         for (int s = 1; s < kMaxContributors && n_w * s + n_t <= max_clusters && blocks / s >= shortest; ++s) {
-            int ts = (max_clusters - n_w * s) / n_t;
+            int ts = ((max_clusters < kMaxClusters ? max_clusters : kMaxClusters - 1) - n_w * s) / n_t;     // (there are partial tiles for one cluster less)
             if (ts > kMaxContributors) ts = kMaxContributors;
-            if (ts > Q.main_blocks / kMinRange) ts = Q.main_blocks / kMinRange;
-            if (ts < 2) ts = 1;
+            if (ts > Q.main_blocks / kMinShare) ts = Q.main_blocks / kMinShare;
+            if (ts < 2 || Q.main_blocks < 2 * kMinRange) ts = 1;
             if (ts == 1 && s == 1) continue;
-            const float t_done = ts == 1 ? t_us : 7.5f + 0.3f * Q.main_blocks / ts + 0.5f * halves * ts;
-            const float w_done = ramp + (halves == 1 ? 0.55f : 0.8f) * blocks / s;
-            const float us = (t_done > w_done ? t_done : w_done) + (s == 1 ? drain : drain + collect(s - 1) + 3.2f);
-            offer({us, halves, n_t * ts + n_w * s, 1, 0, n_t * ts, 0, ts, n_w * blocks});
+            const float t_done = ts == 1 ? t_us : shared_t(ts), w_done = short_us((float)blocks / s);
+            const float us = (t_done > w_done ? t_done : w_done) + (s == 1 ? drain : 4.5f + 3.5f * halves);
+            offer({us, halves, n_t * ts + n_w * s, 1, 0, n_t * ts, 0, ts, n_w * blocks, s});
         }
         // T by clusters of its own, each tile by ts of them, and ranges over all weight tiles for the others: for few channels and many tokens, where one
         // piece in a few is a T tile that the others wait for, and for pieces that come out a little over a row (forward, us, against the
@@ -849,12 +953,12 @@ static int plan_schedule(GemmParams& Q, bool may_cut, int max_clusters, float* e
         // 6144 x 2048, 1500 tokens 54 -> 46).  Ranges of less than half a tile gain nothing (2048 x 4096, 600 tokens 30.4 -> 33.7); nor
         // does a choice that is ahead by less than a microsecond or so (1024 x 11008, 6000 tokens 140 -> 152).
         for (int ts = 1; ts <= kMaxContributors && n_t * ts < max_clusters; ++ts) {
-            if (ts > 1 && ts > Q.main_blocks / kMinRange) break;
+            if (ts > 1 && (ts > Q.main_blocks / kMinShare || Q.main_blocks < 2 * kMinRange)) break;
             const int c = max_clusters - n_t * ts;
             const float range = (float)n_w * blocks / c;
             if (range < shortest || 2.0f * range < blocks) continue;      // (longer with every ts)
-            const float t_done = ts == 1 ? t_us : 7.5f + 0.3f * Q.main_blocks / ts + 0.5f * halves * ts, w_done = ramp + pace * range;
-            offer({(t_done > w_done ? t_done : w_done) + drain + collect((int)((blocks + range - 1) / range)) + 1.5f, halves, max_clusters, 1, 0, n_t * ts, 0, ts, n_w * blocks});
+            const float t_done = ts == 1 ? t_us : shared_t(ts), w_done = ramp + pace * range;
+            offer({(t_done > w_done ? t_done : w_done) + drain + collect((int)((blocks + range - 1) / range)) + 1.5f, halves, max_clusters, 1, 0, n_t * ts, 0, ts, n_w * blocks, 1});
         }
         // Ranges for the last row of pieces, or for the last two.  The clusters' sweeps over the contraction fall out of step
         // inside the ranges, so the part of the token operand that is live there has to stay in L2 (ranges over all tiles of a
@@ -874,7 +978,7 @@ static int plan_schedule(GemmParams& Q, bool may_cut, int max_clusters, float* e
             if ((extra > 0 ? num / max_clusters - extra : num / max_clusters) < shortest) continue;
             const float range = (float)num / max_clusters;
             const int nc = (int)((blocks + range - 1) / range);                  // contributors of a tile, about
-            offer({ramp + pace * (whole * blocks + range) + collect(nc), halves, max_clusters, 1, first, 0, extra, 1, (int)num});
+            offer({ramp + pace * (whole * blocks + range) + collect(nc), halves, max_clusters, 1, first, 0, extra, 1, (int)num, 1});
         }
     }
     Q.halves = best.halves;
@@ -889,6 +993,8 @@ static int plan_schedule(GemmParams& Q, bool may_cut, int max_clusters, float* e
     Q.sk_extra = best.extra;
     Q.sk_num = best.num;
     Q.t_split = best.t_split;
+    Q.w_split = best.w_split;
+    Q.sk_slot0 = best.w_split > 1 ? best.clusters : best.c0;
     if (estimate != nullptr) *estimate = best.us;
     return best.clusters;
 }
@@ -913,13 +1019,36 @@ float fused_estimate(int N, int K, int M, int r, bool mixed, int count) {
     return us * (float)((count + kMaxBatch - 1) / kMaxBatch);
 }
 
-template <int MODE, int NB>
-static lowra_status launch_mode(const GemmParams& G, const BatchMaps& TM, cudaStream_t stream) {
+// How many clusters can be resident at once, and that the kernel may have its shared memory: once per kernel and device.
+template <int MODE, int NB, bool SHARED>
+static lowra_status prepare_fused(cudaLaunchConfig_t& cfg, int* max_clusters) {
     constexpr int CL = kCluster;
-    // per device: the kernel attribute has been set there, and so many clusters can be resident at once
     static std::mutex mutex;
     static bool configured[kMaxDevices] = {false};
     static int max_clusters_of[kMaxDevices] = {0};
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return LOWRA_ERR_CUDA;
+    std::lock_guard<std::mutex> lock(mutex);
+    if (!configured[dev]) {
+        const int sms = device_sm_count();
+        if (sms < CL) return LOWRA_ERR_CUDA;
+        if (cudaFuncSetAttribute(fused_kernel<MODE, NB, SHARED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)kGemmSmemBytes) != cudaSuccess)
+            return LOWRA_ERR_CUDA;
+        // the persistent schedule needs every cluster of the grid resident (a tile waits for T of another)
+        cfg.gridDim = dim3(sms / CL * CL, 1, 1);
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, fused_kernel<MODE, NB, SHARED>, &cfg) != cudaSuccess || n < 1) return LOWRA_ERR_CUDA;
+        max_clusters_of[dev] = n < sms / CL ? n : sms / CL;
+        configured[dev] = true;
+    }
+    *max_clusters = max_clusters_of[dev];
+    return LOWRA_OK;
+}
+
+template <int MODE, int NB>
+static lowra_status launch_mode(const GemmParams& G, const BatchMaps& TM, cudaStream_t stream) {
+    constexpr int CL = kCluster;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -935,35 +1064,27 @@ static lowra_status launch_mode(const GemmParams& G, const BatchMaps& TM, cudaSt
     cfg.stream = stream;
     cfg.attrs = attr;
     cfg.numAttrs = (MODE == kModeDense) ? 1 : 2;
-    int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return LOWRA_ERR_CUDA;
     int max_clusters = 0;
-    {
-        std::lock_guard<std::mutex> lock(mutex);
-        if (!configured[dev]) {
-            const int sms = device_sm_count();
-            if (sms < CL) return LOWRA_ERR_CUDA;
-            if (cudaFuncSetAttribute(fused_kernel<MODE, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)kGemmSmemBytes) != cudaSuccess)
-                return LOWRA_ERR_CUDA;
-            // the persistent schedule needs every cluster of the grid resident (a tile waits for T of another)
-            cfg.gridDim = dim3(sms / CL * CL, 1, 1);
-            int n = 0;
-            if (cudaOccupancyMaxActiveClusters(&n, fused_kernel<MODE, NB>, &cfg) != cudaSuccess || n < 1) return LOWRA_ERR_CUDA;
-            max_clusters_of[dev] = n < sms / CL ? n : sms / CL;
-            configured[dev] = true;
-        }
-        max_clusters = max_clusters_of[dev];
+    lowra_status st = prepare_fused<MODE, NB, false>(cfg, &max_clusters);
+    if (st != LOWRA_OK) return st;
+    if (MODE != kModeDense) {
+        int n = 0;
+        if ((st = prepare_fused<MODE, NB, MODE != kModeDense>(cfg, &n)) != LOWRA_OK) return st;
+        max_clusters = n < max_clusters ? n : max_clusters;
     }
     GemmParams Q = G;
     const int clusters = plan_schedule(Q, MODE != kModeDense, max_clusters);
+    if (Q.t_split > 1)      // (at most 36 T tiles then: their flags fit into the header)
+        for (int i = 0; i < Q.count; ++i) Q.mem[i].flags = Q.flags + kSharedTFlags + Q.mem[i].st0 * CL * kTFlags;
     cfg.gridDim = dim3((unsigned)(clusters * CL), 1, 1);
     KParams<NB> QP;
     KMaps<NB> QM;
     static_cast<GemmCommon&>(QP) = static_cast<const GemmCommon&>(Q);
     for (int i = 0; i < NB; ++i) { QP.mem[i] = Q.mem[i]; QM.m[i] = TM.m[i]; }
-    if (cudaLaunchKernelEx(&cfg, fused_kernel<MODE, NB>, QP, QM) != cudaSuccess) return LOWRA_ERR_CUDA;
-    return LOWRA_OK;
+    const bool shared = Q.t_split > 1 || Q.w_split > 1;
+    const cudaError_t rc = shared ? cudaLaunchKernelEx(&cfg, fused_kernel<MODE, NB, MODE != kModeDense>, QP, QM)
+                                  : cudaLaunchKernelEx(&cfg, fused_kernel<MODE, NB, false>, QP, QM);
+    return rc == cudaSuccess ? LOWRA_OK : LOWRA_ERR_CUDA;
 }
 
 lowra_status launch_fused(int mode, const GemmParams& G, const BatchMaps& TM, cudaStream_t stream) {

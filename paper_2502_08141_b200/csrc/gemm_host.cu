@@ -31,6 +31,7 @@ constexpr size_t kExitsOffset = 128;   //   CTAs of the running call that have l
 constexpr size_t kFlagsOffset = kStatusBytes;
 constexpr size_t kHeaderBytes = 4096;  // status word, numbering, flags
 constexpr int kHeaderFlags = (int)((kHeaderBytes - kFlagsOffset) / 4), kSkFlags = kMaxClusters * kCluster;
+static_assert(kHeaderFlags % 4 == 0 && kSkFlags % 4 == 0, "cleared four at a time");
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
@@ -84,7 +85,7 @@ Workspace plan_workspace(int N, int K, const int* Ms, int count, int r, bool str
     }
     w.off_t_flags = in_header ? kFlagsOffset + kSkFlags * 4 : off;
     w.t_flag_bytes = in_header ? 0 : (size_t)flags * 4;
-    w.n_flags = kSkFlags + (in_header ? flags : 0);
+    w.n_flags = in_header ? kHeaderFlags : kSkFlags;      // (a shared T tile has a flag for every cluster that finishes some of it)
     w.off_items = off + align256(w.t_flag_bytes);
     // room for the deal of one direction, rebuilt by every call that brings none
     const size_t fwd = deal_forward_bytes(N), bwd = deal_backward_bytes(N);

@@ -113,7 +113,9 @@ struct GemmCommon {
     int part_halves;        // (host) halves of a token tile that the slots have room for: 2, or 1, or 0 (no tile is cut)
     uint32_t* sk_flags;     // [clusters][kCluster] raised when a CTA's partial tile is complete
     int halves;             // token tiles of 256 (1) or 512 tokens (2)
-    int t_split;            // > 1: every T tile is cut between so many clusters, which do nothing else
+    int t_split;            // > 1: so many clusters share a T tile, and do nothing else
+    int w_split;            // > 1: so many clusters share a weight tile, from cluster sk_c0 on, and do nothing else
+    int sk_slot0;           // whose place for partial tiles cluster 0 has
     int sk;
     int sk_c0;              // the first cluster that gets a range
     int sk_first;           // first weight tile of the ranges

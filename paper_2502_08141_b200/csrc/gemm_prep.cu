@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(kPrepThreads) prep_kernel(const PrepParams P) 
     if (blockIdx.x == 0) {
         if (threadIdx.x == 0 && P.status != nullptr) *P.status = 0u;   // null: keep what earlier launches recorded
         if (threadIdx.x == 0 && P.exits != nullptr) *P.exits = 0u;
-        for (int i = threadIdx.x; i < P.n_flags; i += kPrepThreads) P.flags[i] = 0u;
+        for (int i = threadIdx.x; i < P.n_flags / 4; i += kPrepThreads) reinterpret_cast<uint4*>(P.flags)[i] = make_uint4(0u, 0u, 0u, 0u);   // (whole fours)
     }
     if (P.group == 64) {
         deal_backward(P, blockIdx.x);

@@ -132,6 +132,26 @@ __device__ __forceinline__ bool flag_wait(const uint32_t* flag, uint32_t want, v
     }
 }
 
+// The same for the first n (at most eight) of eight flags that lie together, 32-byte aligned.
+__device__ __forceinline__ bool flags_wait(const uint32_t* flags, int n, uint32_t want, volatile uint32_t* abort, uint64_t limit_ns) {
+    const uint64_t t0 = globaltimer_ns();
+#pragma unroll 1
+    for (;;) {
+        uint32_t v[8];
+        asm volatile("ld.relaxed.gpu.global.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "l"(flags) : "memory");
+        asm volatile("ld.relaxed.gpu.global.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]) : "l"(flags + 4) : "memory");
+        int up = 0;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) up += i < n && v[i] == want ? 1 : 0;
+        if (up == n) break;
+        __nanosleep(64);
+        if (abort != nullptr && *abort != 0u) return false;
+        if (globaltimer_ns() - t0 > limit_ns) return false;
+    }
+    asm volatile("fence.acq_rel.gpu;" ::: "memory");
+    return true;
+}
+
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
