@@ -10,6 +10,7 @@ Function names are those of the C ABI.
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 from typing import Optional, Tuple
 
@@ -18,6 +19,7 @@ import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "liblowra.so")
+PY_CALLS_PATH = os.path.join(_HERE, "_py_calls.so")
 
 LOWRA_OK = 0
 (LOWRA_ERR_NULL, LOWRA_ERR_SHAPE, LOWRA_ERR_ALIGN, LOWRA_ERR_PREC, LOWRA_ERR_WORKSPACE,
@@ -66,11 +68,23 @@ class _CMember(ctypes.Structure):
 
 
 _lib = None
+_py_calls = None    # the two products' native way (csrc/py_calls.cpp), loaded with the library
+
+
+def _load_py_calls(L: ctypes.CDLL):
+    if not os.path.exists(PY_CALLS_PATH):
+        raise RuntimeError(f"{PY_CALLS_PATH} is missing: build it with `python -m paper_2502_08141_b200.build`")
+    spec = importlib.util.spec_from_file_location("paper_2502_08141_b200._py_calls", PY_CALLS_PATH)
+    module = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(module)
+    address = lambda fn: ctypes.cast(fn, ctypes.c_void_p).value  # noqa: E731
+    module.bind(address(L.lowra_lora_forward), address(L.lowra_lora_backward_input), address(L.lowra_workspace_bytes), address(L.lowra_workspace_init))
+    return module
 
 
 def lib() -> ctypes.CDLL:
     """The loaded shared library; raises if it has not been built."""
-    global _lib
+    global _lib, _py_calls
     if _lib is None:
         if not os.path.exists(LIB_PATH):
             raise RuntimeError(
@@ -146,6 +160,7 @@ def lib() -> ctypes.CDLL:
         L.lowra_diag_wait_expiry.restype = ctypes.c_int
         L.lowra_diag_drop_t_flags.argtypes = [i32]
         L.lowra_diag_drop_t_flags.restype = ctypes.c_int
+        _py_calls = _load_py_calls(L)
         _lib = L
     return _lib
 
@@ -236,6 +251,7 @@ class Layout:
         c.natural_offsets_dev = None
         self.c = c
         self.ref = ctypes.byref(c)
+        self.address = ctypes.addressof(c)
         self.last_size = (-1, -1, 0)   # (tokens, rank) of the last workspace made here, and its size
         self.deal = None
         self.natural_offsets = None
@@ -439,6 +455,12 @@ def lowra_lora_forward(layout: Layout, packed, absmax, maps, X, A, B, s: float,
                        Y: Optional[torch.Tensor] = None, workspace: Optional[torch.Tensor] = None,
                        stream=None) -> torch.Tensor:
     """Y = X . deq(Wq)^T + s (X . A) . B ; X bf16 [M,K], A bf16 [K,r], B bf16 [r,N] -> Y bf16 [M,N]."""
+    if stream is None and _py_calls is not None:
+        done = _py_calls.forward(layout.address, packed, absmax, maps, X, A, B, s, Y, workspace)
+        if done is not None:
+            if done.__class__ is int:
+                _check(done, "lowra_lora_forward")
+            return done
     _dev(X, _BF16, "X")
     _dev(A, _BF16, "A")
     _dev(B, _BF16, "B")
@@ -546,6 +568,12 @@ def lowra_lora_backward_input(layout: Layout, packed, absmax, maps, dY, A, B, s:
                               dX: Optional[torch.Tensor] = None, workspace: Optional[torch.Tensor] = None,
                               stream=None) -> torch.Tensor:
     """dX = dY . deq(Wq) + s (dY . B^T) . A^T ; dY bf16 [M,N] -> dX bf16 [M,K]."""
+    if stream is None and _py_calls is not None:
+        done = _py_calls.backward_input(layout.address, packed, absmax, maps, dY, A, B, s, dX, workspace)
+        if done is not None:
+            if done.__class__ is int:
+                _check(done, "lowra_lora_backward_input")
+            return done
     for t, n in ((dY, "dY"), (A, "A"), (B, "B")):
         _dev(t, torch.bfloat16, n)
     M, r = int(dY.shape[0]), int(A.shape[1])

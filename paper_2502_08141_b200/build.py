@@ -1,4 +1,4 @@
-"""Compile the CUDA sources into ``liblowra.so`` next to this file (sm_100a only)."""
+"""Compile the CUDA sources into ``liblowra.so`` next to this file (sm_100a only), and the Python binding's native part into ``_py_calls.so``."""
 from __future__ import annotations
 
 import glob
@@ -11,6 +11,8 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "liblowra.so")
+PY_CALLS_SOURCE = os.path.join(CSRC, "py_calls.cpp")
+PY_CALLS = os.path.join(HERE, "_py_calls.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -24,11 +26,24 @@ def sources():
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(PY_CALLS):
         return True
-    t = os.path.getmtime(LIB)
-    deps = sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(ROOT, "include", "*.h"))
+    t = min(os.path.getmtime(LIB), os.path.getmtime(PY_CALLS))
+    deps = sources() + [PY_CALLS_SOURCE] + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(ROOT, "include", "*.h"))
     return any(os.path.getmtime(d) > t for d in deps)
+
+
+def _py_calls_command():
+    import sysconfig
+
+    import torch
+    from torch.utils import cpp_extension
+
+    libs = os.path.join(os.path.dirname(torch.__file__), "lib")
+    includes = [ROOT + "/include", sysconfig.get_paths()["include"], *cpp_extension.include_paths(device_type="cuda")]
+    return [shutil.which("g++") or "g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-w", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+            "-DTORCH_API_INCLUDE_EXTENSION_H", *("-I" + i for i in includes), PY_CALLS_SOURCE, "-o", PY_CALLS, "-L" + libs, "-Wl,-rpath," + libs,
+            "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -39,7 +54,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     objdir = os.path.join(HERE, "build")
     os.makedirs(objdir, exist_ok=True)
     objs = []
-    procs = []
+    procs = [(PY_CALLS_SOURCE, subprocess.Popen(_py_calls_command(), stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True))]
     for src in sources():
         obj = os.path.join(objdir, os.path.basename(src)[:-3] + ".o")
         objs.append(obj)
@@ -52,7 +67,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
             sys.stderr.write(f"--- {os.path.basename(src)}\n{out}\n")
         failed |= p.returncode != 0
     if failed:
-        raise RuntimeError("nvcc failed")
+        raise RuntimeError("compilation failed")
     cmd = [nvcc, "-shared", "-o", LIB, *objs, "-lcudart"]
     subprocess.run(cmd, check=True)
     return LIB

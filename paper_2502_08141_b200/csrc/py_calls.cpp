@@ -1,0 +1,111 @@
+// The Python binding's short way into the two products (lowra_lora_forward, lowra_lora_backward_input): tensor checks, the output's and
+// the scratch's memory and the call itself without an interpreted line between them.  A call for few tokens is two launches of 2.5 us each
+// and 10 us on the GPU; with every check, pointer and argument handled by the interpreter its host side took 12 to 14 us.
+//
+// forward / backward_input(layout address, packed, absmax, maps, act, A, B, s, out or None, workspace or None) returns the output,
+// a status that is not LOWRA_OK, or None for everything that is not the ordinary case - other types, other devices, other layouts in memory,
+// shapes that do not fit, subclasses, errors: the caller then takes the interpreted way, which says what is wrong.
+#include <torch/extension.h>
+
+#include <c10/cuda/CUDAFunctions.h>
+#include <c10/cuda/CUDAStream.h>
+
+#include "lowra.h"
+
+namespace {
+
+using Product = lowra_status (*)(const lowra_layout*, const uint8_t*, const float*, const float*, const uint16_t*, int32_t, const uint16_t*,
+                                 const uint16_t*, int32_t, float, uint16_t*, void*, size_t, void*);
+using WorkspaceBytes = size_t (*)(const lowra_layout*, int32_t, int32_t);
+using WorkspaceInit = lowra_status (*)(void*, size_t, void*);
+struct Library {
+    Product forward, backward_input;
+    WorkspaceBytes workspace_bytes;
+    WorkspaceInit workspace_init;
+} library;
+
+bool plain(PyObject* o) { return THPVariable_CheckExact(o); }
+
+bool matrix(const at::Tensor& t, int64_t rows, int64_t cols) {
+    return t.is_cuda() && t.scalar_type() == at::kBFloat16 && t.dim() == 2 && t.size(0) == rows && t.size(1) == cols && t.is_contiguous();
+}
+
+PyObject* product(PyObject* const* args, Py_ssize_t n, bool backward) {
+    if (n != 10 || library.forward == nullptr) Py_RETURN_NONE;
+    for (int i = 1; i <= 6; ++i)
+        if (!plain(args[i])) Py_RETURN_NONE;
+    if ((args[8] != Py_None && !plain(args[8])) || (args[9] != Py_None && !plain(args[9])) || !(PyFloat_CheckExact(args[7]) || PyLong_CheckExact(args[7]))) Py_RETURN_NONE;
+    const lowra_layout* layout = static_cast<const lowra_layout*>(PyLong_AsVoidPtr(args[0]));
+    const double s = PyFloat_AsDouble(args[7]);
+    if (PyErr_Occurred() != nullptr || layout == nullptr) {
+        PyErr_Clear();
+        Py_RETURN_NONE;
+    }
+    try {
+        const at::Tensor &packed = THPVariable_Unpack(args[1]), &absmax = THPVariable_Unpack(args[2]), &maps = THPVariable_Unpack(args[3]);
+        const at::Tensor &act = THPVariable_Unpack(args[4]), &A = THPVariable_Unpack(args[5]), &B = THPVariable_Unpack(args[6]);
+        if (act.dim() != 2 || A.dim() != 2) Py_RETURN_NONE;
+        const int64_t M = act.size(0), r = A.size(1), N = layout->N, K = layout->K;
+        if (!matrix(act, M, backward ? N : K) || !matrix(A, K, r) || !matrix(B, r, N) || M > INT32_MAX || r > INT32_MAX) Py_RETURN_NONE;
+        at::Tensor out = args[8] != Py_None ? THPVariable_Unpack(args[8]) : at::empty({M, backward ? K : N}, act.options().requires_grad(false));
+        void* stream = c10::cuda::getCurrentCUDAStream().stream();
+        at::Tensor workspace;
+        if (args[9] != Py_None) {
+            workspace = THPVariable_Unpack(args[9]);
+        } else {
+            const size_t bytes = library.workspace_bytes(layout, (int32_t)M, (int32_t)r);
+            if (bytes == 0) Py_RETURN_NONE;
+            workspace = at::empty({(int64_t)bytes}, act.options().requires_grad(false).dtype(at::kByte));
+            if (layout->deal_dev != nullptr && library.workspace_init(workspace.data_ptr(), bytes, stream) != LOWRA_OK) Py_RETURN_NONE;   // no prologue launch will clear it
+        }
+        const Product call = backward ? library.backward_input : library.forward;
+        const auto* packed_p = static_cast<const uint8_t*>(packed.data_ptr());
+        const auto *absmax_p = static_cast<const float*>(absmax.data_ptr()), *maps_p = static_cast<const float*>(maps.data_ptr());
+        const auto *act_p = static_cast<const uint16_t*>(act.data_ptr()), *A_p = static_cast<const uint16_t*>(A.data_ptr()), *B_p = static_cast<const uint16_t*>(B.data_ptr());
+        auto* out_p = static_cast<uint16_t*>(out.data_ptr());
+        void* workspace_p = workspace.data_ptr();
+        const size_t workspace_n = (size_t)workspace.numel();
+        lowra_status st;
+        Py_BEGIN_ALLOW_THREADS
+        st = call(layout, packed_p, absmax_p, maps_p, act_p, (int32_t)M, A_p, B_p, (int32_t)r, (float)s, out_p, workspace_p, workspace_n, stream);
+        Py_END_ALLOW_THREADS
+        if (st != LOWRA_OK) return PyLong_FromLong(st);
+        if (args[8] != Py_None) {
+            Py_INCREF(args[8]);
+            return args[8];
+        }
+        return THPVariable_Wrap(std::move(out));
+    } catch (...) {
+        PyErr_Clear();
+        Py_RETURN_NONE;
+    }
+}
+
+PyObject* forward(PyObject*, PyObject* const* args, Py_ssize_t n) { return product(args, n, false); }
+PyObject* backward_input(PyObject*, PyObject* const* args, Py_ssize_t n) { return product(args, n, true); }
+
+// bind(addresses of lowra_lora_forward, lowra_lora_backward_input, lowra_workspace_bytes, lowra_workspace_init)
+PyObject* bind(PyObject*, PyObject* const* args, Py_ssize_t n) {
+    void* p[4] = {};
+    for (int i = 0; i < 4; ++i) {
+        p[i] = i < n ? PyLong_AsVoidPtr(args[i]) : nullptr;
+        if (p[i] == nullptr) {
+            if (PyErr_Occurred() == nullptr) PyErr_SetString(PyExc_ValueError, "bind takes four addresses");
+            return nullptr;
+        }
+    }
+    library = Library{reinterpret_cast<Product>(p[0]), reinterpret_cast<Product>(p[1]), reinterpret_cast<WorkspaceBytes>(p[2]), reinterpret_cast<WorkspaceInit>(p[3])};
+    Py_RETURN_NONE;
+}
+
+PyMethodDef methods[] = {
+    {"forward", (PyCFunction)(void (*)())forward, METH_FASTCALL, nullptr},
+    {"backward_input", (PyCFunction)(void (*)())backward_input, METH_FASTCALL, nullptr},
+    {"bind", (PyCFunction)(void (*)())bind, METH_FASTCALL, nullptr},
+    {nullptr, nullptr, 0, nullptr},
+};
+PyModuleDef module = {PyModuleDef_HEAD_INIT, "_py_calls", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
+
+}  // namespace
+
+PyMODINIT_FUNC PyInit__py_calls() { return PyModule_Create(&module); }
