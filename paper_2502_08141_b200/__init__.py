@@ -2,7 +2,7 @@
 
 Argument marshalling only: every step of the path (encode, decode, fused dequant + LoRA products)
 runs in the CUDA kernels behind the C ABI declared in ``include/lowra.h``.  PyTorch is used for
-device memory and streams, nothing else.  There is no CPU fallback: if the shared library has
+device memory and streams, nothing else.  The two products' own host side is native (``csrc/py_calls.cpp``).  There is no CPU fallback: if the shared library has
 not been built, or the device is not a B200, the calls raise.
 
 Function names are those of the C ABI.

@@ -25,10 +25,11 @@
 // U = s dY B^T) by TMA from the workspace.  T itself is produced by this same kernel: for every token tile there is one
 // extra "T tile" whose operand rows are the ranks, padded to 128.  T tiles come first in the tile order, their epilogue raises
 // a flag per CTA, and the TMA producer of a regular tile waits (bounded) for that flag before it fetches T.  All CTAs are
-// co-resident and a T tile waits for nothing, so the wait cannot deadlock.
+// co-resident and a T tile waits for nothing but the other clusters that share it, so the wait cannot deadlock.
 // Schedule: whole tiles dealt round-robin to the pairs, or (launcher's choice) ranges: equal consecutive pieces of the
 // remaining weight tiles' contraction blocks per pair, partial tiles handed over through a scratch slot and added in the
-// epilogue of the pair that starts the tile (see the schedule in the kernel).
+// epilogue of the pair that starts the tile; or, in calls of few tiles, tiles shared by several pairs, each of which finishes some of
+// the tile's columns (see the schedule in the kernel).
 //
 // Warp roles: 0 = TMA producer, 1 = MMA issuer (in the CTA of rank 0) and TMEM owner, 2-9 = epilogue, 10-25 = dequant.
 // All mbarrier waits are bounded; a wait that runs out sets the status word and every role leaves.
@@ -208,8 +209,8 @@ fused_kernel(const __grid_constant__ KParams<NB> P, const __grid_constant__ KMap
     // whose range starts the tile adds them in its epilogue, in a fixed order.  That piece is always the cluster's last, a slice
     // for somebody else always the first of its range, so collecting rarely waits.
     const bool sk = MODE != kModeDense && P.sk != 0;
-    // Short calls (t_split > 1): the T tiles are what everybody would wait for, so every one of them is cut as well, between
-    // the first clusters, and the weight tiles' ranges belong to the others.
+    // Short calls: the T tiles are what everybody would wait for, so every one of them is shared as well (t_split > 1), by
+    // the first clusters, and the weight tiles belong to the others - in ranges, or each shared by w_split of them.
     const int t_cl = SHARED && P.t_split > 1 ? n_t_tiles * P.t_split : 0;
     const int n_whole = sk ? n_t_tiles + P.sk_first : n_t_tiles + P.tiles_r * super_t;   // pieces dealt round-robin
     const int w_whole = t_cl > 0 ? (cid < t_cl ? 1 : 0) : n_whole > cid ? (n_whole - cid + NC - 1) / NC : 0;   // this cluster's
