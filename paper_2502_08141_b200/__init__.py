@@ -177,13 +177,13 @@ def _check(code: int, where: str) -> None:
 # The raw handle of the current stream without building a Stream object around it (0.1 us against 3.4 us, in calls whose
 # whole host side is a dozen); torch versions without these two take the long way.
 _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
-_current_device = getattr(torch._C, "_cuda_getDevice", None)
+_current_device = getattr(torch._C, "_cuda_getDevice", None) or torch.cuda.current_device
 
 
 def _stream(stream) -> int:
     if stream is not None:
         return stream.cuda_stream
-    if _raw_stream is not None and _current_device is not None:
+    if _raw_stream is not None:
         return _raw_stream(_current_device())
     return torch.cuda.current_stream().cuda_stream
 
@@ -196,7 +196,7 @@ def _ptr(t: Optional[torch.Tensor]) -> int:
 
 
 def _dev(t: torch.Tensor, dtype, name: str) -> torch.Tensor:
-    if t.is_cuda and t.dtype is dtype and t.is_contiguous():
+    if t.is_cuda and t.dtype is dtype and t.is_contiguous() and t.get_device() == _current_device():
         return t
     if not t.is_cuda:
         raise ValueError(f"{name} must be a CUDA tensor")
@@ -204,7 +204,38 @@ def _dev(t: torch.Tensor, dtype, name: str) -> torch.Tensor:
         raise ValueError(f"{name} must be {dtype}, got {t.dtype}")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
+    _here(t, name)
     return t
+
+
+def _here(t: torch.Tensor, name: str) -> None:
+    if t.is_cuda:
+        if t.get_device() != _current_device():
+            raise ValueError(f"{name} is on {t.device}, the call runs on cuda:{_current_device()}")
+    elif not t.is_pinned():
+        raise ValueError(f"{name} must be a CUDA tensor")
+
+
+def _extent(t: Optional[torch.Tensor], least: int, name: str, dtype=None) -> None:
+    """An array that a kernel reads or writes by its address: memory the current device reaches (page-locked host memory is), without gaps,
+    at least `least` elements of `dtype`, or bytes of any type.  None is for the library to refuse."""
+    if t is None:
+        return
+    _here(t, name)
+    if dtype is not None and t.dtype != dtype:
+        raise ValueError(f"{name} must be {dtype}, got {t.dtype}")
+    if not t.is_contiguous():
+        raise ValueError(f"{name} must be contiguous")
+    n = t.numel() if dtype is not None else t.numel() * t.element_size()
+    if n < least:
+        raise ValueError(f"{name}: {n} {'elements' if dtype is not None else 'bytes'}, {least} are needed")
+
+
+def _weight_arrays(layout: Layout, packed, absmax, maps, n_maps: int = 1) -> None:
+    _here(layout.perm, "the layout")
+    _extent(packed, layout.packed_bytes, "packed")
+    _extent(absmax, layout.N * (layout.K // 64), "absmax", torch.float32)
+    _extent(maps, n_maps * layout.N * 16, "maps", torch.float32)
 
 
 # ---------------------------------------------------------------------------------------------
@@ -252,6 +283,7 @@ class Layout:
         self.c = c
         self.ref = ctypes.byref(c)
         self.address = ctypes.addressof(c)
+        self.device_index = self.perm.get_device()
         self.last_size = (-1, -1, 0)   # (tokens, rank) of the last workspace made here, and its size
         self.deal = None
         self.natural_offsets = None
@@ -456,7 +488,7 @@ def lowra_lora_forward(layout: Layout, packed, absmax, maps, X, A, B, s: float,
                        stream=None) -> torch.Tensor:
     """Y = X . deq(Wq)^T + s (X . A) . B ; X bf16 [M,K], A bf16 [K,r], B bf16 [r,N] -> Y bf16 [M,N]."""
     if stream is None and _py_calls is not None:
-        done = _py_calls.forward(layout.address, packed, absmax, maps, X, A, B, s, Y, workspace)
+        done = _py_calls.forward(layout.address, layout.device_index, packed, absmax, maps, X, A, B, s, Y, workspace)
         if done is not None:
             if done.__class__ is int:
                 _check(done, "lowra_lora_forward")
@@ -467,6 +499,9 @@ def lowra_lora_forward(layout: Layout, packed, absmax, maps, X, A, B, s: float,
     M, r = X.shape[0], A.shape[1]
     if X.shape != (M, layout.K) or A.shape != (layout.K, r) or B.shape != (r, layout.N):
         raise ValueError("shape mismatch")
+    _weight_arrays(layout, packed, absmax, maps)
+    _extent(Y, M * layout.N, "Y", _BF16)
+    _extent(workspace, 0, "workspace")     # (its size is the library's to judge)
     if Y is None:
         Y = X.new_empty((M, layout.N))
     if workspace is None:
@@ -569,7 +604,7 @@ def lowra_lora_backward_input(layout: Layout, packed, absmax, maps, dY, A, B, s:
                               stream=None) -> torch.Tensor:
     """dX = dY . deq(Wq) + s (dY . B^T) . A^T ; dY bf16 [M,N] -> dX bf16 [M,K]."""
     if stream is None and _py_calls is not None:
-        done = _py_calls.backward_input(layout.address, packed, absmax, maps, dY, A, B, s, dX, workspace)
+        done = _py_calls.backward_input(layout.address, layout.device_index, packed, absmax, maps, dY, A, B, s, dX, workspace)
         if done is not None:
             if done.__class__ is int:
                 _check(done, "lowra_lora_backward_input")
@@ -579,6 +614,9 @@ def lowra_lora_backward_input(layout: Layout, packed, absmax, maps, dY, A, B, s:
     M, r = int(dY.shape[0]), int(A.shape[1])
     if tuple(dY.shape) != (M, layout.N) or tuple(A.shape) != (layout.K, r) or tuple(B.shape) != (r, layout.N):
         raise ValueError("shape mismatch")
+    _weight_arrays(layout, packed, absmax, maps)
+    _extent(dX, M * layout.K, "dX", _BF16)
+    _extent(workspace, 0, "workspace")
     if dX is None:
         dX = dY.new_empty((M, layout.K))
     if workspace is None:

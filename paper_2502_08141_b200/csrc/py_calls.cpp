@@ -2,9 +2,10 @@
 // the scratch's memory and the call itself without an interpreted line between them.  A call for few tokens is two launches of 2.5 us each
 // and 10 us on the GPU; with every check, pointer and argument handled by the interpreter its host side took 12 to 14 us.
 //
-// forward / backward_input(layout address, packed, absmax, maps, act, A, B, s, out or None, workspace or None) returns the output,
-// a status that is not LOWRA_OK, or None for everything that is not the ordinary case - other types, other devices, other layouts in memory,
-// shapes that do not fit, subclasses, errors: the caller then takes the interpreted way, which says what is wrong.
+// forward / backward_input(layout address, its device, packed, absmax, maps, act, A, B, s, out or None, workspace or None) returns the output,
+// a status that is not LOWRA_OK, or None for everything that is not the ordinary case - other types, memory of other devices than the
+// current one, other layouts in memory, shapes that do not fit, arrays that are too short, subclasses, errors: the caller then takes the
+// interpreted way, which says what is wrong.
 #include <torch/extension.h>
 
 #include <c10/cuda/CUDAFunctions.h>
@@ -26,32 +27,40 @@ struct Library {
 
 bool plain(PyObject* o) { return THPVariable_CheckExact(o); }
 
-bool matrix(const at::Tensor& t, int64_t rows, int64_t cols) {
-    return t.is_cuda() && t.scalar_type() == at::kBFloat16 && t.dim() == 2 && t.size(0) == rows && t.size(1) == cols && t.is_contiguous();
+// memory of device `dev` without gaps
+bool on(const at::Tensor& t, int64_t dev) { return t.is_cuda() && t.get_device() == dev && t.is_contiguous(); }
+bool matrix(const at::Tensor& t, int64_t rows, int64_t cols, int64_t dev) {
+    return on(t, dev) && t.scalar_type() == at::kBFloat16 && t.dim() == 2 && t.size(0) == rows && t.size(1) == cols;
 }
+bool array(const at::Tensor& t, at::ScalarType type, int64_t least, int64_t dev) { return on(t, dev) && t.scalar_type() == type && t.numel() >= least; }
 
 PyObject* product(PyObject* const* args, Py_ssize_t n, bool backward) {
-    if (n != 10 || library.forward == nullptr) Py_RETURN_NONE;
-    for (int i = 1; i <= 6; ++i)
+    if (n != 11 || library.forward == nullptr) Py_RETURN_NONE;
+    for (int i = 2; i <= 7; ++i)
         if (!plain(args[i])) Py_RETURN_NONE;
-    if ((args[8] != Py_None && !plain(args[8])) || (args[9] != Py_None && !plain(args[9])) || !(PyFloat_CheckExact(args[7]) || PyLong_CheckExact(args[7]))) Py_RETURN_NONE;
+    const bool out_given = args[9] != Py_None, workspace_given = args[10] != Py_None;
+    if ((out_given && !plain(args[9])) || (workspace_given && !plain(args[10])) || !(PyFloat_CheckExact(args[8]) || PyLong_CheckExact(args[8]))) Py_RETURN_NONE;
     const lowra_layout* layout = static_cast<const lowra_layout*>(PyLong_AsVoidPtr(args[0]));
-    const double s = PyFloat_AsDouble(args[7]);
+    const long dev = PyLong_AsLong(args[1]);
+    const double s = PyFloat_AsDouble(args[8]);
     if (PyErr_Occurred() != nullptr || layout == nullptr) {
         PyErr_Clear();
         Py_RETURN_NONE;
     }
     try {
-        const at::Tensor &packed = THPVariable_Unpack(args[1]), &absmax = THPVariable_Unpack(args[2]), &maps = THPVariable_Unpack(args[3]);
-        const at::Tensor &act = THPVariable_Unpack(args[4]), &A = THPVariable_Unpack(args[5]), &B = THPVariable_Unpack(args[6]);
-        if (act.dim() != 2 || A.dim() != 2) Py_RETURN_NONE;
-        const int64_t M = act.size(0), r = A.size(1), N = layout->N, K = layout->K;
-        if (!matrix(act, M, backward ? N : K) || !matrix(A, K, r) || !matrix(B, r, N) || M > INT32_MAX || r > INT32_MAX) Py_RETURN_NONE;
-        at::Tensor out = args[8] != Py_None ? THPVariable_Unpack(args[8]) : at::empty({M, backward ? K : N}, act.options().requires_grad(false));
+        const at::Tensor &packed = THPVariable_Unpack(args[2]), &absmax = THPVariable_Unpack(args[3]), &maps = THPVariable_Unpack(args[4]);
+        const at::Tensor &act = THPVariable_Unpack(args[5]), &A = THPVariable_Unpack(args[6]), &B = THPVariable_Unpack(args[7]);
+        if (act.dim() != 2 || A.dim() != 2 || dev != c10::cuda::current_device()) Py_RETURN_NONE;
+        const int64_t M = act.size(0), r = A.size(1), N = layout->N, K = layout->K, cols = backward ? K : N;
+        if (!matrix(act, M, backward ? N : K, dev) || !matrix(A, K, r, dev) || !matrix(B, r, N, dev) || M > INT32_MAX || r > INT32_MAX) Py_RETURN_NONE;
+        if (!on(packed, dev) || packed.nbytes() < layout->packed_bytes || !array(absmax, at::kFloat, N * (K / 64), dev) || !array(maps, at::kFloat, N * 16, dev)) Py_RETURN_NONE;
+        if (out_given && !array(THPVariable_Unpack(args[9]), at::kBFloat16, M * cols, dev)) Py_RETURN_NONE;
+        if (workspace_given && !on(THPVariable_Unpack(args[10]), dev)) Py_RETURN_NONE;
+        at::Tensor out = out_given ? THPVariable_Unpack(args[9]) : at::empty({M, cols}, act.options().requires_grad(false));
         void* stream = c10::cuda::getCurrentCUDAStream().stream();
         at::Tensor workspace;
-        if (args[9] != Py_None) {
-            workspace = THPVariable_Unpack(args[9]);
+        if (workspace_given) {
+            workspace = THPVariable_Unpack(args[10]);
         } else {
             const size_t bytes = library.workspace_bytes(layout, (int32_t)M, (int32_t)r);
             if (bytes == 0) Py_RETURN_NONE;
@@ -70,9 +79,9 @@ PyObject* product(PyObject* const* args, Py_ssize_t n, bool backward) {
         st = call(layout, packed_p, absmax_p, maps_p, act_p, (int32_t)M, A_p, B_p, (int32_t)r, (float)s, out_p, workspace_p, workspace_n, stream);
         Py_END_ALLOW_THREADS
         if (st != LOWRA_OK) return PyLong_FromLong(st);
-        if (args[8] != Py_None) {
-            Py_INCREF(args[8]);
-            return args[8];
+        if (out_given) {
+            Py_INCREF(args[9]);
+            return args[9];
         }
         return THPVariable_Wrap(std::move(out));
     } catch (...) {
