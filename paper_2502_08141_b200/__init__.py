@@ -84,7 +84,7 @@ def _load_py_calls(L: ctypes.CDLL):
 
 def lib() -> ctypes.CDLL:
     """The loaded shared library; raises if it has not been built."""
-    global _lib, _py_calls
+    global _lib, _py_calls, _fits
     if _lib is None:
         if not os.path.exists(LIB_PATH):
             raise RuntimeError(
@@ -161,6 +161,7 @@ def lib() -> ctypes.CDLL:
         L.lowra_diag_drop_t_flags.argtypes = [i32]
         L.lowra_diag_drop_t_flags.restype = ctypes.c_int
         _py_calls = _load_py_calls(L)
+        _fits = _py_calls.fits
         _lib = L
     return _lib
 
@@ -195,8 +196,9 @@ def _ptr(t: Optional[torch.Tensor]) -> int:
     return 0 if t is None else t.data_ptr()
 
 
-def _dev(t: torch.Tensor, dtype, name: str) -> torch.Tensor:
-    if t.is_cuda and t.dtype is dtype and t.is_contiguous() and t.get_device() == _current_device():
+def _dev(t: torch.Tensor, dtype, name: str, least: int = 0) -> torch.Tensor:
+    """A CUDA tensor of `dtype`, contiguous, on the current device, of at least `least` elements."""
+    if t.is_cuda and t.dtype is dtype and t.is_contiguous() and t.numel() >= least and t.get_device() == _current_device():
         return t
     if not t.is_cuda:
         raise ValueError(f"{name} must be a CUDA tensor")
@@ -205,6 +207,8 @@ def _dev(t: torch.Tensor, dtype, name: str) -> torch.Tensor:
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
     _here(t, name)
+    if t.numel() < least:
+        raise ValueError(f"{name}: {t.numel()} elements, {least} are needed")
     return t
 
 
@@ -231,8 +235,22 @@ def _extent(t: Optional[torch.Tensor], least: int, name: str, dtype=None) -> Non
         raise ValueError(f"{name}: {n} {'elements' if dtype is not None else 'bytes'}, {least} are needed")
 
 
+def _no_verdict(*_) -> bool:
+    return False
+
+
+# Whether (tensor or None, element type, least length) ... are all as the kernels want them (csrc/py_calls.cpp, once the library is loaded).  No is
+# not a verdict: the checks above, which say what is wrong, then take their turn.
+_fits = _no_verdict
+
+
+def _layout_here(layout: Layout) -> None:
+    if layout.device_index != _current_device():
+        _here(layout.perm, "the layout")
+
+
 def _weight_arrays(layout: Layout, packed, absmax, maps, n_maps: int = 1) -> None:
-    _here(layout.perm, "the layout")
+    _layout_here(layout)
     _extent(packed, layout.packed_bytes, "packed")
     _extent(absmax, layout.N * (layout.K // 64), "absmax", torch.float32)
     _extent(maps, n_maps * layout.N * 16, "maps", torch.float32)
@@ -284,6 +302,7 @@ class Layout:
         self.ref = ctypes.byref(c)
         self.address = ctypes.addressof(c)
         self.device_index = self.perm.get_device()
+        self.n_absmax, self.n_tables, self.n_weights = self.N * (self.K // 64), self.N * 16, self.N * self.K
         self.last_size = (-1, -1, 0)   # (tokens, rank) of the last workspace made here, and its size
         self.deal = None
         self.natural_offsets = None
@@ -310,20 +329,38 @@ class Layout:
         return self
 
 
+def _check_encode(layout: Layout, W, thresholds, packed, absmax) -> None:
+    if not _fits(layout.device_index, W, "f", 0, thresholds, "f", 0, packed, "u", layout.packed_bytes, absmax, "f", layout.n_absmax):
+        _layout_here(layout)
+        _dev(W, torch.float32, "W")
+        _dev(thresholds, torch.float32, "thresholds")
+        if packed is not None:
+            _dev(packed, torch.uint8, "packed", layout.packed_bytes)
+        if absmax is not None:
+            _dev(absmax, torch.float32, "absmax", layout.n_absmax)
+    if tuple(W.shape) != (layout.N, layout.K) or tuple(thresholds.shape) != (layout.N, 16):
+        raise ValueError("shape mismatch")
+
+
+def _check_decode(layout: Layout, packed, absmax, maps, out) -> None:
+    if not _fits(layout.device_index, packed, "u", layout.packed_bytes, absmax, "f", layout.n_absmax, maps, "f", layout.n_tables, out, "h", layout.n_weights):
+        _layout_here(layout)
+        _dev(packed, torch.uint8, "packed", layout.packed_bytes)
+        _dev(absmax, torch.float32, "absmax", layout.n_absmax)
+        _dev(maps, torch.float32, "maps", layout.n_tables)
+        if out is not None:
+            _dev(out, torch.bfloat16, "out", layout.n_weights)
+
+
 def lowra_encode(layout: Layout, W: torch.Tensor, thresholds: torch.Tensor,
                  packed: Optional[torch.Tensor] = None, absmax: Optional[torch.Tensor] = None,
                  stream=None) -> Tuple[torch.Tensor, torch.Tensor]:
     """W fp32 [N,K], thresholds fp32 [N,16] -> packed uint8 [packed_bytes], absmax fp32 [N,K/64]."""
-    _dev(W, torch.float32, "W")
-    _dev(thresholds, torch.float32, "thresholds")
-    if tuple(W.shape) != (layout.N, layout.K) or tuple(thresholds.shape) != (layout.N, 16):
-        raise ValueError("shape mismatch")
+    _check_encode(layout, W, thresholds, packed, absmax)
     if packed is None:
         packed = torch.empty(max(layout.packed_bytes, 16), dtype=torch.uint8, device=W.device)
     if absmax is None:
         absmax = torch.empty((layout.N, layout.K // 64), dtype=torch.float32, device=W.device)
-    _dev(packed, torch.uint8, "packed")
-    _dev(absmax, torch.float32, "absmax")
     code = lib().lowra_encode(layout.ref, _ptr(W), _ptr(thresholds), _ptr(packed), _ptr(absmax), _stream(stream))
     _check(code, "lowra_encode")
     return packed, absmax
@@ -332,12 +369,9 @@ def lowra_encode(layout: Layout, W: torch.Tensor, thresholds: torch.Tensor,
 def lowra_decode(layout: Layout, packed: torch.Tensor, absmax: torch.Tensor, maps: torch.Tensor,
                  out: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """-> bf16 [N, K], original row order."""
-    _dev(packed, torch.uint8, "packed")
-    _dev(absmax, torch.float32, "absmax")
-    _dev(maps, torch.float32, "maps")
+    _check_decode(layout, packed, absmax, maps, out)
     if out is None:
         out = torch.empty((layout.N, layout.K), dtype=torch.bfloat16, device=packed.device)
-    _dev(out, torch.bfloat16, "out")
     code = lib().lowra_decode(layout.ref, _ptr(packed), _ptr(absmax), _ptr(maps), _ptr(out), _stream(stream))
     _check(code, "lowra_decode")
     return out
@@ -355,18 +389,13 @@ def lowra_encode_group(members, stream=None):
     outs = []
     for i, m in enumerate(members):
         layout, W, thr = m["layout"], m["W"], m["thresholds"]
-        _dev(W, torch.float32, "W")
-        _dev(thr, torch.float32, "thresholds")
-        if tuple(W.shape) != (layout.N, layout.K) or tuple(thr.shape) != (layout.N, 16):
-            raise ValueError("shape mismatch")
         packed = m.get("packed")
         absmax = m.get("absmax")
+        _check_encode(layout, W, thr, packed, absmax)
         if packed is None:
             packed = torch.empty(max(layout.packed_bytes, 16), dtype=torch.uint8, device=W.device)
         if absmax is None:
             absmax = torch.empty((layout.N, layout.K // 64), dtype=torch.float32, device=W.device)
-        _dev(packed, torch.uint8, "packed")
-        _dev(absmax, torch.float32, "absmax")
         arr[i].layout = ctypes.pointer(layout.c)
         arr[i].W_dev, arr[i].tables_dev = W.data_ptr(), thr.data_ptr()
         arr[i].packed_dev, arr[i].absmax_dev, arr[i].W_bf16_dev = packed.data_ptr(), absmax.data_ptr(), None
@@ -383,13 +412,10 @@ def lowra_decode_group(members, stream=None):
     outs = []
     for i, m in enumerate(members):
         layout, packed, absmax, maps = m["layout"], m["packed"], m["absmax"], m["maps"]
-        _dev(packed, torch.uint8, "packed")
-        _dev(absmax, torch.float32, "absmax")
-        _dev(maps, torch.float32, "maps")
         out = m.get("out")
+        _check_decode(layout, packed, absmax, maps, out)
         if out is None:
             out = torch.empty((layout.N, layout.K), dtype=torch.bfloat16, device=packed.device)
-        _dev(out, torch.bfloat16, "out")
         arr[i].layout = ctypes.pointer(layout.c)
         arr[i].W_dev, arr[i].tables_dev = None, maps.data_ptr()
         arr[i].packed_dev, arr[i].absmax_dev, arr[i].W_bf16_dev = packed.data_ptr(), absmax.data_ptr(), out.data_ptr()
@@ -404,7 +430,13 @@ def lowra_learn_codebooks(layout: Layout, W: torch.Tensor, init_levels, init_thr
     """Weighted Lloyd-Max per row at the row's precision -> (maps fp32 [N,16], thresholds fp32 [N,16]).
 
     init_levels / init_thresholds: host arrays [3, 16] float64 (rows: 1-, 2-, 4-bit starting tables)."""
-    _dev(W, torch.float32, "W")
+    if not _fits(layout.device_index, W, "f", layout.n_weights, maps, "f", layout.n_tables, thresholds, "f", layout.n_tables):
+        _layout_here(layout)
+        _dev(W, torch.float32, "W", layout.n_weights)
+        if maps is not None:
+            _dev(maps, torch.float32, "maps", layout.n_tables)
+        if thresholds is not None:
+            _dev(thresholds, torch.float32, "thresholds", layout.n_tables)
     y0 = np.ascontiguousarray(init_levels, dtype=np.float64)
     t0 = np.ascontiguousarray(init_thresholds, dtype=np.float64)
     if y0.shape != (3, 16) or t0.shape != (3, 16):
@@ -413,8 +445,6 @@ def lowra_learn_codebooks(layout: Layout, W: torch.Tensor, init_levels, init_thr
         maps = torch.empty((layout.N, 16), dtype=torch.float32, device=W.device)
     if thresholds is None:
         thresholds = torch.empty((layout.N, 16), dtype=torch.float32, device=W.device)
-    _dev(maps, torch.float32, "maps")
-    _dev(thresholds, torch.float32, "thresholds")
     code = lib().lowra_learn_codebooks(layout.ref, _ptr(W), y0.ctypes.data_as(ctypes.c_void_p),
                                        t0.ctypes.data_as(ctypes.c_void_p), int(iterations), _ptr(maps),
                                        _ptr(thresholds), _stream(stream))
@@ -427,8 +457,12 @@ def lowra_learn_codebooks_all(W: torch.Tensor, init_levels, init_thresholds, ite
                               stream=None) -> Tuple[torch.Tensor, torch.Tensor]:
     """Every row of W learnt at 1, 2 and 4 bits in one pass -> (maps3, thresholds3) fp32 [3, N, 16], the input
     format of lowra_channel_errors."""
-    _dev(W, torch.float32, "W")
     N, K = int(W.shape[0]), int(W.shape[1])
+    if not _fits(W.get_device(), W, "f", 0, maps3, "f", 0, thresholds3, "f", 0):
+        _dev(W, torch.float32, "W")
+        for t, name in ((maps3, "maps3"), (thresholds3, "thresholds3")):
+            if t is not None:
+                _dev(t, torch.float32, name)
     y0 = np.ascontiguousarray(init_levels, dtype=np.float64)
     t0 = np.ascontiguousarray(init_thresholds, dtype=np.float64)
     if y0.shape != (3, 16) or t0.shape != (3, 16):
@@ -437,8 +471,6 @@ def lowra_learn_codebooks_all(W: torch.Tensor, init_levels, init_thresholds, ite
         maps3 = torch.empty((3, N, 16), dtype=torch.float32, device=W.device)
     if thresholds3 is None:
         thresholds3 = torch.empty((3, N, 16), dtype=torch.float32, device=W.device)
-    _dev(maps3, torch.float32, "maps3")
-    _dev(thresholds3, torch.float32, "thresholds3")
     if tuple(maps3.shape) != (3, N, 16) or tuple(thresholds3.shape) != (3, N, 16):
         raise ValueError("maps3 and thresholds3 must be [3, N, 16]")
     code = lib().lowra_learn_codebooks_all(N, K, _ptr(W), y0.ctypes.data_as(ctypes.c_void_p),
@@ -525,8 +557,12 @@ def _batch(fn_name: str, members, s: float, workspace: torch.Tensor, backward: b
     r = int(members[0]["A"].shape[1])
     for i, m in enumerate(members):
         lay = m["layout"]
-        for key in ("act", "A", "B", "out"):
-            _dev(m[key], torch.bfloat16, key)
+        if not _fits(lay.device_index, m["act"], "h", 0, m["A"], "h", 0, m["B"], "h", 0, m["out"], "h", 0, m["packed"], "B", lay.packed_bytes,
+                     m["absmax"], "f", lay.n_absmax, m["maps"], "f", lay.n_tables, workspace, "B", 0):
+            for key in ("act", "A", "B", "out"):
+                _dev(m[key], torch.bfloat16, key)
+            _weight_arrays(lay, m["packed"], m["absmax"], m["maps"])
+            _extent(workspace, 0, "workspace")
         act_cols, out_cols = (lay.N, lay.K) if backward else (lay.K, lay.N)
         if (tuple(m["act"].shape) != (M, act_cols) or tuple(m["out"].shape) != (M, out_cols) or
                 tuple(m["A"].shape) != (lay.K, r) or tuple(m["B"].shape) != (r, lay.N)):
@@ -556,10 +592,15 @@ def lowra_lora_forward_adapters(layout: Layout, packed, absmax, maps, X, group_s
                                 stream=None) -> torch.Tensor:
     """Several adapters on one quantised base weight: maps fp32 [n, N, 16], A bf16 [n, K, r], B bf16 [n, r, N];
     adapter a owns the token rows group_start[a] .. group_start[a + 1] of X (host sequence of n + 1 ints)."""
-    for t, nm in ((X, "X"), (A, "A"), (B, "B")):
-        _dev(t, torch.bfloat16, nm)
-    _dev(maps, torch.float32, "maps")
     n, M, r = int(maps.shape[0]), int(X.shape[0]), int(A.shape[2])
+    if not _fits(layout.device_index, X, "h", 0, A, "h", 0, B, "h", 0, maps, "f", 0, packed, "B", layout.packed_bytes, absmax, "f", layout.n_absmax,
+                 Y, "h", M * layout.N, workspace, "B", 0):
+        for t, nm in ((X, "X"), (A, "A"), (B, "B")):
+            _dev(t, torch.bfloat16, nm)
+        _dev(maps, torch.float32, "maps")
+        _weight_arrays(layout, packed, absmax, maps, 0)
+        _extent(Y, M * layout.N, "Y", _BF16)
+        _extent(workspace, 0, "workspace")
     if (tuple(maps.shape) != (n, layout.N, 16) or tuple(X.shape) != (M, layout.K) or tuple(A.shape) != (n, layout.K, r)
             or tuple(B.shape) != (n, r, layout.N)):
         raise ValueError("shape mismatch")
@@ -586,9 +627,14 @@ def lowra_lora_forward_static(layout: Layout, packed, absmax, maps, X, A, B, s: 
     must not overlap on the GPU.  Raises LowraError(LOWRA_ERR_LIMIT) when the problem needs more scratch.
     `status_out`: optional int32/uint32 device tensor of one element that receives the device status word.
     This wrapper allocates Y only if the caller passes none; the library call itself allocates nothing."""
-    for t, n in ((X, "X"), (A, "A"), (B, "B")):
-        _dev(t, torch.bfloat16, n)
     M, r = int(X.shape[0]), int(A.shape[1])
+    if not _fits(layout.device_index, X, "h", 0, A, "h", 0, B, "h", 0, packed, "B", layout.packed_bytes, absmax, "f", layout.n_absmax,
+                 maps, "f", layout.n_tables, Y, "h", M * layout.N, status_out, "B", 4):
+        for t, n in ((X, "X"), (A, "A"), (B, "B")):
+            _dev(t, torch.bfloat16, n)
+        _weight_arrays(layout, packed, absmax, maps)
+        _extent(Y, M * layout.N, "Y", _BF16)
+        _extent(status_out, 4, "status_out")
     if tuple(X.shape) != (M, layout.K) or tuple(A.shape) != (layout.K, r) or tuple(B.shape) != (r, layout.N):
         raise ValueError("shape mismatch")
     if Y is None:
@@ -644,10 +690,15 @@ def lowra_reorder_rows(layout: Layout, to_natural: bool, offsets: torch.Tensor, 
                        absmax_out: Optional[torch.Tensor] = None, stream=None):
     """Grouped <-> natural row order of the packed codes and the absmax rows.  `offsets`: the natural offsets
     as an int64 / uint64 device tensor [N + 1].  Returns (packed_out, absmax_out)."""
-    _dev(packed, torch.uint8, "packed")
-    _dev(absmax, torch.float32, "absmax")
+    n_absmax = layout.N * (layout.K // 64)
+    _layout_here(layout)
+    _dev(packed, torch.uint8, "packed", layout.packed_bytes)
+    _dev(absmax, torch.float32, "absmax", n_absmax)
     if not offsets.is_cuda or offsets.element_size() != 8 or offsets.numel() != layout.N + 1:
         raise ValueError("offsets must be a 64-bit device tensor of N + 1 entries")
+    _extent(offsets, 8 * (layout.N + 1), "offsets")
+    _extent(packed_out, layout.packed_bytes, "packed_out")
+    _extent(absmax_out, n_absmax, "absmax_out", torch.float32)
     if packed_out is None:
         packed_out = torch.empty_like(packed)
     if absmax_out is None:
@@ -663,9 +714,13 @@ def lowra_quant_error(layout: Layout, W: torch.Tensor, maps: torch.Tensor, thres
                       want_residual: bool = False, stream=None):
     """Per-channel summed square error (fp64 [N]) of quantising W with these tables, and optionally the
     residual W - W_hat (fp32 [N,K]).  Returns (sse, residual or None)."""
-    _dev(W, torch.float32, "W")
-    _dev(maps, torch.float32, "maps")
-    _dev(thresholds, torch.float32, "thresholds")
+    if not _fits(layout.device_index, W, "f", 0, maps, "f", 0, thresholds, "f", 0, sse, "d", layout.N, residual, "f", layout.n_weights):
+        _layout_here(layout)
+        _dev(W, torch.float32, "W")
+        _dev(maps, torch.float32, "maps")
+        _dev(thresholds, torch.float32, "thresholds")
+        _extent(sse, layout.N, "sse", torch.float64)
+        _extent(residual, layout.n_weights, "residual", torch.float32)
     if tuple(W.shape) != (layout.N, layout.K) or tuple(maps.shape) != (layout.N, 16) or tuple(thresholds.shape) != (layout.N, 16):
         raise ValueError("shape mismatch")
     if sse is None:
@@ -681,10 +736,12 @@ def lowra_quant_error(layout: Layout, W: torch.Tensor, maps: torch.Tensor, thres
 def lowra_channel_errors(W: torch.Tensor, maps3: torch.Tensor, thresholds3: torch.Tensor,
                          sse3: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """Summed square error of every row of W under 1, 2 and 4 bits (fp64 [N,3]); tables fp32 [3,N,16]."""
-    _dev(W, torch.float32, "W")
-    _dev(maps3, torch.float32, "maps3")
-    _dev(thresholds3, torch.float32, "thresholds3")
     N, K = int(W.shape[0]), int(W.shape[1])
+    if not _fits(W.get_device(), W, "f", 0, maps3, "f", 0, thresholds3, "f", 0, sse3, "d", 3 * N):
+        _dev(W, torch.float32, "W")
+        _dev(maps3, torch.float32, "maps3")
+        _dev(thresholds3, torch.float32, "thresholds3")
+        _extent(sse3, 3 * N, "sse3", torch.float64)
     if tuple(maps3.shape) != (3, N, 16) or tuple(thresholds3.shape) != (3, N, 16):
         raise ValueError("shape mismatch")
     if sse3 is None:
@@ -702,10 +759,14 @@ def lowra_lora_backward_adapters(X, dY, A, B, s: float, dA: Optional[torch.Tenso
                                  dB: Optional[torch.Tensor] = None, workspace: Optional[torch.Tensor] = None,
                                  stream=None) -> Tuple[torch.Tensor, torch.Tensor]:
     """dA = s X^T (dY B^T) [K,r] and dB = s (X A)^T dY [r,N]; all operands bf16 on the device."""
-    for t, n in ((X, "X"), (dY, "dY"), (A, "A"), (B, "B")):
-        _dev(t, torch.bfloat16, n)
     M, K = int(X.shape[0]), int(X.shape[1])
     N, r = int(dY.shape[1]), int(A.shape[1])
+    if not _fits(X.get_device(), X, "h", 0, dY, "h", 0, A, "h", 0, B, "h", 0, dA, "h", K * r, dB, "h", r * N, workspace, "B", 0):
+        for t, n in ((X, "X"), (dY, "dY"), (A, "A"), (B, "B")):
+            _dev(t, torch.bfloat16, n)
+        _extent(dA, K * r, "dA", _BF16)
+        _extent(dB, r * N, "dB", _BF16)
+        _extent(workspace, 0, "workspace")
     if tuple(dY.shape) != (M, N) or tuple(A.shape) != (K, r) or tuple(B.shape) != (r, N):
         raise ValueError("shape mismatch")
     if dA is None:
@@ -741,10 +802,14 @@ def lowra_lora_backward_adapters_reuse(X, dY, T, U, r: int, dA: Optional[torch.T
                                        stream=None) -> Tuple[torch.Tensor, torch.Tensor]:
     """dA = X^T U [K, r] and dB = T^T dY [r, N] from the down-projections T, U (bf16 [M, rp]) that the forward and the
     backward-input call left in their workspaces (lowra_workspace_projection): X and dY are read once."""
-    for t, n in ((X, "X"), (dY, "dY"), (T, "T"), (U, "U")):
-        _dev(t, torch.bfloat16, n)
     M, K, N = int(X.shape[0]), int(X.shape[1]), int(dY.shape[1])
     rp = (int(r) + 63) // 64 * 64
+    if not _fits(X.get_device(), X, "h", 0, dY, "h", 0, T, "h", 0, U, "h", 0, dA, "h", K * r, dB, "h", r * N, workspace, "B", 0):
+        for t, n in ((X, "X"), (dY, "dY"), (T, "T"), (U, "U")):
+            _dev(t, torch.bfloat16, n)
+        _extent(dA, K * r, "dA", _BF16)
+        _extent(dB, r * N, "dB", _BF16)
+        _extent(workspace, 0, "workspace")
     if tuple(dY.shape) != (M, N) or tuple(T.shape) != (M, rp) or tuple(U.shape) != (M, rp):
         raise ValueError("shape mismatch")
     if dA is None:
@@ -788,6 +853,9 @@ def lowra_dense_nt(P: torch.Tensor, Q: torch.Tensor, C: Optional[torch.Tensor] =
     _dev(Q, torch.bfloat16, "Q")
     M, K = P.shape
     N = Q.shape[0]
+    _dev(Q, torch.bfloat16, "Q", N * K)
+    _extent(C, M * N, "C", torch.bfloat16)
+    _extent(workspace, 0, "workspace")
     if C is None:
         C = torch.empty((M, N), dtype=torch.bfloat16, device=P.device)
     if workspace is None:

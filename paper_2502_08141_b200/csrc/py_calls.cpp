@@ -1,5 +1,5 @@
 // The Python binding's short way into the two products (lowra_lora_forward, lowra_lora_backward_input): tensor checks, the output's and
-// the scratch's memory and the call itself without an interpreted line between them.  A call for few tokens is two launches of 2.5 us each
+// the scratch's memory and the call itself without an interpreted line between them; and the tensor checks of the other calls.  A call for few tokens is two launches of 2.5 us each
 // and 10 us on the GPU; with every check, pointer and argument handled by the interpreter its host side took 12 to 14 us.
 //
 // forward / backward_input(layout address, its device, packed, absmax, maps, act, A, B, s, out or None, workspace or None) returns the output,
@@ -93,6 +93,34 @@ PyObject* product(PyObject* const* args, Py_ssize_t n, bool backward) {
 PyObject* forward(PyObject*, PyObject* const* args, Py_ssize_t n) { return product(args, n, false); }
 PyObject* backward_input(PyObject*, PyObject* const* args, Py_ssize_t n) { return product(args, n, true); }
 
+// fits(device, then for each array: tensor or None, element type, least number of elements) -> whether every one is a plain tensor on that
+// device, which is the current one, without gaps, of that type and long enough; None fits.  Types: 'B' bytes of any type, 'u' uint8, 'h' bf16,
+// 'f' fp32, 'd' fp64.  The other calls' checks, a tenth of a microsecond an array where the interpreter takes one; what does not fit is looked at
+// by the interpreter, which says what is wrong.
+PyObject* fits(PyObject*, PyObject* const* args, Py_ssize_t n) {
+    const long dev = n % 3 == 1 ? PyLong_AsLong(args[0]) : -1;
+    bool good = dev >= 0;
+    try {
+        good = good && dev == c10::cuda::current_device();
+        for (Py_ssize_t i = 1; good && i < n; i += 3) {
+            if (args[i] == Py_None) continue;
+            const Py_UCS4 type = PyUnicode_Check(args[i + 1]) && PyUnicode_GET_LENGTH(args[i + 1]) == 1 ? PyUnicode_READ_CHAR(args[i + 1], 0) : 0;
+            const int64_t least = PyLong_AsLongLong(args[i + 2]);
+            if (!plain(args[i])) { good = false; break; }
+            const at::Tensor& t = THPVariable_Unpack(args[i]);
+            if (type == 'B') good = on(t, dev) && (int64_t)t.nbytes() >= least;
+            else good = type != 0 && array(t, type == 'u' ? at::kByte : type == 'h' ? at::kBFloat16 : type == 'f' ? at::kFloat : at::kDouble, least, dev);
+        }
+    } catch (...) {
+        good = false;
+    }
+    if (PyErr_Occurred() != nullptr) {
+        PyErr_Clear();
+        good = false;
+    }
+    return PyBool_FromLong(good);
+}
+
 // bind(addresses of lowra_lora_forward, lowra_lora_backward_input, lowra_workspace_bytes, lowra_workspace_init)
 PyObject* bind(PyObject*, PyObject* const* args, Py_ssize_t n) {
     void* p[4] = {};
@@ -110,6 +138,7 @@ PyObject* bind(PyObject*, PyObject* const* args, Py_ssize_t n) {
 PyMethodDef methods[] = {
     {"forward", (PyCFunction)(void (*)())forward, METH_FASTCALL, nullptr},
     {"backward_input", (PyCFunction)(void (*)())backward_input, METH_FASTCALL, nullptr},
+    {"fits", (PyCFunction)(void (*)())fits, METH_FASTCALL, nullptr},
     {"bind", (PyCFunction)(void (*)())bind, METH_FASTCALL, nullptr},
     {nullptr, nullptr, 0, nullptr},
 };
