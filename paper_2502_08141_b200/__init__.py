@@ -12,6 +12,8 @@ from __future__ import annotations
 import ctypes
 import importlib.util
 import os
+import sysconfig
+import warnings
 from typing import Optional, Tuple
 
 import numpy as np
@@ -19,7 +21,9 @@ import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "liblowra.so")
-PY_CALLS_PATH = os.path.join(_HERE, "_py_calls.so")
+# The extension module holds on to the C++ interface of the Python and the torch that it was compiled against: both are in its name, and another
+# interpreter, which does not find its own, takes the interpreted way.
+PY_CALLS_PATH = os.path.join(_HERE, f"_py_calls.{sysconfig.get_config_var('SOABI')}.torch-{torch.__version__}.so")
 
 LOWRA_OK = 0
 (LOWRA_ERR_NULL, LOWRA_ERR_SHAPE, LOWRA_ERR_ALIGN, LOWRA_ERR_PREC, LOWRA_ERR_WORKSPACE,
@@ -72,11 +76,16 @@ _py_calls = None    # the two products' native way (csrc/py_calls.cpp), loaded w
 
 
 def _load_py_calls(L: ctypes.CDLL):
-    if not os.path.exists(PY_CALLS_PATH):
-        raise RuntimeError(f"{PY_CALLS_PATH} is missing: build it with `python -m paper_2502_08141_b200.build`")
-    spec = importlib.util.spec_from_file_location("paper_2502_08141_b200._py_calls", PY_CALLS_PATH)
-    module = importlib.util.module_from_spec(spec)
-    spec.loader.exec_module(module)
+    """The extension module, or None, with a warning, where there is none for this interpreter: every call then takes the interpreted way, whose host
+    side takes a few microseconds more."""
+    try:
+        spec = importlib.util.spec_from_file_location("paper_2502_08141_b200._py_calls", PY_CALLS_PATH)
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
+    except ImportError as e:
+        warnings.warn(f"no native binding for this Python and torch ({e}): calls take the interpreted way; `python -m paper_2502_08141_b200.build` makes one",
+                      RuntimeWarning, stacklevel=3)
+        return None
     address = lambda fn: ctypes.cast(fn, ctypes.c_void_p).value  # noqa: E731
     module.bind(address(L.lowra_lora_forward), address(L.lowra_lora_backward_input), address(L.lowra_workspace_bytes), address(L.lowra_workspace_init))
     return module
@@ -161,7 +170,8 @@ def lib() -> ctypes.CDLL:
         L.lowra_diag_drop_t_flags.argtypes = [i32]
         L.lowra_diag_drop_t_flags.restype = ctypes.c_int
         _py_calls = _load_py_calls(L)
-        _fits = _py_calls.fits
+        if _py_calls is not None:
+            _fits = _py_calls.fits
         _lib = L
     return _lib
 

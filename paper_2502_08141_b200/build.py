@@ -1,4 +1,5 @@
-"""Compile the CUDA sources into ``liblowra.so`` next to this file (sm_100a only), and the Python binding's native part into ``_py_calls.so``."""
+"""Compile the CUDA sources into ``liblowra.so`` next to this file (sm_100a only), and the Python binding's native part into a
+``_py_calls.*.so`` whose name says for which Python and torch."""
 from __future__ import annotations
 
 import glob
@@ -7,12 +8,13 @@ import shutil
 import subprocess
 import sys
 
+from . import PY_CALLS_PATH as PY_CALLS
+
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "liblowra.so")
 PY_CALLS_SOURCE = os.path.join(CSRC, "py_calls.cpp")
-PY_CALLS = os.path.join(HERE, "_py_calls.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -53,23 +55,27 @@ def build(force: bool = False, verbose: bool = False) -> str:
     nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
     objdir = os.path.join(HERE, "build")
     os.makedirs(objdir, exist_ok=True)
+    run = lambda cmd: subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)  # noqa: E731
+    py_calls = run(_py_calls_command())
     objs = []
-    procs = [(PY_CALLS_SOURCE, subprocess.Popen(_py_calls_command(), stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True))]
+    procs = []
     for src in sources():
         obj = os.path.join(objdir, os.path.basename(src)[:-3] + ".o")
         objs.append(obj)
-        cmd = [nvcc, *NVCC_FLAGS, "-I", os.path.join(ROOT, "include"), "-I", CSRC, "-c", src, "-o", obj]
-        procs.append((src, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
-    failed = False
-    for src, p in procs:
+        procs.append((src, run([nvcc, *NVCC_FLAGS, "-I", os.path.join(ROOT, "include"), "-I", CSRC, "-c", src, "-o", obj])))
+
+    def finished(src, p) -> bool:
         out, _ = p.communicate()
         if verbose or p.returncode != 0:
             sys.stderr.write(f"--- {os.path.basename(src)}\n{out}\n")
-        failed |= p.returncode != 0
-    if failed:
+        return p.returncode == 0
+
+    done = [finished(src, p) for src, p in procs]
+    if all(done):
+        subprocess.run([nvcc, "-shared", "-o", LIB, *objs, "-lcudart"], check=True)
+    # (last: where it does not compile, the library is there all the same, and the calls take the interpreted way)
+    if not finished(PY_CALLS_SOURCE, py_calls) or not all(done):
         raise RuntimeError("compilation failed")
-    cmd = [nvcc, "-shared", "-o", LIB, *objs, "-lcudart"]
-    subprocess.run(cmd, check=True)
     return LIB
 
 
