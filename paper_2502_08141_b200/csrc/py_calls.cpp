@@ -34,6 +34,12 @@ bool matrix(const at::Tensor& t, int64_t rows, int64_t cols, int64_t dev) {
 }
 bool array(const at::Tensor& t, at::ScalarType type, int64_t least, int64_t dev) { return on(t, dev) && t.scalar_type() == type && t.numel() >= least; }
 
+// Other Python threads run while one of these lives.
+struct Released {
+    PyThreadState* state = PyEval_SaveThread();
+    ~Released() { PyEval_RestoreThread(state); }
+};
+
 PyObject* product(PyObject* const* args, Py_ssize_t n, bool backward) {
     if (n != 11 || library.forward == nullptr) Py_RETURN_NONE;
     for (int i = 2; i <= 7; ++i)
@@ -56,28 +62,34 @@ PyObject* product(PyObject* const* args, Py_ssize_t n, bool backward) {
         if (!on(packed, dev) || packed.nbytes() < layout->packed_bytes || !array(absmax, at::kFloat, N * (K / 64), dev) || !array(maps, at::kFloat, N * 16, dev)) Py_RETURN_NONE;
         if (out_given && !array(THPVariable_Unpack(args[9]), at::kBFloat16, M * cols, dev)) Py_RETURN_NONE;
         if (workspace_given && !on(THPVariable_Unpack(args[10]), dev)) Py_RETURN_NONE;
-        at::Tensor out = out_given ? THPVariable_Unpack(args[9]) : at::empty({M, cols}, act.options().requires_grad(false));
-        void* stream = c10::cuda::getCurrentCUDAStream().stream();
-        at::Tensor workspace;
-        if (workspace_given) {
-            workspace = THPVariable_Unpack(args[10]);
-        } else {
-            const size_t bytes = library.workspace_bytes(layout, (int32_t)M, (int32_t)r);
-            if (bytes == 0) Py_RETURN_NONE;
-            workspace = at::empty({(int64_t)bytes}, act.options().requires_grad(false).dtype(at::kByte));
-            if (layout->deal_dev != nullptr && library.workspace_init(workspace.data_ptr(), bytes, stream) != LOWRA_OK) Py_RETURN_NONE;   // no prologue launch will clear it
-        }
         const Product call = backward ? library.backward_input : library.forward;
         const auto* packed_p = static_cast<const uint8_t*>(packed.data_ptr());
         const auto *absmax_p = static_cast<const float*>(absmax.data_ptr()), *maps_p = static_cast<const float*>(maps.data_ptr());
         const auto *act_p = static_cast<const uint16_t*>(act.data_ptr()), *A_p = static_cast<const uint16_t*>(A.data_ptr()), *B_p = static_cast<const uint16_t*>(B.data_ptr());
-        auto* out_p = static_cast<uint16_t*>(out.data_ptr());
-        void* workspace_p = workspace.data_ptr();
-        const size_t workspace_n = (size_t)workspace.numel();
-        lowra_status st;
-        Py_BEGIN_ALLOW_THREADS
-        st = call(layout, packed_p, absmax_p, maps_p, act_p, (int32_t)M, A_p, B_p, (int32_t)r, (float)s, out_p, workspace_p, workspace_n, stream);
-        Py_END_ALLOW_THREADS
+        const at::TensorOptions options = act.options().requires_grad(false);
+        at::Tensor out, workspace;
+        if (out_given) out = THPVariable_Unpack(args[9]);
+        if (workspace_given) workspace = THPVariable_Unpack(args[10]);
+        lowra_status st = LOWRA_ERR_WORKSPACE;
+        bool called = false;
+        {
+            Released released;      // (allocations included: one that has to ask the driver for memory takes its time)
+            void* stream = c10::cuda::getCurrentCUDAStream().stream();
+            if (!out_given) out = at::empty({M, cols}, options);
+            bool ready = true;
+            if (!workspace_given) {
+                const size_t bytes = library.workspace_bytes(layout, (int32_t)M, (int32_t)r);
+                ready = bytes > 0;
+                if (ready) workspace = at::empty({(int64_t)bytes}, options.dtype(at::kByte));
+                if (ready && layout->deal_dev != nullptr) ready = library.workspace_init(workspace.data_ptr(), bytes, stream) == LOWRA_OK;   // no prologue launch will clear it
+            }
+            if (ready) {
+                st = call(layout, packed_p, absmax_p, maps_p, act_p, (int32_t)M, A_p, B_p, (int32_t)r, (float)s, static_cast<uint16_t*>(out.data_ptr()),
+                          workspace.data_ptr(), (size_t)workspace.numel(), stream);
+                called = true;
+            }
+        }
+        if (!called) Py_RETURN_NONE;
         if (st != LOWRA_OK) return PyLong_FromLong(st);
         if (out_given) {
             Py_INCREF(args[9]);
