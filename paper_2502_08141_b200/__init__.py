@@ -39,7 +39,7 @@ EXPORTS = (
     "lowra_learn_codebooks_all", "lowra_lora_forward_adapters", "lowra_batch_workspace_bytes",
     "lowra_lora_forward_batch", "lowra_lora_backward_input_batch", "lowra_lora_backward_adapters_reuse",
     "lowra_workspace_projection", "lowra_set_wait_limit", "lowra_diag_wait_expiry", "lowra_diag_drop_t_flags",
-    "lowra_encode_group", "lowra_decode_group",
+    "lowra_encode_group", "lowra_decode_group", "lowra_diag_choose",
 )
 
 
@@ -58,6 +58,10 @@ class _CLayout(ctypes.Structure):
         ("precs_dev", ctypes.c_void_p), ("perm_dev", ctypes.c_void_p), ("inv_perm_dev", ctypes.c_void_p),
         ("deal_dev", ctypes.c_void_p), ("natural_offsets_dev", ctypes.c_void_p),
     ]
+
+
+class _CChoice(ctypes.Structure):
+    _fields_ = [(name, ctypes.c_int32) for name in ("few_tokens", "units", "tile_tokens", "clusters", "w_split", "t_split")]
 
 
 class _CGroupMember(ctypes.Structure):
@@ -169,6 +173,8 @@ def lib() -> ctypes.CDLL:
         L.lowra_diag_wait_expiry.restype = ctypes.c_int
         L.lowra_diag_drop_t_flags.argtypes = [i32]
         L.lowra_diag_drop_t_flags.restype = ctypes.c_int
+        L.lowra_diag_choose.argtypes = [lp, i32, vp, i32, i32, i32, ctypes.POINTER(_CChoice)]
+        L.lowra_diag_choose.restype = ctypes.c_int
         _py_calls = _load_py_calls(L)
         if _py_calls is not None:
             _fits = _py_calls.fits
@@ -854,6 +860,15 @@ def lowra_diag_wait_expiry(workspace: torch.Tensor, limit_ns: int, stream=None) 
 def lowra_diag_drop_t_flags(calls: int) -> None:
     """Self test: the next `calls` fused calls do not publish their "down-projection ready" flags and time out."""
     _check(lib().lowra_diag_drop_t_flags(int(calls)), "lowra_diag_drop_t_flags")
+
+
+def lowra_diag_choose(layout: Layout, backward: bool, tokens, r: int, one_weight: bool = False) -> dict:
+    """What a launch for members of these token counts runs (host only): dict(few_tokens, units, tile_tokens, clusters, w_split, t_split)."""
+    counts = np.ascontiguousarray(tokens, dtype=np.int32).reshape(-1)
+    choice = _CChoice()
+    _check(lib().lowra_diag_choose(layout.ref, int(backward), counts.ctypes.data, int(counts.size), int(one_weight), int(r), ctypes.byref(choice)),
+           "lowra_diag_choose")
+    return {name: int(getattr(choice, name)) for name, _ in choice._fields_}
 
 
 def lowra_dense_nt(P: torch.Tensor, Q: torch.Tensor, C: Optional[torch.Tensor] = None,

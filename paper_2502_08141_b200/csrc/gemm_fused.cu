@@ -1020,6 +1020,27 @@ float fused_estimate(int N, int K, int M, int r, bool mixed, int count) {
     return us * (float)((count + kMaxBatch - 1) / kMaxBatch);
 }
 
+// The schedule of a call of `count` members on a whole GPU, its clusters returned.
+int fused_schedule(bool backward, int N, int K, const int32_t* Ms, int count, int r, int* tile_tokens, int* w_split, int* t_split) {
+    GemmParams Q;
+    memset(&Q, 0, sizeof(Q));
+    Q.count = count;
+    for (int i = 0; i < count; ++i) {
+        Q.mem[i].M = Ms[i];
+        Q.M = Ms[i] > Q.M ? Ms[i] : Q.M;
+    }
+    Q.C = backward ? N : K;
+    Q.main_blocks = (Q.C + kTileC - 1) / kTileC;
+    Q.lora_blocks = (r + 63) / 64;
+    Q.tiles_r = ((backward ? K : N) + kPairR - 1) / kPairR;
+    Q.part_halves = 2;
+    const int clusters = plan_schedule(Q, true, kNumSMs / kCluster);
+    *tile_tokens = Q.halves * kHalfT;
+    *w_split = Q.w_split;
+    *t_split = Q.t_split;
+    return clusters;
+}
+
 // How many clusters can be resident at once, and that the kernel may have its shared memory: once per kernel and device.
 template <int MODE, int NB, bool SHARED>
 static lowra_status prepare_fused(cudaLaunchConfig_t& cfg, int* max_clusters) {

@@ -427,6 +427,39 @@ extern "C" lowra_status lowra_lora_backward_input(const lowra_layout* layout, co
                            workspace_dev, workspace_bytes, stream);
 }
 
+extern "C" lowra_status lowra_diag_choose(const lowra_layout* layout, int32_t backward, const int32_t* tokens_host, int32_t count, int32_t one_weight,
+                                          int32_t r, lowra_diag_choice* out) {
+    using namespace lowra;
+    if (!layout || !tokens_host || !out) return LOWRA_ERR_NULL;
+    const int N = layout->N, K = layout->K;
+    if (N < 8 || N % 8 != 0 || K < 128 || K % 128 != 0 || layout->counts[0] + layout->counts[1] + layout->counts[2] != N || !rank_ok(r) || count < 1 ||
+        count > kSmallMembers)
+        return LOWRA_ERR_SHAPE;
+    SmallParams<kSmallMembers> P;
+    memset(&P, 0, sizeof(P));
+    P.N = N;
+    P.K = K;
+    P.count = count;
+    P.one_weight = one_weight != 0 || count == 1;
+    int most = 0;
+    for (int i = 0; i < count; ++i) {
+        if (tokens_host[i] < 1) return LOWRA_ERR_SHAPE;
+        most = tokens_host[i] > most ? tokens_host[i] : most;
+        P.m[i].L = make_row_layout(layout);
+        P.m[i].M = tokens_host[i];
+    }
+    memset(out, 0, sizeof(*out));
+    out->w_split = out->t_split = 1;
+    if (takes_small_path(backward != 0, N, K, most, r, mixes_4_bits(layout))) {
+        out->few_tokens = 1;
+        out->units = small_takes_units(P) ? 1 : 0;
+        return LOWRA_OK;
+    }
+    if (count > kMaxBatch) return LOWRA_ERR_SHAPE;
+    out->clusters = fused_schedule(backward != 0, N, K, tokens_host, count, r, &out->tile_tokens, &out->w_split, &out->t_split);
+    return LOWRA_OK;
+}
+
 static_assert(LOWRA_MAX_BATCH == lowra::kMaxBatch, "header and kernel agree on the batch limit");
 
 extern "C" size_t lowra_batch_workspace_bytes(const lowra_layout* layout, int32_t count, int32_t M, int32_t r) {

@@ -145,6 +145,7 @@ static_assert(kGemmSmemBytes <= 232448, "227 KB of shared memory per CTA");
 
 lowra_status launch_fused(int mode, const GemmParams& G, const BatchMaps& TM, cudaStream_t stream);
 float fused_estimate(int N, int K, int M, int r, bool mixed, int count = 1);
+int fused_schedule(bool backward, int N, int K, const int32_t* Ms, int count, int r, int* tile_tokens, int* w_split, int* t_split);   // what a call would run (diagnostic)
 
 // ---- forward pass for few tokens (gemm_small.cu) --------------------------------------------
 constexpr int kSmallTokens = 64;    // members of up to so many tokens may take it, of 16 and fewer do
@@ -169,6 +170,7 @@ struct SmallParams {
     int one_weight;           // all members have the same layout, codes and absmax (several adapters)
 };
 lowra_status launch_small(const SmallParams<kSmallMembers>& P, cudaStream_t stream);
+bool small_takes_units(const SmallParams<kSmallMembers>& P);     // whether that launch is units_kernel
 
 // One skinny product D [R, rp] = P . Q (see gemm_grad.cu), written in bf16 as out [R, ld_out] or, transposed,
 // as out [n_cols, ld_out].

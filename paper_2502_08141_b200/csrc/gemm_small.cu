@@ -692,16 +692,26 @@ int product_slices(int N, int K) {
     return slices;
 }
 
+// groups of 64 stored rows of one precision (of the member that has the most)
+template <int NB>
+int row_groups(const SmallParams<NB>& P) {
+    int groups = 0;
+    for (int i = 0; i < P.count; ++i) {
+        int n = 0;
+        for (int c = 0; c < 3; ++c) n += (P.m[i].L.class_start[c + 1] - P.m[i].L.class_start[c] + kSmallRows - 1) / kSmallRows;
+        groups = n > groups ? n : groups;
+    }
+    return groups;
+}
+
 template <int NB>
 lowra_status launch_members(const SmallParams<NB>& P, cudaStream_t stream) {
-    int m16 = 0, groups = 0, most = 0;
+    int m16 = 0, most = 0;
+    const int groups = row_groups(P);
     for (int i = 0; i < P.count; ++i) {
         const SmallMember& m = P.m[i];
         m16 += (m.M + 15) / 16;
         most = m.M > most ? m.M : most;
-        int n = 0;
-        for (int c = 0; c < 3; ++c) n += (m.L.class_start[c + 1] - m.L.class_start[c] + kSmallRows - 1) / kSmallRows;
-        groups = n > groups ? n : groups;
     }
     // ---- T: the contraction over up to eight CTAs, 128 indices or more each
     {
@@ -757,6 +767,8 @@ float small_estimate(int N, int K, int M, int count) {
     const float cta_us = 1.7f + 0.4f * (M > 32 ? 3 : (M + 7) / 8 - 4) + 2.7f * n_span / (2.0f * slices) + 6.0f / slices;
     return 6.0f + cta_us * (per_sm / 2 + (per_sm % 2 != 0 ? 0.65f : 0.0f));
 }
+
+bool small_takes_units(const SmallParams<kSmallMembers>& P) { return P.one_weight && units_pay(P, row_groups(P), product_slices(P.N, P.K)); }
 
 // (A call with one member carries 0.3 KB of kernel parameters instead of 1.5 KB, which its launches show.)
 lowra_status launch_small(const SmallParams<kSmallMembers>& P, cudaStream_t stream) {
