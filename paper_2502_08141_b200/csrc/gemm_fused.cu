@@ -54,6 +54,7 @@ constexpr int kPartSlots = kSlotsX + kSlotsW, kMaxContributors = kPartSlots / 2,
 constexpr int kSharedTFlags = (kMaxClusters * kCluster + 7) / 8 * 8;
 static_assert(kMaxContributors <= kTFlags, "a flag for every cluster that shares a T tile");
 constexpr int kRankCols = 128;                   // columns of a T tile: the ranks, padded
+static_assert(2 * kRankCols <= kPairR, "two T tiles in the place of one partial tile");
 constexpr uint32_t kIdesc = ptx::umma_idesc_bf16(kHalfT, kPairR), kIdescT = ptx::umma_idesc_bf16(kHalfT, kRankCols);
 constexpr uint32_t kIdescBmn = 1u << 16;         // operand B MN-major
 
@@ -518,7 +519,10 @@ fused_kernel(const __grid_constant__ KParams<NB> P, const __grid_constant__ KMap
             const int cols = t.is_t ? P.rp : min(kPairR, P.R - r0);   // rows of the tile that exist
             // the columns c0, c0 + 32, ... that this warp takes: half of the tile's; a T tile has few
             const int c_first = t.is_t ? ch * 32 : ch * 128, c_step = t.is_t ? 64 : 32, c_last = t.is_t ? cols : min(cols, ch * 128 + 128);
-            auto part_of = [&](int c) { return P.sk_part + ((size_t)(SHARED && c == 0 ? P.sk_slot0 : c) * CL + crank) * kSkHalfFloats; };   // cluster c's place
+            // Cluster c's place.  Cluster 0 has partial tiles only where it shares a T tile; they lie in cluster 1's place, behind those of its T tile.
+            auto part_of = [&](int c) {
+                return P.sk_part + ((size_t)(SHARED && c == 0 ? 1 : c) * CL + crank) * kSkHalfFloats + (SHARED && c == 0 ? kRankCols * 128 : 0);
+            };
             float* const part = part_of(cid) + my_tok;
             // 32 rows of one token: rounded and stored
             auto put = [&](uint16_t* dst, int left, uint32_t (&v)[32]) {
@@ -939,7 +943,7 @@ static int plan_schedule(GemmParams& Q, bool may_cut, int max_clusters, float* e
         // it, 1.5 more for its second half.
         auto shared_t = [&](int ts) { return 10.7f + 1.5f * halves + 0.42f * Q.main_blocks / ts; };
         for (int s = 1; s < kMaxContributors && n_w * s + n_t <= max_clusters && blocks / s >= shortest; ++s) {
-            int ts = ((max_clusters < kMaxClusters ? max_clusters : kMaxClusters - 1) - n_w * s) / n_t;     // (there are partial tiles for one cluster less)
+            int ts = (max_clusters - n_w * s) / n_t;
             if (ts > kMaxContributors) ts = kMaxContributors;
             if (ts > Q.main_blocks / kMinShare) ts = Q.main_blocks / kMinShare;
             if (ts < 2 || Q.main_blocks < 2 * kMinRange) ts = 1;
@@ -995,7 +999,6 @@ static int plan_schedule(GemmParams& Q, bool may_cut, int max_clusters, float* e
     Q.sk_num = best.num;
     Q.t_split = best.t_split;
     Q.w_split = best.w_split;
-    Q.sk_slot0 = best.w_split > 1 ? best.clusters : best.c0;
     if (estimate != nullptr) *estimate = best.us;
     return best.clusters;
 }

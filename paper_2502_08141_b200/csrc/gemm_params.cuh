@@ -109,13 +109,12 @@ struct GemmCommon {
     int tiles_r;            // tiles of 256 operand rows of a member (all members have one shape)
     // schedule of the tiles that are cut between clusters (set by the launcher; sk == 0: whole tiles, dealt round-robin)
     float* sk_part;         // fp32 partial tiles: for either half of the tokens, [kCluster][256 rows][128 tokens] per cluster.  Points in front of them by
-                            // the place of cluster 0, which has one only where it shares a T tile (sk_slot0).
+                            // the place of cluster 0, which has none of its own.
     int part_halves;        // (host) halves of a token tile that the slots have room for: 2, or 1, or 0 (no tile is cut)
     uint32_t* sk_flags;     // [clusters][kCluster] raised when a CTA's partial tile is complete
     int halves;             // token tiles of 256 (1) or 512 tokens (2)
     int t_split;            // > 1: so many clusters share a T tile, and do nothing else
     int w_split;            // > 1: so many clusters share a weight tile, from cluster sk_c0 on, and do nothing else
-    int sk_slot0;           // the cluster whose place for partial tiles cluster 0 uses (one that needs none, or the one past the last)
     int sk;
     int sk_c0;              // the first cluster that gets a range
     int sk_first;           // first weight tile of the ranges
