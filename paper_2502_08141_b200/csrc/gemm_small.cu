@@ -619,20 +619,34 @@ __global__ void __launch_bounds__(kSmallThreads, 2) units_kernel(const __grid_co
     else work(std::integral_constant<int, 4>());
 }
 
-// Whether a CTA for every group of 64 rows and unit beats one for every slice of it.  Both in microseconds, two CTAs to an SM: of the former 3 and
-// 1.2 for every slice, of the latter 5.5; and 2 (1, 2 bits) to 2.6 (4 bits) for a step.  The long ones leave SMs idle at the end, more so where all
-// are alike.  (Against the slices, us: 4096 x 4096 at 30/50/20 %, 101 tokens in 6 groups 66.0 -> 48.6, 64 in 8 72 -> 46, 60 in 3 34.4 -> 29.9, 16 in
+// Whether a CTA for every group of 64 rows and unit beats one for every slice of it, for a weight of n[0], n[1], n[2] channels at 1, 2 and 4 bits and so many
+// units, the largest member of `most` tokens.  Both in microseconds, two CTAs to an SM: of the former 3 and 1.2 for every slice, of the latter 5.5; and
+// 2 (1, 2 bits) to 2.6 (4 bits) for a step.  The long ones leave SMs idle at the end, more so where all are alike; a few of them with rows of 4 bits, more
+// than 16 tokens and ranks up to 64 are 1.5 slower.  Over 288 calls that take units (256 to 13824 channels, 512 to 13824 features, 2 to 8 groups, single calls of
+// 33 to 64 tokens, ranks 16 to 128, six mixes) they take 0.90 of the slices' time in the mean; the choice is 0.5 % behind the better form, 10 % at most,
+// and 10 calls are more than 3 % behind the slices (25 without the 1.5: 264 x 512, 44 tokens at 2 and 4 bits 7.9 us, 9.1 by units).
+// (Against the slices, us: 4096 x 4096 at 30/50/20 %, 101 tokens in 6 groups 66.0 -> 48.6, 64 in 8 72 -> 46, 60 in 3 34.4 -> 29.9, 16 in
 // 8 48.5 -> 38.7; at 4 bits 101 in 6 66.4 -> 55.4.  Not taken: 4 in 2 there 19.3 -> 19.8, 64 in one 26.9 -> 31.5; 4096 x 11008 of 4 bits 60 in 3 71 -> 83.)
-template <int NB>
-bool units_pay(const SmallParams<NB>& P, int groups, int slices) {
-    int units = 0;
-    for (int i = 0; i < P.count; ++i) units += (P.m[i].M + kUnitTokens - 1) / kUnitTokens;
+bool units_faster(const int* n, int K, int r, int units, int most, int slices) {
     if (units < 2) return false;
+    const int N = n[0] + n[1] + n[2], ctas = ((n[0] + 63) / 64 + (n[1] + 63) / 64 + (n[2] + 63) / 64) * units;
+    const bool alike = n[0] == N || n[1] == N || n[2] == N;
+    const float wide = n[2] > 0 && most > 16 && r <= 64 && ctas <= kNumSMs ? 1.5f : 0.0f;
+    const float step = 2.0f + 0.6f * (float)n[2] / (float)N, steps = 0.5f * (float)((K + kSmallSpan - 1) / kSmallSpan);
+    const float waves = (float)ctas / (2 * kNumSMs), spread = waves * slices, whole = waves + (alike ? 0.35f : 0.15f);
+    return (whole > 1.0f ? whole : 1.0f) * (3.0f + wide + 1.2f * slices + step * steps) < (spread > 1.0f ? spread : 1.0f) * (5.5f + step * steps / slices);
+}
+
+template <int NB>
+bool units_pay(const SmallParams<NB>& P, int slices) {
+    int units = 0, most = 0;
+    for (int i = 0; i < P.count; ++i) {
+        units += (P.m[i].M + kUnitTokens - 1) / kUnitTokens;
+        most = P.m[i].M > most ? P.m[i].M : most;
+    }
     const int* start = P.m[0].L.class_start;
-    const bool alike = start[1] == P.N || (start[1] == 0 && start[2] == P.N) || start[2] == 0;
-    const float step = 2.0f + 0.6f * (float)(start[3] - start[2]) / (float)P.N, steps = 0.5f * (float)((P.K + kSmallSpan - 1) / kSmallSpan);
-    const float waves = (float)(groups * units) / (2 * kNumSMs), spread = waves * slices, whole = waves + (alike ? 0.35f : 0.15f);
-    return (whole > 1.0f ? whole : 1.0f) * (3.0f + 1.2f * slices + step * steps) < (spread > 1.0f ? spread : 1.0f) * (5.5f + step * steps / slices);
+    const int n[3] = {start[1] - start[0], start[2] - start[1], start[3] - start[2]};
+    return units_faster(n, P.K, P.r, units, most, slices);
 }
 
 template <int NB>
@@ -739,7 +753,7 @@ lowra_status launch_members(const SmallParams<NB>& P, cudaStream_t stream) {
     // a step of 256.  The choice depends on the weight's shape alone, so that a member's result does not depend on its company.
     const int n_span = (P.K + kSmallSpan - 1) / kSmallSpan, slices = product_slices(P.N, P.K);
     const int nt8 = most <= 8 ? 1 : most <= 16 ? 2 : most <= 24 ? 3 : 4;
-    if (P.one_weight && units_pay(P, groups, slices)) return launch_units<NB>(P, groups, slices, stream);
+    if (P.one_weight && units_pay(P, slices)) return launch_units<NB>(P, groups, slices, stream);
     int units = 0;
     for (int i = 0; i < P.count; ++i) units += (P.m[i].M + 8 * nt8 - 1) / (8 * nt8);
     // Merged where a CTA's own cost outweighs its steps: slots of one or two steps, few tokens, more CTAs than run at a time.  (Groups of
@@ -768,7 +782,7 @@ float small_estimate(int N, int K, int M, int count) {
     return 6.0f + cta_us * (per_sm / 2 + (per_sm % 2 != 0 ? 0.65f : 0.0f));
 }
 
-bool small_takes_units(const SmallParams<kSmallMembers>& P) { return P.one_weight && units_pay(P, row_groups(P), product_slices(P.N, P.K)); }
+bool small_takes_units(const SmallParams<kSmallMembers>& P) { return P.one_weight && units_pay(P, product_slices(P.N, P.K)); }
 
 // (A call with one member carries 0.3 KB of kernel parameters instead of 1.5 KB, which its launches show.)
 lowra_status launch_small(const SmallParams<kSmallMembers>& P, cudaStream_t stream) {

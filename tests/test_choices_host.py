@@ -51,6 +51,18 @@ def test_groups_of_few_tokens():
     assert lw.lowra_diag_choose(layout, False, [8] * 8, 64)["units"] == 0          # weights of their own
 
 
+@pytest.mark.parametrize("N,K,r,mix,tokens,units", [
+    (264, 512, 16, {2: 0.75, 4: 0.25}, [44], 0),                  # wide units of 4-bit rows: slower than the slices (9.1 us, 7.9)
+    (1720, 512, 48, {4: 1.0}, [34], 0),
+    (4528, 640, 64, {1: 0.5, 2: 0.5}, [58], 1),                   # faster without 4-bit rows (8.6 us, 10.2)
+    (4632, 512, 64, {1: 0.85, 2: 0.15}, [1] * 8, 1),
+    (5800, 640, 64, {1: 0.3, 2: 0.5, 4: 0.2}, [8] * 7, 1),        # and with them in narrow units
+])
+def test_units_where_they_are_faster(N, K, r, mix, tokens, units):
+    assert lw.lowra_diag_choose(layout_of(N, K, mix), False, tokens, r, one_weight=True) == dict(few_tokens=1, units=units, tile_tokens=0, clusters=0,
+                                                                                                 w_split=1, t_split=1)
+
+
 @pytest.mark.parametrize("tokens,r,code", [([0], 64, "SHAPE"), ([1] * 9, 64, "SHAPE"), ([100] * 5, 64, "SHAPE"), ([1], 24, "SHAPE")])
 def test_refusals(tokens, r, code):
     with pytest.raises(lw.LowraError) as e:
