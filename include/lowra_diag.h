@@ -52,12 +52,12 @@ lowra_status lowra_diag_drop_t_flags(int32_t calls);
 /*
  * (No counterpart in the paper.)  What a launch of the forward (backward == 0) or the backward-input pass runs on a whole GPU for `count` members of
  * this layout with tokens_host[i] tokens each: a plain call (count 1), the members of a batch call, or (one_weight != 0) the token groups of
- * lowra_lora_forward_adapters that go into one launch.  Host only: no device is needed, nothing is launched, and layout's device arrays may be NULL.
+ * lowra_lora_forward_adapters that go into one launch, all of them.  Host only: no device is needed, nothing is launched, and layout's device arrays may be NULL.
  * Tests use it to know that a shape reaches the code that they are about.
  * Errors: NULL pointer -> LOWRA_ERR_NULL; a shape the calls refuse, count < 1 or more members than a launch takes -> LOWRA_ERR_SHAPE.
  */
 typedef struct {
-    int32_t few_tokens;  /* 1: the path for few tokens, and there */
+    int32_t few_tokens;  /* 1: the path for few tokens, for every member, and there */
     int32_t units;       /*    1: a CTA does all slices for one unit of up to 32 tokens; 0: a CTA to a slice */
     int32_t tile_tokens; /* otherwise the tensor-core kernel, in tiles of 256 or 512 tokens (0 on the path for few), */
     int32_t clusters;    /*    on so many pairs of SMs, */

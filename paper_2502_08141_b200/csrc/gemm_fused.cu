@@ -905,12 +905,13 @@ fused_kernel(const __grid_constant__ KParams<NB> P, const __grid_constant__ KMap
     }
 }
 
-// Chooses the token tiles (256 or 512 tokens) and the schedule of a call - whole tiles, or ranges behind so many whole weight
-// tiles (see the kernel) - and returns the number of clusters to launch.  What is compared is an estimate of the call's time, in
-// microseconds at full clock, from device timestamps of 256- to 4096-token calls on 4096 x 4096 and 11008 x 4096 weights:
-//   4.5 until the first MMA; 0.6 / 0.8 per contraction block of a 256- / 512-token tile (the smaller one paced by dequantisation,
-//   the larger one by the tensor core); 0.5 / 0.7 of a T tile (paced by its loads); 2.4 per 256 tokens to write a partial tile or to
-//   drain the last accumulator; to collect partial tiles 4.5 and, per 256 tokens, four steps of 1.1 or 0.6 per contributor.
+// Chooses the token tiles (256 or 512 tokens) and the schedule of a call - whole tiles, shared ones, or ranges behind so many whole weight
+// tiles (see the kernel) - and returns the number of clusters to launch.  What is compared is an estimate of the call's time, in microseconds at full
+// clock.  Its figures are a fit to the times of every schedule that 530 calls could take (17 to 8192 tokens, 256 to 13824 channels and features,
+// ranks 16 to 128, six mixes of precisions, both directions), by the errors and by what the choice loses against the best one; estimates are within 7 %
+// of the times (one standard deviation).  On 190 other calls, each in both directions, the choice is 0.5 % behind the best schedule in the mean and more
+// than 5 % behind for 2 % of them.  (With the figures before, from a few shapes: 1.5 %, 10 %; most of it 512-token tiles shared at ranks above 64:
+// backward 2672 x 1152, 1437 tokens, rank 128 34.7 us, now 28.4; forward 5016 x 2944, 404 tokens 36.1, now 30.8.)
 static int plan_schedule(GemmParams& Q, bool may_cut, int max_clusters, float* estimate = nullptr) {
     const int blocks = Q.main_blocks + Q.lora_blocks;
     struct Choice { float us; int halves, clusters, cut, first, c0, extra, t_split, num, w_split; } best = {};
@@ -924,32 +925,30 @@ static int plan_schedule(GemmParams& Q, bool may_cut, int max_clusters, float* e
     // every range keeps a sixth of a tile, so that a tile has at most kMaxContributors contributors
     const int sixth = (blocks + kMaxContributors - 2) / (kMaxContributors - 1), shortest = sixth > kMinRange ? sixth : kMinRange;
     for (int halves = Q.wide_only ? 2 : 1; halves <= (Q.M > kHalfT ? 2 : 1); ++halves) {
-        const float pace = halves == 1 ? 0.6f : 0.8f, t_pace = halves == 1 ? 0.5f : 0.7f;
-        const float ramp = 4.5f, drain = 2.4f * halves;
-        auto collect = [&](int nc) { return 4.5f + 4.0f * halves * (0.6f * nc > 1.1f ? 0.6f * nc : 1.1f); };
+        const float pace = halves == 1 ? 0.51f : 0.76f;         // a contraction block of a weight tile (256 tokens: the dequantising warps'; 512: the tensor core's)
+        auto collect = [&](int nc) { return 4.0f * halves * (0.6f * nc > 1.57f ? 0.6f * nc : 1.57f); };    // four steps per 256 tokens
         const int super_t = tiles_of(halves), n_t = may_cut ? super_t : 0, n_w = Q.tiles_r * super_t, n = n_w + n_t;
-        // when whole T tiles are there (256 tokens: device timestamps of 1800 x 2304, 777 tokens)
-        const float t_us = halves == 1 ? 8.2f + 0.4f * Q.main_blocks : ramp + t_pace * Q.main_blocks + 3.0f;
-        auto short_us = [&](float n) { return 5.0f + (halves == 1 ? 0.52f : 0.8f) * n; };      // MMAs of a cluster's only piece
+        // when T is there: whole tiles, tiles that ts clusters share
+        const float t_us = halves == 1 ? 9.4f + 0.44f * Q.main_blocks : 14.4f + 0.62f * Q.main_blocks;
+        auto shared_t = [&](int ts) { return 7.0f + 0.43f * Q.main_blocks / ts + halves * (6.2f + 1.7f * (Q.lora_blocks - 1)); };
+        auto single_us = [&](float n) { return 8.2f + (halves == 1 ? 0.5f : 0.76f) * n; };                // a cluster's only piece, n blocks
         {   // whole tiles
             const int clusters = n < max_clusters ? n : max_clusters, rows = (n + clusters - 1) / clusters;
-            const float w_us = rows == 1 ? short_us(blocks) : ramp + pace * blocks * rows;
-            offer({(rows == 1 && n_t > 0 && t_us > w_us ? t_us : w_us) + drain, halves, clusters, 0, 0, 0, 0, 1, 0, 1});
+            // (a second row of no more pieces than there are T tiles: they go to the clusters that had one of those, and nobody hands accumulators over)
+            const float w_us = rows == 1 || (rows == 2 && n - clusters <= n_t) ? single_us(blocks * rows) : 14.9f + pace * blocks * rows;
+            offer({(rows == 1 && n_t > 0 && t_us > w_us ? t_us : w_us) - 0.7f * halves, halves, clusters, 0, 0, 0, 0, 1, 0, 1});
         }
         if (!may_cut || halves > Q.part_halves || n_t > max_clusters || blocks < 2 * kMinRange) continue;
         if ((long long)n * blocks * max_clusters >= (1ll << 31)) continue;     // (32-bit arithmetic in the kernel)
-        // Fewer pieces than clusters: s clusters share every weight tile, and those left over the T tiles.  From the end of a shared tile's MMAs to that of its
-        // stores it takes 4.5 and 3.5 for every 256 tokens; a shared T tile 0.42 per block, 9.2 around them and 1.5 for the low-rank blocks behind
-        // it, 1.5 more for its second half.
-        auto shared_t = [&](int ts) { return 10.7f + 1.5f * halves + 0.42f * Q.main_blocks / ts; };
+        // Fewer pieces than clusters: s clusters share every weight tile, and those left over the T tiles.
         for (int s = 1; s < kMaxContributors && n_w * s + n_t <= max_clusters && blocks / s >= shortest; ++s) {
             int ts = (max_clusters - n_w * s) / n_t;
             if (ts > kMaxContributors) ts = kMaxContributors;
             if (ts > Q.main_blocks / kMinShare) ts = Q.main_blocks / kMinShare;
             if (ts < 2 || Q.main_blocks < 2 * kMinRange) ts = 1;
             if (ts == 1 && s == 1) continue;
-            const float t_done = ts == 1 ? t_us : shared_t(ts), w_done = short_us((float)blocks / s);
-            const float us = (t_done > w_done ? t_done : w_done) + (s == 1 ? drain : 4.5f + 3.5f * halves);
+            const float t_done = ts == 1 ? t_us : shared_t(ts), w_done = single_us((float)blocks / s);
+            const float us = (t_done > w_done ? t_done : w_done) + (s == 1 ? -0.7f * halves : 3.5f + 2.5f * halves);
             offer({us, halves, n_t * ts + n_w * s, 1, 0, n_t * ts, 0, ts, n_w * blocks, s});
         }
         // T by clusters of its own, each tile by ts of them, and ranges over all weight tiles for the others: for few channels and many tokens, where one
@@ -962,14 +961,14 @@ static int plan_schedule(GemmParams& Q, bool may_cut, int max_clusters, float* e
             const int c = max_clusters - n_t * ts;
             const float range = (float)n_w * blocks / c;
             if (range < shortest || 2.0f * range < blocks) continue;      // (longer with every ts)
-            const float t_done = ts == 1 ? t_us : shared_t(ts), w_done = ramp + pace * range;
-            offer({(t_done > w_done ? t_done : w_done) + drain + collect((int)((blocks + range - 1) / range)) + 1.5f, halves, max_clusters, 1, 0, n_t * ts, 0, ts, n_w * blocks, 1});
+            const float t_done = ts == 1 ? t_us : shared_t(ts), w_done = 12.1f + pace * range;
+            offer({(t_done > w_done ? t_done : w_done) - 1.4f - 0.7f * halves + collect((int)((blocks + range) / range)), halves, max_clusters, 1, 0, n_t * ts, 0, ts, n_w * blocks, 1});
         }
         // Ranges for the last row of pieces, or for the last two.  The clusters' sweeps over the contraction fall out of step
         // inside the ranges, so the part of the token operand that is live there has to stay in L2 (ranges over all tiles of a
         // 90 MB operand: 6.5 times the DRAM reads, and no gain).
         const int rows = n / max_clusters, n_last = n - rows * max_clusters;
-        const int t_cost = (int)(blocks * t_pace / pace);                       // a T tile, in blocks
+        const int t_cost = (int)(blocks * (halves == 1 ? 0.5f / 0.6f : 0.7f / 0.8f));   // a T tile, in blocks of a weight tile: it is paced by its loads
         for (int whole = rows; whole >= 0 && whole >= rows - 1 && n_last > 0 && rows > 0; --whole) {
             const size_t slab = (size_t)halves * kHalfT * (size_t)Q.C * 2u;   // token operand of one token tile
             const int cut_tiles = n - whole * max_clusters;
@@ -982,8 +981,8 @@ static int plan_schedule(GemmParams& Q, bool may_cut, int max_clusters, float* e
             if (extra < 0 && num / max_clusters < shortest) { extra = 0; num = rest; }
             if ((extra > 0 ? num / max_clusters - extra : num / max_clusters) < shortest) continue;
             const float range = (float)num / max_clusters;
-            const int nc = (int)((blocks + range - 1) / range);                  // contributors of a tile, about
-            offer({ramp + pace * (whole * blocks + range) + collect(nc), halves, max_clusters, 1, first, 0, extra, 1, (int)num, 1});
+            const int nc = (int)((blocks + range) / range);                      // contributors of a tile, about
+            offer({16.7f + pace * (whole * blocks + range) + collect(nc), halves, max_clusters, 1, first, 0, extra, 1, (int)num, 1});
         }
     }
     Q.halves = best.halves;
@@ -1003,10 +1002,8 @@ static int plan_schedule(GemmParams& Q, bool may_cut, int max_clusters, float* e
     return best.clusters;
 }
 
-// The estimate for a forward call of `count` members of M tokens each on a whole GPU.  Where tiles are cut, weights that mix 4-bit channels with
-// others (mixed) take longer than the choice of a schedule counts for (13824 x 5120 at 60/35/5, 65 tokens, 56.5 us for 51.5; with 1 and 2 bits
-// 46.7, all 4 bits 48): what lies above a tile's start and drain counts a quarter more for them.
-float fused_estimate(int N, int K, int M, int r, bool mixed, int count) {
+// The estimate for a forward call of `count` members of M tokens each on a whole GPU.
+float fused_estimate(int N, int K, int M, int r, int count) {
     GemmParams Q;
     memset(&Q, 0, sizeof(Q));
     float us = 0.0f;
@@ -1019,7 +1016,6 @@ float fused_estimate(int N, int K, int M, int r, bool mixed, int count) {
     Q.tiles_r = (N + kPairR - 1) / kPairR;
     Q.part_halves = 2;   // (tiles may be cut)
     plan_schedule(Q, true, kNumSMs / kCluster, &us);
-    if (Q.sk && mixed) us += 0.26f * (us - 7.0f);
     return us * (float)((count + kMaxBatch - 1) / kMaxBatch);
 }
 

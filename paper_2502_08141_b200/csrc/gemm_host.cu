@@ -180,15 +180,55 @@ lowra_status run_small(const MemberArgs* mem, uint16_t* const* T_of, int count, 
 // The diagnostic lowra_diag_drop_t_flags is about flags, which the path for few tokens has none of: it leaves that path out.
 bool dropping_flags() { return g_drop_t_flags.load(std::memory_order_relaxed) != 0; }
 // Up to 16 tokens it is always taken.  From 33 on it dequantises every weight twice, which many channels with short contractions do not repay, and
-// the two estimates decide (64 tokens, forward, few-token path against tensor-core tiles, us: 2048 x 2048 12 - 13.5 against 21 - 25, 4096 x 4096
-// 23 - 26 against 26 - 27; but 8192 x 512 16.9 against 13.1, 13824 x 512 28.7 against 13.3, 6144 x 2048 of 1 and 2 bits 26.6 against 21.9, 5120 x 5120
-// 34 against 29, 5120 x 13824 of 4 bits 70 against 52).  Weights that mix 4-bit channels with others are slower on cut tiles and lean to the
-// few-token path.  At 17 to 32 tokens only the shortest contractions of many channels leave it (32 tokens, 13824 x 256 18.0 against 11.0).
-bool mixes_4_bits(const lowra_layout* L) { return L->counts[2] > 0 && L->counts[2] < L->N; }
-bool takes_small_path(bool backward, int N, int K, int M, int r, bool mixed) {
+// the two estimates decide; tiles of so few tokens take 0.95 of theirs, for there is less to store.  Over 520 calls of 17 to 64 tokens (256 to 13824 channels,
+// 512 to 13824 features, ranks 16 to 128, six mixes) the choice is 0.5 % behind the faster path in the mean (1.3 % with estimates from before units_kernel and
+// shared tiles).  64 tokens, forward, few-token path against tensor-core tiles, us: 2048 x 2048 12 - 13.5 against 21 - 25, 4096 x 4096 23 - 26 against 26 - 27;
+// but 8192 x 512 16.9 against 13.1, 13824 x 512 28.7 against 13.3, 5120 x 13824 of 4 bits 70 against 52; 36 tokens, 7016 x 4608 at 2 and 4 bits 43 against 33.
+// At 17 to 32 tokens only short contractions of many channels leave it (32 tokens, 13824 x 256 18.0 against 11.0; 30, 12256 x 768, rank 128 19.2 against 14.5).
+constexpr float kFewInTiles = 0.95f;
+bool takes_small_path(bool backward, const int32_t* n, int K, int M, int r) {
     if (backward || M > kSmallTokens) return false;
-    return M <= 16 || small_estimate(N, K, M) < fused_estimate(N, K, M, r, mixed);
+    return M <= 16 || small_estimate(n, K, r, M > 32 ? 2 : 1, M) < kFewInTiles * fused_estimate(n[0] + n[1] + n[2], K, M, r, 1);
 }
+
+// Which path the token groups of several adapters take: the one that a call of their own would, but for groups of 33 to 64 in company.  With others in a
+// few-token launch they cost less than alone, and several of them fill a launch of the tensor-core tiles (where they go `together`), which dequantises
+// once per group (4096 x 4096 of 4 bits, 64 tokens in each of 2 / 4 / 8 groups, us: 47 / 86 / 164 against 34 / 41 / 80).  Contractions too short for
+// tiles to be shared gain nothing on the few-token path in company, nor on the other where groups do not go together.
+class GroupPaths {
+    static constexpr int kSharedK = 1536;
+    static constexpr float kLaunchUs = 6.0f, kJoinUs = 2.0f;
+    const int32_t* counts;
+    int K, r;
+    bool company, mid_few = false;
+    int8_t line[kSmallTokens + 1];      // groups of so many tokens: -1 not asked yet
+    bool by_itself(int m) {
+        if (line[m] < 0) line[m] = takes_small_path(false, counts, K, m, r) ? 1 : 0;
+        return line[m] != 0;
+    }
+
+public:
+    GroupPaths(const lowra_layout* L, int32_t rank, const int32_t* start, int n, bool together) : counts(L->counts), K(L->K), r(rank) {
+        memset(line, -1, sizeof(line));
+        int low = 0, mid = 0, many = 0;
+        for (int a = 0; a < n; ++a) {
+            const int m = start[a + 1] - start[a];
+            if (m > kSmallTokens) ++many;
+            else if (m > 32) ++mid;
+            else if (m > 0 && m <= 32 && by_itself(m)) ++low;
+        }
+        company = (together || K >= kSharedK) && (mid > 1 || (mid == 1 && low > 0));
+        if (!company) return;
+        // (a few-token launch takes kSmallMembers groups; where larger groups have a launch of the tiles anyway, these join it)
+        const int N = counts[0] + counts[1] + counts[2], launches = (low + mid - 1) / kSmallMembers - (low > 0 ? (low - 1) / kSmallMembers : 0);
+        const float without = low > 0 ? small_estimate(counts, K, r, low, 32) : 0.0f;
+        const float few = small_estimate(counts, K, r, low + 2 * mid, kSmallTokens) - without + kLaunchUs * launches;
+        const float one = fused_estimate(N, K, kSmallTokens, r, 1);
+        const float tiles = !together ? mid * one : many > 0 ? fused_estimate(N, K, kSmallTokens, r, mid + 1) - one + kJoinUs : fused_estimate(N, K, kSmallTokens, r, mid);
+        mid_few = few < kFewInTiles * tiles;
+    }
+    bool few(int m) { return m >= 1 && m <= kSmallTokens && (company && m > 32 ? mid_few && (K >= kSharedK || by_itself(m)) : by_itself(m)); }
+};
 
 // Forward / backward-input for `count` weights of one shape in one launch (count == 1: the plain calls).  The members
 // may have different token counts (several adapters on one weight: one member per token group).  few_tokens: the path for few tokens is open.
@@ -210,9 +250,14 @@ lowra_status run_members(bool backward, const MemberArgs* mem, int count, int32_
     uint32_t* flags = reinterpret_cast<uint32_t*>(ws + kFlagsOffset);
     uint32_t* t_flags = reinterpret_cast<uint32_t*>(ws + w.off_t_flags);
 
-    bool mixed = false;
-    for (int i = 0; i < count; ++i) mixed = mixed || mixes_4_bits(mem[i].layout);
-    if (few_tokens && !dropping_flags() && takes_small_path(backward, N, K, M, r, mixed)) {   // (M: the largest member's tokens)
+    int32_t counts[3] = {N, 0, 0};      // (of a batch's weights on average)
+    for (int c = 1; c < 3; ++c) {
+        int64_t sum = 0;
+        for (int i = 0; i < count; ++i) sum += mem[i].layout->counts[c];
+        counts[c] = (int32_t)(sum / count);
+        counts[0] -= counts[c];
+    }
+    if (few_tokens && !dropping_flags() && takes_small_path(backward, counts, K, M, r)) {   // (M: the largest member's tokens)
         uint16_t* T_of[kMaxBatch];
         for (int i = 0; i < count; ++i) T_of[i] = reinterpret_cast<uint16_t*>(ws + w.off_T[i]);
         return run_small(mem, T_of, count, r, s, count == 1, workspace, stream);
@@ -450,7 +495,15 @@ extern "C" lowra_status lowra_diag_choose(const lowra_layout* layout, int32_t ba
     }
     memset(out, 0, sizeof(*out));
     out->w_split = out->t_split = 1;
-    if (takes_small_path(backward != 0, N, K, most, r, mixes_4_bits(layout))) {
+    bool few = takes_small_path(backward != 0, layout->counts, K, most, r);
+    if (backward == 0 && one_weight != 0) {
+        int32_t start[kSmallMembers + 1] = {0};
+        for (int i = 0; i < count; ++i) start[i + 1] = start[i] + tokens_host[i];
+        GroupPaths paths(layout, r, start, count, true);
+        few = true;
+        for (int i = 0; i < count; ++i) few = few && paths.few(tokens_host[i]);
+    }
+    if (few) {
         out->few_tokens = 1;
         out->units = small_takes_units(P) ? 1 : 0;
         return LOWRA_OK;
@@ -526,22 +579,13 @@ extern "C" lowra_status lowra_lora_forward_adapters(const lowra_layout* layout, 
                           group_start_host[a + 1] - m0};
     };
     const bool dropping = dropping_flags();   // (asked once: the launches below use the diagnostic's calls up)
-    const bool mixed = mixes_4_bits(layout);
-    auto by_itself = [&](int a) { return !dropping && takes_small_path(false, N, layout->K, group_start_host[a + 1] - group_start_host[a], r, mixed); };
-    // Several groups of 33 to 64 tokens that would take that path each by itself: together they fill the tensor-core tiles' launch, which
-    // dequantises once per group (4096 x 4096 of 4 bits, 64 tokens in each of 2 / 4 / 8 groups, us: 47 / 86 / 164 against 34 / 41 / 80).
-    int few_limit = kSmallTokens;
-    if (together) {
-        int n_mid = 0;
-        for (int a = 0; a < n_adapters; ++a) n_mid += group_start_host[a + 1] - group_start_host[a] > 32 && by_itself(a) ? 1 : 0;
-        if (n_mid > 1 && fused_estimate((int)N, layout->K, kSmallTokens, r, mixed, n_mid) < small_estimate((int)N, layout->K, kSmallTokens, n_mid)) few_limit = 32;
-    }
-    auto is_small = [&](int a) { return group_start_host[a + 1] - group_start_host[a] <= few_limit && by_itself(a); };
+    GroupPaths paths(layout, r, group_start_host, n_adapters, together);
+    auto takes_few = [&](int a) { return !dropping && paths.few(group_start_host[a + 1] - group_start_host[a]); };
     MemberArgs mem[kMaxBatch], few[kSmallMembers];
     uint16_t* few_T[kSmallMembers];
     int n = 0, n_few = 0;
     for (int a = 0; a <= n_adapters; ++a) {
-        if (a < n_adapters && group_start_host[a + 1] > group_start_host[a] && is_small(a)) {
+        if (a < n_adapters && group_start_host[a + 1] > group_start_host[a] && takes_few(a)) {
             if (n_few == 0 && (st = check_members(&(few[0] = member(a)), 1, r, workspace_dev, workspace_bytes, true)) != LOWRA_OK) return st;
             few_T[n_few] = reinterpret_cast<uint16_t*>(static_cast<unsigned char*>(workspace_dev) + kHeaderBytes) +
                            (size_t)group_start_host[a] * (size_t)((r + 63) / 64 * 64);
@@ -554,7 +598,7 @@ extern "C" lowra_status lowra_lora_forward_adapters(const lowra_layout* layout, 
     }
     for (int a = 0; a <= n_adapters; ++a) {
         if (a < n_adapters) {
-            if (group_start_host[a + 1] == group_start_host[a] || is_small(a)) continue;
+            if (group_start_host[a + 1] == group_start_host[a] || takes_few(a)) continue;
             mem[n++] = member(a);
         }
         if (n > 0 && (a == n_adapters || n == (together ? kMaxBatch : 1))) {

@@ -143,7 +143,7 @@ constexpr uint32_t kGemmSmemBytes = kSmemRing + kSmemBarriers;
 static_assert(kGemmSmemBytes <= 232448, "227 KB of shared memory per CTA");
 
 lowra_status launch_fused(int mode, const GemmParams& G, const BatchMaps& TM, cudaStream_t stream);
-float fused_estimate(int N, int K, int M, int r, bool mixed, int count = 1);
+float fused_estimate(int N, int K, int M, int r, int count);
 int fused_schedule(bool backward, int N, int K, const int32_t* Ms, int count, int r, int* tile_tokens, int* w_split, int* t_split);   // what a call would run (diagnostic)
 
 // ---- forward pass for few tokens (gemm_small.cu) --------------------------------------------
@@ -158,7 +158,7 @@ struct SmallMember {
     uint16_t *Y, *T;          // T [M, rp]: s X A, as the fused calls leave it
     int M;
 };
-float small_estimate(int N, int K, int M, int count = 1);
+float small_estimate(const int32_t* n, int K, int r, int units, int most);
 template <int NB>   // members the kernel's parameters have room for
 struct SmallParams {
     SmallMember m[NB];

@@ -771,15 +771,23 @@ lowra_status launch_members(const SmallParams<NB>& P, cudaStream_t stream) {
 
 }  // namespace
 
-// An estimate of a call's time in microseconds for `count` members of 17 to 64 tokens each, fitted to 40 shapes of 256 to 13824 (within 20 % for
-// most): 6 for the projection and the start; then CTAs that take 1.7, 0.4 for every 8 tokens under or over 32 (past 32, where a member has
-// two, 1.2), 2.7 for every span of a slot and 6 / slices for adding up and storing.  Two share an SM; the last one, if alone on its SM,
-// takes 0.65 of that.
-float small_estimate(int N, int K, int M, int count) {
-    const int slices = product_slices(N, K), n_span = (K + kSmallSpan - 1) / kSmallSpan;
-    const int ctas = (N / kSmallRows + 2) * slices * ((M + 31) / 32) * count, per_sm = (ctas + kNumSMs - 1) / kNumSMs;
-    const float cta_us = 1.7f + 0.4f * (M > 32 ? 3 : (M + 7) / 8 - 4) + 2.7f * n_span / (2.0f * slices) + 6.0f / slices;
-    return 6.0f + cta_us * (per_sm / 2 + (per_sm % 2 != 0 ? 0.65f : 0.0f));
+// An estimate of a call's time in microseconds for so many units of up to 32 tokens, the largest member of `most`, on one weight of n[0], n[1], n[2] channels at
+// 1, 2 and 4 bits: 2.8 for the projection and the start, then CTAs, two to an SM.  A step of 256 takes 2.5, 0.45 more at 4 bits; around a CTA's steps and its
+// share of the low-rank term 5.4, and if it is alone on its SM all that takes 0.64 of it.  A CTA that does all slices takes 3.7 and 1.2 for every slice around its
+// steps, of which two halves overlap (0.74), and waits 1.7 for 4-bit rows among others; of three on an SM the third does not wait for both.  Fitted to 520
+// calls (256 to 13824 channels, 512 to 13824 features, ranks 16 to 128, six mixes): within 17 %.
+float small_estimate(const int32_t* n, int K, int r, int units, int most) {
+    const int N = n[0] + n[1] + n[2], slices = product_slices(N, K);
+    const int groups = (n[0] + kSmallRows - 1) / kSmallRows + (n[1] + kSmallRows - 1) / kSmallRows + (n[2] + kSmallRows - 1) / kSmallRows;
+    const float rank = (float)r / 64.0f, step = 2.5f + 0.45f * (float)n[2] / (float)N, steps = 0.5f * (float)((K + kSmallSpan - 1) / kSmallSpan);
+    const bool mixed = n[2] > 0 && n[2] < N;
+    auto per_sm = [](int ctas) { return (ctas + kNumSMs - 1) / kNumSMs; };
+    if (units_faster(n, K, r, units, most, slices)) {
+        const int k = per_sm(groups * units);
+        return 2.8f + (mixed ? 1.7f : 0.0f) + (3.7f + 1.2f * slices + 2.1f * rank + 0.74f * step * steps) * (k == 1 ? 0.64f : k == 2 ? 1.15f : 0.5f * k);
+    }
+    const int k = per_sm(groups * slices * units);
+    return 2.8f + (mixed ? 0.3f : 0.0f) + (5.4f + (2.2f * rank + step * steps) / slices) * (k / 2 + (k % 2 != 0 ? 0.64f : 0.0f));
 }
 
 bool small_takes_units(const SmallParams<kSmallMembers>& P) { return P.one_weight && units_pay(P, product_slices(P.N, P.K)); }
