@@ -949,7 +949,11 @@ static int plan_schedule(GemmParams& Q, bool may_cut, int max_clusters, float* e
             if (ts == 1 && s == 1) continue;
             const float t_done = ts == 1 ? t_us : shared_t(ts), w_done = single_us((float)blocks / s);
             const float us = (t_done > w_done ? t_done : w_done) + (s == 1 ? -0.7f * halves : 3.5f + 2.5f * halves);
-            offer({us, halves, n_t * ts + n_w * s, 1, 0, n_t * ts, 0, ts, n_w * blocks, s});
+            // Tiles of 256 tokens between two or three clusters on (almost) all SMs are finished by the first one: the others leave while it works, and the next
+            // call's CTAs come in (us, shared against this: forward 5888 x 4352, 168 tokens 32.0 -> 27.8, backward 3224 x 8832, 209 tokens 32.9 -> 28.3).  On
+            // fewer SMs the two are alike at two clusters and sharing is ahead from three, by 2 to 15 %; tiles of 512 tokens are always shared (by 5 to 27 %).
+            const bool by_first = halves == 1 && s <= 3 && n_t * ts + n_w * s >= 70;
+            offer({us, halves, n_t * ts + n_w * s, 1, 0, n_t * ts, 0, ts, n_w * blocks, by_first ? 1 : s});
         }
         // T by clusters of its own, each tile by ts of them, and ranges over all weight tiles for the others: for few channels and many tokens, where one
         // piece in a few is a T tile that the others wait for, and for pieces that come out a little over a row (forward, us, against the

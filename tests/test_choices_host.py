@@ -67,7 +67,10 @@ def test_units_where_they_are_faster(N, K, r, mix, tokens, units):
     # 512-token tiles shared by three clusters took 34.7 and 36.1 us, their estimates counted the T tile's second 64 ranks as nothing
     (2672, 1152, 1437, 128, {1: 0.85, 2: 0.15}, True, dict(tile_tokens=256, w_split=1)),         # 28.4
     (5016, 2944, 404, 128, {1: 0.5, 2: 0.5}, False, dict(tile_tokens=256, w_split=1)),           # 30.8
-    (9184, 6016, 77, 64, {1: 0.3, 2: 0.5, 4: 0.2}, True, dict(clusters=74, w_split=3, t_split=2)),   # 45.2; two clusters a tile 54.5
+    (9184, 6016, 77, 64, {1: 0.3, 2: 0.5, 4: 0.2}, True, dict(clusters=74, t_split=2)),          # 45 - 47; two clusters a tile, on 55, 54.5
+    # on all SMs, tiles of 256 tokens: the first cluster of a tile finishes it
+    (5888, 4352, 168, 64, {1: 0.85, 2: 0.15}, False, dict(clusters=74, w_split=1, t_split=5)),   # 27.8; shared 32.0
+    (3224, 8832, 209, 128, {1: 0.85, 2: 0.15}, True, dict(clusters=74, w_split=1, t_split=4)),   # 28.3; shared 32.9
     (4096, 4096, 128, 64, {1: 0.6, 2: 0.4}, False, dict(tile_tokens=256, w_split=4, t_split=7)),
     (7016, 4608, 36, 64, {2: 0.75, 4: 0.25}, False, dict(few_tokens=0)),                          # 33; few-token path 43
     (2048, 2048, 64, 64, {1: 0.6, 2: 0.4}, False, dict(few_tokens=1)),                            # 12; tiles 21

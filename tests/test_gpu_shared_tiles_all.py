@@ -1,5 +1,6 @@
-"""Shared tiles on all 74 pairs of SMs, where cluster 0 keeps its part of a T tile in the place of cluster 1: both directions, one and two halves
-of a token tile, ranks of one and two widths, against fp64 products of the decoded weight, and twice, bit for bit."""
+"""Calls cut over all 74 pairs of SMs, where cluster 0 keeps its part of a shared T tile in the place of cluster 1: both directions, one and two halves
+of a token tile (the weight tiles finished by their first cluster, and shared), ranks of one and two widths, against fp64 products of the
+decoded weight, and twice, bit for bit."""
 import pytest
 import torch
 
@@ -10,9 +11,10 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("N,K,r,M,backward", [
-    (9184, 6016, 64, 77, True),       # 24 tiles by three clusters, T by two
+    (9184, 6016, 64, 77, True),       # 24 tiles by three clusters, T by two (all of them)
     (9216, 9216, 128, 256, True),
-    (6144, 9216, 80, 400, False),     # tiles of 512 tokens
+    (6144, 9216, 80, 400, False),     # tiles of 512 tokens, shared
+    (9216, 6144, 128, 500, True),
     (4608, 9216, 16, 70, True),       # 36 tiles by two clusters
 ])
 def test_against_fp64(N, K, r, M, backward):
@@ -23,7 +25,7 @@ def test_against_fp64(N, K, r, M, backward):
     precs = si.precisions(N, {1: 0.3, 2: 0.5, 4: 0.2}, matrix_id=3)
     layout = lw.Layout(precs, K).build_deal()
     choice = lw.lowra_diag_choose(layout, backward, [M], r)
-    assert choice["clusters"] == 74 and choice["w_split"] > 1 and choice["t_split"] == 2, choice
+    assert choice["clusters"] == 74 and choice["w_split"] == (1 if M <= 256 else 3) and choice["t_split"] == 2, choice
     maps, thr = (torch.from_numpy(t).cuda() for t in si.standin_codebooks(precs))
     packed, absmax = lw.lowra_encode(layout, torch.randn(N, K, device="cuda", generator=gen), thr)
     W = lw.lowra_decode(layout, packed, absmax, maps).double()
