@@ -60,8 +60,11 @@ def refused(call, changes):
             call(**change)
 
 
-def test_codec_learner_and_errors(problem):
+@pytest.mark.parametrize("native", [False, True])
+def test_codec_learner_and_errors(problem, native, monkeypatch):
     p, lw, layout = problem, problem["lw"], problem["layout"]
+    if not native:      # as for an interpreter without an extension module of its own
+        monkeypatch.setattr(lw, "_fits", lw._no_verdict)
     new = lambda *shape, dtype=torch.float32: torch.empty(*shape, dtype=dtype, device="cuda")
     W, thr = torch.randn(N, K, device="cuda"), p["maps"].sort().values
     short_packed, short_absmax = p["packed"][:-1], new(N, K // 64 - 1)
@@ -86,8 +89,11 @@ def test_codec_learner_and_errors(problem):
     refused(lambda **k: lw.lowra_channel_errors(W, three, three, **k), ((dict(sse3=new(N, 2, dtype=torch.float64)), "sse3"),))
 
 
-def test_other_products(problem):
+@pytest.mark.parametrize("native", [False, True])
+def test_other_products(problem, native, monkeypatch):
     p, lw = problem, problem["lw"]
+    if not native:
+        monkeypatch.setattr(lw, "_fits", lw._no_verdict)
     layout = lw.Layout(p["layout"].precs_host, K).build_deal()
     new = lambda *shape, dtype=torch.bfloat16: torch.empty(*shape, dtype=dtype, device="cuda")
     ws = lambda size: lw.lowra_workspace_init(torch.empty(size, dtype=torch.uint8, device="cuda"))
