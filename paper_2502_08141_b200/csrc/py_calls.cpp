@@ -28,7 +28,7 @@ struct Library {
 bool plain(PyObject* o) { return THPVariable_CheckExact(o); }
 
 // memory of device `dev` without gaps
-bool on(const at::Tensor& t, int64_t dev) { return t.is_cuda() && t.get_device() == dev && t.is_contiguous(); }
+bool on(const at::Tensor& t, int64_t dev) { return t.device() == at::Device(at::kCUDA, (c10::DeviceIndex)dev) && t.is_contiguous(); }
 bool matrix(const at::Tensor& t, int64_t rows, int64_t cols, int64_t dev) {
     return on(t, dev) && t.scalar_type() == at::kBFloat16 && t.dim() == 2 && t.size(0) == rows && t.size(1) == cols;
 }
@@ -74,7 +74,7 @@ PyObject* product(PyObject* const* args, Py_ssize_t n, bool backward) {
         bool called = false;
         {
             Released released;      // (allocations included: one that has to ask the driver for memory takes its time)
-            void* stream = c10::cuda::getCurrentCUDAStream().stream();
+            void* stream = c10::cuda::getCurrentCUDAStream((c10::DeviceIndex)dev).stream();
             if (!out_given) out = at::empty({M, cols}, options);
             bool ready = true;
             if (!workspace_given) {
