@@ -9,8 +9,9 @@
 // to the midpoints of neighbouring levels.  Levels and thresholds in fp64, sums in 64-bit fixed point.  Output: the levels rounded to fp32 and the
 // midpoints of those fp32 levels (computed in fp64, rounded to fp32), in [N, 16] tables.
 //
-// Two kernels.  learn_kernel adds the whole row up in every round.  sorted_learn_kernel brings the row's values into order once and
-// then needs a few hundred of them per round; it takes over where the rounds are many or expensive enough (sorted_pays).
+// Three kernels.  learn_kernel adds the whole row up in every round.  ordered_learn_kernel brings every block's values into order and then searches
+// them, a block per lane.  sorted_learn_kernel brings the whole row into order, after which a round takes a few hundred of its values.  The more
+// thresholds and rounds, the more order pays (kernel_for).
 #include <float.h>
 #include <math.h>
 #include <string.h>
@@ -30,14 +31,15 @@ struct LearnParams {
     int row0;             // this launch's rows: stored rows row0 .. row0 + grid - 1
     int turn;             // see enter()
     int bins;             // sorted rows: cells
+    int one;              // 1, which the compiler does not know
     unsigned near_zero;   // see too_coarse
     double init_y[3][16];  // initial levels per class (1, 2, 4 bits)
     double init_t[3][16];  // initial thresholds per class
 };
 
-// The rows of one call may go to two launches, which know nothing of each other's rows.  turn 1, the first of two, lets the second
-// begin once everything before the call is complete; turn 2 does not wait for the first before it begins but before it ends, so that
-// what comes after it may rely on both.  turn 0: a launch by itself.
+// The rows of one call may go to several launches, which know nothing of each other's rows.  turn 1, the first of them, lets the next one
+// begin once everything before the call is complete; turn 2 does not wait for the launch before it to begin but to end, so that
+// what comes after it may rely on all.  turn 0: a launch by itself.
 __device__ __forceinline__ void enter(int turn) {
     if (turn != 2) asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -491,8 +493,8 @@ __global__ void __launch_bounds__(THREADS) learn_kernel(const __grid_constant__ 
 // The order inside a cell is that in which the atomics arrive, which integer sums do not see.
 // What bounds it: shared-memory wavefronts (two atomics and an 8-byte store per element at random places: 24 wavefronts for 32
 // elements, the pipe 77 % busy at T = 0) and, in the rounds, the latency of one warp's steps (about 1000 cycles each, hidden by the
-// other rows of the SM).  Measured against a pass over the row per round, 4096 x 4096, T = 10: 391 -> 105 us at 4 bits, 157 -> 86
-// at 2; 127 -> 80 at 60/35/5 % of 1/2/4 bits (1-bit rows in learn_kernel); three precisions, T = 2: 133 -> 66 us.
+// other rows of the SM).  For 4-bit rows and the three-precision form: 4096 x 4096 of 4 bits, T = 10, 109 us (ordered blocks 140, a pass over the row per
+// round 415); three precisions 127 (181, 624).
 constexpr int kSortedMaxK = 16384;         // 10 to 11 bytes of shared memory per element
 int bins_of(int K) { int n = 256; while (n < K / 6) n *= 2; return n; }
 
@@ -647,10 +649,7 @@ __device__ __forceinline__ void learn_rounds(const LearnParams& P, const float2*
             else learn_sorted<1, CROWDED>(P, sorted, first, run, bins, row_most, y, h);
         }
     } else if (warp == 0) {
-        const int b = P.L.precs[r];
-        if (b == 1) learn_sorted<1, CROWDED>(P, sorted, first, run, bins, row_most, y, h);
-        else if (b == 2) learn_sorted<2, CROWDED>(P, sorted, first, run, bins, row_most, y, h);
-        else learn_sorted<4, CROWDED>(P, sorted, first, run, bins, row_most, y, h);
+        learn_sorted<4, CROWDED>(P, sorted, first, run, bins, row_most, y, h);
     }
 }
 template <bool ALL3>
@@ -809,6 +808,336 @@ __global__ void __launch_bounds__(THREADS, CTAS) sorted_learn_kernel(const __gri
     leave(P.turn);
 }
 
+// ---------------------------------------------------------------------------------------------------------------------------------
+// Rounds on blocks in order.  A lane takes one absmax block (of short rows a half or a quarter), so that all its values have one weight and order is a matter
+// of its registers alone: a sorting network, no atomics, no scattered stores (the order of a whole row costs 24 shared-memory wavefronts for 32
+// elements, below).  The values lie in shared memory as [place][lane], with the sums of w * n before every fourth place; a lane finds a threshold's
+// place in its block by bisection, every look-up free of bank conflicts, adds the few values of the last four below it, and the warp's sums are
+// added up by a halving exchange.  The same sums on the same grid as in the other kernels, hence the same tables bit for bit.
+// What bounds it: instruction issue (60 to 73 % of the slots, with the 16 warps that an SM's shared memory takes): 2400 instructions a warp until the first
+// round, 1360 of them in the network, then 62 for a threshold and 150 for a round.  Measured, 4096 x 4096, T = 10: 82 -> 58 us at
+// 60/35/5 % of 1/2/4 bits (72 -> 48 at 1 bit, 89 -> 58 at 2); three precisions, T = 2: 67.7 -> 56.8.
+// Not taken: two blocks a lane in turn (49 -> 55 us at 1 bit, T = 10: half the warps); rows one after the other in a persistent grid, the next one's load
+// in flight (66: five rows to an SM instead of eight); halves of blocks (a fifth less network, but every threshold twice: 61 -> 70 at 2 bits).
+//
+// Batcher's odd-even merge sort ("Sorting networks and their applications", 1968): layer (p, k), then those after it.  Both a minimum and a maximum go to
+// the half-rate pipe, which bounds the network; so every other maximum is formed on the other one, as what the minimum leaves of the two bit patterns'
+// sum (half of them: 30.5 -> 29.4 us at T = 1; two thirds are more instructions than that wins, 30.6).
+template <int P_, int K_, int PER>
+__device__ __forceinline__ void sort_layers(float (&x)[PER], int one) {
+#pragma unroll
+    for (int i = 0; i < PER - K_; ++i) {
+        if (i >= K_ % P_ && ((i - K_ % P_) & K_) == 0 && i / (2 * P_) == (i + K_) / (2 * P_)) {
+            const float lo = fminf(x[i], x[i + K_]);
+            if ((i & 1) == 0) {
+                x[i + K_] = fmaxf(x[i], x[i + K_]);
+            } else {
+                int hi;
+                asm("mad.lo.s32 %0, %1, %2, %3;" : "=r"(hi) : "r"(__float_as_int(x[i])), "r"(one), "r"(__float_as_int(x[i + K_])));
+                asm("mad.lo.s32 %0, %1, %2, %0;" : "+r"(hi) : "r"(__float_as_int(lo)), "r"(-one));
+                x[i + K_] = __int_as_float(hi);
+            }
+            x[i] = lo;
+        }
+    }
+    if constexpr (K_ > 1) sort_layers<P_, K_ / 2, PER>(x, one);
+    else if constexpr (2 * P_ < PER) sort_layers<2 * P_, 2 * P_, PER>(x, one);
+}
+
+// As warp_sums, for any number of values and none of them held twice: afterwards v[0] of a lane is total number slot(lane).
+template <int NV, int D>
+struct Halve {
+    static __device__ __forceinline__ void sums(long long* v, int lane) {
+        if constexpr (D >= 1) {
+            if constexpr (NV > 1) {
+                constexpr int H = (NV + 1) / 2;
+                const bool upper = (lane & D) != 0;
+#pragma unroll
+                for (int k = 0; k < H; ++k) {
+                    const long long b = k + H < NV ? v[k + H] : 0;
+                    const long long send = upper ? v[k] : b, keep = upper ? b : v[k];
+                    v[k] = keep + __shfl_xor_sync(0xffffffffu, send, D);
+                }
+                Halve<H, D / 2>::sums(v, lane);
+            } else {
+                v[0] += __shfl_xor_sync(0xffffffffu, v[0], D);
+                Halve<1, D / 2>::sums(v, lane);
+            }
+        }
+    }
+    // which of the NV totals that is; -1: none, or one that another lane holds as well
+    static __device__ __forceinline__ int slot(int lane, int n = NV) {
+        if constexpr (D >= 1) {
+            constexpr int H = (NV + 1) / 2;
+            const bool upper = (lane & D) != 0;
+            if constexpr (NV > 1) {
+                const int below = Halve<H, D / 2>::slot(lane, upper ? max(n - H, 0) : min(n, H));
+                return below < 0 ? -1 : below + (upper ? H : 0);
+            } else {
+                return upper ? -1 : Halve<1, D / 2>::slot(lane, n);
+            }
+        } else {
+            return n > 0 ? 0 : -1;
+        }
+    }
+};
+
+// Who looks after which level and the threshold above it: BITS = 1, 2, 4: lane j after level j; 7: all three precisions, lanes 0 to 15, 16 to 19, 20 and 21.
+template <int BITS>
+struct Levels {
+    static constexpr int kLevels = BITS == 7 ? 22 : 1 << BITS, kThresholds = BITS == 7 ? 19 : (1 << BITS) - 1;
+    static __device__ __forceinline__ int cls(int lane) { return BITS == 7 ? (lane < 16 ? 2 : lane < 20 ? 1 : 0) : BITS >> 1; }
+    static __device__ __forceinline__ int level(int lane) { return BITS == 7 ? (lane < 16 ? lane : lane < 20 ? lane - 16 : lane - 20) : lane; }
+    static __device__ __forceinline__ constexpr int lane_of(int q) { return BITS == 7 ? (q < 15 ? q : q < 18 ? q + 1 : q + 2) : q; }
+    static __device__ __forceinline__ int threshold_of(int lane) { return BITS == 7 ? (lane < 15 ? lane : lane < 19 ? lane - 1 : lane - 2) : lane; }
+};
+
+__device__ __forceinline__ long long lds_s64(uint32_t at) {
+    long long v;
+    asm volatile("ld.shared.s64 %0, [%1];" : "=l"(v) : "r"(at));
+    return v;
+}
+
+// What a thread has in order: PER values, 32 apart, and their weight.
+struct Ordered {
+    uint32_t xs;        // this thread's first value
+    uint32_t sums;      // of w n before values 0, 4, 8, ..., 32 apart
+    float weight;
+};
+
+// The mean of the bucket [t_lo, t_hi) by the whole CTA; y if it weighs nothing.  scratch: five words per warp.
+template <int PER, int WARPS>
+__device__ __noinline__ double fine_mean_ordered(Ordered O, float t_lo, float t_hi, bool vanished, double y, long long* scratch) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    auto element = [&](int p) { return make_float2(lds_f32(O.xs + 128 * p), O.weight); };
+    double g = kGrid;
+    if (vanished) {
+        float* most_of = reinterpret_cast<float*>(scratch + 4 * WARPS);
+        float most = largest_weight(element, 0, PER, 1, t_lo, t_hi);
+        if (WARPS > 1) {
+            if (lane == 0) most_of[warp] = most;
+            __syncthreads();
+            for (int w = 0; w < WARPS; ++w) most = fmaxf(most, most_of[w]);
+        }
+        g = grid_of(most);
+        if (!(most > 0.0f)) {
+            __syncthreads();
+            return y;
+        }
+    }
+    Fine f = fine_sums<2>(element, 0, PER, 1, t_lo, t_hi, g);
+    if (WARPS > 1) {
+        if (lane == 0) { scratch[4 * warp] = f.wn; scratch[4 * warp + 1] = f.wn_lo; scratch[4 * warp + 2] = f.w; scratch[4 * warp + 3] = f.w_lo; }
+        __syncthreads();
+        f = Fine{0, 0, 0, 0};
+        for (int w = 0; w < WARPS; ++w) { f.wn += scratch[4 * w]; f.wn_lo += scratch[4 * w + 1]; f.w += scratch[4 * w + 2]; f.w_lo += scratch[4 * w + 3]; }
+        __syncthreads();
+    }
+    return fine_mean(f);
+}
+
+// T rounds and the tables of row r.  Every warp forms all levels and thresholds from all warps' sums, as in learn_row.  The thresholds five at a time: their
+// searches hide one another's latency, and the loop's code stays short (all 19 unrolled, the instruction cache missed).
+template <int BITS, int PER, int WARPS>
+__device__ __forceinline__ void ordered_rounds(const LearnParams& P, const Ordered& O, long long all_n, long long all_w,
+                                               unsigned zero_too, float row_most, long long* red2, int r) {
+    using V = Levels<BITS>;
+    constexpr int NQ = V::kThresholds, kAtOnce = NQ < 5 ? NQ : 5;
+    constexpr int kRed = 2 * (BITS == 7 ? NQ : 15) * WARPS;      // (also room for fine_mean_ordered's scratch)
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int c = V::cls(lane), j = V::level(lane), Lv = 1 << (1 << c);
+    const bool mine = lane < V::kLevels, top = j >= Lv - 1;
+    const int slot = Halve<2 * kAtOnce, 16>::slot(lane);
+    double y = mine ? P.init_y[c][j] : 0.0;
+    float t = mine && !top ? __double2float_ru(P.init_t[c][j]) : INFINITY;
+    const double w = (double)O.weight;
+    const long long wg = grid_weight(w, kGrid);
+    for (int it = 0; it < P.iterations; ++it) {
+        long long* red = red2 + (it & 1) * kRed;
+#pragma unroll 1
+        for (int q0 = 0; q0 < NQ; q0 += kAtOnce) {
+            float tq[kAtOnce];
+            uint32_t at[kAtOnce];
+            int n[kAtOnce];
+            double s[kAtOnce];
+#pragma unroll
+            for (int k = 0; k < kAtOnce; ++k) {
+                tq[k] = __shfl_sync(0xffffffffu, t, V::lane_of(q0 + k));
+                at[k] = O.xs;
+                s[k] = kGrid;
+                n[k] = 0;
+            }
+#pragma unroll
+            for (int h = PER / 2; h >= 4; h /= 2) {
+#pragma unroll
+                for (int k = 0; k < kAtOnce; ++k)
+                    if (lds_f32(at[k] + (h - 1) * 128) < tq[k]) at[k] += h * 128;
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+#pragma unroll
+                for (int k = 0; k < kAtOnce; ++k) {
+                    const float x = lds_f32(at[k] + e * 128);
+                    const double d = (double)x;
+                    if (x < tq[k]) ++n[k];
+                    s[k] = __fma_rd(__hiloint2double(x < tq[k] ? __double2hiint(d) : 0, __double2loint(d)), w, s[k]);   // (see few_buckets)
+                }
+            }
+            long long v[2 * kAtOnce];
+#pragma unroll
+            for (int k = 0; k < kAtOnce; ++k) {
+                const uint32_t before = at[k] - O.xs;
+                v[2 * k] = lds_s64(O.sums + before / 2) + (long long)(grid_bits(s[k]) - grid_bits(kGrid));
+                v[2 * k + 1] = (n[k] + (int)(before / 128)) * wg;
+            }
+            Halve<2 * kAtOnce, 16>::sums(v, lane);
+            if (slot >= 0 && 2 * q0 + slot < 2 * NQ) red[(2 * q0 + slot) * WARPS + warp] = v[0];
+        }
+        if (WARPS > 1) __syncthreads();
+        else __syncwarp();
+        long long fn = all_n, fw = all_w;
+        if (!top) {
+            fn = fw = 0;
+            const int q = V::threshold_of(lane);
+#pragma unroll
+            for (int k = 0; k < WARPS; ++k) { fn += red[2 * q * WARPS + k]; fw += red[(2 * q + 1) * WARPS + k]; }
+        }
+        const long long ln = __shfl_up_sync(0xffffffffu, fn, 1), lw = __shfl_up_sync(0xffffffffu, fw, 1);
+        const double sn = (double)(j == 0 ? fn : fn - ln);
+        const long long sw = j == 0 ? fw : fw - lw;
+        const bool vanished = sw <= 0;
+        if (!vanished) y = sn / (double)sw;
+        for (unsigned left = __ballot_sync(0xffffffffu, mine && too_coarse(sn, P.near_zero, zero_too)); left != 0u; left &= left - 1u) {     // (the same in every warp)
+            const int k = __ffs(left) - 1;
+            const float t_lo = __shfl_sync(0xffffffffu, t, max(k - 1, 0)), t_hi = __shfl_sync(0xffffffffu, t, k);
+            const bool first = __shfl_sync(0xffffffffu, j, k) == 0;
+            const double mean = fine_mean_ordered<PER, WARPS>(O, first ? -INFINITY : t_lo, t_hi, __shfl_sync(0xffffffffu, (int)vanished, k) != 0,
+                                                                  __shfl_sync(0xffffffffu, y, k), red2 + ((it & 1) ^ 1) * kRed);
+            if (lane == k) y = mean;
+        }
+        const double yn = __shfl_down_sync(0xffffffffu, y, 1);
+        const float tn = mine && !top ? __double2float_ru((y + yn) * 0.5) : INFINITY;
+        const bool same = tn == t;
+        t = tn;
+        if (__all_sync(0xffffffffu, same)) break;
+    }
+    if (warp == 0) {
+        const bool bad = !(row_most < INFINITY) && P.iterations > 0;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            if (BITS != 7 && k != BITS >> 1) continue;
+            const int lv = 1 << (1 << k), l0 = BITS == 7 ? (k == 2 ? 0 : k == 1 ? 16 : 20) : 0;
+            const size_t plane = BITS == 7 ? (size_t)k * P.N * kTableStride : 0;
+            const double yl = __shfl_sync(0xffffffffu, y, l0 + min(lane, lv - 1));
+            const float m = lane < lv ? (bad ? __int_as_float(0x7fc00000) : (float)yl) : 0.0f;
+            const float mn = __shfl_down_sync(0xffffffffu, m, 1);
+            if (lane < kTableStride) {
+                P.maps[plane + (size_t)r * kTableStride + lane] = m;
+                P.thresholds[plane + (size_t)r * kTableStride + lane] = (lane + 1 < lv) ? (float)(((double)m + (double)mn) * 0.5) : __int_as_float(0x7f800000);
+            }
+        }
+    }
+}
+
+template <bool ALL3, int PER, int WARPS>
+constexpr size_t ordered_smem() {
+    return (size_t)WARPS * (PER * 32 * 4 + (PER / 4) * 32 * 8 + 2 * 2 * Levels<ALL3 ? 7 : 4>::kThresholds * 8 + 16 + 8);
+}
+
+// WARPS warps, a lane of which has PER values of one block; CTAS of them to an SM.
+template <bool ALL3, int PER, int WARPS, int CTAS>
+__global__ void __launch_bounds__(32 * WARPS, CTAS) ordered_learn_kernel(const __grid_constant__ LearnParams P) {
+    extern __shared__ __align__(16) unsigned char ordered_smem_bytes[];
+    constexpr int kPieces = PER / 4, kLanes = kBlock / PER;     // 16-byte pieces a lane; lanes a block
+    const int K = P.K, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float* xs = reinterpret_cast<float*>(ordered_smem_bytes);                           // [warps][PER][32]; before that, a warp's 32 PER values as they come
+    long long* sums = reinterpret_cast<long long*>(xs + WARPS * PER * 32);              // [warps][PER / 4][32]
+    long long* red2 = sums + WARPS * (PER / 4) * 32;                                    // two buffers of [thresholds][2][warps]
+    long long* totals = red2 + 2 * 2 * Levels<ALL3 ? 7 : 4>::kThresholds * WARPS;       // [warps][2]
+    float* most_of = reinterpret_cast<float*>(totals + 2 * WARPS);                      // [warps][2]
+    enter(P.turn);
+    const int i0 = P.row0 + (int)(gridDim.x - 1 - blockIdx.x);
+    const int r = ALL3 ? i0 : P.L.perm[i0];
+    const float* wrow = P.W + (size_t)r * K;
+    const int first = warp * (PER * 32);
+#pragma unroll
+    for (int u = 0; u < kPieces; ++u) {
+        const int at = first + 4 * (32 * u + lane);
+        if (at < K) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(xs + at)), "l"(wrow + at) : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    const int b = ALL3 ? 0 : P.L.precs[r];
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncwarp();
+    const bool in = first + lane * PER < K;
+    float x[PER];
+    float m = 0.0f;
+#pragma unroll
+    for (int q = 0; q < kPieces; ++q) {       // in an order in which eight lanes meet different banks
+        float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (in) f = *reinterpret_cast<const float4*>(xs + first + PER * lane + 4 * (q ^ (PER >= 32 ? lane & 7 : (lane >> 1) & 3)));
+        x[4 * q] = f.x; x[4 * q + 1] = f.y; x[4 * q + 2] = f.z; x[4 * q + 3] = f.w;
+        m = max_nan(max_nan(m, max_nan(fabsf(f.x), fabsf(f.y))), max_nan(fabsf(f.z), fabsf(f.w)));
+    }
+#pragma unroll
+    for (int d = 1; d < kLanes; d <<= 1) m = max_nan(m, __shfl_xor_sync(0xffffffffu, m, d));
+    const float inv = (m == 0.0f) ? 0.0f : __frcp_rn(m);
+    float most = max_nan(m, __fmul_rn(inv, 0.0f)), least = m > 0.0f ? m : INFINITY;
+#pragma unroll
+    for (int e = 0; e < PER; ++e) x[e] = __fmul_rn(x[e], inv);
+    sort_layers<1, 1, PER>(x, P.one);
+#pragma unroll
+    for (int d = kLanes; d < 32; d <<= 1) {
+        most = max_nan(most, __shfl_xor_sync(0xffffffffu, most, d));
+        least = fminf(least, __shfl_xor_sync(0xffffffffu, least, d));
+    }
+    if (WARPS > 1) {
+        if (lane == 0) { most_of[2 * warp] = most; most_of[2 * warp + 1] = least; }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < WARPS; ++k) { most = max_nan(most, most_of[2 * k]); least = fminf(least, most_of[2 * k + 1]); }
+    } else {
+        __syncwarp();          // the row has been read
+    }
+    const float scale = weight_scale(most), weight = scaled_weight(m, scale);
+    const unsigned zero_too = least < INFINITY && scaled_weight(least, scale) < kVanishing ? 1u : 0u;
+    float* mine = xs + first + lane;
+    long long* before = sums + warp * ((PER / 4) * 32) + lane;
+    long long all[2] = {0, PER * grid_weight((double)weight, kGrid)};
+    {
+        const double w = (double)weight;
+#pragma unroll
+        for (int q = 0; q < PER; q += 16) {
+            double s = kGrid;
+#pragma unroll
+            for (int e = 0; e < 16; ++e) {
+                if ((e & 3) == 0) before[((q + e) / 4) * 32] = all[0] + (long long)(grid_bits(s) - grid_bits(kGrid));
+                mine[(q + e) * 32] = x[q + e];
+                s = __fma_rd((double)x[q + e], w, s);
+            }
+            all[0] += (long long)(grid_bits(s) - grid_bits(kGrid));
+        }
+    }
+#pragma unroll
+    for (int d = 16; d >= 1; d >>= 1) {
+        all[0] += __shfl_xor_sync(0xffffffffu, all[0], d);
+        all[1] += __shfl_xor_sync(0xffffffffu, all[1], d);
+    }
+    if (WARPS > 1) {
+        if (lane == 0) { totals[2 * warp] = all[0]; totals[2 * warp + 1] = all[1]; }
+        __syncthreads();
+        all[0] = all[1] = 0;
+#pragma unroll
+        for (int k = 0; k < WARPS; ++k) { all[0] += totals[2 * k]; all[1] += totals[2 * k + 1]; }
+    }
+    const Ordered O = {(uint32_t)__cvta_generic_to_shared(mine), (uint32_t)__cvta_generic_to_shared(before), weight};
+    if (ALL3) ordered_rounds<7, PER, WARPS>(P, O, all[0], all[1], zero_too, most, red2, r);
+    else if (b == 1) ordered_rounds<1, PER, WARPS>(P, O, all[0], all[1], zero_too, most, red2, r);
+    else if (b == 2) ordered_rounds<2, PER, WARPS>(P, O, all[0], all[1], zero_too, most, red2, r);
+    else ordered_rounds<4, PER, WARPS>(P, O, all[0], all[1], zero_too, most, red2, r);
+    leave(P.turn);
+}
+
 }  // namespace lowra
 
 namespace lowra {
@@ -854,21 +1183,56 @@ lowra_status launch_sorted_kernel(LearnParams& P, int rows, void* stream) {
 
 bool two_long_rows(int K) { return 2 * (sorted_smem_bytes(K) + 1024) <= 228 * 1024; }   // an SM holds two (K <= 11776)
 
-// Whether the rounds of a class together are long enough to pay for the order (c = 0, 1, 2: 1, 2, 4 bits; 3: all of them).  Measured, us, 4096 rows
-// (K = 13824: 3328), learn_kernel against sorted_learn_kernel, after 2, 4 and 10 rounds:
-//             1 bit                              2 bits                             4 bits                              all three, 2 and 10
-//   K=1024    11 16 27       19 22 30            15 24 52       19 22 33            54 98 221        22 30 53           80 311     27 69
-//   K=2048    15 23 41       31 34 42            22 37 79       31 34 46            63 114 271       33 39 57           97 391     36 69
-//   K=4096    24 38 72       57 65 80            37 63 137      57 64 86            95 173 408       62 72 105          149 622    64 122
-//   K=5120    33 50 93       72 81 102           50 83 184      73 82 108           111 202 474      78 91 132          178 748    83 156
-//   K=8192    48 71 135      134 151 195         73 122 270     134 152 201         173 313 733      141 166 238        273 1140   141 247
-//   K=11008   69 99 188      171 187 229         101 167 369    173 189 238         274 491 1143     179 204 278        436 1800   180 278
-//   K=13824   74 106 199     238 263 331         108 175 383    238 264 344         273 494 1160     252 290 403        429 1780   253 416
-// The lines cross where the table below has them; with all three (an assessment) already in the first round.
-bool sorted_pays(int K, int c, int iterations) {
-    if (K > kSortedMaxK || iterations < 1) return false;
-    constexpr int kRounds[3][3] = {{12, 4, 1}, {25, 6, 2}, {43, 9, 2}};
-    return c == 3 || iterations >= kRounds[K <= 5120 ? 0 : two_long_rows(K) ? 1 : 2][c];
+// Which kernel takes a class of rows (c = 0, 1, 2: 1, 2, 4 bits; 3: all of them).  Measured, us, 4096 rows (K >= 13824: 3328) after 2, 4 and 10
+// rounds, learn_kernel / ordered_learn_kernel at 1 and 2 bits, ordered_learn_kernel / sorted_learn_kernel else:
+//             1 bit                            2 bits                           4 bits                            all three
+//   K=512     11/6    15/8    24/12            14/8    23/11   48/20            17/14   28/18   62/28             22/19   38/27   85/48
+//   K=1024    11/9    16/12   27/16            15/10   23/14   49/23            19/21   31/28   68/48             23/27   39/38   90/68
+//   K=2048    16/17   23/20   41/26            23/19   37/22   78/31            29/34   39/40   77/59             33/37   47/46   97/72
+//   K=3072    21/29   31/35   56/47            31/32   50/39   108/58           49/51   70/62   137/93            57/55   87/70   179/112
+//   K=4096    26/30   39/36   72/48            39/33   63/40   138/59           49/63   71/74   140/109           57/67   87/83   181/127
+//   K=5120    34/44   51/52   94/73            50/48   84/59   185/91           75/78   108/93  216/136           87/84   133/103 281/159
+//   K=8192    48/56   71/64   134/90           72/60   121/73  267/113          94/143  140/170 277/245           107/140 172/169 359/247
+//   K=11008   69/99   100/116 188/168          102/106 168/130 369/204          157/180 231/206 462/284           181/183 282/209 592/287
+//   K=13824   74/93   107/110 199/155          106/101 175/124 381/197          153/255 230/296 460/417           178/252 281/294 589/418
+//   K=16384   83/97   119/114 225/162          120/105 197/130 432/209          169/281 263/322 549/443           199/279 328/321 704/445
+// At 1 bit the ordered blocks pay in the fourth round where every lane has a block, later where some have none (K = 3072, 5120), or where an SM
+// holds few warps (K = 8320 to 12288); K up to 2048 is one warp, up to 1024 of short networks.
+enum Kernel { kRowAgain, kOrdered, kSorted };
+int ordered_warps(int K) { return (K + 2047) / 2048; }
+Kernel kernel_for(int K, int c, int iterations) {
+    if (K > kSortedMaxK || iterations < 1) return kRowAgain;
+    if (c == 0) {
+        const bool pays = K <= 1024 || (K <= 2048 ? iterations >= 3 : (iterations - (K > 8192 && K <= 12288 ? 2 : 0)) * K >= 4 * 2048 * ordered_warps(K));
+        return pays ? kOrdered : kRowAgain;
+    }
+    if (c == 1) return K <= 1024 || iterations >= 2 ? kOrdered : kRowAgain;
+    constexpr int kUpTo[] = {512, 1024, 2048, 3072, 4096, 6144, 8192, 11776}, kFour[] = {2, 3, 4, 3, 5, 3, 7, 4, 9}, kAll[] = {2, 4, 4, 2, 4, 2, 4, 3, 5};
+    int i = 0;
+    while (i < 8 && K > kUpTo[i]) ++i;
+    return iterations >= (c == 2 ? kFour : kAll)[i] ? kSorted : kOrdered;
+}
+
+template <bool ALL3, int PER, int WARPS, int CTAS>
+lowra_status launch_ordered_kernel(const LearnParams& P, int rows, void* stream) {
+    static SmemLimit limit = {};
+    return launch_rows(ordered_learn_kernel<ALL3, PER, WARPS, CTAS>, P, rows, 32 * WARPS, ordered_smem<ALL3, PER, WARPS>(), &limit, stream);
+}
+
+// As many rows to an SM as its shared memory takes: 12 KB for 2048 values.
+template <bool ALL3>
+lowra_status launch_ordered(const LearnParams& P, int rows, void* stream) {
+    const int K = P.K;
+    return K <= 512 ? launch_ordered_kernel<ALL3, 16, 1, 32>(P, rows, stream)
+         : K <= 1024 ? launch_ordered_kernel<ALL3, 32, 1, 24>(P, rows, stream)
+         : K <= 2048 ? launch_ordered_kernel<ALL3, 64, 1, 16>(P, rows, stream)
+         : K <= 4096 ? launch_ordered_kernel<ALL3, 64, 2, 8>(P, rows, stream)
+         : K <= 6144 ? launch_ordered_kernel<ALL3, 64, 3, 5>(P, rows, stream)
+         : K <= 8192 ? launch_ordered_kernel<ALL3, 64, 4, 4>(P, rows, stream)
+         : K <= 10240 ? launch_ordered_kernel<ALL3, 64, 5, 3>(P, rows, stream)
+         : K <= 12288 ? launch_ordered_kernel<ALL3, 64, 6, 2>(P, rows, stream)
+         : K <= 14336 ? launch_ordered_kernel<ALL3, 64, 7, 2>(P, rows, stream)
+                      : launch_ordered_kernel<ALL3, 64, 8, 2>(P, rows, stream);
 }
 
 // validation shared by the two entry points is done by the callers; this fills the tables and launches (n1, n2, n4: rows to be
@@ -881,6 +1245,7 @@ lowra_status launch_learn(LearnParams& P, const double* init_levels_host, const 
     if (st != LOWRA_OK) return st;
     int log_k = 0;
     while ((2 << log_k) <= P.K) ++log_k;
+    P.one = 1;
     P.near_zero = (unsigned)(1023 + 24 + log_k) << 20;
     for (int c = 0; c < 3; ++c)
         for (int j = 0; j < 16; ++j) {
@@ -888,34 +1253,40 @@ lowra_status launch_learn(LearnParams& P, const double* init_levels_host, const 
             P.init_t[c][j] = init_thresholds_host[c * 16 + j];
         }
     // stored rows are in the order of their precisions: the last `sorted` of them go to the sorted kernel
-    int sorted = 0;
-    if (ALL3) {
-        sorted = sorted_pays(P.K, 3, P.iterations) ? P.N : 0;
-    } else {
-        if (sorted_pays(P.K, 2, P.iterations)) sorted += n4;
-        if (sorted_pays(P.K, 1, P.iterations)) sorted += n2;
-        if (sorted_pays(P.K, 0, P.iterations)) sorted += n1;
+    Kernel kernel[3];
+    for (int c = 0; c < 3; ++c) kernel[c] = kernel_for(P.K, ALL3 ? 3 : c, P.iterations);
+    // Stored rows are in the order of their precisions, and more bits want more order: a launch for every kernel that has classes, the last classes' first
+    // (in turns; see enter()).
+    const int n[3] = {n1, n2, n4};
+    int end = P.N;
+    P.turn = 0;
+    for (int c = ALL3 ? 0 : 2; end > 0; ) {
+        const Kernel k = kernel[c];
+        int rows = ALL3 ? P.N : 0;
+        for (; !ALL3 && c >= 0 && (kernel[c] == k || n[c] == 0); --c) rows += n[c];
+        if (rows == 0) continue;
+        if (rows < P.N) P.turn = end == P.N ? 1 : 2;
+        P.row0 = end - rows;
+        end -= rows;
+        if (k == kOrdered) {
+            st = launch_ordered<ALL3>(P, rows, stream);
+        } else if (k == kSorted) {
+            // As many CTAs to an SM as its shared memory takes, for the phases of one row leave what bounds the others idle.  The registers
+            // go with that: 16 elements a thread up to K = 8192; beyond it two rows of 512 threads beat one of 1024 (K = 11008: 152
+            // against 232 us) as long as two fit.
+            st = P.K <= 4096       ? launch_sorted_kernel<ALL3, 256, 16, 5>(P, rows, stream)
+               : P.K <= 5120       ? launch_sorted_kernel<ALL3, 320, 16, 4>(P, rows, stream)
+               : P.K <= 8192       ? launch_sorted_kernel<ALL3, 512, 16, 2>(P, rows, stream)
+               : two_long_rows(P.K) ? launch_sorted_kernel<ALL3, 512, 32, 2>(P, rows, stream)
+                                    : launch_sorted_kernel<ALL3, 1024, 16, 1>(P, rows, stream);
+        } else {
+            const bool four = (ALL3 || (kernel[2] == kRowAgain && n4 > 0)) && P.iterations > 0;
+            st = four ? launch_learn_kernel<ALL3, true, 128>(P, rows, stream)
+               : P.K <= 4096 ? launch_learn_kernel<ALL3, false, 64>(P, rows, stream) : launch_learn_kernel<ALL3, false, 128>(P, rows, stream);
+        }
+        if (st != LOWRA_OK) return st;
     }
-    const bool two = sorted > 0 && sorted < P.N;
-    if (sorted > 0) {
-        P.row0 = P.N - sorted;
-        P.turn = two ? 1 : 0;
-        // As many CTAs to an SM as its shared memory takes, for the phases of one row leave what bounds the others idle.  The registers
-        // go with that: 16 elements a thread up to K = 8192; beyond it two rows of 512 threads beat one of 1024 (K = 11008: 152
-        // against 232 us) as long as two fit.
-        st = P.K <= 4096       ? launch_sorted_kernel<ALL3, 256, 16, 5>(P, sorted, stream)
-           : P.K <= 5120       ? launch_sorted_kernel<ALL3, 320, 16, 4>(P, sorted, stream)
-           : P.K <= 8192       ? launch_sorted_kernel<ALL3, 512, 16, 2>(P, sorted, stream)
-           : two_long_rows(P.K) ? launch_sorted_kernel<ALL3, 512, 32, 2>(P, sorted, stream)
-                                : launch_sorted_kernel<ALL3, 1024, 16, 1>(P, sorted, stream);
-        if (st != LOWRA_OK || !two) return st;
-    }
-    const int rows = P.N - sorted;
-    P.row0 = 0;
-    P.turn = two ? 2 : 0;
-    const bool four = (ALL3 || (!two && n4 > 0)) && P.iterations > 0;
-    return four ? launch_learn_kernel<ALL3, true, 128>(P, rows, stream)
-         : P.K <= 4096 ? launch_learn_kernel<ALL3, false, 64>(P, rows, stream) : launch_learn_kernel<ALL3, false, 128>(P, rows, stream);
+    return LOWRA_OK;
 }
 
 }  // namespace
