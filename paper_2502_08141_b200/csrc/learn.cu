@@ -898,6 +898,11 @@ __device__ __forceinline__ long long lds_s64(uint32_t at) {
     return v;
 }
 
+// (by the instruction's own predicate; see threshold_place)
+__device__ __forceinline__ void add_if_below(uint32_t& a, uint32_t by, float x, float t) {
+    asm("{\n\t.reg .pred p;\n\tsetp.lt.f32 p, %1, %2;\n\t@p add.u32 %0, %0, %3;\n\t}" : "+r"(a) : "f"(x), "f"(t), "r"(by));
+}
+
 // What a thread has in order: PER values, 32 apart, and their weight.
 struct Ordered {
     uint32_t xs;        // this thread's first value
@@ -958,20 +963,19 @@ __device__ __forceinline__ void ordered_rounds(const LearnParams& P, const Order
         for (int q0 = 0; q0 < NQ; q0 += kAtOnce) {
             float tq[kAtOnce];
             uint32_t at[kAtOnce];
-            int n[kAtOnce];
+            uint32_t n[kAtOnce];
             double s[kAtOnce];
 #pragma unroll
             for (int k = 0; k < kAtOnce; ++k) {
                 tq[k] = __shfl_sync(0xffffffffu, t, V::lane_of(q0 + k));
                 at[k] = O.xs;
                 s[k] = kGrid;
-                n[k] = 0;
+                n[k] = 0u;
             }
 #pragma unroll
             for (int h = PER / 2; h >= 4; h /= 2) {
 #pragma unroll
-                for (int k = 0; k < kAtOnce; ++k)
-                    if (lds_f32(at[k] + (h - 1) * 128) < tq[k]) at[k] += h * 128;
+                for (int k = 0; k < kAtOnce; ++k) add_if_below(at[k], h * 128, lds_f32(at[k] + (h - 1) * 128), tq[k]);
             }
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
@@ -979,7 +983,7 @@ __device__ __forceinline__ void ordered_rounds(const LearnParams& P, const Order
                 for (int k = 0; k < kAtOnce; ++k) {
                     const float x = lds_f32(at[k] + e * 128);
                     const double d = (double)x;
-                    if (x < tq[k]) ++n[k];
+                    n[k] += x < tq[k] ? 1u : 0u;
                     s[k] = __fma_rd(__hiloint2double(x < tq[k] ? __double2hiint(d) : 0, __double2loint(d)), w, s[k]);   // (see few_buckets)
                 }
             }
@@ -988,7 +992,7 @@ __device__ __forceinline__ void ordered_rounds(const LearnParams& P, const Order
             for (int k = 0; k < kAtOnce; ++k) {
                 const uint32_t before = at[k] - O.xs;
                 v[2 * k] = lds_s64(O.sums + before / 2) + (long long)(grid_bits(s[k]) - grid_bits(kGrid));
-                v[2 * k + 1] = (n[k] + (int)(before / 128)) * wg;
+                v[2 * k + 1] = (long long)(n[k] + before / 128) * wg;
             }
             Halve<2 * kAtOnce, 16>::sums(v, lane);
             if (slot >= 0 && 2 * q0 + slot < 2 * NQ) red[(2 * q0 + slot) * WARPS + warp] = v[0];
