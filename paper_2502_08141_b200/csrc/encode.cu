@@ -139,11 +139,7 @@ __device__ __forceinline__ void encode_chunk(const EncodeParams& P, int p, int c
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const float n = __fmul_rn(x[4 * q + i], inv);
-                uint32_t a = t7 <= n ? t_at + 32u : t_at;
-                a += lds_f32(a + 12u) <= n ? 16u : 0u;
-                a += lds_f32(a + 4u) <= n ? 8u : 0u;
-                a += lds_f32(a) <= n ? 4u : 0u;
-                sum += a << (4 * i);
+                sum += threshold_place(t_at, t7, n) << (4 * i);
             }
             const uint32_t codes = (sum - t_at * 0x1111u) >> 2;
             w[q >> 1] = (q & 1) ? w[q >> 1] | (codes << 16) : codes;

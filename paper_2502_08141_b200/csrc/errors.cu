@@ -17,9 +17,9 @@
 // time.  At 1 and 2 bits the two or four values w_hat are formed once per half block and picked by comparison; at 4 bits
 // a branch-free binary search finds the level.  The residual is written over the weights in shared memory and leaves in one bulk copy
 // per chunk.
-// What bounds it: memory at 1 and 2 bits (5120 x 5120 at 85/15 % with the residual 44.6 -> 37.3 us, 85 % of the copy rate; without it 26.2 ->
-// 20.7), the half-rate pipe for comparisons, selections and address arithmetic at 4 bits and for all three precisions at once (4096 x 4096: 29.1 ->
-// 21.1 and 40.7 -> 31 us).
+// What bounds it: memory at 1 and 2 bits (5120 x 5120 at 85/15 % with the residual 37 us, 85 % of the copy rate; without it 19.8), instruction
+// issue at 4 bits and for all three precisions at once (48 instructions an element in 73 % of the slots; 4096 x 4096: 21.6 -> 19.6 us with conditional
+// additions and subtractions instead of selections, and what comes in pairs in packed instructions; 31.6 -> 28.4, a value normalised once for all).
 #include "row_stream.cuh"
 
 namespace lowra {
@@ -38,60 +38,122 @@ struct ErrParams {
     float* residual;          // [N, K] or null
 };
 
+// What is left of x after the value its bucket stands for, 1 bit (two values) and 2 bits (four): every candidate's difference, the last whose
+// threshold is <= n stands.  Comparisons and selections go to the half-rate pipe, conditional subtractions to the other one.
+__device__ __forceinline__ float residual_of(float x, float n, const float (&w)[2], const float (&t)[1]) {
+    float r;
+    asm("{\n\t.reg .pred p;\n\tsetp.le.f32 p, %4, %5;\n\tsub.rn.f32 %0, %1, %2;\n\t@p sub.rn.f32 %0, %1, %3;\n\t}"
+        : "=&f"(r) : "f"(x), "f"(w[0]), "f"(w[1]), "f"(t[0]), "f"(n));
+    return r;
+}
+__device__ __forceinline__ float residual_of(float x, float n, const float (&w)[4], const float (&t)[3]) {
+    float r;
+    asm("{\n\t.reg .pred p, q, s;\n\tsetp.le.f32 p, %6, %9;\n\tsetp.le.f32 q, %7, %9;\n\tsetp.le.f32 s, %8, %9;\n\tsub.rn.f32 %0, %1, %2;\n\t"
+        "@p sub.rn.f32 %0, %1, %3;\n\t@q sub.rn.f32 %0, %1, %4;\n\t@s sub.rn.f32 %0, %1, %5;\n\t}"
+        : "=&f"(r) : "f"(x), "f"(w[0]), "f"(w[1]), "f"(w[2]), "f"(w[3]), "f"(t[0]), "f"(t[1]), "f"(t[2]), "f"(n));
+    return r;
+}
+
+// A row's codebook at B bits for one half block: the values its buckets stand for there (1 and 2 bits), and the thresholds; or (4 bits) where
+// levels and thresholds lie, which a binary search on addresses reads.
+template <int B>
+struct HalfBlock {
+    float w[1 << B], t[(1 << B) - 1];
+    __device__ __forceinline__ HalfBlock(const float* y, float m) {
+#pragma unroll
+        for (int k = 0; k < (1 << B); ++k) w[k] = __uint_as_float(pack_bf16x2(0.0f, __fmul_rn(y[k], m)) & 0xFFFF0000u);
+#pragma unroll
+        for (int k = 0; k + 1 < (1 << B); ++k) t[k] = y[kTableStride + k];
+    }
+    __device__ __forceinline__ float residual(float x, float n) const { return residual_of(x, n, w, t); }
+};
+template <>
+struct HalfBlock<4> {
+    uint32_t at;
+    float t7, m;
+    __device__ __forceinline__ HalfBlock(const float* y, float m_) : at((uint32_t)__cvta_generic_to_shared(y + kTableStride)), t7(y[kTableStride + 7]), m(m_) {}
+    __device__ __forceinline__ float residual(float x, float n) const {
+        const uint32_t a = threshold_place(at, t7, n);
+        return __fsub_rn(x, __uint_as_float(pack_bf16x2(0.0f, __fmul_rn(lds_f32(a - 4u * kTableStride), m))));
+    }
+};
+
+// Two fp32 operations in one instruction, each rounded as by itself.
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+    float2 d;
+    asm("{\n\t.reg .b64 a, b, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tmul.rn.f32x2 d, a, b;\n\tmov.b64 {%0, %1}, d;\n\t}"
+        : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+    float2 d;
+    asm("{\n\t.reg .b64 a, b, c, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tmov.b64 c, {%6, %7};\n\tfma.rn.f32x2 d, a, b, c;\n\tmov.b64 {%0, %1}, d;\n\t}"
+        : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    return d;
+}
+
+template <bool PACKED>
+__device__ __forceinline__ float2 normalised(float a, float b, float inv) {
+    return PACKED ? mul2(make_float2(a, b), make_float2(inv, inv)) : make_float2(__fmul_rn(a, inv), __fmul_rn(b, inv));
+}
+
+// Error of four neighbouring elements: four squares in fp32, then into the fp64 sum.  PACKED: without residuals to keep, where instructions bound the kernel (three
+// precisions 31 -> 28.4 us on 4096 x 4096); residuals next to one another for both purposes cost moves (at 4 bits 24.4 -> 28.1).
+template <bool PACKED>
+__device__ __forceinline__ double four_squares(const float (&r)[4]) {
+    if (!PACKED) return (double)__fadd_rn(__fmaf_rn(r[0], r[0], __fmul_rn(r[1], r[1])), __fmaf_rn(r[2], r[2], __fmul_rn(r[3], r[3])));
+    const float2 even = make_float2(r[0], r[2]), odd = make_float2(r[1], r[3]);
+    const float2 s = fma2(even, even, mul2(odd, odd));
+    return (double)__fadd_rn(s.x, s.y);
+}
+
 // Error of a lane's part of a block at B bits (inv: what normalises it; m: the block's absmax; y: the row's levels in shared memory, its
 // thresholds behind them); with RES the residuals take the weights' places.  The number of thresholds <= n picks the level
 // (thresholds sorted, as the encoder assumes).
 template <int B, bool RES, int PER>
 __device__ __forceinline__ double half_block_error(float (&x)[PER], float inv, float m, const float* y) {
-    const float* t = y + kTableStride;
+    const HalfBlock<B> book(y, m);
     double acc = 0.0;
-    float wh[B == 4 ? 1 : 1 << B], th[B == 4 ? 1 : (1 << B) - 1];
-    if (B <= 2) {
-#pragma unroll
-        for (int k = 0; k < (1 << B); ++k) wh[k] = __uint_as_float(pack_bf16x2(0.0f, __fmul_rn(y[k], m)) & 0xFFFF0000u);
-#pragma unroll
-        for (int k = 0; k + 1 < (1 << B); ++k) th[k] = t[k];
-    }
-    const float t7 = t[7];
-    const uint32_t t_at = (uint32_t)__cvta_generic_to_shared(t);
 #pragma unroll
     for (int q = 0; q < PER / 4; ++q) {
-        float res[4];
+        float r[4];
 #pragma unroll
         for (int e = 0; e < 4; e += 2) {
-            const float n0 = __fmul_rn(x[4 * q + e], inv), n1 = __fmul_rn(x[4 * q + e + 1], inv);
-            float w0, w1;
-            if (B <= 2) {
-                auto pick = [&](float n) {
-                    if (B == 1) return th[0] <= n ? wh[1] : wh[0];
-                    const bool hi = th[B == 2 ? 1 : 0] <= n;
-                    const bool lo = (hi ? th[B == 2 ? 2 : 0] : th[0]) <= n;
-                    const float a = hi ? wh[B == 2 ? 2 : 0] : wh[0], b = hi ? wh[B == 2 ? 3 : 0] : wh[1];
-                    return lo ? b : a;
-                };
-                w0 = pick(n0);
-                w1 = pick(n1);
-            } else {
-                // binary search on shared-memory addresses: the thresholds lie behind the levels
-                auto level = [&](float n) {
-                    uint32_t a = t7 <= n ? t_at + 32u : t_at;
-                    a += lds_f32(a + 12u) <= n ? 16u : 0u;
-                    a += lds_f32(a + 4u) <= n ? 8u : 0u;
-                    a += lds_f32(a) <= n ? 4u : 0u;
-                    return lds_f32(a - 4u * kTableStride);
-                };
-                const uint32_t h = pack_bf16x2(__fmul_rn(level(n0), m), __fmul_rn(level(n1), m));
-                w0 = __uint_as_float(h << 16);
-                w1 = __uint_as_float(h & 0xFFFF0000u);
-            }
-            res[e] = __fsub_rn(x[4 * q + e], w0);
-            res[e + 1] = __fsub_rn(x[4 * q + e + 1], w1);
+            const float2 n = normalised<!RES>(x[4 * q + e], x[4 * q + e + 1], inv);
+            r[e] = book.residual(x[4 * q + e], n.x);
+            r[e + 1] = book.residual(x[4 * q + e + 1], n.y);
         }
-        // four squares in fp32, then into the fp64 sum
-        acc += (double)__fadd_rn(__fmaf_rn(res[0], res[0], __fmul_rn(res[1], res[1])), __fmaf_rn(res[2], res[2], __fmul_rn(res[3], res[3])));
-        if (RES) { x[4 * q] = res[0]; x[4 * q + 1] = res[1]; x[4 * q + 2] = res[2]; x[4 * q + 3] = res[3]; }
+        acc += four_squares<!RES>(r);
+        if (RES) { x[4 * q] = r[0]; x[4 * q + 1] = r[1]; x[4 * q + 2] = r[2]; x[4 * q + 3] = r[3]; }
     }
     return acc;
+}
+// At all three precisions: the tables one behind the other.
+template <int PER>
+__device__ __forceinline__ void half_block_errors(const float (&x)[PER], float inv, float m, const float* y, double (&acc)[3]) {
+    const HalfBlock<1> one_bit(y, m);
+    const HalfBlock<2> two_bits(y + 32, m);
+    const HalfBlock<4> four_bits(y + 64, m);
+    double sum[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+    for (int q = 0; q < PER / 4; ++q) {
+        float r[3][4];
+#pragma unroll
+        for (int e = 0; e < 4; e += 2) {
+            const float2 n2 = normalised<true>(x[4 * q + e], x[4 * q + e + 1], inv);
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const float v = x[4 * q + e + i], n = i ? n2.y : n2.x;
+                r[0][e + i] = one_bit.residual(v, n);
+                r[1][e + i] = two_bits.residual(v, n);
+                r[2][e + i] = four_bits.residual(v, n);
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) sum[k] += four_squares<true>(r[k]);
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) acc[k] += sum[k];
 }
 
 // sum over the warp, in a fixed order
@@ -172,9 +234,7 @@ __device__ __forceinline__ void error_rows(const Params& P, int N, int K) {
             const float inv = (m == 0.0f) ? 0.0f : __frcp_rn(m);
             if (in) {
                 if constexpr (NP == 3) {
-                    acc[0] += half_block_error<1, false, PER>(x, inv, m, tables);
-                    acc[1] += half_block_error<2, false, PER>(x, inv, m, tables + 32);
-                    acc[2] += half_block_error<4, false, PER>(x, inv, m, tables + 64);
+                    half_block_errors<PER>(x, inv, m, tables, acc);
                 } else {
                     const int p = N - 1 - ((int)blockIdx.x + at.i * (int)gridDim.x);
                     if (p < P.L.class_start[1]) acc[0] += half_block_error<1, RES, PER>(x, inv, m, tables);

@@ -87,6 +87,21 @@ __device__ __forceinline__ float lds_f32(uint32_t at) {
     return v;
 }
 
+// Binary search among 15 sorted thresholds in shared memory at t_at, the middle one in t7: the address of the first that is above n (of the sixteenth place if
+// none is).  The additions are conditional by the instruction's own predicate, one each instead of a selection and an addition (written as plain
+// conditions, nvcc 12.9 makes wrong code of it in encode.cu: some values one bucket too high).
+__device__ __forceinline__ uint32_t threshold_place(uint32_t t_at, float t7, float n) {
+    uint32_t a = t_at;
+    auto step = [&](float t, uint32_t by) {
+        asm("{\n\t.reg .pred p;\n\tsetp.le.f32 p, %1, %2;\n\t@p add.u32 %0, %0, %3;\n\t}" : "+r"(a) : "f"(t), "f"(n), "r"(by));
+    };
+    step(t7, 32u);
+    step(lds_f32(a + 12u), 16u);
+    step(lds_f32(a + 4u), 8u);
+    step(lds_f32(a), 4u);
+    return a;
+}
+
 __device__ __forceinline__ uint4 ld_stream_v4(const void* p) {
     uint4 v;
     asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
