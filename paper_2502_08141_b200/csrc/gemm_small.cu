@@ -3,7 +3,7 @@
 // With a handful of tokens the work is reading the weight's codes once (1 - 2 bits per weight), a few microseconds of memory
 // time: what counts is how many SMs share it and how long the longest chain of dependent steps is.  The persistent
 // tensor-core kernel (gemm_fused.cu) has tiles of 256 channels and 256 tokens, of which a 4096 x 4096 weight is 16: cut in four, their
-// slices handed over, it takes 26 us for 1 token as for 65.  Here two launches share the work finely instead (1 token 10.1, 16 tokens 13.3):
+// slices handed over, it takes 26 us for 1 token as for 65.  Here two launches share the work finely instead (1 token 9.6, 16 tokens 11.9):
 //   project_kernel   T = bf16(s X A): a CTA per 16 tokens and slice of the contraction, the slices of a cluster added up
 //                    through distributed shared memory.
 //   small_kernel     a CTA takes 64 stored rows of one precision and a slice of the contraction, its warps 16 rows and half
@@ -322,8 +322,8 @@ __device__ __forceinline__ void multiply_rows(int K, const SmallMember& W, int m
 //           which the others' warps write into its shared memory;
 //   MERGED: one CTA does all slices of a group, each half of its warps every other half of them.  For grids of several waves: a CTA costs
 //           about 4 us beside its steps (its launch in a cluster, the way from a row's number to its codes, a barrier of the cluster).
-template <int NT8, int NB, bool MERGED>
-__global__ void __launch_bounds__(kSmallThreads, 2) small_kernel(const __grid_constant__ SmallParams<NB> P, const int slices) {
+template <int NT8, int NB, bool MERGED, int CTAS>
+__global__ void __launch_bounds__(kSmallThreads, CTAS) small_kernel(const __grid_constant__ SmallParams<NB> P, const int slices) {
     extern __shared__ __align__(128) unsigned char small_smem[];
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (!MERGED) cluster_arrive();   // "this CTA runs": waited for before its shared memory is written from elsewhere
@@ -332,7 +332,7 @@ __global__ void __launch_bounds__(kSmallThreads, 2) small_kernel(const __grid_co
     float* sums = reinterpret_cast<float*>(small_smem + 2 * kTokenBytes);   // spread: [slots][tokens][share of the rows]; MERGED: see end()
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const int rank = MERGED ? 0 : (int)ptx::cluster_ctarank();
-    int grp = MERGED ? (int)blockIdx.x : (int)blockIdx.x / slices;
+    int grp = MERGED ? (int)blockIdx.x : ((int)gridDim.x - 1 - (int)blockIdx.x) / slices;     // (spread: the long rows of 4 bits first)
     const Unit un = unit_at(P, (int)blockIdx.y, kTokens);
     const SmallMember& W = P.m[un.member];
     // the group's rows: 64 neighbouring stored rows of one precision class
@@ -678,11 +678,11 @@ lowra_status launch_units(const SmallParams<NB>& P, int groups, int slices, cuda
     return cudaLaunchKernelEx(&cfg, units_kernel<NB>, P, order, slices) == cudaSuccess ? LOWRA_OK : LOWRA_ERR_CUDA;
 }
 
-template <int NT8, int NB, bool MERGED>
+template <int NT8, int NB, bool MERGED, int CTAS>
 lowra_status launch_product(const SmallParams<NB>& P, int groups, int units, int slices, cudaStream_t stream) {
     const size_t smem = 4u * (8 * NT8) * kSmallSpan * 2u + (MERGED ? (2 + slices / 2) * (8 * NT8) * kMergedPitch * 4u : 2u * (8 * NT8) * kSmallRows * 4u);
     static SmemLimit limit = {};
-    if (ensure_smem_limit(reinterpret_cast<const void*>(small_kernel<NT8, NB, MERGED>), smem, &limit) != LOWRA_OK) return LOWRA_ERR_CUDA;
+    if (ensure_smem_limit(reinterpret_cast<const void*>(small_kernel<NT8, NB, MERGED, CTAS>), smem, &limit) != LOWRA_OK) return LOWRA_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -696,7 +696,7 @@ lowra_status launch_product(const SmallParams<NB>& P, int groups, int units, int
     cfg.stream = stream;
     cfg.attrs = attr;
     cfg.numAttrs = MERGED ? 1 : 2;
-    return cudaLaunchKernelEx(&cfg, small_kernel<NT8, NB, MERGED>, P, slices) == cudaSuccess ? LOWRA_OK : LOWRA_ERR_CUDA;
+    return cudaLaunchKernelEx(&cfg, small_kernel<NT8, NB, MERGED, CTAS>, P, slices) == cudaSuccess ? LOWRA_OK : LOWRA_ERR_CUDA;
 }
 
 int product_slices(int N, int K) {
@@ -704,6 +704,19 @@ int product_slices(int N, int K) {
     int slices = 1;
     while (slices < 8 && 4 * slices <= n_span && 2 * slices * by_shape <= 3 * kNumSMs) slices *= 2;
     return slices;
+}
+
+// Whether the spread form runs three CTAs to an SM, at 80 registers (some of which spill, most at 4 bits), or two at 128: for so many CTAs beside so
+// many of the projection, `four` of N channels at 4 bits.  Three where two do not fit in one wave - clusters of eight leave SMs of a GPC over - and for short
+// steps at few tokens, which wait for memory rather than for instructions.  Two against three, us (rows of 4 bits first in both; before, they were last: in brackets):
+// 60/35/5 %, 1 token: 11008 x 4096 19.6 -> 16.4 (24.7), 13824 x 5120 22.5 -> 19.6 (28.1), 6144 x 4096 16.4 -> 11.7 (18.2), 5120 x 13824 30.2 -> 24.6 (36.5), 2048 x 4096
+// 12.8 -> 10.0 (14.0), 4096 x 4096 10.25 -> 9.6; 16 tokens: 11008 x 4096 24.9 -> 19.7 (30.5), 4096 x 4096 13.0 -> 11.9.  Two where they fit and steps are long
+// (4096 x 11008, 16 tokens 18.9, three 20.1; 24 tokens 20.6, 28.3) and with most rows at 4 bits (13824 x 5120, 16 tokens 30.9, three 33.9; 4096 x 4096, 1 token 10.5, 11.5),
+// unless short steps take two waves (6144 x 4096 of 4 bits, 1 token 19.0, three 14.7).
+bool three_pay(int four, int N, int n_span, int slices, int ctas, int projection, int nt8) {
+    if (nt8 > 3) return false;                           // (no shared memory for a third)
+    const bool fit = ctas + projection <= (slices == 8 ? 272 : slices == 4 ? 280 : 2 * kNumSMs), short_steps = n_span <= 2 * (2 * slices);
+    return fit ? short_steps && nt8 <= 2 && four <= N / 8 : short_steps || four <= N / 2;
 }
 
 // groups of 64 stored rows of one precision (of the member that has the most)
@@ -761,12 +774,14 @@ lowra_status launch_members(const SmallParams<NB>& P, cudaStream_t stream) {
     // tokens a group 64 in 2 38.5 against 34.8; on 4096 x 11008 - slots of five steps - 6 in 3 54.5 against 46.1; one group 18.8 against 10.6.)
     if constexpr (NB > 1) {
         if (slices > 1 && nt8 <= 2 && n_span <= 2 * (2 * slices) && groups * slices * units > 2 * kNumSMs)
-            return nt8 == 1 ? launch_product<1, NB, true>(P, groups, units, slices, stream) : launch_product<2, NB, true>(P, groups, units, slices, stream);
+            return nt8 == 1 ? launch_product<1, NB, true, 2>(P, groups, units, slices, stream) : launch_product<2, NB, true, 2>(P, groups, units, slices, stream);
     }
-    if (nt8 == 1) return launch_product<1, NB, false>(P, groups, units, slices, stream);
-    if (nt8 == 2) return launch_product<2, NB, false>(P, groups, units, slices, stream);
-    if (nt8 == 3) return launch_product<3, NB, false>(P, groups, units, slices, stream);
-    return launch_product<4, NB, false>(P, groups, units, slices, stream);
+    const int* start = P.m[0].L.class_start;
+    const bool three = three_pay(start[3] - start[2], P.N, n_span, slices, groups * slices * units, 8 * m16, nt8);
+    if (nt8 == 1) return three ? launch_product<1, NB, false, 3>(P, groups, units, slices, stream) : launch_product<1, NB, false, 2>(P, groups, units, slices, stream);
+    if (nt8 == 2) return three ? launch_product<2, NB, false, 3>(P, groups, units, slices, stream) : launch_product<2, NB, false, 2>(P, groups, units, slices, stream);
+    if (nt8 == 3) return three ? launch_product<3, NB, false, 3>(P, groups, units, slices, stream) : launch_product<3, NB, false, 2>(P, groups, units, slices, stream);
+    return launch_product<4, NB, false, 2>(P, groups, units, slices, stream);
 }
 
 }  // namespace
