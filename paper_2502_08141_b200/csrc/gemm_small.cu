@@ -790,7 +790,7 @@ lowra_status launch_members(const SmallParams<NB>& P, cudaStream_t stream) {
 // 1, 2 and 4 bits: 2.8 for the projection and the start, then CTAs, two to an SM.  A step of 256 takes 2.5, 0.45 more at 4 bits; around a CTA's steps and its
 // share of the low-rank term 5.4, and if it is alone on its SM all that takes 0.64 of it.  A CTA that does all slices takes 3.7 and 1.2 for every slice around its
 // steps, of which two halves overlap (0.74), and waits 1.7 for 4-bit rows among others; of three on an SM the third does not wait for both.  Fitted to 520
-// calls (256 to 13824 channels, 512 to 13824 features, ranks 16 to 128, six mixes): within 17 %.
+// calls (256 to 13824 channels, 512 to 13824 features, ranks 16 to 128, six mixes): within 18 %.  Where three CTAs share an SM in one wave, 0.85 of that.
 float small_estimate(const int32_t* n, int K, int r, int units, int most) {
     const int N = n[0] + n[1] + n[2], slices = product_slices(N, K);
     const int groups = (n[0] + kSmallRows - 1) / kSmallRows + (n[1] + kSmallRows - 1) / kSmallRows + (n[2] + kSmallRows - 1) / kSmallRows;
@@ -801,8 +801,9 @@ float small_estimate(const int32_t* n, int K, int r, int units, int most) {
         const int k = per_sm(groups * units);
         return 2.8f + (mixed ? 1.7f : 0.0f) + (3.7f + 1.2f * slices + 2.1f * rank + 0.74f * step * steps) * (k == 1 ? 0.64f : k == 2 ? 1.15f : 0.5f * k);
     }
-    const int k = per_sm(groups * slices * units);
-    return 2.8f + (mixed ? 0.3f : 0.0f) + (5.4f + (2.2f * rank + step * steps) / slices) * (k / 2 + (k % 2 != 0 ? 0.64f : 0.0f));
+    const int k = per_sm(groups * slices * units), n_span = (K + kSmallSpan - 1) / kSmallSpan;
+    const float three = three_pay(n[2], N, n_span, slices, groups * slices * units, 8 * ((most + 15) / 16), (most + 7) / 8) ? 0.85f : 1.0f;
+    return 2.8f + (mixed ? 0.3f : 0.0f) + three * (5.4f + (2.2f * rank + step * steps) / slices) * (k / 2 + (k % 2 != 0 ? 0.64f : 0.0f));
 }
 
 bool small_takes_units(const SmallParams<kSmallMembers>& P) { return P.one_weight && units_pay(P, product_slices(P.N, P.K)); }
