@@ -450,9 +450,14 @@ __global__ void __launch_bounds__(kSmallThreads, CTAS) small_kernel(const __grid
 // and does all slices of the contraction.  No cluster, and every unit is as many eights of tokens wide as it has.  The halves of the warps take a
 // slot of every slice each; the second half hands its sums to the first one's threads, which hold the same places, add them up in the
 // order of the other two forms - a group's result does not depend on its company, nor on the kernel - and store them.
-// The CTAs go out in the order of their length: rows of 4 bits first, and a weight's largest unit before its others.
+// The CTAs go out in the order of their length, so that the last ones, which leave SMs idle, are short: by precision and width of the unit together
+// (unit_cost; by precision alone 26 % of the SMs' time was idle: six groups of 101 tokens on 4096 x 4096 at 30/50/20 % 51 -> 43.8 us, at 85/15 % 45.9 -> 39.6).
 constexpr int kUnitTokens = 32;
-struct UnitOrder { uint8_t member[2 * kSmallMembers], first[2 * kSmallMembers]; };   // units: member, and its first token in units
+constexpr int kUnitRuns = 3 * 2 * kSmallMembers;
+struct UnitOrder {                               // runs of CTAs: a unit's row groups of one precision
+    int32_t count, end[kUnitRuns];               // end: the first CTA after the run
+    uint8_t member[kUnitRuns], first[kUnitRuns], cls[kUnitRuns];     // the unit's member, and its first token in units
+};
 
 __device__ __forceinline__ void barrier_arrive(int id, int threads) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
 
@@ -592,19 +597,18 @@ __device__ __forceinline__ void unit_rows(const SmallParams<NB>& P, const SmallM
     }
 }
 
-// Grid: (units, row groups).
 template <int NB>
 __global__ void __launch_bounds__(kSmallThreads, 2) units_kernel(const __grid_constant__ SmallParams<NB> P, const __grid_constant__ UnitOrder order, const int slices) {
     extern __shared__ __align__(128) unsigned char small_smem[];
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const SmallMember& W = P.m[order.member[blockIdx.x]];
-    const int m0 = order.first[blockIdx.x] * kUnitTokens;
-    int grp = (int)(gridDim.y - 1 - blockIdx.y), c = 0;
-    for (; c < 2; ++c) {
-        const int n = (W.L.class_start[c + 1] - W.L.class_start[c] + kSmallRows - 1) / kSmallRows;
-        if (grp < n) break;
-        grp -= n;
+    int run = 0, above = order.count - 1;
+    while (run < above) {
+        const int mid = (run + above) >> 1;
+        if ((int)blockIdx.x < order.end[mid]) above = mid;
+        else run = mid + 1;
     }
+    const SmallMember& W = P.m[order.member[run]];
+    const int m0 = order.first[run] * kUnitTokens, c = order.cls[run], grp = (int)blockIdx.x - (run > 0 ? order.end[run - 1] : 0);
     const int p0 = W.L.class_start[c] + grp * kSmallRows + (int)((threadIdx.x >> 5) & 3) * 16, p_end = W.L.class_start[c + 1];
     const int tokens = W.M - m0;
     auto work = [&](auto bits) {
@@ -625,7 +629,7 @@ __global__ void __launch_bounds__(kSmallThreads, 2) units_kernel(const __grid_co
 // than 16 tokens and ranks up to 64 are 1.5 slower.  Over 288 calls that take units (256 to 13824 channels, 512 to 13824 features, 2 to 8 groups, single calls of
 // 33 to 64 tokens, ranks 16 to 128, six mixes) they take 0.90 of the slices' time in the mean; the choice is 0.5 % behind the better form, 10 % at most,
 // and 10 calls are more than 3 % behind the slices (25 without the 1.5: 264 x 512, 44 tokens at 2 and 4 bits 7.9 us, 9.1 by units).
-// (Against the slices, us: 4096 x 4096 at 30/50/20 %, 101 tokens in 6 groups 66.0 -> 48.6, 64 in 8 72 -> 46, 60 in 3 34.4 -> 29.9, 16 in
+// (Against the slices, us: 4096 x 4096 at 30/50/20 %, 101 tokens in 6 groups 66.0 -> 48.6 (43 in order of length), 64 in 8 72 -> 46, 60 in 3 34.4 -> 29.9, 16 in
 // 8 48.5 -> 38.7; at 4 bits 101 in 6 66.4 -> 55.4.  Not taken: 4 in 2 there 19.3 -> 19.8, 64 in one 26.9 -> 31.5; 4096 x 11008 of 4 bits 60 in 3 71 -> 83.)
 bool units_faster(const int* n, int K, int r, int units, int most, int slices) {
     if (units < 2) return false;
@@ -649,19 +653,40 @@ bool units_pay(const SmallParams<NB>& P, int slices) {
     return units_faster(n, P.K, P.r, units, most, slices);
 }
 
+// How long a CTA takes at so many bits (class) and eights of tokens, relative to the others (us on 4096 features, several at a time).
+float unit_cost(int cls, int eights) {
+    constexpr float kCost[3][4] = {{13.7f, 17.0f, 18.8f, 22.4f}, {19.7f, 23.7f, 25.9f, 28.9f}, {27.0f, 30.0f, 33.0f, 36.5f}};
+    return kCost[cls][eights - 1];
+}
+
 template <int NB>
-lowra_status launch_units(const SmallParams<NB>& P, int groups, int slices, cudaStream_t stream) {
-    UnitOrder order;
-    int units = 0, widest = 1;
-    for (int size = kUnitTokens; size > 0; size -= 8)          // 32 to 25 tokens first
-        for (int i = 0; i < P.count; ++i)
-            for (int u = 0; u * kUnitTokens < P.m[i].M; ++u) {
-                const int left = P.m[i].M - u * kUnitTokens, n = left < kUnitTokens ? left : kUnitTokens;
-                if (n > size || n <= size - 8) continue;
-                order.member[units] = (uint8_t)i;
-                order.first[units++] = (uint8_t)u;
-                widest = (n + 7) / 8 > widest ? (n + 7) / 8 : widest;
+lowra_status launch_units(const SmallParams<NB>& P, int slices, cudaStream_t stream) {
+    struct Run { float cost; int groups; uint8_t member, first, cls; } runs[kUnitRuns];
+    int n = 0, widest = 1;
+    for (int i = 0; i < P.count; ++i) {
+        const SmallMember& m = P.m[i];
+        for (int u = 0; u * kUnitTokens < m.M; ++u) {
+            const int left = m.M - u * kUnitTokens, eights = left < kUnitTokens ? (left + 7) / 8 : kUnitTokens / 8;
+            widest = eights > widest ? eights : widest;
+            for (int c = 0; c < 3; ++c) {
+                const Run run = {unit_cost(c, eights), (m.L.class_start[c + 1] - m.L.class_start[c] + kSmallRows - 1) / kSmallRows, (uint8_t)i, (uint8_t)u, (uint8_t)c};
+                if (run.groups == 0) continue;
+                int at = n++;
+                for (; at > 0 && runs[at - 1].cost < run.cost; --at) runs[at] = runs[at - 1];
+                runs[at] = run;
             }
+        }
+    }
+    UnitOrder order;
+    order.count = n;
+    int ctas = 0;
+    for (int i = 0; i < n; ++i) {
+        ctas += runs[i].groups;
+        order.end[i] = ctas;
+        order.member[i] = runs[i].member;
+        order.first[i] = runs[i].first;
+        order.cls[i] = runs[i].cls;
+    }
     const size_t smem = 4u * (8 * widest) * kSmallSpan * 2u + 3u * 4 * widest * 128 * 4u;
     static SmemLimit limit = {};
     if (ensure_smem_limit(reinterpret_cast<const void*>(units_kernel<NB>), smem, &limit) != LOWRA_OK) return LOWRA_ERR_CUDA;
@@ -669,7 +694,7 @@ lowra_status launch_units(const SmallParams<NB>& P, int groups, int slices, cuda
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.gridDim = dim3((unsigned)units, (unsigned)groups, 1);
+    cfg.gridDim = dim3((unsigned)ctas, 1, 1);
     cfg.blockDim = dim3(kSmallThreads, 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
@@ -766,7 +791,7 @@ lowra_status launch_members(const SmallParams<NB>& P, cudaStream_t stream) {
     // a step of 256.  The choice depends on the weight's shape alone, so that a member's result does not depend on its company.
     const int n_span = (P.K + kSmallSpan - 1) / kSmallSpan, slices = product_slices(P.N, P.K);
     const int nt8 = most <= 8 ? 1 : most <= 16 ? 2 : most <= 24 ? 3 : 4;
-    if (P.one_weight && units_pay(P, slices)) return launch_units<NB>(P, groups, slices, stream);
+    if (P.one_weight && units_pay(P, slices)) return launch_units<NB>(P, slices, stream);
     int units = 0;
     for (int i = 0; i < P.count; ++i) units += (P.m[i].M + 8 * nt8 - 1) / (8 * nt8);
     // Merged where a CTA's own cost outweighs its steps: slots of one or two steps, few tokens, more CTAs than run at a time.  (Groups of
