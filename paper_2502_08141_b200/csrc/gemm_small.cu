@@ -59,16 +59,21 @@ __device__ __forceinline__ uint4 ld_shared_v4(uint32_t saddr) {
     return v;
 }
 __device__ __forceinline__ void st_cluster_f32(uint32_t caddr, float v) { asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(caddr), "f"(v) : "memory"); }
+__device__ __forceinline__ void st_cluster_f4(uint32_t caddr, float4 v) {
+    asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(caddr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+}
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
 // ------------------------------------------------------------------------------------------------ T = bf16(s X A)
 constexpr int kProjectBatch = 4;        // steps of 16 contraction indices a warp fetches at a time
 
-// bytes of A a CTA fetches at a time (more than its warps' sums, 512 r, which later take the same place)
+// bytes of A a CTA fetches at a time (more than its warps' sums, 512 (r + 8), which later take the same place)
 __host__ __device__ constexpr size_t project_fetch_bytes(int r) { return (size_t)(kSmallThreads / 32) * kProjectBatch * 16 * (r * 2 + 16); }
 
-// Grid: (slices of the contraction = cluster, tiles of 16 tokens of all members).
+// Grid: (slices of the contraction = cluster, tiles of 16 tokens of all members).  What bounds it: latency, all of which the product waits for.  No division on the
+// way (by powers of two: shifts), sums padded and in wide accesses: 16 tokens on 4096 x 4096 with the product 11.9 -> 11.0 us a call, rank 128 and 30 tokens on
+// 2048 x 2048 13.1 -> 10.9; in units_kernel, which found its slices' bounds by 64-bit divisions, six groups of 101 tokens on 4096 x 4096 43.8 -> 39.8.
 template <int NB>
 __global__ void __launch_bounds__(kSmallThreads) project_kernel(const __grid_constant__ SmallParams<NB> P) {
     extern __shared__ __align__(16) unsigned char project_smem[];
@@ -82,7 +87,8 @@ __global__ void __launch_bounds__(kSmallThreads) project_kernel(const __grid_con
     const Unit un = unit_at(P, (int)blockIdx.y, 16);
     const SmallMember& W = P.m[un.member];
     const int n_steps = P.K / 16;
-    const int s0 = (int)((long long)slice * n_steps / slices), s1 = (int)((long long)(slice + 1) * n_steps / slices);
+    const int slices_log = 31 - __clz(slices);
+    const int s0 = (int)(((long long)slice * n_steps) >> slices_log), s1 = (int)(((long long)(slice + 1) * n_steps) >> slices_log);
     const int pitch = P.r * 2 + 16;                                   // bytes per contraction index of A in shared memory
     unsigned char* mine = project_smem + (size_t)warp * (kProjectBatch * 16 * pitch);
     const int n_j8 = P.r / 8;
@@ -102,10 +108,9 @@ __global__ void __launch_bounds__(kSmallThreads) project_kernel(const __grid_con
             const int st = first + u * kWarps;
             xa[u][0] = xa[u][1] = xa[u][2] = xa[u][3] = 0u;
             if (st < s1) {
-                for (int c = lane; c < 16 * n_j8; c += 32) {
-                    const int k = c / n_j8, j = c - k * n_j8;
+                const int k = lane & 15;
+                for (int j = lane >> 4; j < n_j8; j += 2)
                     cp_async_16_zfill(ptx::smem_u32(mine + (u * 16 + k) * pitch + j * 16), W.A + (size_t)(st * 16 + k) * P.r + j * 8, true);
-                }
                 if (v0) { xa[u][0] = __ldg(x0 + st * 8); xa[u][2] = __ldg(x0 + st * 8 + 4); }
                 if (v1) { xa[u][1] = __ldg(x1 + st * 8); xa[u][3] = __ldg(x1 + st * 8 + 4); }
             }
@@ -130,41 +135,47 @@ __global__ void __launch_bounds__(kSmallThreads) project_kernel(const __grid_con
     }
     // the warps' sums, then the CTA's, then the cluster's, each in a fixed order
     __syncthreads();
-    float* red = reinterpret_cast<float*>(project_smem);              // [warps][16 tokens][r]
+    float* red = reinterpret_cast<float*>(project_smem);              // [warps][16 tokens][r + 8]: half a warp's stores meet different banks
+    const int red_pitch = P.r + 8;
 #pragma unroll
     for (int j = 0; j < 16; ++j) {
         if (j >= n_j8) break;
-        float* d = red + (warp * 16 + g) * P.r + j * 8 + 2 * t;
-        d[0] = acc[j][0]; d[1] = acc[j][1];
-        d[8 * P.r] = acc[j][2]; d[8 * P.r + 1] = acc[j][3];
+        float* d = red + (warp * 16 + g) * red_pitch + j * 8 + 2 * t;
+        *reinterpret_cast<float2*>(d) = make_float2(acc[j][0], acc[j][1]);
+        *reinterpret_cast<float2*>(d + 8 * red_pitch) = make_float2(acc[j][2], acc[j][3]);
     }
     __syncthreads();
-    // every CTA of the cluster owns a share of the sums: its own sums of a share go into the owner's shared memory
-    const int share = 16 * P.r / slices;
+    // every CTA of the cluster owns a share of the sums, 16 / slices tokens: its own sums of a share go into the owner's shared memory
+    const int rows_log = 4 - slices_log, share = P.r << rows_log;
     float* sums = reinterpret_cast<float*>(project_smem + project_fetch_bytes(P.r));   // [slices][share]: behind what this CTA may still be reading
     const uint32_t recv = ptx::smem_u32(sums);
     cluster_wait();
-    for (int i = threadIdx.x; i < 16 * P.r; i += kSmallThreads) {
-        float sum = 0.0f;
+    const int row = (int)threadIdx.x >> 4, col0 = 4 * ((int)threadIdx.x & 15);        // sixteen threads to a token, four ranks each
+    for (int col = col0; col < P.r; col += 64) {
+        float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int w = 0; w < kWarps; ++w) sum += red[w * 16 * P.r + i];
-        const int owner = i / share;
-        st_cluster_f32(ptx::map_to_cta(recv + (uint32_t)(slice * share + i - owner * share) * 4u, (uint32_t)owner), sum);
+        for (int w = 0; w < kWarps; ++w) {
+            const float4 v = *reinterpret_cast<const float4*>(red + (w * 16 + row) * red_pitch + col);
+            sum.x += v.x; sum.y += v.y; sum.z += v.z; sum.w += v.w;
+        }
+        const uint32_t at = recv + (uint32_t)(slice * share + (row & ((1 << rows_log) - 1)) * P.r + col) * 4u;
+        st_cluster_f4(ptx::map_to_cta(at, (uint32_t)(row >> rows_log)), sum);
     }
     ptx::cluster_sync();
-    for (int i = 2 * (int)threadIdx.x; i < share; i += 2 * kSmallThreads) {   // pairs of neighbouring ranks
-        const int e = slice * share + i, row = e / P.r, col = e - row * P.r;
-        if (un.m0 + row >= W.M) continue;
-        float a = 0.0f, b = 0.0f;
-        for (int c = 0; c < slices; ++c) { a += sums[c * share + i]; b += sums[c * share + i + 1]; }
-        *reinterpret_cast<uint32_t*>(W.T + (size_t)(un.m0 + row) * P.rp + col) = pack_bf16x2(P.s * a, P.s * b);
+    const int mine_row = un.m0 + (slice << rows_log) + row;
+    if (row < (1 << rows_log) && mine_row < W.M) {
+        for (int col = col0; col < P.r; col += 64) {
+            float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int c = 0; c < slices; ++c) {
+                const float4 b = *reinterpret_cast<const float4*>(sums + c * share + row * P.r + col);
+                a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w;
+            }
+            *reinterpret_cast<uint2*>(W.T + (size_t)mine_row * P.rp + col) = make_uint2(pack_bf16x2(P.s * a.x, P.s * a.y), pack_bf16x2(P.s * a.z, P.s * a.w));
+        }
     }
     // columns between the rank and its padded width are zero
-    const int pad = P.rp - P.r;
-    for (int i = slice * kSmallThreads + (int)threadIdx.x; i < 16 * pad; i += slices * kSmallThreads) {
-        const int row = i / pad;
-        if (un.m0 + row < W.M) W.T[(size_t)(un.m0 + row) * P.rp + P.r + (i - row * pad)] = 0;
-    }
+    if (slice == 0 && un.m0 + row < W.M)
+        for (int col = P.r + col0; col < P.rp; col += 64) *reinterpret_cast<uint2*>(W.T + (size_t)(un.m0 + row) * P.rp + col) = make_uint2(0u, 0u);
 }
 
 // ------------------------------------------------------------------------------------------------ the product
@@ -243,7 +254,8 @@ __device__ __forceinline__ void multiply_rows(int K, const SmallMember& W, int m
     constexpr int c = B >> 1;
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const int n_span = (K + kSmallSpan - 1) / kSmallSpan, nb = K / kBlock;
-    auto bound = [&](int slot) { return (int)((long long)slot * n_span / slots); };
+    const int slots_log = 31 - __clz(slots);          // (a power of two; n_span is below 2^27: K is an int32)
+    auto bound = [&](int slot) { return (int)(((long long)slot * n_span) >> slots_log); };
     const int b0 = bound(slot0), b1 = bound(slot1);
     // rows g and g + 8 of the warp's sixteen
     const bool live0 = p0 + g < p_end, live1 = p0 + g + 8 < p_end;
@@ -332,7 +344,7 @@ __global__ void __launch_bounds__(kSmallThreads, CTAS) small_kernel(const __grid
     float* sums = reinterpret_cast<float*>(small_smem + 2 * kTokenBytes);   // spread: [slots][tokens][share of the rows]; MERGED: see end()
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const int rank = MERGED ? 0 : (int)ptx::cluster_ctarank();
-    int grp = MERGED ? (int)blockIdx.x : ((int)gridDim.x - 1 - (int)blockIdx.x) / slices;     // (spread: the long rows of 4 bits first)
+    int grp = MERGED ? (int)blockIdx.x : ((int)gridDim.x - 1 - (int)blockIdx.x) >> (31 - __clz(slices));     // (spread: the long rows of 4 bits first)
     const Unit un = unit_at(P, (int)blockIdx.y, kTokens);
     const SmallMember& W = P.m[un.member];
     // the group's rows: 64 neighbouring stored rows of one precision class
@@ -466,7 +478,8 @@ __device__ __forceinline__ void unit_rows(const SmallParams<NB>& P, const SmallM
     constexpr uint32_t kStep = 8u * NT8 * kSmallSpan * 2u;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, half = warp >> 2;
     const int K = P.K, n_span = (K + kSmallSpan - 1) / kSmallSpan, nb = K / kBlock, slots = 2 * slices;
-    auto bound = [&](int slot) { return (int)((long long)slot * n_span / slots); };
+    const int slots_log = 31 - __clz(slots);          // (a power of two; n_span is below 2^27: K is an int32)
+    auto bound = [&](int slot) { return (int)(((long long)slot * n_span) >> slots_log); };
     const bool live0 = p0 + g < p_end, live1 = p0 + g + 8 < p_end;
     const int q0 = live0 ? p0 + g : p_end - 1, q1 = live1 ? p0 + g + 8 : p_end - 1;
     const int r0 = __ldg(W.L.perm + q0), r1 = __ldg(W.L.perm + q1);
@@ -737,11 +750,11 @@ int product_slices(int N, int K) {
 // 60/35/5 %, 1 token: 11008 x 4096 19.6 -> 16.4 (24.7), 13824 x 5120 22.5 -> 19.6 (28.1), 6144 x 4096 16.4 -> 11.7 (18.2), 5120 x 13824 30.2 -> 24.6 (36.5), 2048 x 4096
 // 12.8 -> 10.0 (14.0), 4096 x 4096 10.25 -> 9.6; 16 tokens: 11008 x 4096 24.9 -> 19.7 (30.5), 4096 x 4096 13.0 -> 11.9.  Two where they fit and steps are long
 // (4096 x 11008, 16 tokens 18.9, three 20.1; 24 tokens 20.6, 28.3) and with most rows at 4 bits (13824 x 5120, 16 tokens 30.9, three 33.9; 4096 x 4096, 1 token 10.5, 11.5),
-// unless short steps take two waves (6144 x 4096 of 4 bits, 1 token 19.0, three 14.7).
+// unless short steps take two waves (6144 x 4096 of 4 bits, 1 token 19.0, three 14.7); and where an SM has one CTA at most (4096 x 768, 16 tokens 7.6, 8.6).
 bool three_pay(int four, int N, int n_span, int slices, int ctas, int projection, int nt8) {
     if (nt8 > 3) return false;                           // (no shared memory for a third)
     const bool fit = ctas + projection <= (slices == 8 ? 272 : slices == 4 ? 280 : 2 * kNumSMs), short_steps = n_span <= 2 * (2 * slices);
-    return fit ? short_steps && nt8 <= 2 && four <= N / 8 : short_steps || four <= N / 2;
+    return fit ? (slices > 1 || ctas > kNumSMs) && short_steps && nt8 <= 2 && four <= N / 8 : short_steps || four <= N / 2;
 }
 
 // groups of 64 stored rows of one precision (of the member that has the most)
