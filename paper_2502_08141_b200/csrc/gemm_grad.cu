@@ -14,6 +14,9 @@
 //     K-major  (the contraction index is contiguous: X for T, dY and B for U)   one box of [rows][64 c]
 //     MN-major (the row / column index is contiguous: A for T; X, dY, U, T for the gradients)   boxes of [64 c][64 rows]
 // warp 0 = TMA, warp 1 = MMA issue, warps 2-5 = epilogue and reduction.  All waits are bounded.
+// What bounds it: reading P at 4096 tokens (11008 x 4096 with the projections at hand 24 us, one reading of X and dY 18.6); the chain set-up, first tiles,
+// cluster barrier, reduction for short ones.  With the two issuing warps in step and no division on the way, us, with the projections at hand / in full:
+// 4096 x 4096 at 2048 tokens 10.4 -> 9.5 / 20.5 -> 18.8, 1800 x 2304 at 777 7.9 -> 6.6 / 15.2 -> 13.8, 13824 x 5120 at 1000 12.5 -> 9.2 / 26.9 -> 21.7.
 #include "gemm_params.cuh"
 #include "ptx.cuh"
 
@@ -51,7 +54,7 @@ __device__ __forceinline__ void add_slices(const SkinnyProduct& P, const float* 
     uint32_t from[S];
 #pragma unroll
     for (int p = 0; p < S; ++p) from[p] = ptx::map_to_cta(ptx::smem_u32(part), (uint32_t)p);
-    const int c4n = rp / 4;                                          // 16 or 32
+    const int c4_log = rp > 64 ? 5 : 4;                              // rp / 4: 16 or 32
 #pragma unroll 1
     for (int half = 0; half < (rp / 64) * (16 / kLoads); ++half) {
         float4 v[kPlaces][S];
@@ -61,8 +64,8 @@ __device__ __forceinline__ void add_slices(const SkinnyProduct& P, const float* 
             if (!P.transposed) {
                 // out [R, ld_out]: four neighbouring columns per thread
                 const int u = t + 128 * (half * kPlaces + k);
-                row[k] = row_base + u / c4n;
-                col[k] = (u % c4n) * 4;
+                row[k] = row_base + (u >> c4_log);
+                col[k] = (u & ((1 << c4_log) - 1)) * 4;
             } else {
                 // out [n_cols, ld_out] = D^T.  A warp takes 8 rows x 16 columns of D: its loads read whole 64-byte runs of
                 // a row, its stores write 8 neighbouring elements (rows of D) of 16 rows of out.
@@ -109,7 +112,8 @@ skinny_kernel(const __grid_constant__ SkinnyPair A, const int S) {
     const int r0 = ((int)blockIdx.x - (second ? A.tiles0 : 0)) * 128;
     const uint32_t crank = ptx::cluster_ctarank();            // which slice of the contraction
     const int n_blocks = (P.C + 63) / 64;
-    const int kb0 = (int)((long long)crank * n_blocks / S), kb1 = (int)((long long)(crank + 1) * n_blocks / S);
+    const int s_log = 31 - __clz(S);                          // (a power of two: no division before the first load)
+    const int kb0 = (int)(((long long)crank * n_blocks) >> s_log), kb1 = (int)(((long long)(crank + 1) * n_blocks) >> s_log);
     const int n_my = kb1 - kb0;
     const uint32_t stage_bytes = kSkinnySmemP + (uint32_t)rp * 128u;   // 24 or 32 KB
     const int stages = (int)(kSkinnyRing / stage_bytes);                  // 4 or 3
@@ -140,13 +144,15 @@ skinny_kernel(const __grid_constant__ SkinnyPair A, const int S) {
     if (failed) {
         // shared memory not aligned as the swizzled tiles need: nothing is loaded or multiplied
     } else if (warp == 0) {
-        if (lane == 0) {
-            int issued = 0;
-            for (int i = 0; i < n_my; ++i) {
-                const int s = i % stages, kb = kb0 + i;
-                if (!ptx::mbar_wait(&bars->empty[s], ((i / stages) & 1u) ^ 1u, abort_flag, A.wait_ns)) { failed = true; bars->abort = 1u; break; }
-                unsigned char* p_s = base + s * stage_bytes;
-                unsigned char* q_s = p_s + kSkinnySmemP;
+        // The whole warp walks through the loop, one lane issues (as in the fused kernel: a loop of a single lane takes twice the time).
+        const bool leader = ptx::elect_one();
+        int s = 0, issued = 0;
+        uint32_t ph = 0;
+        for (int kb = kb0; kb < kb1; ++kb) {
+            if (!ptx::mbar_wait_lanes(&bars->empty[s], ph ^ 1u, abort_flag, A.wait_ns)) { failed = true; bars->abort = 1u; break; }
+            unsigned char* p_s = base + s * stage_bytes;
+            unsigned char* q_s = p_s + kSkinnySmemP;
+            if (leader) {
                 ptx::mbar_arrive_expect_tx(&bars->full[s], stage_bytes);
                 // rows, columns and contraction indices past the end of a matrix read as zero
                 if (P.a_mn) {
@@ -156,35 +162,42 @@ skinny_kernel(const __grid_constant__ SkinnyPair A, const int S) {
                     ptx::tma_load_2d(p_s, &P.tmP, kb * 64, r0, &bars->full[s]);
                 }
                 if (P.b_mn) {
-                    for (int h = 0; h < rp / 64; ++h) ptx::tma_load_2d(q_s + h * 8192, &P.tmQ, h * 64, kb * 64, &bars->full[s]);
+                    ptx::tma_load_2d(q_s, &P.tmQ, 0, kb * 64, &bars->full[s]);
+                    if (rp > 64) ptx::tma_load_2d(q_s + 8192, &P.tmQ, 64, kb * 64, &bars->full[s]);
                 } else {
                     ptx::tma_load_2d(q_s, &P.tmQ, kb * 64, 0, &bars->full[s]);
                 }
-                issued = i + 1;
             }
-            if (failed) {   // let the copies in flight land before the shared memory is given back
-                for (int back = 1; back <= stages && back <= issued; ++back)
-                    ptx::mbar_wait(&bars->full[(issued - back) % stages], ((issued - back) / stages) & 1u, nullptr, 2000000ull);
-            }
+            __syncwarp();
+            ++issued;
+            if (++s == stages) { s = 0; ph ^= 1u; }
+        }
+        if (failed && lane == 0) {   // let the copies in flight land before the shared memory is given back
+            for (int back = 1; back <= stages && back <= issued; ++back)
+                ptx::mbar_wait(&bars->full[(issued - back) % stages], ((issued - back) / stages) & 1u, nullptr, 2000000ull);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            const uint32_t idesc = ptx::umma_idesc_bf16(128, rp) | (P.a_mn ? (1u << 15) : 0u) | (P.b_mn ? (1u << 16) : 0u);
-            const uint32_t a_step = P.a_mn ? 128u : 2u, b_step = P.b_mn ? 128u : 2u;   // 16 contraction indices further
-            for (int i = 0; i < n_my; ++i) {
-                const int s = i % stages;
-                if (!ptx::mbar_wait(&bars->full[s], (i / stages) & 1u, abort_flag, A.wait_ns)) { failed = true; bars->abort = 1u; break; }
-                ptx::tc_fence_after();
-                const uint32_t p_addr = ptx::smem_u32(base + s * stage_bytes);
-                const uint32_t q_addr = p_addr + kSkinnySmemP;
-                const uint64_t adesc = P.a_mn ? ptx::umma_desc_mn_sw128(p_addr, 8192u) : ptx::umma_desc_k_sw128(p_addr);
-                const uint64_t bdesc = P.b_mn ? ptx::umma_desc_mn_sw128(q_addr, 8192u) : ptx::umma_desc_k_sw128(q_addr);
+        const bool leader = ptx::elect_one();
+        const uint32_t idesc = ptx::umma_idesc_bf16(128, rp) | (P.a_mn ? (1u << 15) : 0u) | (P.b_mn ? (1u << 16) : 0u);
+        const uint32_t a_step = P.a_mn ? 128u : 2u, b_step = P.b_mn ? 128u : 2u;   // 16 contraction indices further
+        int s = 0;
+        uint32_t ph = 0;
+        for (int i = 0; i < n_my; ++i) {
+            if (!ptx::mbar_wait_lanes(&bars->full[s], ph, abort_flag, A.wait_ns)) { failed = true; bars->abort = 1u; break; }
+            ptx::tc_fence_after();
+            const uint32_t p_addr = ptx::smem_u32(base + s * stage_bytes);
+            const uint32_t q_addr = p_addr + kSkinnySmemP;
+            const uint64_t adesc = P.a_mn ? ptx::umma_desc_mn_sw128(p_addr, 8192u) : ptx::umma_desc_k_sw128(p_addr);
+            const uint64_t bdesc = P.b_mn ? ptx::umma_desc_mn_sw128(q_addr, 8192u) : ptx::umma_desc_k_sw128(q_addr);
+            if (leader) {
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk)
                     ptx::umma_bf16(tmem_base, adesc + a_step * kk, bdesc + b_step * kk, idesc, (i | kk) != 0 ? 1u : 0u);
                 ptx::umma_commit(&bars->empty[s]);
+                if (i + 1 == n_my) ptx::umma_commit(&bars->tmem_full);
             }
-            if (!failed && n_my > 0) ptx::umma_commit(&bars->tmem_full);
+            __syncwarp();
+            if (++s == stages) { s = 0; ph ^= 1u; }
         }
     } else {
         // ------------------------------------------------------------------ TMEM -> fp32 partial tile in shared memory
