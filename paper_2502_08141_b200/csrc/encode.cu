@@ -7,9 +7,9 @@
 // 32-element segments are 144 bytes apart, so neither the writes nor the reads collide on a bank).  The block
 // maximum is one shuffle away; codes are accumulated as bit planes of sign bits:
 //   "thresholds <= n" is counted through the sign of n - t (exact: a difference of two floats has the sign of
-//   the exact difference, and equal values give +0, so a value on a threshold takes the upper bucket; n is
-//   first passed through n + 0.0 so that a negative zero cannot come out below a threshold of +0),
-//   1 bit : one subtract and one funnel shift per element,
+//   the exact difference, and equal values give +0, so a value on a threshold takes the upper bucket; what is added is -t, a
+//   zero as +0, so that a negative zero cannot come out below a threshold of +0),
+//   1 bit : one multiplication, half a packed addition and one funnel shift per element,
 //   2 bits: three sign planes (one per threshold; sorted thresholds) combined into the two code planes with
 //           two logic ops per 32 elements, then interleaved,
 //   4 bits: branch-free binary search over the row's 15 thresholds, which lie in the warp's slice of shared memory
@@ -40,11 +40,9 @@ struct EncodeParams {
     uint32_t n_tasks;
 };
 
-// sign bit of (n - t) pushed into `plane` from the right: after 32 pushes (elements 31 .. 0) bit i of the
+// sign bit of d = n - t pushed into `plane` from the right: after 32 pushes (elements 31 .. 0) bit i of the
 // plane says "element i is below t"
-__device__ __forceinline__ uint32_t push_below(uint32_t plane, float n, float t) {
-    return __funnelshift_l(__float_as_uint(__fsub_rn(n, t)), plane, 1);
-}
+__device__ __forceinline__ uint32_t push_sign(uint32_t plane, float d) { return __funnelshift_l(__float_as_uint(d), plane, 1); }
 
 // bits of x (16 of them) spread to the even positions
 __device__ __forceinline__ uint32_t spread16(uint32_t x) {
@@ -106,19 +104,28 @@ __device__ __forceinline__ void encode_chunk(const EncodeParams& P, int p, int c
     const float inv = (m == 0.0f) ? 0.0f : __frcp_rn(m);
 
     uint8_t* dst = P.packed + packed_row_offset(P.L, c, p, r) + (size_t)(e0 + lane * 32) * B / 8;
+    // Two elements at a time; m0, m1, m2: the thresholds negated, a zero to +0 (so that n + m is +0 for n = -0, too).  Two single multiplications: a packed one
+    // and the packed addition behind it become one fused operation in the assembler (nvcc 12.9), which skips the rounding of n.
+    auto normalised = [&](float a, float b) { return make_float2(__fmul_rn(a, inv), __fmul_rn(b, inv)); };
     if (B == 1) {
+        const float m0 = 0.0f - t0;
         uint32_t below = 0u;
 #pragma unroll
-        for (int i = 31; i >= 0; --i) below = push_below(below, __fadd_rn(__fmul_rn(x[i], inv), 0.0f), t0);
+        for (int i = 30; i >= 0; i -= 2) {
+            const float2 d = add2(normalised(x[i], x[i + 1]), make_float2(m0, m0));
+            below = push_sign(push_sign(below, d.y), d.x);
+        }
         if (live) *reinterpret_cast<uint32_t*>(dst) = ~below;
     } else if (B == 2) {
+        const float m0 = 0.0f - t0, m1 = 0.0f - t1, m2 = 0.0f - t2;
         uint32_t s0 = 0u, s1 = 0u, s2 = 0u;   // element i is below threshold 0 / 1 / 2
 #pragma unroll
-        for (int i = 31; i >= 0; --i) {
-            const float n = __fadd_rn(__fmul_rn(x[i], inv), 0.0f);
-            s0 = push_below(s0, n, t0);
-            s1 = push_below(s1, n, t1);
-            s2 = push_below(s2, n, t2);
+        for (int i = 30; i >= 0; i -= 2) {
+            const float2 n = normalised(x[i], x[i + 1]);
+            const float2 d0 = add2(n, make_float2(m0, m0)), d1 = add2(n, make_float2(m1, m1)), d2 = add2(n, make_float2(m2, m2));
+            s0 = push_sign(push_sign(s0, d0.y), d0.x);
+            s1 = push_sign(push_sign(s1, d1.y), d1.x);
+            s2 = push_sign(push_sign(s2, d2.y), d2.x);
         }
         // sorted thresholds: code = number of thresholds <= n; high bit = not below t1, low bit = not below t2
         // (upper half) or not below t0 (lower half)
@@ -137,9 +144,10 @@ __device__ __forceinline__ void encode_chunk(const EncodeParams& P, int p, int c
         for (int q = 0; q < 8; ++q) {
             uint32_t sum = 0u;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const float n = __fmul_rn(x[4 * q + i], inv);
-                sum += threshold_place(t_at, t7, n) << (4 * i);
+            for (int i = 0; i < 4; i += 2) {
+                const float2 n = mul2(make_float2(x[4 * q + i], x[4 * q + i + 1]), make_float2(inv, inv));
+                sum += threshold_place(t_at, t7, n.x) << (4 * i);
+                sum += threshold_place(t_at, t7, n.y) << (4 * i + 4);
             }
             const uint32_t codes = (sum - t_at * 0x1111u) >> 2;
             w[q >> 1] = (q & 1) ? w[q >> 1] | (codes << 16) : codes;
