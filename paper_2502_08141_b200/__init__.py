@@ -461,8 +461,8 @@ def lowra_learn_codebooks(layout: Layout, W: torch.Tensor, init_levels, init_thr
         maps = torch.empty((layout.N, 16), dtype=torch.float32, device=W.device)
     if thresholds is None:
         thresholds = torch.empty((layout.N, 16), dtype=torch.float32, device=W.device)
-    code = lib().lowra_learn_codebooks(layout.ref, _ptr(W), y0.ctypes.data_as(ctypes.c_void_p),
-                                       t0.ctypes.data_as(ctypes.c_void_p), int(iterations), _ptr(maps),
+    code = lib().lowra_learn_codebooks(layout.ref, _ptr(W), y0.ctypes.data,
+                                       t0.ctypes.data, int(iterations), _ptr(maps),
                                        _ptr(thresholds), _stream(stream))
     _check(code, "lowra_learn_codebooks")
     return maps, thresholds
@@ -489,8 +489,8 @@ def lowra_learn_codebooks_all(W: torch.Tensor, init_levels, init_thresholds, ite
         thresholds3 = torch.empty((3, N, 16), dtype=torch.float32, device=W.device)
     if tuple(maps3.shape) != (3, N, 16) or tuple(thresholds3.shape) != (3, N, 16):
         raise ValueError("maps3 and thresholds3 must be [3, N, 16]")
-    code = lib().lowra_learn_codebooks_all(N, K, _ptr(W), y0.ctypes.data_as(ctypes.c_void_p),
-                                           t0.ctypes.data_as(ctypes.c_void_p), int(iterations), _ptr(maps3),
+    code = lib().lowra_learn_codebooks_all(N, K, _ptr(W), y0.ctypes.data,
+                                           t0.ctypes.data, int(iterations), _ptr(maps3),
                                            _ptr(thresholds3), _stream(stream))
     _check(code, "lowra_learn_codebooks_all")
     return maps3, thresholds3

@@ -1202,15 +1202,19 @@ bool two_long_rows(int K) { return 2 * (sorted_smem_bytes(K) + 1024) <= 228 * 10
 //   K=16384   83/97   119/114 225/162          120/105 197/130 432/209          169/281 263/322 549/443           199/279 328/321 704/445
 // At 1 bit the ordered blocks pay in the fourth round where every lane has a block, later where some have none (K = 3072, 5120), or where an SM
 // holds few warps (K = 8320 to 12288); K up to 2048 is one warp, up to 1024 of short networks.
+// A few rows to an SM (`few`: four at most) wait for the longest chain, and a warp's network is longer than the eight warps' way to the order of a whole row
+// (256 rows, T = 2, us, ordered against sorted, 4 bits and all three: K = 2048 10.8 7.8, 12.0 8.5; K = 3584 9.6 8.6, 10.8 9.1) or, of 2048 values at 2 bits, than rounds
+// through the row (6.4 4.7).
 enum Kernel { kRowAgain, kOrdered, kSorted };
 int ordered_warps(int K) { return (K + 2047) / 2048; }
-Kernel kernel_for(int K, int c, int iterations) {
+Kernel kernel_for(int K, int c, int iterations, bool few) {
     if (K > kSortedMaxK || iterations < 1) return kRowAgain;
     if (c == 0) {
         const bool pays = K <= 1024 || (K <= 2048 ? iterations >= 3 : (iterations - (K > 8192 && K <= 12288 ? 2 : 0)) * K >= 4 * 2048 * ordered_warps(K));
         return pays ? kOrdered : kRowAgain;
     }
-    if (c == 1) return K <= 1024 || iterations >= 2 ? kOrdered : kRowAgain;
+    if (c == 1) return K <= 1024 || iterations >= (few && K <= 2048 ? 4 : K > 8192 && K <= 12288 ? 3 : 2) ? kOrdered : kRowAgain;
+    if (few && K > 1024 && K <= 6144 && iterations >= 2) return kSorted;
     constexpr int kUpTo[] = {512, 1024, 2048, 3072, 4096, 6144, 8192, 11776}, kFour[] = {2, 3, 4, 3, 5, 3, 7, 4, 9}, kAll[] = {2, 4, 4, 2, 4, 2, 4, 3, 5};
     int i = 0;
     while (i < 8 && K > kUpTo[i]) ++i;
@@ -1258,7 +1262,9 @@ lowra_status launch_learn(LearnParams& P, const double* init_levels_host, const 
         }
     // stored rows are in the order of their precisions: the last `sorted` of them go to the sorted kernel
     Kernel kernel[3];
-    for (int c = 0; c < 3; ++c) kernel[c] = kernel_for(P.K, ALL3 ? 3 : c, P.iterations);
+    for (int c = 0; c < 3; ++c) kernel[c] = kernel_for(P.K, ALL3 ? 3 : c, P.iterations, P.N <= 4 * kNumSMs);
+    // (one launch fewer counts for more than the rows' kernel where these are few: 535 x 2048 at 60/35/5, T = 2 10.2 -> 7.8 us)
+    if (!ALL3 && P.N <= 8 * kNumSMs && kernel[0] == kRowAgain && kernel[1] == kOrdered && n1 > 0 && n2 > 0) kernel[0] = kOrdered;
     // Stored rows are in the order of their precisions, and more bits want more order: a launch for every kernel that has classes, the last classes' first
     // (in turns; see enter()).
     const int n[3] = {n1, n2, n4};
