@@ -1210,11 +1210,11 @@ int ordered_warps(int K) { return (K + 2047) / 2048; }
 Kernel kernel_for(int K, int c, int iterations, bool few) {
     if (K > kSortedMaxK || iterations < 1) return kRowAgain;
     if (c == 0) {
-        const bool pays = K <= 1024 || (K <= 2048 ? iterations >= 3 : (iterations - (K > 8192 && K <= 12288 ? 2 : 0)) * K >= 4 * 2048 * ordered_warps(K));
+        const bool pays = K <= 1024 || (K <= 2048 ? iterations >= (few ? 4 : 3) : (iterations - (K > 8192 && K <= 12288 ? 2 : 0)) * K >= 4 * 2048 * ordered_warps(K));
         return pays ? kOrdered : kRowAgain;
     }
     if (c == 1) return K <= 1024 || iterations >= (few && K <= 2048 ? 4 : K > 8192 && K <= 12288 ? 3 : 2) ? kOrdered : kRowAgain;
-    if (few && K > 1024 && K <= 6144 && iterations >= 2) return kSorted;
+    if (few && iterations >= 2 && ((K > 1024 && K <= 6144) || (c == 3 && K > 8192 && K <= 11776))) return kSorted;      // (five warps: two on one scheduler)
     constexpr int kUpTo[] = {512, 1024, 2048, 3072, 4096, 6144, 8192, 11776}, kFour[] = {2, 3, 4, 3, 5, 3, 7, 4, 9}, kAll[] = {2, 4, 4, 2, 4, 2, 4, 3, 5};
     int i = 0;
     while (i < 8 && K > kUpTo[i]) ++i;
