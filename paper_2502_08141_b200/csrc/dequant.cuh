@@ -24,18 +24,19 @@ __device__ __forceinline__ uint32_t pick_bytes(uint32_t a, uint32_t b, uint32_t 
 
 template <int B> struct Scaled;
 template <> struct Scaled<1> {
-    uint32_t base, d, f;     // both halves: the smaller pattern; the difference of the patterns; 0x10001 if level 0 is the larger one
+    // Both halves: the pattern L of level 0; H - L modulo 2^32, which may be negative: L + b (H - L), for a bit b, is one of the two patterns, so nothing is
+    // carried from the low half to the high one, whichever is the larger.
+    uint32_t base, d;
     __device__ __forceinline__ void set(const float* y, float a) {
-        const uint32_t LH = pack_bf16x2(__fmul_rn(y[0], a), __fmul_rn(y[1], a));
-        const uint32_t L = LH & 0xFFFFu, H = LH >> 16, lo = min(L, H);
-        base = lo * 0x10001u; d = max(L, H) - lo; f = (L > H) ? 0x10001u : 0u;
+        const uint32_t LH = pack_bf16x2(__fmul_rn(y[0], a), __fmul_rn(y[1], a)), L = LH & 0xFFFFu;
+        base = L * 0x10001u; d = (LH >> 16) - L;
     }
     // elements 16 q .. 16 q + 15 of the block whose codes are w[0 .. 1]
     __device__ __forceinline__ void expand16(const uint32_t* w, int q, uint32_t (&o)[8]) const {
         const uint32_t h = (q & 1) ? (w[q >> 1] >> 16) : (w[q >> 1] & 0xFFFFu);
         const uint32_t z = h | (h << 15);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) o[i] = (((z >> (2 * i)) & 0x10001u) ^ f) * d + base;
+        for (int i = 0; i < 8; ++i) o[i] = ((z >> (2 * i)) & 0x10001u) * d + base;
     }
 };
 template <> struct Scaled<2> {
