@@ -733,7 +733,7 @@ lowra_status launch_product(const SmallParams<NB>& P, int groups, int units, int
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cfg.attrs = attr;
-    cfg.numAttrs = MERGED ? 1 : 2;
+    cfg.numAttrs = MERGED || slices == 1 ? 1 : 2;           // (a CTA is a cluster of its own without being told, and 0.4 us less host time)
     return cudaLaunchKernelEx(&cfg, small_kernel<NT8, NB, MERGED, CTAS>, P, slices) == cudaSuccess ? LOWRA_OK : LOWRA_ERR_CUDA;
 }
 
