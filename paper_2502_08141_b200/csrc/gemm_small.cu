@@ -3,7 +3,7 @@
 // With a handful of tokens the work is reading the weight's codes once (1 - 2 bits per weight), a few microseconds of memory
 // time: what counts is how many SMs share it and how long the longest chain of dependent steps is.  The persistent
 // tensor-core kernel (gemm_fused.cu) has tiles of 256 channels and 256 tokens, of which a 4096 x 4096 weight is 16: cut in four, their
-// slices handed over, it takes 26 us for 1 token as for 65.  Here two launches share the work finely instead (1 token 9.6, 16 tokens 11.9):
+// slices handed over, it takes 26 us for 1 token as for 65.  Here two launches share the work finely instead (1 token 9.1, 16 tokens 11.0):
 //   project_kernel   T = bf16(s X A): a CTA per 16 tokens and slice of the contraction, the slices of a cluster added up
 //                    through distributed shared memory.
 //   small_kernel     a CTA takes 64 stored rows of one precision and a slice of the contraction, its warps 16 rows and half
@@ -14,7 +14,8 @@
 //                    simply its own next four elements, for the weights and for the tokens alike.  The tokens of the slice
 //                    lie in shared memory.  Slices are added up as above; the low-rank term enters as further steps of
 //                    the same accumulation.
-// It starts while project_kernel runs and waits for it only before the low-rank term (programmatic dependent launch).
+// It starts while project_kernel runs and waits for it only before the low-rank term (programmatic dependent launch).  For a small weight with a low rank
+// every CTA of small_kernel forms T itself, and there is no other launch.
 // No flags, no waits that need a limit, any number of such calls may share the GPU.
 #include <type_traits>
 
@@ -70,6 +71,13 @@ constexpr int kProjectBatch = 4;        // steps of 16 contraction indices a war
 
 // bytes of A a CTA fetches at a time (more than its warps' sums, 512 (r + 8), which later take the same place)
 __host__ __device__ constexpr size_t project_fetch_bytes(int r) { return (size_t)(kSmallThreads / 32) * kProjectBatch * 16 * (r * 2 + 16); }
+
+// slices of the projection's contraction: up to eight, 128 indices or more each
+__host__ __device__ constexpr int project_slices(int K) {
+    int slices = 1;
+    while (slices < 8 && K >= 256 * slices) slices *= 2;
+    return slices;
+}
 
 // Grid: (slices of the contraction = cluster, tiles of 16 tokens of all members).  What bounds it: latency, all of which the product waits for.  No division on the
 // way (by powers of two: shifts), sums padded and in wide accesses: 16 tokens on 4096 x 4096 with the product 11.9 -> 11.0 us a call, rank 128 and 30 tokens on
@@ -328,21 +336,100 @@ __device__ __forceinline__ void multiply_rows(int K, const SmallMember& W, int m
     }
 }
 
+// T of up to 16 tokens by one CTA of the product, for itself: a weight so small that the projection's launch costs more.  A lies in shared memory as in memory,
+// behind it are the warps' sums [slices][warps][16 tokens][r + 8] and T [16][r + 8]; the tokens are those staged for the product (one step per slot).  The same sums in
+// the same order as project_kernel's.  Ends with a barrier.
+constexpr int kOwnK = 512, kOwnRank = 32, kOwnSlices = 4;
+static_assert(project_slices(kOwnK) == kOwnSlices && project_slices(kOwnK - 1) < kOwnSlices, "slices");
+struct OwnT {
+    unsigned char* a;
+    float* sums;
+    uint16_t* T;
+    static __host__ __device__ constexpr size_t bytes(int K, int r) { return (size_t)K * r * 2 + (size_t)project_slices(K) * 8 * 16 * (r + 8) * 4 + 16 * (r + 8) * 2; }
+    __device__ OwnT(unsigned char* smem, int K, int r) : a(smem), sums(reinterpret_cast<float*>(smem + K * r * 2)), T(reinterpret_cast<uint16_t*>(sums + (K < 256 ? 1 : K < 512 ? 2 : 4) * 8 * 16 * (r + 8))) {}
+    __device__ __forceinline__ void fetch(const uint16_t* A, int K, int r) const {
+        for (int i = threadIdx.x; i < K * r / 8; i += kSmallThreads) cp_async_16_zfill(ptx::smem_u32(a) + 16u * i, A + 8 * i, true);
+        ptx::cp_async_commit();
+    }
+    // x_of(step of 256): where its tokens are staged
+    template <int NT8, typename X>
+    __device__ __forceinline__ void form(int K, int r, float s, X x_of) const {
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+        const int log = K < 256 ? 0 : K < 512 ? 1 : 2, n_steps = K / 16;
+        ptx::cp_async_wait<0>();
+        __syncthreads();
+#pragma unroll 1
+        for (int c = 0; c < 1 << log; ++c) {
+            float acc[kOwnRank / 8][4];
+#pragma unroll
+            for (int j = 0; j < kOwnRank / 8; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.0f;
+#pragma unroll 1
+            for (int st = ((c * n_steps) >> log) + warp; st < ((c + 1) * n_steps) >> log; st += 8) {
+                const int k = st * 16 % kSmallSpan;
+                uint32_t x[4] = {0u, 0u, 0u, 0u};
+                const uint32_t at = x_of(st / 16) + token_piece(lane & (NT8 == 1 ? 7 : 15), k / 64, k % 64 / 8 + (NT8 == 1 ? lane >> 3 & 1 : lane >> 4));
+                if (NT8 == 1) asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];" : "=r"(x[0]), "=r"(x[2]) : "r"(at) : "memory");
+                else asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(x[0]), "=r"(x[1]), "=r"(x[2]), "=r"(x[3]) : "r"(at) : "memory");
+                const uint32_t a_row = ptx::smem_u32(a) + (uint32_t)((st * 16 + (lane & 15)) * r * 2 + (lane >> 4) * 16);
+#pragma unroll
+                for (int j = 0; j < kOwnRank / 8; j += 2) {
+                    if (8 * j >= r) break;
+                    uint32_t b0, b1, b2, b3;
+                    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(b0), "=r"(b1), "=r"(b2), "=r"(b3) : "r"(a_row + 16u * j) : "memory");
+                    mma_bf16(acc[j], x[0], x[1], x[2], x[3], b0, b1);
+                    mma_bf16(acc[j + 1], x[0], x[1], x[2], x[3], b2, b3);
+                }
+            }
+            float* d = sums + ((c * 8 + warp) * 16 + g) * (r + 8) + 2 * t;
+#pragma unroll
+            for (int j = 0; j < kOwnRank / 8; ++j) {
+                if (8 * j >= r) break;
+                *reinterpret_cast<float2*>(d + 8 * j) = make_float2(acc[j][0], acc[j][1]);
+                *reinterpret_cast<float2*>(d + 8 * (r + 8) + 8 * j) = make_float2(acc[j][2], acc[j][3]);
+            }
+        }
+        __syncthreads();
+        const int row = (int)threadIdx.x >> 3, col = 4 * ((int)threadIdx.x & 7);
+        if (row < 16 && col < r) {
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+            for (int c = 0; c < 1 << log; ++c) {
+                float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int w = 0; w < 8; ++w) {
+                    const float4 b = *reinterpret_cast<const float4*>(sums + ((c * 8 + w) * 16 + row) * (r + 8) + col);
+                    sum.x += b.x; sum.y += b.y; sum.z += b.z; sum.w += b.w;
+                }
+                v.x += sum.x; v.y += sum.y; v.z += sum.z; v.w += sum.w;
+            }
+            *reinterpret_cast<uint2*>(T + row * (r + 8) + col) = make_uint2(pack_bf16x2(s * v.x, s * v.y), pack_bf16x2(s * v.z, s * v.w));
+        }
+        __syncthreads();
+    }
+};
+
 // Grid: (row groups, for each the slices of the contraction; token tiles of all members).  Every slice has two slots, whose sums are added up
 // first, then the slices' sums one after the other; where that happens does not change the result:
 //   spread: a slice per CTA, a slot per half of its warps; the slices of a group are a cluster, and every CTA of it adds up a share of the rows,
 //           which the others' warps write into its shared memory;
 //   MERGED: one CTA does all slices of a group, each half of its warps every other half of them.  For grids of several waves: a CTA costs
 //           about 4 us beside its steps (its launch in a cluster, the way from a row's number to its codes, a barrier of the cluster).
-template <int NT8, int NB, bool MERGED, int CTAS>
+// OWN: one slice, and every CTA forms T itself (OwnT); no launch goes before this one.
+template <int NT8, int NB, bool MERGED, int CTAS, bool OWN>
 __global__ void __launch_bounds__(kSmallThreads, CTAS) small_kernel(const __grid_constant__ SmallParams<NB> P, const int slices) {
     extern __shared__ __align__(128) unsigned char small_smem[];
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (OWN) {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        if (P.clear_status && blockIdx.x == 0 && threadIdx.x == 0) *P.status = 0u;
+    }
     if (!MERGED) cluster_arrive();   // "this CTA runs": waited for before its shared memory is written from elsewhere
     constexpr int kTokens = 8 * NT8;
     constexpr uint32_t kTokenBytes = 2u * kTokens * kSmallSpan * 2u;     // two steps of one half of the warps
     float* sums = reinterpret_cast<float*>(small_smem + 2 * kTokenBytes);   // spread: [slots][tokens][share of the rows]; MERGED: see end()
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const OwnT own(reinterpret_cast<unsigned char*>(sums + 2 * kTokens * kSmallRows), P.K, P.r);
+    if (OWN) own.fetch(P.m[0].A, P.K, P.r);
     const int rank = MERGED ? 0 : (int)ptx::cluster_ctarank();
     int grp = MERGED ? (int)blockIdx.x : ((int)gridDim.x - 1 - (int)blockIdx.x) >> (31 - __clz(slices));     // (spread: the long rows of 4 bits first)
     const Unit un = unit_at(P, (int)blockIdx.y, kTokens);
@@ -379,7 +466,16 @@ __global__ void __launch_bounds__(kSmallThreads, CTAS) small_kernel(const __grid
         if (slot * 16 < P.r) fetch_up(slot);
     };
     auto end = [&](int slot, float (&acc)[NT8][4]) {
-        asm volatile("griddepcontrol.wait;" ::: "memory");               // T is in place
+        if constexpr (OWN) {             // (a warp has one slot, of one step at most: the second of two steps is the second half's)
+            const uint32_t staged = ptx::smem_u32(small_smem);
+            const bool two = P.K > kSmallSpan;
+            own.form<NT8>(P.K, P.r, P.s, [&](int step) { return staged + (two && step == 0 ? 0u : kTokenBytes); });
+            const int m = (int)threadIdx.x >> 4, col = 4 * ((int)threadIdx.x & 15);          // (the padded rank is 64)
+            if (blockIdx.x == 0 && m < W.M)  // for the gradients
+                *reinterpret_cast<uint2*>(W.T + (size_t)m * P.rp + col) = col < P.r ? *reinterpret_cast<const uint2*>(own.T + m * (P.r + 8) + col) : make_uint2(0u, 0u);
+        } else {
+            asm volatile("griddepcontrol.wait;" ::: "memory");           // T is in place
+        }
         for (int i = slot; i * 16 < P.r; i += slots) {
             if (i != slot) fetch_up(i);
             const uint32_t a0 = raw[0] | (raw[1] << 16), a1 = raw[4] | (raw[5] << 16), a2 = raw[2] | (raw[3] << 16), a3 = raw[6] | (raw[7] << 16);
@@ -387,7 +483,11 @@ __global__ void __launch_bounds__(kSmallThreads, CTAS) small_kernel(const __grid
             for (int nt = 0; nt < NT8; ++nt) {
                 const int m = un.m0 + nt * 8 + g;
                 uint32_t b0 = 0u, b1 = 0u;
-                if (m < W.M) {
+                if (OWN) {
+                    const uint32_t* tr = reinterpret_cast<const uint32_t*>(own.T + (nt * 8 + g) * (P.r + 8) + i * 16) + t;
+                    b0 = tr[0];
+                    b1 = tr[4];
+                } else if (m < W.M) {
                     const uint32_t* tr = reinterpret_cast<const uint32_t*>(W.T + (size_t)m * P.rp + i * 16) + t;
                     b0 = __ldcg(tr);
                     b1 = __ldcg(tr + 4);
@@ -716,11 +816,12 @@ lowra_status launch_units(const SmallParams<NB>& P, int slices, cudaStream_t str
     return cudaLaunchKernelEx(&cfg, units_kernel<NB>, P, order, slices) == cudaSuccess ? LOWRA_OK : LOWRA_ERR_CUDA;
 }
 
-template <int NT8, int NB, bool MERGED, int CTAS>
+template <int NT8, int NB, bool MERGED, int CTAS, bool OWN = false>
 lowra_status launch_product(const SmallParams<NB>& P, int groups, int units, int slices, cudaStream_t stream) {
-    const size_t smem = 4u * (8 * NT8) * kSmallSpan * 2u + (MERGED ? (2 + slices / 2) * (8 * NT8) * kMergedPitch * 4u : 2u * (8 * NT8) * kSmallRows * 4u);
+    const size_t smem = 4u * (8 * NT8) * kSmallSpan * 2u + (MERGED ? (2 + slices / 2) * (8 * NT8) * kMergedPitch * 4u : 2u * (8 * NT8) * kSmallRows * 4u) +
+                        (OWN ? OwnT::bytes(P.K, P.r) : 0);
     static SmemLimit limit = {};
-    if (ensure_smem_limit(reinterpret_cast<const void*>(small_kernel<NT8, NB, MERGED, CTAS>), smem, &limit) != LOWRA_OK) return LOWRA_ERR_CUDA;
+    if (ensure_smem_limit(reinterpret_cast<const void*>(small_kernel<NT8, NB, MERGED, CTAS, OWN>), smem, &limit) != LOWRA_OK) return LOWRA_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -734,7 +835,7 @@ lowra_status launch_product(const SmallParams<NB>& P, int groups, int units, int
     cfg.stream = stream;
     cfg.attrs = attr;
     cfg.numAttrs = MERGED || slices == 1 ? 1 : 2;           // (a CTA is a cluster of its own without being told, and 0.4 us less host time)
-    return cudaLaunchKernelEx(&cfg, small_kernel<NT8, NB, MERGED, CTAS>, P, slices) == cudaSuccess ? LOWRA_OK : LOWRA_ERR_CUDA;
+    return cudaLaunchKernelEx(&cfg, small_kernel<NT8, NB, MERGED, CTAS, OWN>, P, slices) == cudaSuccess ? LOWRA_OK : LOWRA_ERR_CUDA;
 }
 
 int product_slices(int N, int K) {
@@ -778,10 +879,16 @@ lowra_status launch_members(const SmallParams<NB>& P, cudaStream_t stream) {
         m16 += (m.M + 15) / 16;
         most = m.M > most ? m.M : most;
     }
+    const int n_span = (P.K + kSmallSpan - 1) / kSmallSpan, slices = product_slices(P.N, P.K);
+    // Small weights, low ranks: what a launch costs the host (2.7 us) is more than T costs every CTA (512 x 512, 16 tokens, rank 16 8.0 -> 5.9 us a call; the
+    // GPU takes 4.7 us for the two launches and 5.4 for the one).  Not where many CTAs would read much of A (4096 x 384, 16 tokens, rank 32: 7.8, 8.6).
+    if constexpr (NB == 1) {
+        if (slices == 1 && P.K <= kOwnK && P.r <= kOwnRank && most <= 16 && groups <= (P.r <= 16 ? kNumSMs : 40))
+            return most <= 8 ? launch_product<1, NB, false, 2, true>(P, groups, 1, 1, stream) : launch_product<2, NB, false, 2, true>(P, groups, 1, 1, stream);
+    }
     // ---- T: the contraction over up to eight CTAs, 128 indices or more each
     {
-        int slices = 1;
-        while (slices < 8 && P.K >= 256 * slices) slices *= 2;
+        const int slices = project_slices(P.K);
         const size_t smem = project_fetch_bytes(P.r) + (size_t)16 * P.r * 4;
         static SmemLimit limit = {};
         if (ensure_smem_limit(reinterpret_cast<const void*>(project_kernel<NB>), smem, &limit) != LOWRA_OK) return LOWRA_ERR_CUDA;
@@ -802,7 +909,6 @@ lowra_status launch_members(const SmallParams<NB>& P, cudaStream_t stream) {
     }
     // ---- the product: slices of the contraction until the grid is about three CTAs per two places, as long as every warp keeps
     // a step of 256.  The choice depends on the weight's shape alone, so that a member's result does not depend on its company.
-    const int n_span = (P.K + kSmallSpan - 1) / kSmallSpan, slices = product_slices(P.N, P.K);
     const int nt8 = most <= 8 ? 1 : most <= 16 ? 2 : most <= 24 ? 3 : 4;
     if (P.one_weight && units_pay(P, slices)) return launch_units<NB>(P, slices, stream);
     int units = 0;
