@@ -205,7 +205,7 @@ size_t lowra_workspace_bytes(const lowra_layout* layout, int32_t M, int32_t r);
  * dequantising warps sorted by precision.  With layout->deal_dev == NULL every call works that out again in
  * a small prologue launch, which also clears the status word and the flags in the workspace.  With
  * layout->deal_dev pointing at a buffer filled by lowra_deal_build the fused kernel is the only launch
- * of a call (2-3 us less per call on a B200; forward calls of up to 64 tokens mostly take another path, of two launches, which needs no
+ * of a call (2-3 us less per call on a B200; forward calls of up to 64 tokens mostly take another path, of one or two launches, which needs no
  * deal); the workspace then has to be initialised once with
  * lowra_workspace_init before its first use, is written by these calls only, and its status word is no
  * longer cleared per call: lowra_device_status reports the first failure since the initialisation.
@@ -302,7 +302,7 @@ lowra_status lowra_lora_backward_input_batch(const lowra_member* members_host, i
  * [group_start_host[a], group_start_host[a + 1]) of X and Y, and for those rows
  *     Y = X . deq_a(Wq)^T + s * (X . A_a) . B_a
  * with deq_a the dequantisation through adapter a's mappings.  One call routes every group to its tables.  Groups of few tokens (up to 16
- * always, up to 64 by the weight's shape and precisions) go first, eight to two launches, with or without a deal.  Of the others up to
+ * always, up to 64 by the weight's shape and precisions) go first, eight to one or two launches, with or without a deal.  Of the others up to
  * LOWRA_MAX_BATCH run in one fused launch (their tiles dealt to the SMs together, so that small groups fill the
  * GPU between them) when the layout carries a deal and the workspace has lowra_batch_workspace_bytes(layout,
  * LOWRA_MAX_BATCH, M, r) bytes; otherwise every group is a launch of its own.  Groups of up to 16 tokens are bit for bit what a call of their
