@@ -76,7 +76,7 @@ class _CMember(ctypes.Structure):
 
 
 _lib = None
-_py_calls = None    # the two products' native way (csrc/py_calls.cpp), loaded with the library
+_py_calls = None    # the products' and the gradients' native way (csrc/py_calls.cpp), loaded with the library
 
 
 def _load_py_calls(L: ctypes.CDLL):
@@ -91,7 +91,9 @@ def _load_py_calls(L: ctypes.CDLL):
                       RuntimeWarning, stacklevel=3)
         return None
     address = lambda fn: ctypes.cast(fn, ctypes.c_void_p).value  # noqa: E731
-    module.bind(address(L.lowra_lora_forward), address(L.lowra_lora_backward_input), address(L.lowra_workspace_bytes), address(L.lowra_workspace_init))
+    module.bind(*(address(fn) for fn in (L.lowra_lora_forward, L.lowra_lora_backward_input, L.lowra_workspace_bytes, L.lowra_workspace_init, L.lowra_lora_forward_batch,
+                                         L.lowra_lora_backward_input_batch, L.lowra_lora_backward_adapters, L.lowra_lora_backward_adapters_reuse,
+                                         L.lowra_adapter_workspace_bytes, L.lowra_workspace_projection)))
     return module
 
 
@@ -567,6 +569,12 @@ def lowra_batch_workspace_bytes(layout: Layout, count: int, M: int, r: int) -> i
 
 def _batch(fn_name: str, members, s: float, workspace: torch.Tensor, backward: bool, stream=None):
     """members: sequence of dicts with layout, packed, absmax, maps, act, A, B, out (device tensors)."""
+    if stream is None and _py_calls is not None:
+        done = _py_calls.batch(backward, members, s, workspace)
+        if done is not None:
+            if done.__class__ is int:
+                _check(done, fn_name)
+            return done
     n = len(members)
     arr = (_CMember * n)()
     M = int(members[0]["act"].shape[0])
@@ -775,6 +783,12 @@ def lowra_lora_backward_adapters(X, dY, A, B, s: float, dA: Optional[torch.Tenso
                                  dB: Optional[torch.Tensor] = None, workspace: Optional[torch.Tensor] = None,
                                  stream=None) -> Tuple[torch.Tensor, torch.Tensor]:
     """dA = s X^T (dY B^T) [K,r] and dB = s (X A)^T dY [r,N]; all operands bf16 on the device."""
+    if stream is None and _py_calls is not None:
+        done = _py_calls.gradients(X, dY, A, B, s, dA, dB, workspace)
+        if done is not None:
+            if done.__class__ is int:
+                _check(done, "lowra_lora_backward_adapters")
+            return done
     M, K = int(X.shape[0]), int(X.shape[1])
     N, r = int(dY.shape[1]), int(A.shape[1])
     if not _fits(X.get_device(), X, "h", 0, dY, "h", 0, A, "h", 0, B, "h", 0, dA, "h", K * r, dB, "h", r * N, workspace, "B", 0):
@@ -804,6 +818,10 @@ def lowra_lora_backward_adapters(X, dY, A, B, s: float, dA: Optional[torch.Tenso
 def lowra_workspace_projection(workspace: torch.Tensor, M: int, r: int, member: int = 0) -> torch.Tensor:
     """The down-projection (s X A after a forward call, s dY B^T after a backward-input call) that the last fused call
     left in `workspace`: a bf16 [M, rp] view into the workspace, rp = r rounded up to 64."""
+    if _py_calls is not None:
+        done = _py_calls.projection(workspace, M, r, member)
+        if done is not None:
+            return done
     _dev(workspace, torch.uint8, "workspace")
     p = lib().lowra_workspace_projection(_ptr(workspace), int(member), int(M), int(r))
     if not p:
@@ -818,6 +836,12 @@ def lowra_lora_backward_adapters_reuse(X, dY, T, U, r: int, dA: Optional[torch.T
                                        stream=None) -> Tuple[torch.Tensor, torch.Tensor]:
     """dA = X^T U [K, r] and dB = T^T dY [r, N] from the down-projections T, U (bf16 [M, rp]) that the forward and the
     backward-input call left in their workspaces (lowra_workspace_projection): X and dY are read once."""
+    if stream is None and _py_calls is not None:
+        done = _py_calls.gradients_reuse(X, dY, T, U, r, dA, dB, workspace)
+        if done is not None:
+            if done.__class__ is int:
+                _check(done, "lowra_lora_backward_adapters_reuse")
+            return done
     M, K, N = int(X.shape[0]), int(X.shape[1]), int(dY.shape[1])
     rp = (int(r) + 63) // 64 * 64
     if not _fits(X.get_device(), X, "h", 0, dY, "h", 0, T, "h", 0, U, "h", 0, dA, "h", K * r, dB, "h", r * N, workspace, "B", 0):
