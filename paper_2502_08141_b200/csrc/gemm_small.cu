@@ -338,7 +338,7 @@ __device__ __forceinline__ void multiply_rows(int K, const SmallMember& W, int m
 
 // T of up to 16 tokens by one CTA of the product, for itself: a weight so small that the projection's launch costs more.  A lies in shared memory as in memory,
 // behind it are the warps' sums [slices][warps][16 tokens][r + 8] and T [16][r + 8]; the tokens are those staged for the product (one step per slot).  The same sums in
-// the same order as project_kernel's.  Ends with a barrier.
+// the same order as project_kernel's, the slices' steps side by side (one after the other 0.15 - 0.3 us longer).  Ends with a barrier.
 constexpr int kOwnK = 512, kOwnRank = 32, kOwnSlices = 4;
 static_assert(project_slices(kOwnK) == kOwnSlices && project_slices(kOwnK - 1) < kOwnSlices, "slices");
 struct OwnT {
@@ -358,8 +358,9 @@ struct OwnT {
         const int log = K < 256 ? 0 : K < 512 ? 1 : 2, n_steps = K / 16;
         ptx::cp_async_wait<0>();
         __syncthreads();
-#pragma unroll 1
-        for (int c = 0; c < 1 << log; ++c) {
+#pragma unroll
+        for (int c = 0; c < kOwnSlices; ++c) {
+            if (c >= 1 << log) break;
             float acc[kOwnRank / 8][4];
 #pragma unroll
             for (int j = 0; j < kOwnRank / 8; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.0f;
@@ -392,8 +393,9 @@ struct OwnT {
         const int row = (int)threadIdx.x >> 3, col = 4 * ((int)threadIdx.x & 7);
         if (row < 16 && col < r) {
             float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 1
-            for (int c = 0; c < 1 << log; ++c) {
+#pragma unroll
+            for (int c = 0; c < kOwnSlices; ++c) {
+                if (c >= 1 << log) break;
                 float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
                 for (int w = 0; w < 8; ++w) {
@@ -880,8 +882,8 @@ lowra_status launch_members(const SmallParams<NB>& P, cudaStream_t stream) {
         most = m.M > most ? m.M : most;
     }
     const int n_span = (P.K + kSmallSpan - 1) / kSmallSpan, slices = product_slices(P.N, P.K);
-    // Small weights, low ranks: what a launch costs the host (2.7 us) is more than T costs every CTA (512 x 512, 16 tokens, rank 16 8.0 -> 5.9 us a call; the
-    // GPU takes 4.7 us for the two launches and 5.4 for the one).  Not where many CTAs would read much of A (4096 x 384, 16 tokens, rank 32: 7.8, 8.6).
+    // Small weights, low ranks: what a launch costs the host (2.7 us) is more than T costs every CTA (512 x 512, 16 tokens, rank 16 8.0 -> 5.8 us a call; the
+    // GPU takes 4.7 us for the two launches and 5.2 for the one).  Not where many CTAs would read much of A (4096 x 384, 16 tokens, rank 32: 7.8, 8.6).
     if constexpr (NB == 1) {
         if (slices == 1 && P.K <= kOwnK && P.r <= kOwnRank && most <= 16 && groups <= (P.r <= 16 ? kNumSMs : 40))
             return most <= 8 ? launch_product<1, NB, false, 2, true>(P, groups, 1, 1, stream) : launch_product<2, NB, false, 2, true>(P, groups, 1, 1, stream);
