@@ -109,6 +109,15 @@ constexpr float kVanishing = 0x1p-44f;   // scaled weights from here on are abov
 struct Fine {
     long long wn, wn_lo, w, w_lo;
 };
+__device__ __forceinline__ void add_up(Fine& f) {       // over the warp
+#pragma unroll
+    for (int d = 16; d >= 1; d >>= 1) {
+        f.wn += __shfl_xor_sync(0xffffffffu, f.wn, d);
+        f.wn_lo += __shfl_xor_sync(0xffffffffu, f.wn_lo, d);
+        f.w += __shfl_xor_sync(0xffffffffu, f.w, d);
+        f.w_lo += __shfl_xor_sync(0xffffffffu, f.w_lo, d);
+    }
+}
 template <int UNROLL, typename F>
 __device__ __forceinline__ Fine fine_sums(F element, int p0, int p1, int step, float t_lo, float t_hi, double g) {
     const double g2 = g * 0x1p-46;
@@ -124,13 +133,7 @@ __device__ __forceinline__ Fine fine_sums(F element, int p0, int p1, int step, f
         f.wn_lo += (long long)(grid_bits(__dadd_rd(__fma_rn(n, w, -__dsub_rn(a, g)), g2)) - grid_bits(g2));
         f.w_lo += (long long)(grid_bits(__dadd_rn(__dsub_rn(w, __dsub_rn(b, g)), g2)) - grid_bits(g2));
     }
-#pragma unroll
-    for (int d = 16; d >= 1; d >>= 1) {
-        f.wn += __shfl_xor_sync(0xffffffffu, f.wn, d);
-        f.wn_lo += __shfl_xor_sync(0xffffffffu, f.wn_lo, d);
-        f.w += __shfl_xor_sync(0xffffffffu, f.w, d);
-        f.w_lo += __shfl_xor_sync(0xffffffffu, f.w_lo, d);
-    }
+    add_up(f);
     return f;
 }
 template <typename F>
@@ -910,15 +913,38 @@ struct Ordered {
     float weight;
 };
 
-// The mean of the bucket [t_lo, t_hi) by the whole CTA; y if it weighs nothing.  scratch: five words per warp.
+// As fine_sums, for `count` values of one weight, 32 apart in shared memory from `at` on.
+__device__ __forceinline__ Fine fine_sums_of(float weight, uint32_t at, int count, double g) {
+    const double g2 = g * 0x1p-46, w = (double)weight, b = __dadd_rn(w, g);
+    Fine f = {0, 0, count * (long long)(grid_bits(b) - grid_bits(g)),
+              count * (long long)(grid_bits(__dadd_rn(__dsub_rn(w, __dsub_rn(b, g)), g2)) - grid_bits(g2))};
+    for (int p = 0; p < count; ++p, at += 128) {
+        const double n = (double)lds_f32(at), a = __fma_rd(n, w, g);
+        f.wn += (long long)(grid_bits(a) - grid_bits(g));
+        f.wn_lo += (long long)(grid_bits(__dadd_rd(__fma_rn(n, w, -__dsub_rn(a, g)), g2)) - grid_bits(g2));
+    }
+    add_up(f);
+    return f;
+}
+
+// The mean of the bucket [t_lo, t_hi) by the whole CTA; y if it weighs nothing.  scratch: five words per warp.  A thread's part of the bucket lies together:
+// two bisections find it.
 template <int PER, int WARPS>
 __device__ __noinline__ double fine_mean_ordered(Ordered O, float t_lo, float t_hi, bool vanished, double y, long long* scratch) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    auto element = [&](int p) { return make_float2(lds_f32(O.xs + 128 * p), O.weight); };
+    uint32_t at = O.xs, end = O.xs;
+#pragma unroll
+    for (int h = PER / 2; h >= 1; h /= 2) {
+        add_if_below(at, h * 128, lds_f32(at + (h - 1) * 128), t_lo);
+        add_if_below(end, h * 128, lds_f32(end + (h - 1) * 128), t_hi);
+    }
+    add_if_below(at, 128, lds_f32(at), t_lo);
+    add_if_below(end, 128, lds_f32(end), t_hi);
+    const int count = end > at ? (int)(end - at) / 128 : 0;
     double g = kGrid;
     if (vanished) {
         float* most_of = reinterpret_cast<float*>(scratch + 4 * WARPS);
-        float most = largest_weight(element, 0, PER, 1, t_lo, t_hi);
+        float most = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(count > 0 ? O.weight : 0.0f)));      // (none is negative)
         if (WARPS > 1) {
             if (lane == 0) most_of[warp] = most;
             __syncthreads();
@@ -930,7 +956,7 @@ __device__ __noinline__ double fine_mean_ordered(Ordered O, float t_lo, float t_
             return y;
         }
     }
-    Fine f = fine_sums<2>(element, 0, PER, 1, t_lo, t_hi, g);
+    Fine f = fine_sums_of(O.weight, at, count, g);
     if (WARPS > 1) {
         if (lane == 0) { scratch[4 * warp] = f.wn; scratch[4 * warp + 1] = f.wn_lo; scratch[4 * warp + 2] = f.w; scratch[4 * warp + 3] = f.w_lo; }
         __syncthreads();
