@@ -13,6 +13,7 @@
 // them, a block per lane.  sorted_learn_kernel brings the whole row into order, after which a round takes a few hundred of its values.  The more
 // thresholds and rounds, the more order pays (kernel_for).
 #include <float.h>
+#include <limits.h>
 #include <math.h>
 #include <string.h>
 
@@ -1228,23 +1229,36 @@ bool two_long_rows(int K) { return 2 * (sorted_smem_bytes(K) + 1024) <= 228 * 10
 //   K=16384   83/97   119/114 225/162          120/105 197/130 432/209          169/281 263/322 549/443           199/279 328/321 704/445
 // At 1 bit the ordered blocks pay in the fourth round where every lane has a block, later where some have none (K = 3072, 5120), or where an SM
 // holds few warps (K = 8320 to 12288); K up to 2048 is one warp, up to 1024 of short networks.
-// A few rows to an SM (`few`: four at most) wait for the longest chain, and a warp's network is longer than the eight warps' way to the order of a whole row
-// (256 rows, T = 2, us, ordered against sorted, 4 bits and all three: K = 2048 10.8 7.8, 12.0 8.5; K = 3584 9.6 8.6, 10.8 9.1) or, of 2048 values at 2 bits, than rounds
-// through the row (6.4 4.7).
+// A few rows to an SM (per_sm) wait for the longest chain, and a warp's network is longer than the eight warps' way to the order of a whole row, or, of 2048 values
+// at 1 and 2 bits, than rounds through the row.  Ordered against sorted, us, at 4 bits, one round / two: 296 rows of 1152 8.0 6.1 / 9.2 6.9, of 2048 8.1 6.6 / 9.1 7.7, of
+// 4096 8.6 8.1; 1600 rows of 2048 12.0 16.3.  Rows that leave most of their last warp without a block (1152, 2176 values) gain little from it with any number.  Of 1794 calls for
+// each column (23 lengths, 40 to 4096 rows) the choice is 0.4 % behind the better kernel in the mean, 18 % at most (at 1 bit 1.7).
 enum Kernel { kRowAgain, kOrdered, kSorted };
 int ordered_warps(int K) { return (K + 2047) / 2048; }
-Kernel kernel_for(int K, int c, int iterations, bool few) {
+// Rows of up to `up_to` values: by their whole order from round `few` on with up to `rows` of them to an SM, from round `many` on with more.
+struct SortedFrom { int up_to, rows, few, many; };
+constexpr SortedFrom kFour[] = {{512, 8, 2, 2}, {1024, 8, 2, 3}, {1536, 6, 1, 2}, {2048, 5, 1, 4}, {2560, 0, 1, 1}, {3072, 2, 1, 2}, {4096, 2, 1, 4}, {5120, 4, 2, 3},
+                                {6144, 2, 2, 10}, {8192, 2, 2, 6}, {10240, 2, 3, 4}, {11776, 0, 4, 4}, {kSortedMaxK, 1, 4, 10}};
+constexpr SortedFrom kAll[] = {{512, 8, INT_MAX, 2}, {1024, 8, 10, 4}, {1536, 6, 1, 2}, {2048, 5, 1, 4}, {2560, 0, 1, 1}, {3072, 3, 1, 2}, {4096, 2, 1, 3}, {5120, 2, 1, 2},
+                               {6144, 2, 1, 4}, {8192, 2, 2, 4}, {10240, 2, 2, 3}, {11776, 0, 3, 3}, {kSortedMaxK, 1, 3, 6}};
+Kernel kernel_for(int K, int c, int iterations, int rows) {
     if (K > kSortedMaxK || iterations < 1) return kRowAgain;
+    const int per_sm = (rows + kNumSMs - 1) / kNumSMs;
     if (c == 0) {
-        const bool pays = K <= 1024 || (K <= 2048 ? iterations >= (few ? 4 : 3) : (iterations - (K > 8192 && K <= 12288 ? 2 : 0)) * K >= 4 * 2048 * ordered_warps(K));
+        const bool pays = K <= 1024 ? K <= 512 || iterations >= 2 || per_sm > 5 : K <= 2048 ? iterations >= (per_sm <= 4 ? 6 : 3)
+                        : (iterations - (K > 8192 && K <= 12288 ? 2 : 0)) * K >= 4 * 2048 * ordered_warps(K);
         return pays ? kOrdered : kRowAgain;
     }
-    if (c == 1) return K <= 1024 || iterations >= (few && K <= 2048 ? 4 : K > 8192 && K <= 12288 ? 3 : 2) ? kOrdered : kRowAgain;
-    if (few && iterations >= 2 && ((K > 1024 && K <= 6144) || (c == 3 && K > 8192 && K <= 11776))) return kSorted;      // (five warps: two on one scheduler)
-    constexpr int kUpTo[] = {512, 1024, 2048, 3072, 4096, 6144, 8192, 11776}, kFour[] = {2, 3, 4, 3, 5, 3, 7, 4, 9}, kAll[] = {2, 4, 4, 2, 4, 2, 4, 3, 5};
-    int i = 0;
-    while (i < 8 && K > kUpTo[i]) ++i;
-    return iterations >= (c == 2 ? kFour : kAll)[i] ? kSorted : kOrdered;
+    if (c == 1) {
+        const bool idle = per_sm <= 2;
+        const int from = K <= 1024 ? 1 : K <= 2048 ? (per_sm <= 4 ? 4 : 2) : K <= 3072 && idle ? 4 : (K <= 6144 && idle) || K <= 2560 || (K > 8192 && K <= 12288) ? 3 : 2;
+        return iterations >= from ? kOrdered : kRowAgain;
+    }
+    const SortedFrom* line = c == 2 ? kFour : kAll;
+    while (K > line->up_to) ++line;
+    // (five rows of two warps leave one scheduler more to do than another; in the order of whole rows an SM has five at a time)
+    const int many = K > 2560 && K <= 4096 && per_sm == 5 ? 2 : line->many;
+    return iterations >= (per_sm <= line->rows ? line->few : many) ? kSorted : kOrdered;
 }
 
 template <bool ALL3, int PER, int WARPS, int CTAS>
@@ -1286,11 +1300,19 @@ lowra_status launch_learn(LearnParams& P, const double* init_levels_host, const 
             P.init_y[c][j] = init_levels_host[c * 16 + j];
             P.init_t[c][j] = init_thresholds_host[c * 16 + j];
         }
-    // stored rows are in the order of their precisions: the last `sorted` of them go to the sorted kernel
+    const int per_sm = (P.N + kNumSMs - 1) / kNumSMs;
     Kernel kernel[3];
-    for (int c = 0; c < 3; ++c) kernel[c] = kernel_for(P.K, ALL3 ? 3 : c, P.iterations, P.N <= 4 * kNumSMs);
-    // (one launch fewer counts for more than the rows' kernel where these are few: 535 x 2048 at 60/35/5, T = 2 10.2 -> 7.8 us)
-    if (!ALL3 && P.N <= 8 * kNumSMs && kernel[0] == kRowAgain && kernel[1] == kOrdered && n1 > 0 && n2 > 0) kernel[0] = kOrdered;
+    for (int c = 0; c < 3; ++c) {
+        // (one round: the others' rows are done soon, and the last 4-bit row counts: 444 x 3072 at 30/50/20 9.5 -> 7.5 us)
+        const bool alone = c == 2 && P.iterations == 1 && per_sm <= (P.K <= 2048 ? 8 : P.K <= 4096 ? 5 : 0);
+        kernel[c] = kernel_for(P.K, ALL3 ? 3 : c, P.iterations, !ALL3 && alone ? n4 : P.N);
+    }
+    // One launch fewer counts for more than the rows' kernel where these are few (535 x 2048 at 60/35/5, T = 4 11.7 -> 10.2 us): the blocks' order for the 1-bit rows as well
+    // or, for two rounds of no more 2-bit rows than of 1 bit, none for the 2-bit rows (740 x 2176 at 50/50 9.5 -> 8.4 us, 888 x 4224 at 85/15 14.2 -> 11.1).
+    if (!ALL3 && per_sm <= 8 && kernel[0] == kRowAgain && kernel[1] == kOrdered && n1 > 0 && n2 > 0) {
+        const bool row = P.iterations == 2 && n1 >= n2 && ((P.K <= 3072 && per_sm <= 6) || (P.K > 4096 && P.K <= 6144 && per_sm >= 6 && n1 >= 2 * n2));
+        (row ? kernel[1] : kernel[0]) = row ? kRowAgain : kOrdered;
+    }
     // Stored rows are in the order of their precisions, and more bits want more order: a launch for every kernel that has classes, the last classes' first
     // (in turns; see enter()).
     const int n[3] = {n1, n2, n4};

@@ -1,4 +1,4 @@
-"""The learner's time: rows whose blocks differ widely.
+"""The learner's time: rows whose blocks differ widely, and one round beside two.
 
 A block 10^6 times heavier than the others leaves nearly every bucket below what the fixed-point sums resolve, so that each is added up again.  In blocks whose values lie
 in order a bucket's are found by bisection; a walk through every block for every such bucket took 2.1 to 2.7 times the usual.
@@ -51,3 +51,13 @@ def test_rows_of_unequal_blocks(N, K, bits, T):
     run = _learner(N, K, bits, W)
     usual, unequal = _us(lambda: run(T)), _us(lambda: run(T, heavy))
     assert unequal <= 1.8 * usual, (usual, unequal)
+
+
+@pytest.mark.parametrize("bits", [4, 0])
+@pytest.mark.parametrize("N,K", [(148, 1152), (296, 1152), (296, 1536), (148, 2048)])
+def test_one_round_takes_no_longer_than_two(N, K, bits):
+    """A few rows go through the order of the whole row from the first round on, not from the second (where blocks' order took 1.1 times as long for one round as that for
+    two)."""
+    run = _learner(N, K, bits, torch.randn(N, K, device="cuda", generator=torch.Generator(device="cuda").manual_seed(K)) * 0.02)
+    one, two = _us(lambda: run(1)), _us(lambda: run(2))
+    assert one <= two, (one, two)
