@@ -847,17 +847,20 @@ int product_slices(int N, int K) {
     return slices;
 }
 
-// Whether the spread form runs three CTAs to an SM, at 80 registers (some of which spill, most at 4 bits), or two at 128: for so many CTAs beside so
-// many of the projection, `four` of N channels at 4 bits.  Three where two do not fit in one wave - clusters of eight leave SMs of a GPC over - and for short
-// steps at few tokens, which wait for memory rather than for instructions.  Two against three, us (rows of 4 bits first in both; before, they were last: in brackets):
-// 60/35/5 %, 1 token: 11008 x 4096 19.6 -> 16.4 (24.7), 13824 x 5120 22.5 -> 19.6 (28.1), 6144 x 4096 16.4 -> 11.7 (18.2), 5120 x 13824 30.2 -> 24.6 (36.5), 2048 x 4096
-// 12.8 -> 10.0 (14.0), 4096 x 4096 10.25 -> 9.6; 16 tokens: 11008 x 4096 24.9 -> 19.7 (30.5), 4096 x 4096 13.0 -> 11.9.  Two where they fit and steps are long
-// (4096 x 11008, 16 tokens 18.9, three 20.1; 24 tokens 20.6, 28.3) and with most rows at 4 bits (13824 x 5120, 16 tokens 30.9, three 33.9; 4096 x 4096, 1 token 10.5, 11.5),
-// unless short steps take two waves (6144 x 4096 of 4 bits, 1 token 19.0, three 14.7); and where an SM has one CTA at most (4096 x 768, 16 tokens 7.6, 8.6).
-bool three_pay(int four, int N, int n_span, int slices, int ctas, int projection, int nt8) {
+// Whether a grid of so many CTAs beside so many of the projection runs in one wave, two to an SM (clusters of eight and four leave SMs of a GPC over).
+bool two_fit(int slices, int ctas, int projection) { return ctas + projection <= (slices == 8 ? 272 : slices == 4 ? 280 : 2 * kNumSMs); }
+
+// Whether the spread form runs three CTAs to an SM, at 80 registers (some of which spill, most at 4 bits), or two at 128: `four` of N channels at 4 bits.  Measured
+// over 32 shapes, six mixes, ranks 16 to 128, 1 to 24 tokens; two against three, us, in a captured graph:
+//   two do not fit in one wave   three (6144 x 4096 at 60/35/5, 16 tokens, rank 64 16.4 13.1; all mixes and ranks 0.70 to 1.09 of the time), but for long steps with most rows at 4 bits
+//   two fit                      two (1024 x 2048 at 60/35/5, 16 tokens, rank 16 5.4 6.2; 4096 x 1024, rank 32 6.3 7.2), but for four slices on nearly all SMs and short steps at
+//                                ranks 48 and 64, from 9 tokens on without 4-bit rows (4096 x 4096 at 85/15, 16 tokens, rank 64 10.7 10.1), and 32 with up to 8 tokens and none
+bool three_pay(int four, int N, int r, int n_span, int slices, int ctas, int projection, int nt8) {
     if (nt8 > 3) return false;                           // (no shared memory for a third)
-    const bool fit = ctas + projection <= (slices == 8 ? 272 : slices == 4 ? 280 : 2 * kNumSMs), short_steps = n_span <= 2 * (2 * slices);
-    return fit ? (slices > 1 || ctas > kNumSMs) && short_steps && nt8 <= 2 && four <= N / 8 : short_steps || four <= N / 2;
+    const bool short_steps = n_span <= 2 * (2 * slices);
+    if (!two_fit(slices, ctas, projection)) return short_steps || four <= N / 2;
+    if (slices != 4 || ctas < 128 || !short_steps || r > 64 || nt8 > 2) return false;
+    return nt8 == 1 ? (four == 0 ? r > 16 : four <= N / 8 && r > 32) : four == 0 && r > 32;
 }
 
 // groups of 64 stored rows of one precision (of the member that has the most)
@@ -923,7 +926,7 @@ lowra_status launch_members(const SmallParams<NB>& P, cudaStream_t stream) {
             return nt8 == 1 ? launch_product<1, NB, true, 2>(P, groups, units, slices, stream) : launch_product<2, NB, true, 2>(P, groups, units, slices, stream);
     }
     const int* start = P.m[0].L.class_start;
-    const bool three = three_pay(start[3] - start[2], P.N, n_span, slices, groups * slices * units, 8 * m16, nt8);
+    const bool three = three_pay(start[3] - start[2], P.N, P.r, n_span, slices, groups * slices * units, 8 * m16, nt8);
     if (nt8 == 1) return three ? launch_product<1, NB, false, 3>(P, groups, units, slices, stream) : launch_product<1, NB, false, 2>(P, groups, units, slices, stream);
     if (nt8 == 2) return three ? launch_product<2, NB, false, 3>(P, groups, units, slices, stream) : launch_product<2, NB, false, 2>(P, groups, units, slices, stream);
     if (nt8 == 3) return three ? launch_product<3, NB, false, 3>(P, groups, units, slices, stream) : launch_product<3, NB, false, 2>(P, groups, units, slices, stream);
@@ -936,7 +939,8 @@ lowra_status launch_members(const SmallParams<NB>& P, cudaStream_t stream) {
 // 1, 2 and 4 bits: 2.8 for the projection and the start, then CTAs, two to an SM.  A step of 256 takes 2.5, 0.45 more at 4 bits; around a CTA's steps and its
 // share of the low-rank term 5.4, and if it is alone on its SM all that takes 0.64 of it.  A CTA that does all slices takes 3.7 and 1.2 for every slice around its
 // steps, of which two halves overlap (0.74), and waits 1.7 for 4-bit rows among others; of three on an SM the third does not wait for both.  Fitted to 520
-// calls (256 to 13824 channels, 512 to 13824 features, ranks 16 to 128, six mixes): within 18 %.  Where three CTAs share an SM in one wave, 0.85 of that.
+// calls (256 to 13824 channels, 512 to 13824 features, ranks 16 to 128, six mixes): within 18 %.  Where two CTAs to an SM are more than one wave (and three may
+// share it), 0.85 of that.
 float small_estimate(const int32_t* n, int K, int r, int units, int most) {
     const int N = n[0] + n[1] + n[2], slices = product_slices(N, K);
     const int groups = (n[0] + kSmallRows - 1) / kSmallRows + (n[1] + kSmallRows - 1) / kSmallRows + (n[2] + kSmallRows - 1) / kSmallRows;
@@ -948,7 +952,8 @@ float small_estimate(const int32_t* n, int K, int r, int units, int most) {
         return 2.8f + (mixed ? 1.7f : 0.0f) + (3.7f + 1.2f * slices + 2.1f * rank + 0.74f * step * steps) * (k == 1 ? 0.64f : k == 2 ? 1.15f : 0.5f * k);
     }
     const int k = per_sm(groups * slices * units), n_span = (K + kSmallSpan - 1) / kSmallSpan;
-    const float three = three_pay(n[2], N, n_span, slices, groups * slices * units, 8 * ((most + 15) / 16), (most + 7) / 8) ? 0.85f : 1.0f;
+    const bool packed = most <= 24 && !two_fit(slices, groups * slices * units, 8 * ((most + 15) / 16)) && (n_span <= 2 * (2 * slices) || n[2] <= N / 2);
+    const float three = packed ? 0.85f : 1.0f;
     return 2.8f + (mixed ? 0.3f : 0.0f) + three * (5.4f + (2.2f * rank + step * steps) / slices) * (k / 2 + (k % 2 != 0 ? 0.64f : 0.0f));
 }
 
