@@ -875,6 +875,20 @@ int row_groups(const SmallParams<NB>& P) {
     return groups;
 }
 
+// Whether every CTA of a small weight (`groups` CTAs, `four` channels of 4 bits) forms T itself instead of a launch before it.  That saves a launch, 2.5 us of host time, and costs every
+// CTA the reading of A and a chain of its own.  One launch against two, us, called from the host / in a captured graph, where launches cost little:
+//   up to 256 features         512 x 256 at 50/50, 16 tokens, rank 16 4.8 6.2 / 4.4 4.6; 8192 x 256 at 50/50 0.71 - 0.92 / 0.94 - 1.05 of the time, of 4 bits, rank
+//                              16 0.88 - 1.03 / 1.08 - 1.20
+//   384 and 512                512 x 512 at 50/50, rank 16, 8 tokens 4.9 6.2 / 4.5 4.1, 16 tokens 0.94 / 1.12 of the time; not at more than 40 or 80 groups of rows, each reading so
+//                              much of A (4096 x 384 of 4 bits, 16 tokens 7.5 6.2 / 6.0 5.6), nor with slow rows and many tokens or ranks (512 x 512 of 4 bits, 16
+//                              tokens, rank 32 1.12 / 1.14)
+bool forms_own_t(int K, int r, int tokens, int groups, int four) {
+    if (K > kOwnK || r > kOwnRank || tokens > 16) return false;
+    const bool slow = four > 0;
+    if (K <= 256) return groups <= (r > 16 ? 40 : slow ? 80 : kNumSMs);
+    return (tokens <= 8 || !slow) && (r <= 16 || (tokens <= 8 && !slow)) && groups <= (r <= 16 && tokens <= 8 && !slow ? 80 : 40);
+}
+
 template <int NB>
 lowra_status launch_members(const SmallParams<NB>& P, cudaStream_t stream) {
     int m16 = 0, most = 0;
@@ -885,10 +899,9 @@ lowra_status launch_members(const SmallParams<NB>& P, cudaStream_t stream) {
         most = m.M > most ? m.M : most;
     }
     const int n_span = (P.K + kSmallSpan - 1) / kSmallSpan, slices = product_slices(P.N, P.K);
-    // Small weights, low ranks: what a launch costs the host (2.7 us) is more than T costs every CTA (512 x 512, 16 tokens, rank 16 8.0 -> 5.8 us a call; the
-    // GPU takes 4.7 us for the two launches and 5.2 for the one).  Not where many CTAs would read much of A (4096 x 384, 16 tokens, rank 32: 7.8, 8.6).
     if constexpr (NB == 1) {
-        if (slices == 1 && P.K <= kOwnK && P.r <= kOwnRank && most <= 16 && groups <= (P.r <= 16 ? kNumSMs : 40))
+        const int* start = P.m[0].L.class_start;
+        if (slices == 1 && forms_own_t(P.K, P.r, most, groups, start[3] - start[2]))
             return most <= 8 ? launch_product<1, NB, false, 2, true>(P, groups, 1, 1, stream) : launch_product<2, NB, false, 2, true>(P, groups, 1, 1, stream);
     }
     // ---- T: the contraction over up to eight CTAs, 128 indices or more each

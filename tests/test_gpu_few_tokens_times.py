@@ -47,3 +47,10 @@ def test_sixteen_tokens_take_no_longer_than_seventeen(N, K, r):
     mix = {1: 0.6, 2: 0.35, 4: 0.05}
     few, more = (_forward_us(N, K, mix, r, M) for M in (16, 17))
     assert few <= more, (few, more)
+
+
+@pytest.mark.parametrize("mix", [{2: 0.75, 4: 0.25}, {1: 0.3, 2: 0.5, 4: 0.2}])
+def test_rank_16_takes_no_longer_than_rank_32(mix):
+    """A weight of many channels whose CTAs all formed the projection at rank 16: 1.3 of the time at rank 32, for which it is a launch of its own."""
+    low, high = (_forward_us(8192, 384, mix, r, 1) for r in (16, 32))
+    assert low <= high, (low, high)
