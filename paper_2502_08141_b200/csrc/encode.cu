@@ -104,8 +104,9 @@ __device__ __forceinline__ void encode_chunk(const EncodeParams& P, int p, int c
     const float inv = (m == 0.0f) ? 0.0f : __frcp_rn(m);
 
     uint8_t* dst = P.packed + packed_row_offset(P.L, c, p, r) + (size_t)(e0 + lane * 32) * B / 8;
-    // Two elements at a time; m0, m1, m2: the thresholds negated, a zero to +0 (so that n + m is +0 for n = -0, too).  Two single multiplications: a packed one
-    // and the packed addition behind it become one fused operation in the assembler (nvcc 12.9), which skips the rounding of n.
+    // Two elements at a time; m0, m1, m2: the thresholds negated, a zero to +0 (so that n + m is +0 for n = -0, too).  Two single multiplications: with
+    // a packed one before the packed addition, nvcc 12.9, values on a threshold fell into the wrong bucket, as if n had not been rounded
+    // (tests/test_gpu_encode_thresholds.py).
     auto normalised = [&](float a, float b) { return make_float2(__fmul_rn(a, inv), __fmul_rn(b, inv)); };
     if (B == 1) {
         const float m0 = 0.0f - t0;

@@ -1149,6 +1149,7 @@ __global__ void __launch_bounds__(32 * WARPS, CTAS) ordered_learn_kernel(const _
             all[0] += (long long)(grid_bits(s) - grid_bits(kGrid));
         }
     }
+    __syncwarp();       // (see lds_f32)
 #pragma unroll
     for (int d = 16; d >= 1; d >>= 1) {
         all[0] += __shfl_xor_sync(0xffffffffu, all[0], d);

@@ -81,6 +81,8 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
     return r;
 }
 
+// A shared-memory read by address.  The compiler keeps it in its place among other volatile instructions, not among plain stores: between a store that it
+// reads and this there has to be a barrier, if only of the warp (a "memory" clobber would hold up everything around it).
 __device__ __forceinline__ float lds_f32(uint32_t at) {
     float v;
     asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(at));
@@ -108,8 +110,9 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
 }
 
 // Binary search among 15 sorted thresholds in shared memory at t_at, the middle one in t7: the address of the first that is above n (of the sixteenth place if
-// none is).  The additions are conditional by the instruction's own predicate, one each instead of a selection and an addition (written as plain
-// conditions, nvcc 12.9 makes wrong code of it in encode.cu: some values one bucket too high).
+// none is).  The additions are conditional by the instruction's own predicate, one each instead of a selection and an addition.  Written as plain
+// conditions (`if (t <= n) a += by`), nvcc 12.9, the encoder's 4-bit codes came out one too high for some values, with and without a "memory" clobber on the reads; not so as
+// selections, nor in errors.cu.  The cause is open; tests/test_gpu_encode_thresholds.py and test_gpu_encode_decode.py show it.
 __device__ __forceinline__ uint32_t threshold_place(uint32_t t_at, float t7, float n) {
     uint32_t a = t_at;
     auto step = [&](float t, uint32_t by) {
