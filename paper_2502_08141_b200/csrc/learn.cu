@@ -1231,14 +1231,14 @@ bool two_long_rows(int K) { return 2 * (sorted_smem_bytes(K) + 1024) <= 228 * 10
 // At 1 bit the ordered blocks pay in the fourth round where every lane has a block, later where some have none (K = 3072, 5120), or where an SM
 // holds few warps (K = 8320 to 12288); K up to 2048 is one warp, up to 1024 of short networks.
 // A few rows to an SM (per_sm) wait for the longest chain, and a warp's network is longer than the eight warps' way to the order of a whole row, or, of 2048 values
-// at 1 and 2 bits, than rounds through the row.  Ordered against sorted, us, at 4 bits, one round / two: 296 rows of 1152 8.0 6.1 / 9.2 6.9, of 2048 8.1 6.6 / 9.1 7.7, of
+// at 1 and 2 bits, than rounds through the row.  Ordered against sorted, us, at 4 bits, one round / two: 296 rows of 1152 8.0 6.1 / 9.6 7.1, of 2048 8.1 6.6 / 9.6 8.2, of
 // 4096 8.6 8.1; 1600 rows of 2048 12.0 16.3.  Rows that leave most of their last warp without a block (1152, 2176 values) gain little from it with any number.  Of 1794 calls for
-// each column (23 lengths, 40 to 4096 rows) the choice is 0.4 % behind the better kernel in the mean, 18 % at most (at 1 bit 1.7).
+// each column (23 lengths, 40 to 4096 rows) the choice is 0.3 % behind the better kernel in the mean, 18 % at most (at 2 bits 0.6, at 1 bit 1.7).
 enum Kernel { kRowAgain, kOrdered, kSorted };
 int ordered_warps(int K) { return (K + 2047) / 2048; }
 // Rows of up to `up_to` values: by their whole order from round `few` on with up to `rows` of them to an SM, from round `many` on with more.
 struct SortedFrom { int up_to, rows, few, many; };
-constexpr SortedFrom kFour[] = {{512, 8, 2, 2}, {1024, 8, 2, 3}, {1536, 6, 1, 2}, {2048, 5, 1, 4}, {2560, 0, 1, 1}, {3072, 2, 1, 2}, {4096, 2, 1, 4}, {5120, 4, 2, 3},
+constexpr SortedFrom kFour[] = {{512, 8, 2, 2}, {1024, 8, 3, 3}, {1536, 6, 1, 2}, {2048, 5, 1, 4}, {2560, 0, 1, 1}, {3072, 2, 1, 3}, {4096, 2, 1, 5}, {5120, 4, 2, 3},
                                 {6144, 2, 2, 10}, {8192, 2, 2, 6}, {10240, 2, 3, 4}, {11776, 0, 4, 4}, {kSortedMaxK, 1, 4, 10}};
 constexpr SortedFrom kAll[] = {{512, 8, INT_MAX, 2}, {1024, 8, 10, 4}, {1536, 6, 1, 2}, {2048, 5, 1, 4}, {2560, 0, 1, 1}, {3072, 3, 1, 2}, {4096, 2, 1, 3}, {5120, 2, 1, 2},
                                {6144, 2, 1, 4}, {8192, 2, 2, 4}, {10240, 2, 2, 3}, {11776, 0, 3, 3}, {kSortedMaxK, 1, 3, 6}};
@@ -1258,7 +1258,7 @@ Kernel kernel_for(int K, int c, int iterations, int rows) {
     const SortedFrom* line = c == 2 ? kFour : kAll;
     while (K > line->up_to) ++line;
     // (five rows of two warps leave one scheduler more to do than another; in the order of whole rows an SM has five at a time)
-    const int many = K > 2560 && K <= 4096 && per_sm == 5 ? 2 : line->many;
+    const int many = K > 2560 && K <= 4096 && (per_sm == 5 || (K <= 3072 && per_sm == 6)) ? 2 : line->many;
     return iterations >= (per_sm <= line->rows ? line->few : many) ? kSorted : kOrdered;
 }
 
@@ -1304,9 +1304,11 @@ lowra_status launch_learn(LearnParams& P, const double* init_levels_host, const 
     const int per_sm = (P.N + kNumSMs - 1) / kNumSMs;
     Kernel kernel[3];
     for (int c = 0; c < 3; ++c) {
-        // (one round: the others' rows are done soon, and the last 4-bit row counts: 444 x 3072 at 30/50/20 9.5 -> 7.5 us)
-        const bool alone = c == 2 && P.iterations == 1 && per_sm <= (P.K <= 2048 ? 8 : P.K <= 4096 ? 5 : 0);
-        kernel[c] = kernel_for(P.K, ALL3 ? 3 : c, P.iterations, !ALL3 && alone ? n4 : P.N);
+        kernel[c] = kernel_for(P.K, ALL3 ? 3 : c, P.iterations, P.N);
+        if (ALL3 || c < 2 || 2 * n4 > P.N || P.K <= 1024) continue;
+        // 4-bit rows in company are the longest: of a few rows the last one counts (444 x 3072 at 30/50/20, one round 9.5 -> 7.5 us; 535 x 6144 at 60/35/5, six 19.1 -> 14.4)
+        if (P.iterations == 1 && per_sm <= (P.K <= 2048 ? 8 : P.K <= 4096 ? 5 : 0)) kernel[c] = kernel_for(P.K, c, 1, n4);
+        if (P.K <= 6144 && (P.iterations == 2 ? per_sm <= 4 : P.iterations > 2 && per_sm <= (P.K <= 4096 ? 4 : 5))) kernel[c] = kSorted;
     }
     // One launch fewer counts for more than the rows' kernel where these are few (535 x 2048 at 60/35/5, T = 4 11.7 -> 10.2 us): the blocks' order for the 1-bit rows as well
     // or, for two rounds of no more 2-bit rows than of 1 bit, none for the 2-bit rows (740 x 2176 at 50/50 9.5 -> 8.4 us, 888 x 4224 at 85/15 14.2 -> 11.1).
