@@ -38,8 +38,9 @@ struct ErrParams {
     float* residual;          // [N, K] or null
 };
 
-// What is left of x after the value its bucket stands for, 1 bit (two values) and 2 bits (four): every candidate's difference, the last whose
-// threshold is <= n stands.  Comparisons and selections go to the half-rate pipe, conditional subtractions to the other one.
+// What is left of x after the value its bucket stands for, 1 bit (two values) and 2 bits (four): every candidate's difference, the last one that the encoder's search
+// passes through stands (at 2 bits the middle threshold first, then the one on its side, so that codes and errors agree in whatever order the thresholds are).
+// Comparisons and selections go to the half-rate pipe, conditional subtractions to the other one.
 __device__ __forceinline__ float residual_of(float x, float n, const float (&w)[2], const float (&t)[1]) {
     float r;
     asm("{\n\t.reg .pred p;\n\tsetp.le.f32 p, %4, %5;\n\tsub.rn.f32 %0, %1, %2;\n\t@p sub.rn.f32 %0, %1, %3;\n\t}"
@@ -48,8 +49,8 @@ __device__ __forceinline__ float residual_of(float x, float n, const float (&w)[
 }
 __device__ __forceinline__ float residual_of(float x, float n, const float (&w)[4], const float (&t)[3]) {
     float r;
-    asm("{\n\t.reg .pred p, q, s;\n\tsetp.le.f32 p, %6, %9;\n\tsetp.le.f32 q, %7, %9;\n\tsetp.le.f32 s, %8, %9;\n\tsub.rn.f32 %0, %1, %2;\n\t"
-        "@p sub.rn.f32 %0, %1, %3;\n\t@q sub.rn.f32 %0, %1, %4;\n\t@s sub.rn.f32 %0, %1, %5;\n\t}"
+    asm("{\n\t.reg .pred p, q, s;\n\tsetp.le.f32 p, %7, %9;\n\tsetp.le.and.f32 q, %6, %9, !p;\n\tsetp.le.and.f32 s, %8, %9, p;\n\tsub.rn.f32 %0, %1, %2;\n\t"
+        "@q sub.rn.f32 %0, %1, %3;\n\t@p sub.rn.f32 %0, %1, %4;\n\t@s sub.rn.f32 %0, %1, %5;\n\t}"
         : "=&f"(r) : "f"(x), "f"(w[0]), "f"(w[1]), "f"(w[2]), "f"(w[3]), "f"(t[0]), "f"(t[1]), "f"(t[2]), "f"(n));
     return r;
 }
