@@ -875,18 +875,17 @@ int row_groups(const SmallParams<NB>& P) {
     return groups;
 }
 
-// Whether every CTA of a small weight (`groups` CTAs, `four` channels of 4 bits) forms T itself instead of a launch before it.  That saves a launch, 2.5 us of host time, and costs every
-// CTA the reading of A and a chain of its own.  One launch against two, us, called from the host / in a captured graph, where launches cost little:
-//   up to 256 features         512 x 256 at 50/50, 16 tokens, rank 16 4.8 6.2 / 4.4 4.6; 8192 x 256 at 50/50 0.71 - 0.92 / 0.94 - 1.05 of the time, of 4 bits, rank
-//                              16 0.88 - 1.03 / 1.08 - 1.20
-//   384 and 512                512 x 512 at 50/50, rank 16, 8 tokens 4.9 6.2 / 4.5 4.1, 16 tokens 0.94 / 1.12 of the time; not at more than 40 or 80 groups of rows, each reading so
-//                              much of A (4096 x 384 of 4 bits, 16 tokens 7.5 6.2 / 6.0 5.6), nor with slow rows and many tokens or ranks (512 x 512 of 4 bits, 16
-//                              tokens, rank 32 1.12 / 1.14)
+// Whether every CTA of a small weight (`groups` CTAs, `four` channels of 4 bits) forms T itself instead of a launch before it.  That saves a launch, 2.5 us of host time, which all
+// calls show that allocate their output and scratch, and costs every CTA the reading of A and a chain of its own, which shows where the host is ahead.  One launch against two, us, nothing
+// kept / output and workspace kept / in a captured graph:
+//   512 x 512 at 50/50, rank 16, 8 tokens   5.4 8.0 / 4.9 5.9 / 4.5 4.0      256 x 256 at 50/50, rank 16, 16 tokens   5.3 7.7 / 4.6 5.7 / 4.2 4.5
+//   at 60/35/5, rank 32, 16 tokens          6.8 8.0 / 6.8 5.9 / 6.4 5.6      4096 x 384 of 4 bits, rank 16, 16 tokens 6.9 7.9 / 7.6 6.1 / 5.9 5.6
+// Not with ranks above 16 on more than 40 groups of rows, which each read so much of A (4096 x 384 at 60/35/5, rank 32, 16 tokens 8.7 7.9 / 8.6 7.1 / 7.4 6.2), nor above 256
+// features with slow rows on more than 40 for more than 8 tokens (3072 x 512 of 4 bits, rank 16, 9 tokens 6.9 8.0 / 7.9 5.9 / 5.9 5.2) or 80 for fewer (8192 x 384 at 60/35/5, rank
+// 16, 1 token 5.5 8.0 / 6.5 5.9 / 6.0 4.5).
 bool forms_own_t(int K, int r, int tokens, int groups, int four) {
     if (K > kOwnK || r > kOwnRank || tokens > 16) return false;
-    const bool slow = four > 0;
-    if (K <= 256) return groups <= (r > 16 ? 40 : slow ? 80 : kNumSMs);
-    return (tokens <= 8 || !slow) && (r <= 16 || (tokens <= 8 && !slow)) && groups <= (r <= 16 && tokens <= 8 && !slow ? 80 : 40);
+    return groups <= (r > 16 ? 40 : K <= 256 || four == 0 ? kNumSMs : tokens > 8 ? 40 : 80);
 }
 
 template <int NB>

@@ -54,3 +54,9 @@ def test_rank_16_takes_no_longer_than_rank_32(mix):
     """A weight of many channels whose CTAs all formed the projection at rank 16: 1.3 of the time at rank 32, for which it is a launch of its own."""
     low, high = (_forward_us(8192, 384, mix, r, 1) for r in (16, 32))
     assert low <= high, (low, high)
+
+
+def test_slow_rows_and_many_tokens():
+    """Likewise 49 groups of rows, some of 4 bits: 16 tokens took 1.1 of the time of 17."""
+    few, more = (_forward_us(3072, 512, {1: 0.6, 2: 0.35, 4: 0.05}, 16, M) for M in (16, 17))
+    assert few <= more, (few, more)
