@@ -1252,7 +1252,7 @@ Kernel kernel_for(int K, int c, int iterations, int rows) {
     }
     if (c == 1) {
         const bool idle = per_sm <= 2;
-        const int from = K <= 1024 ? 1 : K <= 2048 ? (per_sm <= 4 ? 4 : 2) : K <= 3072 && idle ? 4 : (K <= 6144 && idle) || K <= 2560 || (K > 8192 && K <= 12288) ? 3 : 2;
+        const int from = K <= 1024 ? 1 : K <= 2048 ? (per_sm <= 4 ? 4 : 2) : K <= 3072 && idle ? 4 : (K <= 6144 && idle) || (K > 8192 && K <= 12288) ? 3 : 2;
         return iterations >= from ? kOrdered : kRowAgain;
     }
     const SortedFrom* line = c == 2 ? kFour : kAll;
@@ -1260,6 +1260,16 @@ Kernel kernel_for(int K, int c, int iterations, int rows) {
     // (five rows of two warps leave one scheduler more to do than another; in the order of whole rows an SM has five at a time)
     const int many = K > 2560 && K <= 4096 && (per_sm == 5 || (K <= 3072 && per_sm == 6)) ? 2 : line->many;
     return iterations >= (per_sm <= line->rows ? line->few : many) ? kSorted : kOrdered;
+}
+
+// 4-bit rows, n4 of N, among others of more than 1024 values.  They are the longest, and of a few rows the last one counts (444 x 3072 at 30/50/20, one round 9.5 -> 7.5 us; 535 x 6144
+// at 60/35/5, six 19.1 -> 14.4).  Otherwise they go by the whole row's order later than by themselves, for that is a launch more: 2.5 us of the 12 that a short call takes the host
+// (600 x 2048 at 60/35/5, two rounds 15 -> 12.3).
+Kernel four_in_company(int K, int iterations, int N, int n4) {
+    const int per_sm = (N + kNumSMs - 1) / kNumSMs;
+    if (K > kSortedMaxK || iterations < 2) return kernel_for(K, 2, iterations, per_sm <= (K <= 2048 ? 8 : K <= 4096 ? 5 : 0) ? n4 : N);
+    const int from = K <= 6144 && per_sm <= 4 ? 2 : K <= 2048 ? 4 : K <= 3072 ? 3 : K <= 4096 ? 5 : K <= 6144 ? 3 : K <= 8192 ? 7 : K <= 11776 ? 4 : 9;
+    return iterations >= from ? kSorted : kOrdered;
 }
 
 template <bool ALL3, int PER, int WARPS, int CTAS>
@@ -1303,17 +1313,14 @@ lowra_status launch_learn(LearnParams& P, const double* init_levels_host, const 
         }
     const int per_sm = (P.N + kNumSMs - 1) / kNumSMs;
     Kernel kernel[3];
-    for (int c = 0; c < 3; ++c) {
-        kernel[c] = kernel_for(P.K, ALL3 ? 3 : c, P.iterations, P.N);
-        if (ALL3 || c < 2 || 2 * n4 > P.N || P.K <= 1024) continue;
-        // 4-bit rows in company are the longest: of a few rows the last one counts (444 x 3072 at 30/50/20, one round 9.5 -> 7.5 us; 535 x 6144 at 60/35/5, six 19.1 -> 14.4)
-        if (P.iterations == 1 && per_sm <= (P.K <= 2048 ? 8 : P.K <= 4096 ? 5 : 0)) kernel[c] = kernel_for(P.K, c, 1, n4);
-        if (P.K <= 6144 && (P.iterations == 2 ? per_sm <= 4 : P.iterations > 2 && per_sm <= (P.K <= 4096 ? 4 : 5))) kernel[c] = kSorted;
-    }
+    for (int c = 0; c < 3; ++c) kernel[c] = kernel_for(P.K, ALL3 ? 3 : c, P.iterations, P.N);
+    if (!ALL3 && 2 * n4 <= P.N && P.K > 1024) kernel[2] = four_in_company(P.K, P.iterations, P.N, n4);
     // One launch fewer counts for more than the rows' kernel where these are few (535 x 2048 at 60/35/5, T = 4 11.7 -> 10.2 us): the blocks' order for the 1-bit rows as well
-    // or, for two rounds of no more 2-bit rows than of 1 bit, none for the 2-bit rows (740 x 2176 at 50/50 9.5 -> 8.4 us, 888 x 4224 at 85/15 14.2 -> 11.1).
+    // or, for two rounds of no more 2-bit rows than of 1 bit, none for the 2-bit rows (740 x 2176 at 50/50 9.5 -> 8.4 us, 888 x 4224 at 85/15 14.2 -> 11.1) unless the 4-bit rows
+    // go by it.
     if (!ALL3 && per_sm <= 8 && kernel[0] == kRowAgain && kernel[1] == kOrdered && n1 > 0 && n2 > 0) {
-        const bool row = P.iterations == 2 && n1 >= n2 && ((P.K <= 3072 && per_sm <= 6) || (P.K > 4096 && P.K <= 6144 && per_sm >= 6 && n1 >= 2 * n2));
+        const bool row = P.iterations == 2 && n1 >= n2 && (n4 == 0 || kernel[2] != kOrdered) &&
+                         ((P.K <= 3072 && per_sm <= 6) || (P.K > 4096 && P.K <= 6144 && per_sm >= 6 && n1 >= 2 * n2));
         (row ? kernel[1] : kernel[0]) = row ? kRowAgain : kOrdered;
     }
     // Stored rows are in the order of their precisions, and more bits want more order: a launch for every kernel that has classes, the last classes' first
