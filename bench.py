@@ -980,7 +980,7 @@ def run_reference(args):
 # small single-kernel cases for profiler captures (a few hundred MB on the device, three launches each)
 # --------------------------------------------------------------------------------------------------
 CASES = ("forward", "backward", "forward4096", "backward_gate", "forward_4bit", "backward_4bit", "forward_1bit", "backward_1bit",
-         "codec", "decode_layer", "learn", "adapters", "adapters_reuse", "errors")
+         "codec", "decode_layer", "learn", "learn_all", "adapters", "adapters_reuse", "errors", "few_tokens")
 
 
 def run_case(case: str) -> None:
@@ -988,7 +988,7 @@ def run_case(case: str) -> None:
     at that precision); forward4096: 4096 tokens (136 pieces: tiles cut between SMs);
     backward_gate: 11008 x 4096 at 4096 tokens (last row of tiles cut); codec: decode + encode of an 11008 x 4096
     matrix; decode_layer: the seven decodes of a Llama-7B layer back to back; learn: codebook learner, 4096 x 4096,
-    10 rounds; adapters: gradients of the low-rank factors, 4096 x 11008, 4096 tokens (adapters_reuse: from given projections); errors: per-channel
+    10 rounds (learn_all: at all three precisions, 2 rounds, and the errors); few_tokens: one token, and 101 tokens of six adapters on a weight at 30/50/20, 4096 x 4096; adapters: gradients of the low-rank factors, 4096 x 11008, 4096 tokens (adapters_reuse: from given projections); errors: per-channel
     quantisation error with and without the residual, 11008 x 4096."""
     import torch
 
@@ -1034,7 +1034,7 @@ def run_case(case: str) -> None:
         torch.cuda.synchronize()
         print("decode_layer ok")
         return
-    mix = {4: 1.0} if case.endswith("_4bit") else {1: 1.0} if case.endswith("_1bit") else cfg.mix
+    mix = {4: 1.0} if case.endswith("_4bit") else {1: 1.0} if case.endswith("_1bit") else {1: 0.3, 2: 0.5, 4: 0.2} if case == "few_tokens" else cfg.mix
     base = case.split("_")[0] if case.endswith("bit") else case
     N, K = (11008, 4096) if base in ("codec", "errors", "backward_gate") else (4096, 4096)
     M = 4096 if base in ("forward4096", "backward_gate") else 2048
@@ -1049,6 +1049,13 @@ def run_case(case: str) -> None:
             lw.lowra_learn_codebooks(layout, W, y0, t0, LLOYD_ITERS)
         torch.cuda.synchronize()
         print("learn ok")
+        return
+    if base == "learn_all":
+        y0, t0 = si.initial_codebooks()
+        for _ in range(3):
+            lw.lowra_channel_errors(W, *lw.lowra_learn_codebooks_all(W, y0, t0, 2))
+        torch.cuda.synchronize()
+        print("learn_all ok")
         return
     if base == "errors":
         sse = torch.empty(N, dtype=torch.float64, device="cuda")
@@ -1067,6 +1074,22 @@ def run_case(case: str) -> None:
             lw.lowra_encode(layout, W, thr_d, packed=packed, absmax=absmax)
         torch.cuda.synchronize()
         print("codec ok")
+        return
+    if base == "few_tokens":
+        sizes = [4, 30, 9, 17, 25, 16]
+        n, M = len(sizes), sum(sizes)
+        layout.build_deal()
+        X = torch.randn(M, K, device="cuda", generator=gen).bfloat16()
+        A = (torch.randn(n, K, r, device="cuda", generator=gen) * 0.01).bfloat16()
+        B = (torch.randn(n, r, N, device="cuda", generator=gen) * 0.01).bfloat16()
+        ws = lw.lowra_workspace_init(torch.empty(lw.lowra_batch_workspace_bytes(layout, 4, M, r), dtype=torch.uint8, device="cuda"))
+        for _ in range(3):
+            lw.lowra_lora_forward(layout, packed, absmax, maps_d, X[:1], A[0], B[0], s, workspace=ws)
+            lw.lowra_lora_forward_adapters(layout, packed, absmax, maps_d.expand(n, N, 16).contiguous(), X, [0, *np.cumsum(sizes)], A, B, s, workspace=ws)
+        status = lw.lowra_device_status(ws)
+        print("few_tokens status", status)
+        if status != 0:
+            raise SystemExit(1)
         return
     fwd = base in ("forward", "forward4096")
     act = torch.randn(M, K if fwd else N, device="cuda", generator=gen).bfloat16()

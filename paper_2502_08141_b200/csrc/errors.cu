@@ -14,12 +14,12 @@
 // additions in fp32: 3 * 2^-24 more), typically far closer.
 //
 // Traffic: 4 bytes per element read (+ 4 written with the residual), streamed as row_stream.cuh says: a lane works on half an absmax block at a
-// time.  At 1 and 2 bits the two or four values w_hat are formed once per half block and picked by comparison; at 4 bits
+// time.  At 1 and 2 bits the two or four values w_hat are formed once per half block, and every one is subtracted under its own condition; at 4 bits
 // a branch-free binary search finds the level.  The residual is written over the weights in shared memory and leaves in one bulk copy
 // per chunk.
-// What bounds it: memory at 1 and 2 bits (5120 x 5120 at 85/15 % with the residual 37 us, 85 % of the copy rate; without it 19.8), instruction
-// issue at 4 bits and for all three precisions at once (48 instructions an element in 73 % of the slots; 4096 x 4096: 21.6 -> 19.6 us with conditional
-// additions and subtractions instead of selections, and what comes in pairs in packed instructions; 31.6 -> 28.4, a value normalised once for all).
+// What bounds it: memory at 1 and 2 bits (5120 x 5120 at 85/15 % with the residual 36.8 us, 87 % of the copy rate; without it 19.5), instruction
+// issue at 4 bits and for all three precisions at once (45 instructions an element in 74 % of the slots; 4096 x 4096: 20.4 -> 18.5 us with conditional
+// additions and subtractions instead of selections, and what comes in pairs in packed instructions; 30.9 -> 27.6, a value normalised once for all).
 #include "row_stream.cuh"
 
 namespace lowra {
@@ -85,7 +85,7 @@ __device__ __forceinline__ float2 normalised(float a, float b, float inv) {
 }
 
 // Error of four neighbouring elements: four squares in fp32, then into the fp64 sum.  PACKED: without residuals to keep, where instructions bound the kernel (three
-// precisions 31 -> 28.4 us on 4096 x 4096); residuals next to one another for both purposes cost moves (at 4 bits 24.4 -> 28.1).
+// precisions on 4096 x 4096); residuals next to one another for both purposes cost moves (at 4 bits 24.4 -> 28.1).
 template <bool PACKED>
 __device__ __forceinline__ double four_squares(const float (&r)[4]) {
     if (!PACKED) return (double)__fadd_rn(__fmaf_rn(r[0], r[0], __fmul_rn(r[1], r[1])), __fmaf_rn(r[2], r[2], __fmul_rn(r[3], r[3])));

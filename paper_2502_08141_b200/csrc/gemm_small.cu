@@ -3,7 +3,7 @@
 // With a handful of tokens the work is reading the weight's codes once (1 - 2 bits per weight), a few microseconds of memory
 // time: what counts is how many SMs share it and how long the longest chain of dependent steps is.  The persistent
 // tensor-core kernel (gemm_fused.cu) has tiles of 256 channels and 256 tokens, of which a 4096 x 4096 weight is 16: cut in four, their
-// slices handed over, it takes 26 us for 1 token as for 65.  Here two launches share the work finely instead (1 token 9.1, 16 tokens 11.0):
+// slices handed over, it takes 26 us for 1 token as for 65.  Here two launches share the work finely instead (1 token 8.9, 16 tokens 10.7):
 //   project_kernel   T = bf16(s X A): a CTA per 16 tokens and slice of the contraction, the slices of a cluster added up
 //                    through distributed shared memory.
 //   small_kernel     a CTA takes 64 stored rows of one precision and a slice of the contraction, its warps 16 rows and half

@@ -71,7 +71,7 @@ __device__ __forceinline__ void warp_sums(long long (&v)[NV], int lane) {
 }
 
 // ---------------------------------------------------------------------------------------------------------------------------------
-// The arithmetic of both kernels.  A bucket's sums of w and of w * n are formed on a grid, so that they do not depend on the order
+// The arithmetic of all kernels.  A bucket's sums of w and of w * n are formed on a grid, so that they do not depend on the order
 // of the additions: results are reproducible, and the same whichever kernel takes the row.  Let the row's largest weight be below
 // 2^e.  fp64 numbers from 64 * 2^e to 128 * 2^e are multiples of u = 2^(e - 46), and adding to g = 96 * 2^e takes w (to nearest) and w * n
 // (down) to that grid: s + w * n, one fused multiply-add rounding down, is s plus w * n taken down, whatever s is, so that a
@@ -815,12 +815,13 @@ __global__ void __launch_bounds__(THREADS, CTAS) sorted_learn_kernel(const __gri
 // ---------------------------------------------------------------------------------------------------------------------------------
 // Rounds on blocks in order.  A lane takes one absmax block (of short rows a half or a quarter), so that all its values have one weight and order is a matter
 // of its registers alone: a sorting network, no atomics, no scattered stores (the order of a whole row costs 24 shared-memory wavefronts for 32
-// elements, below).  The values lie in shared memory as [place][lane], with the sums of w * n before every fourth place; a lane finds a threshold's
+// elements, above).  The values lie in shared memory as [place][lane], with the sums of w * n before every fourth place; a lane finds a threshold's
 // place in its block by bisection, every look-up free of bank conflicts, adds the few values of the last four below it, and the warp's sums are
 // added up by a halving exchange.  The same sums on the same grid as in the other kernels, hence the same tables bit for bit.
 // What bounds it: instruction issue (60 to 73 % of the slots, with the 16 warps that an SM's shared memory takes): 2400 instructions a warp until the first
-// round, 1360 of them in the network, then 62 for a threshold and 150 for a round.  Measured, 4096 x 4096, T = 10: 82 -> 58 us at
-// 60/35/5 % of 1/2/4 bits (72 -> 48 at 1 bit, 89 -> 58 at 2); three precisions, T = 2: 67.7 -> 56.8.
+// round, 1360 of them in the network, then 62 for a threshold and 150 for a round.  Against rounds through
+// the row and the whole row's order, 4096 x 4096, T = 10: 80 -> 57 us at 60/35/5 % of 1/2/4 bits (70 -> 45 at 1 bit, 86 -> 56 at 2); three precisions, T = 2: 65.5 -> 54.1.
+// Rows with one block 10^6 times heavier, nearly every bucket of which is added up again (fine_mean_ordered): 81 us, 121 with every block walked through for every bucket.
 // Not taken: two blocks a lane in turn (49 -> 55 us at 1 bit, T = 10: half the warps); rows one after the other in a persistent grid, the next one's load
 // in flight (66: five rows to an SM instead of eight); halves of blocks (a fifth less network, but every threshold twice: 61 -> 70 at 2 bits).
 //

@@ -2,7 +2,7 @@
 // tensor checks, the outputs' and the scratch's memory and the call itself without an interpreted line between them; and the tensor checks of the other calls.
 // A call for few tokens is one or two launches of 2.5 us each and 5 to 9 us on the GPU; with every check, pointer and argument handled by the interpreter
 // its host side took 12 to 14 us.  Host time of the others (256 x 512, 128 tokens, rank 48), us: a batch of three 16.3 -> 5.2, gradients 17.3 -> 8.6, from kept
-// projections 13.5 -> 6.4, such a projection's view 5.2 -> 1.6; a training step of three weights 138 -> 66.
+// projections 13.5 -> 6.4, such a projection's view 5.2 -> 1.6; a training step of three weights 135 -> 66.
 //
 // forward / backward_input(layout address, its device, packed, absmax, maps, act, A, B, s, out or None, workspace or None) returns the output,
 // a status that is not LOWRA_OK, or None for everything that is not the ordinary case - other types, memory of other devices than the

@@ -1,7 +1,7 @@
 """The learner with many rows: blocks in order for several rounds, three kernels in one call, and what each kernel's slow ways must not lose or cost.
 
 Which kernel takes a row depends on the number of rows.  With 1200 of them (nine to an SM)
-  all precisions and 4 bits   go by the blocks' order in the first round; in later ones where the tables in kernel_for say so (2048, 4096, 6144 values: to the second or third)
+  all precisions and 4 bits   go by the blocks' order in the first round; in later ones where the tables in kernel_for say so (2048, 4096, 6144 values: to the second or third at least)
   2 bits                      from the second round on; 1 bit: 1152 to 2048 values from the third, 4096 from the fourth
 while a call of 148 of them takes 4-bit rows of 1152 to 6144 values through the whole row's order and the others through the row in every round.  One fixed-point grid: the same
 tables bit for bit.
