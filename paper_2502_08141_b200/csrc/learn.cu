@@ -13,7 +13,6 @@
 // them, a block per lane.  sorted_learn_kernel brings the whole row into order, after which a round takes a few hundred of its values.  The more
 // thresholds and rounds, the more order pays (kernel_for).
 #include <float.h>
-#include <limits.h>
 #include <math.h>
 #include <string.h>
 
@@ -1234,15 +1233,16 @@ bool two_long_rows(int K) { return 2 * (sorted_smem_bytes(K) + 1024) <= 228 * 10
 // A few rows to an SM (per_sm) wait for the longest chain, and a warp's network is longer than the eight warps' way to the order of a whole row, or, of 2048 values
 // at 1 and 2 bits, than rounds through the row.  Ordered against sorted, us, at 4 bits, one round / two: 296 rows of 1152 8.0 6.1 / 9.6 7.1, of 2048 8.1 6.6 / 9.6 8.2, of
 // 4096 8.6 8.1; 1600 rows of 2048 12.0 16.3.  Rows that leave most of their last warp without a block (1152, 2176 values) gain little from it with any number.  Of 1794 calls for
-// each column (23 lengths, 40 to 4096 rows) the choice is 0.3 % behind the better kernel in the mean, 18 % at most (at 2 bits 0.6, at 1 bit 1.7).
+// each column (23 lengths, 40 to 4096 rows) the choice is 0.8 % (4 bits), 1.7 (all, 1 bit) and 0.6 (2 bits) behind the better kernel in the mean: where the two are close, the order of
+// whole rows is left out, for rows of few values, crowded in one cell, take it up to three times as long (296 pruned rows of 8192, two rounds 17.0 46.2).
 enum Kernel { kRowAgain, kOrdered, kSorted };
 int ordered_warps(int K) { return (K + 2047) / 2048; }
 // Rows of up to `up_to` values: by their whole order from round `few` on with up to `rows` of them to an SM, from round `many` on with more.
 struct SortedFrom { int up_to, rows, few, many; };
-constexpr SortedFrom kFour[] = {{512, 8, 2, 2}, {1024, 8, 3, 3}, {1536, 6, 1, 2}, {2048, 5, 1, 4}, {2560, 0, 1, 1}, {3072, 2, 1, 3}, {4096, 2, 1, 5}, {5120, 4, 2, 3},
-                                {6144, 2, 2, 10}, {8192, 2, 2, 6}, {10240, 2, 3, 4}, {11776, 0, 4, 4}, {kSortedMaxK, 1, 4, 10}};
-constexpr SortedFrom kAll[] = {{512, 8, INT_MAX, 2}, {1024, 8, 10, 4}, {1536, 6, 1, 2}, {2048, 5, 1, 4}, {2560, 0, 1, 1}, {3072, 3, 1, 2}, {4096, 2, 1, 3}, {5120, 2, 1, 2},
-                               {6144, 2, 1, 4}, {8192, 2, 2, 4}, {10240, 2, 2, 3}, {11776, 0, 3, 3}, {kSortedMaxK, 1, 3, 6}};
+constexpr SortedFrom kFour[] = {{512, 8, 2, 2}, {1024, 8, 3, 3}, {1536, 6, 1, 2}, {2048, 5, 1, 4}, {2560, 2, 1, 2}, {3072, 2, 1, 3}, {4096, 2, 2, 5}, {5120, 4, 2, 3},
+                                {6144, 2, 2, 10}, {8192, 0, 7, 7}, {11776, 0, 4, 4}, {kSortedMaxK, 0, 9, 9}};
+constexpr SortedFrom kAll[] = {{512, 8, 2, 2}, {1024, 8, 4, 4}, {1536, 6, 1, 2}, {2048, 5, 1, 4}, {2560, 2, 1, 2}, {3072, 3, 1, 2}, {4096, 2, 2, 3}, {5120, 2, 2, 2},
+                               {6144, 2, 2, 4}, {8192, 0, 4, 4}, {10240, 2, 2, 3}, {11776, 0, 3, 3}, {kSortedMaxK, 0, 5, 5}};
 Kernel kernel_for(int K, int c, int iterations, int rows) {
     if (K > kSortedMaxK || iterations < 1) return kRowAgain;
     const int per_sm = (rows + kNumSMs - 1) / kNumSMs;
@@ -1252,14 +1252,14 @@ Kernel kernel_for(int K, int c, int iterations, int rows) {
         return pays ? kOrdered : kRowAgain;
     }
     if (c == 1) {
-        const bool idle = per_sm <= 2;
-        const int from = K <= 1024 ? 1 : K <= 2048 ? (per_sm <= 4 ? 4 : 2) : K <= 3072 && idle ? 4 : (K <= 6144 && idle) || (K > 8192 && K <= 12288) ? 3 : 2;
+        const int from = K <= 1024 ? 1 : K <= 2048 ? (per_sm <= 4 ? 4 : 2) : K <= 3072 && per_sm <= 2 ? 4 : K > 8192 && K <= 12288 ? 3 : 2;
         return iterations >= from ? kOrdered : kRowAgain;
     }
     const SortedFrom* line = c == 2 ? kFour : kAll;
     while (K > line->up_to) ++line;
-    // (five rows of two warps leave one scheduler more to do than another; in the order of whole rows an SM has five at a time)
-    const int many = K > 2560 && K <= 4096 && (per_sm == 5 || (K <= 3072 && per_sm == 6)) ? 2 : line->many;
+    // (In the order of whole rows an SM has five at a time; and in company - encoded or assessed right behind - up to five rows of two warps each crowd on the SMs that the kernel
+    // before leaves first: 400 x 3072 of 4 bits, two rounds and encode 17.7 us, by the whole rows' order 15.3.)
+    const int many = K > 2560 && K <= 4096 && (per_sm <= 5 || (K <= 3072 && per_sm == 6)) ? 2 : line->many;
     return iterations >= (per_sm <= line->rows ? line->few : many) ? kSorted : kOrdered;
 }
 
@@ -1316,14 +1316,8 @@ lowra_status launch_learn(LearnParams& P, const double* init_levels_host, const 
     Kernel kernel[3];
     for (int c = 0; c < 3; ++c) kernel[c] = kernel_for(P.K, ALL3 ? 3 : c, P.iterations, P.N);
     if (!ALL3 && 2 * n4 <= P.N && P.K > 1024) kernel[2] = four_in_company(P.K, P.iterations, P.N, n4);
-    // One launch fewer counts for more than the rows' kernel where these are few (535 x 2048 at 60/35/5, T = 4 11.7 -> 10.2 us): the blocks' order for the 1-bit rows as well
-    // or, for two rounds of no more 2-bit rows than of 1 bit, none for the 2-bit rows (740 x 2176 at 50/50 9.5 -> 8.4 us, 888 x 4224 at 85/15 14.2 -> 11.1) unless the 4-bit rows
-    // go by it.
-    if (!ALL3 && per_sm <= 8 && kernel[0] == kRowAgain && kernel[1] == kOrdered && n1 > 0 && n2 > 0) {
-        const bool row = P.iterations == 2 && n1 >= n2 && (n4 == 0 || kernel[2] != kOrdered) &&
-                         ((P.K <= 3072 && per_sm <= 6) || (P.K > 4096 && P.K <= 6144 && per_sm >= 6 && n1 >= 2 * n2));
-        (row ? kernel[1] : kernel[0]) = row ? kRowAgain : kOrdered;
-    }
+    // (one launch fewer counts for more than the rows' kernel where these are few: 535 x 2048 at 60/35/5, T = 4 11.7 -> 10.2 us)
+    if (!ALL3 && per_sm <= 8 && kernel[0] == kRowAgain && kernel[1] == kOrdered && n1 > 0 && n2 > 0) kernel[0] = kOrdered;
     // Stored rows are in the order of their precisions, and more bits want more order: a launch for every kernel that has classes, the last classes' first
     // (in turns; see enter()).
     const int n[3] = {n1, n2, n4};

@@ -3,7 +3,8 @@
 Which kernel takes a row depends on the number of rows.  With 1200 of them (nine to an SM)
   all precisions and 4 bits   go by the blocks' order in the first round; in later ones where the tables in kernel_for say so (2048, 4096, 6144 values: to the second or third at least)
   2 bits                      from the second round on; 1 bit: 1152 to 2048 values from the third, 4096 from the fourth
-while a call of 148 of them takes 4-bit rows of 1152 to 6144 values through the whole row's order and the others through the row in every round.  One fixed-point grid: the same
+while a call of 148 of them takes 4-bit rows of 1152 to 6144 values through the whole row's order (above 3072 values from the second round on) and most of the others through the row in
+every round.  One fixed-point grid: the same
 tables bit for bit.
 """
 import numpy as np
@@ -80,8 +81,7 @@ def test_three_kernels_in_one_call():
 
 @pytest.mark.parametrize("K", [1024, 4096, 8192, 11008])
 def test_weights_below_the_grid_in_the_whole_rows_order(K):
-    """Buckets whose elements all lie in blocks 2^-60 to 2^-100 as heavy as the row's heaviest, for ten rounds: both forms bring the whole row into order (1024 to 8192 values; of
-    11008 the three-precision form), and both agree with the oracle."""
+    """Buckets whose elements all lie in blocks 2^-60 to 2^-100 as heavy as the row's heaviest, for ten rounds: both forms bring the whole row into order, and both agree with the oracle."""
     import paper_2502_08141_b200 as lw
 
     rng = np.random.default_rng(K + 2)
